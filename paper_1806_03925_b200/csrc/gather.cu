@@ -52,8 +52,10 @@ template <int N> __device__ __forceinline__ void store_x(__nv_bfloat16* dst, con
     else *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
 }
 
-// x / n for a small positive integer n held as nf, with rinv = 1 / nf: the product x * rinv corrected by one
-// exact residual step, which yields the correctly rounded quotient (infinities and NaNs pass through).
+// x / n for a small positive integer n held as nf, with rinv = 1 / nf rounded to nearest: the product x * rinv corrected
+// by one exact residual step (Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", IBM
+// J. Res. Dev. 34 (1990), theorem on the final step of a division: with a correctly rounded reciprocal the corrected
+// quotient is the correctly rounded one).  Infinities and NaNs pass through.
 __device__ __forceinline__ float div_by_count(float x, float nf, float rinv) {
     const float q = x * rinv;
     const float q2 = fmaf(fmaf(-q, nf, x), rinv, q);
