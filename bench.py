@@ -48,8 +48,8 @@ def measured_peaks():
     return dict(hbm_gbs=6650.0, bf16_tflops=1590.0, bf16_sustained=1400.0, source="fallback")
 
 
-# fp32 FMA peak of the plain-ALU head: 148 SMs x 128 lanes x 2 flop x max SM clock
-ALU_F32_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
+# an fp32 product of an fp32 head is six bf16 tensor-core products
+F32_PRODUCTS = 6
 
 
 class ClockSampler:
@@ -204,17 +204,16 @@ def roofline_for(name, ms_per_launch, p, stats, peaks):
         return {"kernel": name, "bound": "hbm", "achieved": round(ach, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": round(ach / peaks["hbm_gbs"], 4), "traffic": traffic, "traffic_source": source,
                 "peak_source": peaks["source"], "work_per_launch": work}
-    if name.startswith("simt_gemm") or name.startswith("tc_gemm"):
+    if name.startswith(("tc_gemm", "tc3_gemm")):
         # The head's products are dense contractions: rated by their flops against the tensor peak (bf16 heads; the
-        # sustained figure, since they run inside a long step) or the fp32 FMA peak (fp32 heads).  memory_frac is
+        # sustained figure, since they run inside a long step; a sixth of it for fp32 heads).  memory_frac is
         # the secondary figure: every operand and the output once, over the measured copy rate.
         flops, nbytes = models["gemm"][name.rsplit("_", 1)[1]]
-        if name.startswith("tc_gemm"):
-            peak, bound, src = peaks["bf16_sustained"] or peaks["bf16_tflops"], "tensor", peaks["source"] + " (sustained bf16)"
-        else:
-            peak, bound, src = ALU_F32_TFLOPS, "alu", "148 SMs x 128 FMA lanes x 2 x 1.965 GHz"
+        peak, bound, src = peaks["bf16_sustained"] or peaks["bf16_tflops"], "tensor", peaks["source"] + " (sustained bf16)"
+        if name.startswith("tc3_gemm"):
+            peak, src = peak / F32_PRODUCTS, src + " / %d" % F32_PRODUCTS
         ach = flops / sec / 1e12
-        traffic, source = ncu_traffic(name, p, None) if bound == "tensor" else (None, "fp32 head: no capture")
+        traffic, source = ncu_traffic(name, p, None)
         return {"kernel": name, "bound": bound, "achieved": round(ach, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
                 "frac": round(ach / peak, 4), "traffic": traffic, "traffic_source": source,
                 "peak_source": src, "work_per_launch": flops, "memory_frac": round(nbytes / sec / 1e9 / peaks["hbm_gbs"], 4)}
@@ -231,11 +230,11 @@ def step_roofline(p, stats, ms_per_step, peaks):
     fan = [p.d_in] + list(p.hidden)
     flops = 6.0 * stats["B"] * (sum(fan[l] * fan[l + 1] for l in range(len(p.hidden))) + fan[-1])
     sec = ms_per_step * 1e-3
-    tensor_peak = (peaks["bf16_sustained"] or peaks["bf16_tflops"]) if p.head_dtype == "bf16" else ALU_F32_TFLOPS
+    tensor_peak = (peaks["bf16_sustained"] or peaks["bf16_tflops"]) / (1 if p.head_dtype == "bf16" else F32_PRODUCTS)
     return {"bytes_per_step": round(nbytes), "flops_per_step": round(flops),
             "hbm_GB/s": round(nbytes / sec / 1e9, 1), "hbm_frac": round(nbytes / sec / 1e9 / peaks["hbm_gbs"], 4),
             "math_TFLOP/s": round(flops / sec / 1e12, 2), "math_frac": round(flops / sec / 1e12 / tensor_peak, 4),
-            "math_peak": round(tensor_peak, 1), "math_bound": "tensor" if p.head_dtype == "bf16" else "alu",
+            "math_peak": round(tensor_peak, 1), "math_bound": "tensor",
             "lower_bound_ms": round(max(nbytes / (peaks["hbm_gbs"] * 1e9), flops / (tensor_peak * 1e12)) * 1e3, 4),
             "peak_source": peaks["source"]}
 
@@ -490,7 +489,7 @@ def run_ours(args):
     roof = None
     for kd in kernels:
         r = roofline_for(kd["name"], kd["ms_per_launch"], p, stats, peaks)
-        if r["bound"] in ("hbm", "tensor", "alu"):
+        if r["bound"] in ("hbm", "tensor"):
             roof = r
             roof["share_of_step"] = round(kd["share"], 4)
             break
@@ -530,7 +529,7 @@ def run_ours(args):
             "roofline": roof,
             "roofline_step": step_roofline(p, stats, ms / K, peaks),
             "products": [roofline_for(k["name"], k["ms_per_launch"], p, stats, peaks) for k in kernels
-                         if k["name"].startswith(("tc_gemm", "simt_gemm"))],
+                         if k["name"].startswith(("tc_gemm", "tc3_gemm"))],
             "kernels": [{"name": k["name"], "ms_per_step": round(k["ms_per_step"], 4), "share": round(k["share"], 4),
                          "launches_per_step": round(k["launches_per_step"], 2)} for k in kernels],
             "hbm_kernels": hbm_kernels,

@@ -47,11 +47,17 @@ static int validate_config(const gear_config& c) {
     return GEAR_OK;
 }
 
+static int64_t param_count(const gear_config& c) {
+    int64_t n = 0, fan = 2 * c.emb_dim + c.dfv_dim + c.fast_dim;
+    for (int l = 0; l < c.n_hidden; ++l) { n += fan * c.hidden[l] + c.hidden[l]; fan = c.hidden[l]; }
+    return n + fan + 1;
+}
+
 int plan_workspace(const gear_config& c, WsPlan* p) {
     memset(p, 0, sizeof(*p));
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t at = off; off = align_up(off + bytes, 256); return at; };
-    const size_t hsz = c.head_dtype == GEAR_BF16 ? 2 : 4;
+    const size_t hsz = c.head_dtype == GEAR_BF16 ? 2 : 6;      // three bf16 planes per fp32 value
     const int d_in = 2 * c.emb_dim + c.dfv_dim + c.fast_dim;
     const size_t B = (size_t)c.max_batch;
     p->ready_cap = c.ready_cap > 0 ? c.ready_cap : c.max_nnz;
@@ -64,13 +70,13 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
     for (int l = 0; l < c.n_hidden; ++l) {
         p->h[l] = take(B * c.hidden[l] * hsz);
         p->da[l] = take(B * c.hidden[l] * hsz);
-        p->wb[l] = take((size_t)fan * c.hidden[l] * 2);
-        p->wbt[l] = take((size_t)fan * c.hidden[l] * 2);
+        p->wb[l] = take((size_t)fan * c.hidden[l] * hsz);
+        p->wbt[l] = take((size_t)fan * c.hidden[l] * hsz);
         fan = c.hidden[l];
     }
     p->dz = take(B * 4);
     p->loss_part = take((size_t)p->loss_blocks * 4);
-    p->colsum_part = take((size_t)CS_BLOCKS * 1024 * 4);
+    if (c.head_dtype == GEAR_F32) p->head_grad = take((size_t)param_count(c) * 4);
     p->sort_n[0] = p->sort_n[1] = c.max_batch;
     p->sort_n[2] = c.max_nnz;
     p->sort_n[3] = p->ready_cap;
@@ -97,12 +103,6 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
     return GEAR_OK;
 }
 
-static int64_t param_count(const gear_config& c) {
-    int64_t n = 0, fan = 2 * c.emb_dim + c.dfv_dim + c.fast_dim;
-    for (int l = 0; l < c.n_hidden; ++l) { n += fan * c.hidden[l] + c.hidden[l]; fan = c.hidden[l]; }
-    return n + fan + 1;
-}
-
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 // the ctx's side stream and fork/join events (host-side driver objects, no device memory)
@@ -113,6 +113,8 @@ static void release_host_objects(gear_ctx_impl& c) {
     if (c.ev_dx) cudaEventDestroy(c.ev_dx);
     c.ev_dx = nullptr;
     if (c.side_stream) cudaStreamDestroy(c.side_stream);
+    delete_tma_cache(c.tma);
+    c.tma = nullptr;
     c.ev_fork = c.ev_join = c.ev_gather = nullptr;
     c.side_stream = nullptr;
 }
@@ -167,7 +169,8 @@ int gear_init_tables(gear_ctx** out_ctx, const gear_config* cfg, const gear_buff
     c.d_in = 2 * cfg->emb_dim + cfg->dfv_dim + cfg->fast_dim;
     c.n_params = param_count(*cfg);
     c.alive = true;
-    c.tc_state = nullptr;
+    c.tma = new_tma_cache();
+    if (!c.tma) { delete ctx; return arg_fail("out of host memory"); }
     c.gbs.device_counter = &c.state()->grid_barrier;
     c.gbs.host_base = 0;
     c.img_sorted = false;
@@ -270,11 +273,10 @@ int gear_forward_backward(gear_ctx* ctx, const gear_batch* batch, float lr, cons
         if (e != cudaSuccess) return cuda_fail(e, "fork");
         join_pending = true;
     }
-    // bf16 copies of the head's weights: first on the caller's stream, ahead of the gather.  The gather keeps every SM
-    // busy for its whole duration, so a small kernel on another stream would get its blocks placed only when the gather
-    // ends, and the first product of the head would wait for it.
-    const bool weights_early = b.B > 0 && c.cfg.head_dtype == GEAR_BF16;
-    if (weights_early) {
+    // The weights in the form the head's products read: first on the caller's stream, ahead of the gather.  The gather keeps
+    // every SM busy for its whole duration, so a small kernel on another stream would get its blocks placed only when the
+    // gather ends, and the first product of the head would wait for it.
+    if (b.B > 0) {
         e = launch_round_weights(c, st);
         if (e != cudaSuccess) return abandon(e, "weight copies");
     }
@@ -336,8 +338,8 @@ int gear_forward_backward(gear_ctx* ctx, const gear_batch* batch, float lr, cons
                                    k.o->url_m, k.o->url_v, where);
         return launch_emb_reduce(c, k.sorted_buf, k.B, ut, ht, k.o->dX, c.d_in, alpha, where);
     };
-    const HeadHooks hooks{weights_early, scatter, &sc};
-    e = launch_head_simt(c, b, o, st, hooks);
+    const HeadHooks hooks{scatter, &sc};
+    e = launch_head(c, b, o, st, hooks);
     if (e != cudaSuccess) return abandon(e, "head");
     if (o.dfv_grad && b.B > 0) {
         e = launch_dfv_grad_rows(c, o.dX, o.row_view, o.inv_n, b.nnz, o.dfv_grad, st);

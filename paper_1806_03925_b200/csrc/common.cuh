@@ -100,6 +100,20 @@ __device__ __forceinline__ float4 ld_stream_f4(const float* p) {
     return v;
 }
 
+// An fp32 matrix held as three bf16 matrices `stride` elements apart, whose sum it is (head_tc3.cu)
+struct Planes { __nv_bfloat16* p; int64_t stride; };
+
+// two fp32 values as three packed pairs of bf16 (each part rounded to nearest; the three parts of a value sum to it)
+__device__ __forceinline__ void split3_pair(float x, float y, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
+    const __nv_bfloat162 h0 = __floats2bfloat162_rn(x, y);
+    p0 = *reinterpret_cast<const uint32_t*>(&h0);
+    const float rx = x - __uint_as_float(p0 << 16), ry = y - __uint_as_float(p0 & 0xffff0000u);
+    const __nv_bfloat162 h1 = __floats2bfloat162_rn(rx, ry);
+    p1 = *reinterpret_cast<const uint32_t*>(&h1);
+    const __nv_bfloat162 h2 = __floats2bfloat162_rn(rx - __uint_as_float(p1 << 16), ry - __uint_as_float(p1 & 0xffff0000u));
+    p2 = *reinterpret_cast<const uint32_t*>(&h2);
+}
+
 // vector reduction: *p += v without a return value (sm_90+)
 __device__ __forceinline__ void red_add_f4(float* p, float4 v) {
     asm volatile("red.global.add.v4.f32 [%0], {%1,%2,%3,%4};"

@@ -37,19 +37,31 @@ template <> struct Chunk<__nv_bfloat16> {
     }
 };
 
-template <int N> __device__ __forceinline__ void store_x(float* dst, const float* v) {
-#pragma unroll
-    for (int k = 0; k < N; k += 4) st_f4(dst + k, make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]));
-}
-template <int N> __device__ __forceinline__ void store_x(__nv_bfloat16* dst, const float* v) {
-    uint32_t w[N / 2];
+// N (4 or 8) values of a row of the head input at X + off: rounded to bf16 (HB: bf16 heads) or as three bf16 planes,
+// `stride` apart; and, if asked for, a copy of them at xd + off, in bf16 or fp32.
+template <bool HB, int N> __device__ __forceinline__ void store_x(__nv_bfloat16* X, int64_t stride, void* xd, int64_t off, const float* v) {
+    constexpr int PLANES = HB ? 1 : 3;
+    uint32_t w[3][N / 2];
 #pragma unroll
     for (int k = 0; k < N / 2; ++k) {
-        __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
-        w[k] = *reinterpret_cast<uint32_t*>(&h);
+        if constexpr (HB) {
+            __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
+            w[0][k] = *reinterpret_cast<uint32_t*>(&h);
+        } else split3_pair(v[2 * k], v[2 * k + 1], w[0][k], w[1][k], w[2][k]);
     }
-    if constexpr (N == 8) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
-    else *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
+    auto put = [&](__nv_bfloat16* dst, const uint32_t* q) {
+        if constexpr (N == 8) *reinterpret_cast<uint4*>(dst) = make_uint4(q[0], q[1], q[2], q[3]);
+        else *reinterpret_cast<uint2*>(dst) = make_uint2(q[0], q[1]);
+    };
+#pragma unroll
+    for (int p = 0; p < PLANES; ++p) put(X + p * stride + off, w[p]);
+    if (xd) {
+        if constexpr (HB) put(static_cast<__nv_bfloat16*>(xd) + off, w[0]);
+        else {
+#pragma unroll
+            for (int k = 0; k < N; k += 4) st_f4(static_cast<float*>(xd) + off + k, make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]));
+        }
+    }
 }
 
 // x / n for a small positive integer n held as nf, with rinv = 1 / nf rounded to nearest: the product x * rinv corrected
@@ -69,7 +81,7 @@ struct GatherArgs {
     const float* fast;          // [B][F] the views' own dense input (F > 0)
     int64_t nnz;
     const int32_t* user_id; const int32_t* url_id; const int32_t* img_off; const int32_t* img_id;
-    void* X; void* x_debug;
+    __nv_bfloat16* X; int64_t x_stride; void* x_debug;      // X: bf16, or three planes x_stride apart
     int32_t* row_view; float* inv_n;
     DevState* state;
 };
@@ -133,7 +145,7 @@ __device__ __forceinline__ ViewRec load_view(const GatherArgs& a, int b) {
 // and keeps two stages of look-ahead in registers: the record of the view after next and the image IDs of
 // the next view are requested before the current view's rows are summed, so that per view only one memory
 // round trip (the rows themselves) is exposed.
-template <typename TD, typename TX, int NQ, bool FULL>
+template <typename TD, bool HB, int NQ, bool FULL>
 __global__ void __launch_bounds__(GP_WARPS * 32, NQ <= 2 ? 3 : 2)
 gather_pool_kernel(const GatherArgs a) {
     wait_for_predecessor();
@@ -161,8 +173,7 @@ gather_pool_kernel(const GatherArgs a) {
         const int ids_nxt = load_ids(nxt, 0);
         const ViewRec nxt2 = load_view(a, b + 2 * W);
 
-        TX* __restrict__ x = static_cast<TX*>(a.X) + (int64_t)b * Din;
-        TX* __restrict__ xd = a.x_debug ? static_cast<TX*>(a.x_debug) + (int64_t)b * Din : nullptr;
+        const int64_t x0 = (int64_t)b * Din;
         int uid = cur.uid, hid = cur.hid, s = cur.s, n = cur.n;
         if (uid < 0 || uid >= a.user_vocab) { uid = -1; flags |= GEAR_DEV_BAD_ID; }
         if (hid < 0 || hid >= a.url_vocab) { hid = -1; flags |= GEAR_DEV_BAD_ID; }
@@ -226,8 +237,7 @@ gather_pool_kernel(const GatherArgs a) {
         // ---- write the row of X
         if (lane < 2 * ce) {
             const float f[4] = {emb.x, emb.y, emb.z, emb.w};
-            store_x<4>(x + lane * 4, f);
-            if (xd) store_x<4>(xd + lane * 4, f);
+            store_x<HB, 4>(a.X, a.x_stride, a.x_debug, x0 + lane * 4, f);
         }
         for (int c = 32 + lane; c < 2 * ce; c += 32) {             // embedding rows wider than 32 chunks in total
             const bool is_url = c >= ce;
@@ -236,8 +246,7 @@ gather_pool_kernel(const GatherArgs a) {
             float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
             if (id >= 0) t = __ldg(reinterpret_cast<const float4*>(table + (int64_t)id * a.E + (is_url ? c - ce : c) * 4));
             const float f[4] = {t.x, t.y, t.z, t.w};
-            store_x<4>(x + c * 4, f);
-            if (xd) store_x<4>(xd + c * 4, f);
+            store_x<HB, 4>(a.X, a.x_stride, a.x_debug, x0 + c * 4, f);
         }
         const float nf = (float)n, rinv = n > 0 ? 1.0f / nf : 0.f;
 #pragma unroll
@@ -247,8 +256,7 @@ gather_pool_kernel(const GatherArgs a) {
                 float o[PER];
 #pragma unroll
                 for (int k = 0; k < PER; ++k) o[k] = n > 0 ? div_by_count(acc[q][k], nf, rinv) : 0.f;
-                store_x<PER>(x + 2 * a.E + ch * PER, o);
-                if (xd) store_x<PER>(xd + 2 * a.E + ch * PER, o);
+                store_x<HB, PER>(a.X, a.x_stride, a.x_debug, x0 + 2 * a.E + ch * PER, o);
             }
         }
         if (a.inv_n && lane == 0) a.inv_n[b] = rinv;
@@ -256,8 +264,7 @@ gather_pool_kernel(const GatherArgs a) {
         for (int c = lane * 8; c < a.F; c += 256) {
             const float4 f0 = ld_stream_f4(a.fast + (int64_t)b * a.F + c), f1 = ld_stream_f4(a.fast + (int64_t)b * a.F + c + 4);
             const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-            store_x<8>(x + 2 * a.E + a.D + c, f);
-            if (xd) store_x<8>(xd + 2 * a.E + a.D + c, f);
+            store_x<HB, 8>(a.X, a.x_stride, a.x_debug, x0 + 2 * a.E + a.D + c, f);
         }
 
         cur = nxt; nxt = nxt2; ids_cur = ids_nxt;
@@ -265,7 +272,7 @@ gather_pool_kernel(const GatherArgs a) {
     if (flags) atomicOr(&a.state->status, flags);
 }
 
-template <typename TD, typename TX>
+template <typename TD, bool HB>
 static cudaError_t dispatch_nq(const GatherArgs& a, cudaStream_t st, Profiler* prof) {
     constexpr int PER = Chunk<TD>::PER;
     const int n_chunks = a.D / PER;
@@ -277,8 +284,8 @@ static cudaError_t dispatch_nq(const GatherArgs& a, cudaStream_t st, Profiler* p
     // FULL only when a row fills the instantiated width exactly (n_chunks == NQ * 32): every lane then owns a chunk of
     // every DFV row; widths that round up to the next instantiation (3, 5, 6, 7 chunks per lane) keep the guard
 #define GEAR_GATHER(NQ) do { \
-        if (n_chunks == NQ * 32) launch_dependent(gather_pool_kernel<TD, TX, NQ, true>, dim3(grid), dim3(GP_WARPS * 32), 0, st, a); \
-        else launch_dependent(gather_pool_kernel<TD, TX, NQ, false>, dim3(grid), dim3(GP_WARPS * 32), 0, st, a); } while (0)
+        if (n_chunks == NQ * 32) launch_dependent(gather_pool_kernel<TD, HB, NQ, true>, dim3(grid), dim3(GP_WARPS * 32), 0, st, a); \
+        else launch_dependent(gather_pool_kernel<TD, HB, NQ, false>, dim3(grid), dim3(GP_WARPS * 32), 0, st, a); } while (0)
     if (nq <= 1) GEAR_GATHER(1);
     else if (nq <= 2) GEAR_GATHER(2);
     else if (nq <= 4) GEAR_GATHER(4);
@@ -295,13 +302,13 @@ cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* 
     a.user_vocab = c.cfg.user_vocab; a.url_vocab = c.cfg.url_vocab; a.img_vocab = c.cfg.img_vocab;
     a.E = c.cfg.emb_dim; a.D = c.cfg.dfv_dim; a.B = b.B; a.nnz = b.nnz; a.F = c.cfg.fast_dim; a.fast = b.fast;
     a.user_id = b.user_id; a.url_id = b.url_id; a.img_off = b.img_off; a.img_id = b.img_id;
-    a.X = c.at<void>(c.ws.x); a.x_debug = x_debug; a.row_view = row_view; a.inv_n = inv_n;
+    a.X = c.at<__nv_bfloat16>(c.ws.x); a.x_stride = (int64_t)c.cfg.max_batch * c.d_in; a.x_debug = x_debug; a.row_view = row_view; a.inv_n = inv_n;
     a.state = c.state();
     const bool dbf = c.cfg.dfv_dtype == GEAR_BF16, xbf = c.cfg.head_dtype == GEAR_BF16;
-    if (dbf && xbf) return dispatch_nq<__nv_bfloat16, __nv_bfloat16>(a, st, &c.prof);
-    if (dbf && !xbf) return dispatch_nq<__nv_bfloat16, float>(a, st, &c.prof);
-    if (!dbf && xbf) return dispatch_nq<float, __nv_bfloat16>(a, st, &c.prof);
-    return dispatch_nq<float, float>(a, st, &c.prof);
+    if (dbf && xbf) return dispatch_nq<__nv_bfloat16, true>(a, st, &c.prof);
+    if (dbf && !xbf) return dispatch_nq<__nv_bfloat16, false>(a, st, &c.prof);
+    if (!dbf && xbf) return dispatch_nq<float, true>(a, st, &c.prof);
+    return dispatch_nq<float, false>(a, st, &c.prof);
 }
 
 }  // namespace gear

@@ -23,22 +23,19 @@
 //                                                as a TMA reduction: the copy engine adds it to the matrix)
 // No cluster launch and no multicast.  Every wait is bounded: on a timeout the kernel records an error
 // code, leaves its loops, frees its tensor memory and returns.
-#include <cuda.h>
-
-#include <mutex>
+#include <new>
 
 #include "common.cuh"
 #include "internal.h"
+#include "tc_ptx.cuh"
 
 namespace gear {
 
-constexpr int TC_BM = 128;
 constexpr int TC_BK = 64;                 // 64 bf16 = 128 bytes = one swizzle row
 // Epilogue warps per CTA (a multiple of four: each warp reaches one quarter of the tensor-memory lanes).
 constexpr int tc_threads(int ew) { return 64 + 32 * ew; }
 constexpr int TC_MAX_N = 1024;            // widest output the column-sum partials cover
 constexpr int TC_MASK_BLOCK = 32 * 64;    // a warp's ReLU-mask block for 32 columns: 32 rows of 64 bytes (two per warp)
-constexpr uint32_t TC_SPIN_LIMIT = 1u << 22;
 
 enum { TC_EPI_BIAS_RELU = 0, TC_EPI_MASK = 1, TC_EPI_F32 = 2, TC_EPI_RED = 3 };
 
@@ -70,132 +67,6 @@ struct TcArgs {
     float* colsum;            // ReLU-mask epilogue: colsum[n] += sum over rows of the stored output (may be null)
     int32_t* err;             // device word that receives a non-zero code on a timeout
 };
-
-// ---------------------------------------------------------------- PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count));
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" :: "r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
-}
-// Arrival that orders nothing but the barrier itself: the epilogue hands its accumulator buffer back with this one,
-// so that the hand-over does not wait for the tile's global stores to drain (tensor-memory reads are complete by
-// then: tcgen05.wait::ld, then tcgen05.fence::before_thread_sync).
-__device__ __forceinline__ void mbar_arrive_relaxed(uint32_t bar) {
-    asm volatile("mbarrier.arrive.relaxed.cta.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
-}
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-                 "selp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-// Bounded wait.  Returns false (and records `code`) if the phase never completed.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* err, int code) {
-    for (uint32_t i = 0; i < TC_SPIN_LIMIT; ++i) {
-        if (mbar_try(bar, parity)) return true;
-        if (i > 64) __nanosleep(32);
-        if ((i & 1023u) == 1023u && *reinterpret_cast<volatile int32_t*>(err) != 0) return false;
-    }
-    atomicCAS(err, 0, code);
-    return false;
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
-    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-                 :: "r"(dst), "l"(map), "r"(bar), "r"(x), "r"(y) : "memory");
-}
-
-// Store of a shared-memory box (128-byte swizzle) into the output matrix; parts of the box past the matrix edge are
-// dropped by the copy engine.  Bulk groups belong to the issuing thread: the same lane commits and waits.
-__device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];"
-                 :: "l"(map), "r"(src), "r"(x), "r"(y) : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-// The same with an L2 eviction policy for the lines written.
-__device__ __forceinline__ void tma_store_2d_hint(const CUtensorMap* map, uint32_t src, int x, int y, uint64_t policy) {
-    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%2, %3}], [%1], %4;"
-                 :: "l"(map), "r"(src), "r"(x), "r"(y), "l"(policy) : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-// The same box added to the matrix instead of stored (fp32 adds by the copy engine, whole rows of the box at a time).
-__device__ __forceinline__ void tma_reduce_add_2d(const CUtensorMap* map, uint32_t src, int x, int y) {
-    asm volatile("cp.reduce.async.bulk.tensor.2d.global.shared::cta.add.tile.bulk_group [%0, {%2, %3}], [%1];"
-                 :: "l"(map), "r"(src), "r"(x), "r"(y) : "memory");
-    asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-template <int PENDING>
-__device__ __forceinline__ void tma_store_wait_read() {
-    asm volatile("cp.async.bulk.wait_group.read %0;" :: "n"(PENDING) : "memory");
-}
-__device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void sts_u4(uint32_t addr, const uint4& v) {
-    asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" :: "r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" :: "r"(bar) : "memory");
-}
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate) {
-    asm volatile("{\n\t.reg .pred p;\n\t"
-                 "setp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 :: "r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
-}
-__device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-                 "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(taddr) : "memory");
-}
-// Waits for the tensor-memory reads issued so far.  The registers are passed through so that no use of
-// them can be scheduled ahead of the wait.
-__device__ __forceinline__ void tc_wait_ld(uint32_t (&r)[32]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
-                   "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
-                   "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-                 :: "memory");
-}
-
-__device__ __forceinline__ float4 ldg_f4(const float* p) { return __ldg(reinterpret_cast<const float4*>(p)); }
-__device__ __forceinline__ uint4 ldg_u4(const void* p) { return __ldg(reinterpret_cast<const uint4*>(p)); }
-
-// Shared-memory matrix descriptor, 128-byte swizzle, sm_100 format (version 1).
-//   K-major operand : rows of 128 bytes, 8-row groups 1024 bytes apart (SBO); LBO unused.
-//   MN-major operand: 64-element (128-byte) slabs along M/N, `lbo` bytes apart; 8-deep K groups 1024 bytes apart.
-__device__ __forceinline__ uint64_t smem_desc(uint32_t addr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3ffffu) >> 4);
-    d |= (uint64_t)((lbo_bytes >> 4) & 0x3fffu) << 16;
-    d |= (uint64_t)((sbo_bytes >> 4) & 0x3fffu) << 32;
-    d |= (uint64_t)1 << 46;            // descriptor version
-    d |= (uint64_t)2 << 61;            // SWIZZLE_128B
-    return d;
-}
-
-// Instruction descriptor: bf16 x bf16 -> fp32, M = 128, N = BN.
-__host__ __device__ constexpr uint32_t instr_desc(int bn, bool mn_major) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((mn_major ? 1u : 0u) << 15) | ((mn_major ? 1u : 0u) << 16) |
-           ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
-}
 
 // Epilogue of one finished accumulator buffer `a`, as run by one of the epilogue warps: warp w reads
 // tensor-memory lanes 32 * (w % 4) .. + 31 (its rows of the tile); the EW / 4 warps of a lane quarter split the
@@ -557,99 +428,50 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 static EncodeTiledFn encode_fn() {
-    static EncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static EncodeTiledFn fn = [] {
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return reinterpret_cast<EncodeTiledFn>(p);
+    }();
     return fn;
 }
 
-// A step encodes the same eighteen maps every time (operands and outputs live at fixed places in the workspace): a
-// small table of the most recent encodings saves the driver calls.  A map depends on the key alone.
-struct MapKey { const void* ptr; int64_t rows, cols, ld; int box_rows, f32; };
-struct MapCache {
-    static constexpr int N = 64;
-    std::mutex mu;
-    MapKey key[N];
-    CUtensorMap map[N];
-    int used = 0, next = 0;
-    bool find(const MapKey& k, CUtensorMap* out) {
-        std::lock_guard<std::mutex> lock(mu);
-        for (int i = 0; i < used; ++i)
-            if (key[i].ptr == k.ptr && key[i].rows == k.rows && key[i].cols == k.cols && key[i].ld == k.ld &&
-                key[i].box_rows == k.box_rows && key[i].f32 == k.f32) { *out = map[i]; return true; }
+bool TmaCache::get(CUtensorMap* out, const TmaSpec& k) {
+    for (int i = 0; i < used_; ++i)
+        if (key_[i] == k) { *out = map_[i]; return true; }
+    EncodeTiledFn fn = encode_fn();
+    if (!fn) return false;
+    const cuuint64_t esz = k.f32 ? 4 : 2;
+    cuuint64_t dims[3] = {(cuuint64_t)k.cols, (cuuint64_t)k.rows, (cuuint64_t)k.planes};
+    cuuint64_t strides[2] = {(cuuint64_t)k.ld * esz, (cuuint64_t)k.plane_stride * esz};
+    cuuint32_t box[3] = {(cuuint32_t)k.box_cols, (cuuint32_t)k.box_rows, (cuuint32_t)k.planes};
+    cuuint32_t estr[3] = {1, 1, 1};
+    if (fn(out, k.f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, k.planes > 1 ? 3 : 2,
+           const_cast<void*>(k.ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+           k.swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return false;
-    }
-    void put(const MapKey& k, const CUtensorMap& m) {
-        std::lock_guard<std::mutex> lock(mu);
-        const int i = used < N ? used++ : (next = (next + 1) % N);
-        key[i] = k; map[i] = m;
-    }
-};
-static MapCache g_maps;
-
-static bool make_map_f32(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows);
-static bool encode_bf16(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows);
-
-// bf16 matrix [rows][cols] with leading dimension ld (elements); box = box_rows x 64 columns, 128-byte swizzle.
-// Out-of-range parts of a box read as zero.
-static bool make_map(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-    const MapKey k{ptr, rows, cols, ld, box_rows, 0};
-    if (g_maps.find(k, m)) return true;
-    if (!encode_bf16(m, ptr, rows, cols, ld, box_rows)) return false;
-    g_maps.put(k, *m);
-    return true;
-}
-static bool encode_bf16(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// fp32 matrix [rows][cols] with leading dimension ld (elements); box = box_rows x 32 columns, 128-byte swizzle.
-static bool make_map_f32(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
-    const MapKey k{ptr, rows, cols, ld, box_rows, 1};
-    if (g_maps.find(k, m)) return true;
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
-    cuuint32_t box[2] = {32, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    if (fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return false;
-    g_maps.put(k, *m);
+    const int i = used_ < N ? used_++ : (next_ = (next_ + 1) % N);
+    key_[i] = k; map_[i] = *out;
     return true;
 }
 
-// bf16 matrix [rows][cols] read in boxes of 32 rows x 32 columns (64 bytes a row), 64-byte swizzle: the ReLU mask.
-static bool make_map_mask(CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld) {
-    const MapKey k{ptr, rows, cols, ld, 32, 2};
-    if (g_maps.find(k, m)) return true;
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-    cuuint32_t box[2] = {32, 32};
-    cuuint32_t estr[2] = {1, 1};
-    if (fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-           CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return false;
-    g_maps.put(k, *m);
-    return true;
+TmaCache* new_tma_cache() { return new (std::nothrow) TmaCache; }
+void delete_tma_cache(TmaCache* t) { delete t; }
+
+// bf16 matrix in boxes of box_rows x 64 columns; fp32 matrix in boxes of 32 x 32 (both 128 bytes a row); the ReLU mask, a
+// bf16 matrix in boxes of 32 x 32 (64 bytes a row)
+static bool make_map(const gear_ctx_impl& c, CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
+    return c.tma->get(m, TmaSpec{ptr, rows, cols, ld, 0, 1, box_rows, 64, 0, 128});
+}
+static bool make_map_f32(const gear_ctx_impl& c, CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld) {
+    return c.tma->get(m, TmaSpec{ptr, rows, cols, ld, 0, 1, 32, 32, 1, 128});
+}
+static bool make_map_mask(const gear_ctx_impl& c, CUtensorMap* m, const void* ptr, int64_t rows, int64_t cols, int64_t ld) {
+    return c.tma->get(m, TmaSpec{ptr, rows, cols, ld, 0, 1, 32, 32, 0, 64});
 }
 
 template <int BN, bool MN, int EPI, int EW>
@@ -676,30 +498,30 @@ static cudaError_t launch_bn(int bn, const CUtensorMap& ma, const CUtensorMap& m
                      : launch_variant<128, MN, EPI, EW>(ma, mb, mo, mm, g, st);
 }
 
-cudaError_t tc_gemm_kmajor(Profiler* prof, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
+cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
                            const __nv_bfloat16* W, int64_t ldw, int epi, void* out, int64_t ldo, const float* bias,
-                           const __nv_bfloat16* mask, int64_t ldm, float* colsum, int32_t* err, cudaStream_t st) {
+                           const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     // column tiles of 256 or 128; the fp32 output (dX) also has 192, which fits a width like 384 without a half-empty tile
     int bn = N > 128 ? 256 : 128;
     if (epi == TC_EPI_F32 && N > 128 && ceil_div(N, 192) * 192 < ceil_div(N, 256) * 256) bn = 192;
     CUtensorMap ma, mb, mo;
-    if (!make_map(&ma, A, M, K, lda, TC_BM) || !make_map(&mb, W, N, K, ldw, bn)) return cudaErrorInvalidValue;
+    if (!make_map(c, &ma, A, M, K, lda, TC_BM) || !make_map(c, &mb, W, N, K, ldw, bn)) return cudaErrorInvalidValue;
     // the output leaves in boxes of 32 rows x 128 bytes
-    if (!(epi == TC_EPI_F32 ? make_map_f32(&mo, out, M, N, ldo, 32) : make_map(&mo, out, M, N, ldo, 32))) return cudaErrorInvalidValue;
+    if (!(epi == TC_EPI_F32 ? make_map_f32(c, &mo, out, M, N, ldo) : make_map(c, &mo, out, M, N, ldo, 32))) return cudaErrorInvalidValue;
     TcArgs g;
     g.M = M; g.N = N; g.K = K;
     g.m_tiles = (int)ceil_div(M, TC_BM); g.n_tiles = (int)ceil_div(N, bn); g.k_splits = 1;
     g.kb_per_split = (int)ceil_div(K, TC_BK);
-    g.out = out; g.ldo = ldo; g.bias = bias; g.mask = mask; g.ldm = ldm; g.err = err;
+    g.out = out; g.ldo = ldo; g.bias = bias; g.mask = mask; g.ldm = ldm; g.err = &c.state()->tc_error;
     g.colsum = (epi == TC_EPI_MASK && N <= TC_MAX_N) ? colsum : nullptr;
     if (epi == TC_EPI_MASK && colsum != nullptr && g.colsum == nullptr) return cudaErrorInvalidValue;
-    KernelScope ks(prof, name, st);
+    KernelScope ks(&c.prof, name, st);
     switch (epi) {
     case TC_EPI_BIAS_RELU: return launch_bn<false, TC_EPI_BIAS_RELU>(bn, ma, mb, mo, ma /*unused*/, g, st);
     case TC_EPI_MASK: {
         CUtensorMap mm;
-        if (!mask || !make_map_mask(&mm, mask, M, N, ldm)) return cudaErrorInvalidValue;
+        if (!mask || !make_map_mask(c, &mm, mask, M, N, ldm)) return cudaErrorInvalidValue;
         return launch_bn<false, TC_EPI_MASK>(bn, ma, mb, mo, mm, g, st);
     }
     default:
@@ -708,13 +530,13 @@ cudaError_t tc_gemm_kmajor(Profiler* prof, const char* name, int M, int N, int K
     }
 }
 
-cudaError_t tc_gemm_mnmajor(Profiler* prof, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
-                            const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo, int32_t* err,
+cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
+                            const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo,
                             cudaStream_t st) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     const int bn = N > 128 ? 256 : 128;
     CUtensorMap ma, mb, mo;
-    if (!make_map(&ma, A, K, M, lda, 64) || !make_map(&mb, Bm, K, N, ldb, 64) || !make_map_f32(&mo, out, M, N, ldo, 32))
+    if (!make_map(c, &ma, A, K, M, lda, 64) || !make_map(c, &mb, Bm, K, N, ldb, 64) || !make_map_f32(c, &mo, out, M, N, ldo))
         return cudaErrorInvalidValue;
     TcArgs g;
     g.M = M; g.N = N; g.K = K;
@@ -726,8 +548,8 @@ cudaError_t tc_gemm_mnmajor(Profiler* prof, const char* name, int M, int N, int 
     if (splits < 1) splits = 1;
     g.kb_per_split = (int)ceil_div(total_kb, splits);
     g.k_splits = (int)ceil_div(total_kb, g.kb_per_split);
-    g.out = out; g.ldo = ldo; g.bias = nullptr; g.mask = nullptr; g.ldm = 0; g.colsum = nullptr; g.err = err;
-    KernelScope ks(prof, name, st);
+    g.out = out; g.ldo = ldo; g.bias = nullptr; g.mask = nullptr; g.ldm = 0; g.colsum = nullptr; g.err = &c.state()->tc_error;
+    KernelScope ks(&c.prof, name, st);
     return launch_bn<true, TC_EPI_RED>(bn, ma, mb, mo, ma /*unused*/, g, st);
 }
 

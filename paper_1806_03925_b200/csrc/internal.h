@@ -13,19 +13,19 @@ namespace gear {
 constexpr int EXP_TILE = 8192;     // entries of the timestamp table per block of the expiry scan's write pass
 constexpr int EXP_MARK_TILE = 2048; // ... and per block (and per count) of its mark pass
 constexpr int MAX_LAYERS = 2;
-constexpr int CS_BLOCKS = 296;      // blocks of the column-sum kernel (two per SM)
 
 // Byte offsets into the caller's workspace.  Everything is 256-byte aligned.
 struct WsPlan {
     size_t state;                       // DevState
-    size_t x;                           // [max_batch][d_in]      head dtype: head input
-    size_t h[MAX_LAYERS];               // [max_batch][hidden[l]] head dtype: post-ReLU activations
-    size_t da[MAX_LAYERS];              // [max_batch][hidden[l]] head dtype: gradient at the pre-activation
+    // the head's matrices: bf16 (bf16 heads) or three bf16 planes of an fp32 matrix, one behind the other (fp32 heads)
+    size_t x;                           // [max_batch][d_in]      head input
+    size_t h[MAX_LAYERS];               // [max_batch][hidden[l]] post-ReLU activations
+    size_t da[MAX_LAYERS];              // [max_batch][hidden[l]] gradient at the pre-activation
     size_t dz;                          // [max_batch] fp32
     size_t loss_part;                   // [loss_blocks] fp32 per-block partial losses
-    size_t colsum_part;                 // [CS_BLOCKS][1024] fp32 per-block partial column sums
-    size_t wb[MAX_LAYERS];              // bf16 head: W_l as [in][out]
-    size_t wbt[MAX_LAYERS];             // bf16 head: W_l as [out][in]
+    size_t head_grad;                   // fp32 head: the parameters' gradient, when the caller's array is not 16-byte aligned
+    size_t wb[MAX_LAYERS];              // W_l as [in][out]
+    size_t wbt[MAX_LAYERS];             // W_l as [out][in]
     // four sets of sort buffers: user IDs, URL IDs (max_batch each), image IDs (max_nnz), ready queue (ready_cap)
     size_t sort_keys[4][2], sort_vals[4][2];
     size_t sort_hist[4], sort_tot[4];
@@ -48,6 +48,10 @@ struct WsPlan {
 
 int plan_workspace(const gear_config& c, WsPlan* p);
 
+class TmaCache;
+TmaCache* new_tma_cache();
+void delete_tma_cache(TmaCache* t);
+
 struct gear_ctx_impl {
     gear_config cfg;
     gear_buffers buf;
@@ -66,7 +70,7 @@ struct gear_ctx_impl {
         else { cudaStreamSynchronize(seen_stream[0]); seen_stream[0] = st; }     // a fifth stream: retire the oldest
     }
     bool alive;
-    void* tc_state;     // tensor-core head state (tensor maps), owned by head_tc.cu; may be null
+    TmaCache* tma;      // tensor maps of the head's products (tc_ptx.cuh)
     cudaStream_t side_stream;          // runs the ID sort of a step beside the gather and the head
     cudaEvent_t ev_fork, ev_join;
     mutable Profiler prof;
@@ -117,22 +121,28 @@ cudaError_t launch_fill_ts(int64_t* ts, int64_t n, uint64_t seed, int64_t expire
 cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* row_view, float* inv_n,
                           void* x_debug, cudaStream_t st);
 
-// head_simt.cu: forward + backward of the head (fp32 FMA products, or the tensor-core products of head_tc.cu).
-// weights_ready: the bf16 copies of the weights have been made already (launch_round_weights earlier on the same stream).  after_dx(arg) is called once dX has been enqueued, before the last weight-gradient product.
-struct HeadHooks { bool weights_ready; cudaError_t (*after_dx)(void*); void* arg; };
-cudaError_t launch_head_simt(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o, cudaStream_t st,
-                             const HeadHooks& hooks);
+// head.cu: forward + backward of the head.  The weights' copies must have been made earlier on the same stream
+// (launch_round_weights).  after_dx(arg) is called once dX has been enqueued, before the last weight-gradient product.
+struct HeadHooks { cudaError_t (*after_dx)(void*); void* arg; };
+cudaError_t launch_head(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o, cudaStream_t st, const HeadHooks& hooks);
 cudaError_t launch_round_weights(const gear_ctx_impl& c, cudaStream_t st);
 
 // head_tc.cu: bf16 products on tcgen05 tensor cores.  epi: 0 bias+ReLU -> bf16, 1 ReLU mask -> bf16, 2 plain fp32.
 // colsum (epi 1 only, may be null): colsum[n] += sum over the rows of the stored (rounded) output.
-cudaError_t tc_gemm_kmajor(Profiler* prof, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
+cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
                            const __nv_bfloat16* W, int64_t ldw, int epi, void* out, int64_t ldo, const float* bias,
-                           const __nv_bfloat16* mask, int64_t ldm, float* colsum, int32_t* err, cudaStream_t st);
+                           const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st);
 // out[M][N] (fp32) += A[K][M]^T . Bm[K][N]
-cudaError_t tc_gemm_mnmajor(Profiler* prof, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
-                            const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo, int32_t* err,
-                            cudaStream_t st);
+cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
+                            const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo, cudaStream_t st);
+
+// head_tc3.cu: the same products of fp32 matrices held as three bf16 planes.  epi 0 and 1 write planes, 2 plain fp32; the mask
+// is the leading plane of the activations.
+cudaError_t tc3_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,
+                            const Planes& W, int64_t ldw, int epi, const Planes& out_planes, float* out_f32, int64_t ldo,
+                            const float* bias, const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st);
+cudaError_t tc3_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,
+                             const Planes& Bm, int64_t ldb, float* out, int64_t ldo, cudaStream_t st);
 
 // emb_scatter.cu
 // table[id] += alpha * (sum of the dX rows of the views with that id) for the user and the URL-hash table, given the

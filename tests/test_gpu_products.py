@@ -1,0 +1,31 @@
+"""fp32 head on the tensor cores (three bf16 planes per matrix) at the edges of its tiles, against the oracle at the fp32
+tolerance (1e-5 of the largest value of a tensor)."""
+import pytest
+import torch
+
+from paper_1806_03925_b200.workloads import F32, PRESETS, BatchSource
+
+pytestmark = pytest.mark.gpu
+
+
+# row tiles are 128 views, column tiles 64 or 128 wide, the reduction goes in steps of 32 and is cut into segments of 256
+# terms from 544 on; weight gradients reduce over the batch
+@pytest.mark.parametrize("B,E,D,hidden", [
+    (1, 4, 8, (8,)),                        # one view, narrowest layers: one tile, most of it past the edge
+    (127, 12, 40, (64,)), (129, 12, 48, (72, 8)),          # one row short of / past a tile; 64 and 72 columns
+    (256, 16, 480, (136, 120)),             # head input 512 wide: two segments' worth in one, columns one step past 128
+    (640, 16, 512, (128, 64)),              # head input 544 wide: the first width that is cut into segments
+    (20_000, 4, 24, (1024,)),               # widest layer, a long reduction over the batch
+])
+def test_fp32_products_at_tile_edges(B, E, D, hidden):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from gpu_harness import Pair
+    p = PRESETS["skew"].scaled(emb_dim=E, dfv_dim=D, dfv_dtype=F32, head_dtype=F32, hidden=hidden, M=3, user_vocab=3000,
+                               url_vocab=2000, img_vocab=4000, expire=2)
+    batch = BatchSource(p, B).batch(0, B)
+    pair = Pair(p, [batch], seed=1, want_emb_grad=True)
+    try:
+        pair.step_and_compare(batch, now=1)
+    finally:
+        pair.close()
