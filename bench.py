@@ -204,7 +204,7 @@ def roofline_for(name, ms_per_launch, p, stats, peaks):
         return {"kernel": name, "bound": "hbm", "achieved": round(ach, 1), "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": round(ach / peaks["hbm_gbs"], 4), "traffic": traffic, "traffic_source": source,
                 "peak_source": peaks["source"], "work_per_launch": work}
-    if name.startswith(("tc_gemm", "tc3_gemm")):
+    if name.startswith(("tc_gemm", "tc3_gemm", "f32_gemm")):
         # The head's products are dense contractions: rated by their flops against the tensor peak (bf16 heads; the
         # sustained figure, since they run inside a long step; a sixth of it for fp32 heads).  memory_frac is
         # the secondary figure: every operand and the output once, over the measured copy rate.
@@ -529,7 +529,7 @@ def run_ours(args):
             "roofline": roof,
             "roofline_step": step_roofline(p, stats, ms / K, peaks),
             "products": [roofline_for(k["name"], k["ms_per_launch"], p, stats, peaks) for k in kernels
-                         if k["name"].startswith(("tc_gemm", "tc3_gemm"))],
+                         if k["name"].startswith(("tc_gemm", "tc3_gemm", "f32_gemm"))],
             "kernels": [{"name": k["name"], "ms_per_step": round(k["ms_per_step"], 4), "share": round(k["share"], 4),
                          "launches_per_step": round(k["launches_per_step"], 2)} for k in kernels],
             "hbm_kernels": hbm_kernels,

@@ -18,6 +18,7 @@
  *   gear_collect_ready        event 6: hand over the averaged gradient of
  *                             every completed group.
  *   gear_accumulate_collect   events 5 and 6 as one call.
+ *   gear_step                 events 1 to 6 and the expiry scan as one call.
  *   gear_refresh_dfv          Section 1 / Section 3: recomputed DFVs replace
  *                             expired ones and restart their clocks.
  *   gear_dense_forward /      events 2-3 and the second half of event 6 for a
@@ -44,6 +45,8 @@
  *     GEAR_DEV_BAD_ID bit of the device status word.
  *   - Calls on one ctx must be issued from one host thread at a time and on
  *     one stream (or on streams the caller orders with events).
+ *   - A call whose kernels and streams are the same as before (a training loop's) is replayed as a CUDA graph with the new
+ *     batch's pointers and sizes; a stream that its owner is capturing gets the kernels one by one.
  */
 #ifndef GEAR_H
 #define GEAR_H
@@ -253,6 +256,24 @@ int gear_accumulate_collect(gear_ctx* ctx, const int32_t* img_id, const float* g
  */
 int gear_collect_expired(gear_ctx* ctx, int64_t now, int restamp, int32_t* ids, int64_t cap,
                          int64_t* d_n, int64_t* h_n, void* stream);
+
+/*
+ * One whole step in one call: the same results as gear_forward_backward, then gear_accumulate_collect with
+ * (NULL, dX + 2 * emb_dim, d_in, row_view, inv_n, nnz) and gear_collect_expired, with the lists and counts of `lists`.
+ * What does not depend on one another runs side by side; the host pays for one call.  out->row_view and out->inv_n are
+ * required.  scan_beside != 0: the expiry scan runs beside the training kernels, else behind them.  h_n (host, [2],
+ * optional): the two counts, with one wait for both; GEAR_ERR_CAPACITY if a list was too small (see the calls named).
+ */
+typedef struct {
+    int32_t* ids; int32_t* seq; float* avg;     /* averages handed over: [cap], [cap], [cap][dfv_dim] */
+    int64_t  cap;
+    int64_t* d_n;                               /* device count, optional */
+    int32_t* expired;                           /* expired images: [expired_cap] */
+    int64_t  expired_cap;
+    int64_t* d_expired;                         /* device count, optional */
+} gear_step_lists;
+int gear_step(gear_ctx* ctx, const gear_batch* batch, float lr, const gear_step_out* out, const gear_step_lists* lists,
+              int64_t now, int restamp, int scan_beside, int64_t* h_n, void* stream);
 
 /*
  * Refresh of cached inference results (Section 1, second point; Section 3: a Dense Feature Vector whose cached

@@ -27,7 +27,7 @@ EXPORTS = ("gear_workspace_bytes", "gear_init_tables", "gear_forward_backward", 
            "gear_collect_ready", "gear_collect_expired", "gear_status", "gear_destroy", "gear_fill_uniform",
            "gear_last_error", "gear_profile_enable", "gear_profile_read", "gear_launch_count",
            "gear_collect_expired_static", "gear_refresh_dfv", "gear_accumulate_collect", "gear_dense_forward",
-           "gear_dense_backward", "gear_adam_dense", "gear_fetch_rows", "gear_apply_emb_grad", "gear_profile_timeline")
+           "gear_dense_backward", "gear_adam_dense", "gear_fetch_rows", "gear_apply_emb_grad", "gear_profile_timeline", "gear_step")
 GEAR_STATIC_EXPIRY_MAX_VOCAB = 16777216
 
 
@@ -68,6 +68,11 @@ class gear_step_out(C.Structure):
                 ("user_m", C.c_void_p), ("user_v", C.c_void_p), ("url_m", C.c_void_p), ("url_v", C.c_void_p)]
 
 
+class gear_step_lists(C.Structure):
+    _fields_ = [("ids", C.c_void_p), ("seq", C.c_void_p), ("avg", C.c_void_p), ("cap", C.c_int64), ("d_n", C.c_void_p),
+                ("expired", C.c_void_p), ("expired_cap", C.c_int64), ("d_expired", C.c_void_p)]
+
+
 _lib = None
 
 
@@ -94,6 +99,9 @@ def load() -> C.CDLL:
     L.gear_collect_ready.argtypes = [vp, vp, vp, vp, i64, vp, C.POINTER(i64), vp]
     L.gear_accumulate_collect.restype = C.c_int
     L.gear_accumulate_collect.argtypes = [vp, vp, vp, i64, vp, vp, i64, vp, vp, vp, i64, vp, C.POINTER(i64), vp]
+    L.gear_step.restype = C.c_int
+    L.gear_step.argtypes = [vp, C.POINTER(gear_batch), C.c_float, C.POINTER(gear_step_out), C.POINTER(gear_step_lists), i64, C.c_int,
+                            C.c_int, C.POINTER(i64), vp]
     L.gear_fetch_rows.restype = C.c_int
     L.gear_fetch_rows.argtypes = [vp, i32, vp, i64, vp, vp]
     L.gear_apply_emb_grad.restype = C.c_int
@@ -147,9 +155,14 @@ def _p(t: Optional[torch.Tensor]):
     return C.c_void_p(t.data_ptr())
 
 
+def _raw_stream(stream: Optional[torch.cuda.Stream]) -> int:
+    """The cudaStream_t of a stream (None: the current one of the current device; asked for as a plain number, which is a
+    tenth of the cost of building a torch.cuda.Stream object)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()) if stream is None else stream.cuda_stream
+
+
 def _stream(stream: Optional[torch.cuda.Stream]):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    return C.c_void_p(_raw_stream(stream))
 
 
 def make_config(user_vocab, url_vocab, img_vocab, emb_dim, dfv_dim, dfv_dtype, head_dtype, hidden, M, expire,
@@ -266,6 +279,24 @@ def gear_accumulate_collect(ctx, img_id, grads_ptr: int, ld: int, src_row, scale
                                           _p(ids), _p(seq), _p(avg), cap, _p(d_n), C.byref(h) if sync else None,
                                           _stream(stream)), "gear_accumulate_collect")
     return h.value if sync else None
+
+
+def make_step_lists(ids, seq, avg, cap: int, expired, expired_cap: int, d_n=None, d_expired=None) -> gear_step_lists:
+    o = gear_step_lists()
+    for name, t in (("ids", ids), ("seq", seq), ("avg", avg), ("d_n", d_n), ("expired", expired), ("d_expired", d_expired)):
+        setattr(o, name, None if t is None else _p(t).value)
+    o.cap, o.expired_cap = cap, expired_cap
+    return o
+
+
+def gear_step_structs(ctx, bt: gear_batch, lr: float, o: gear_step_out, lists: gear_step_lists, now: int, restamp: bool = True,
+                      scan_beside: bool = True, sync: bool = False, stream=None):
+    """The whole step as one call; returns (averages handed over, images listed) when sync, else (None, None)."""
+    h = (C.c_int64 * 2)() if sync else None
+    rc = (_lib or load()).gear_step(ctx, bt, lr, o, lists, now, 1 if restamp else 0, 1 if scan_beside else 0, h, _raw_stream(stream))
+    if rc != GEAR_OK:
+        _check(rc, "gear_step")
+    return (h[0], h[1]) if sync else (None, None)
 
 
 def gear_collect_expired(ctx, now: int, restamp: bool, ids, cap: int, d_n=None, sync: bool = True,

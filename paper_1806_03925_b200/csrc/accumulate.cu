@@ -15,6 +15,7 @@
 //   4. plan pass: the flags again, now with their global prefix: group g starts at grp_start[g]; complete
 //      groups get consecutive ready-queue slots (a counter-threshold stream compaction: ballot-free block
 //      scan of the "count reaches M" predicate).
+//      Arrays of at most 32768 rows are sorted and planned by one kernel instead (sort_small.cu).
 //   5. reduce pass: a warp sums the rows of each of its groups (fp32, arrival order, whole rows staged through
 //      shared memory by asynchronous copies, addressed through the sort permutation) and either writes the
 //      average to its queue slot or, for the open group, the running sum and count back to the table.  The
@@ -211,7 +212,8 @@ acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, int 
 }
 
 struct RowGather {
-    const float* grads; int64_t ld; const int2* pmeta;      // pmeta[p] = (source row, scale bits) of sorted position p
+    const float* grads; int64_t ld;
+    const int2* pmeta;             // pmeta[p] = (source row, scale bits) of sorted position p
 };
 
 // What a lane knows about "its" group of a span: own rows [start, start + len), then zlen rows from zstart.
@@ -250,15 +252,14 @@ struct ItemDesc { uint32_t addr_lo, addr_hi; float scale; int meta; };
 // FULL: a row is exactly NQ * 512 bytes, so no lane is ever idle.
 template <int NQ, int S, bool FULL>
 __global__ void __launch_bounds__(256, NQ <= 2 ? 3 : 2)
-acc_reduce_kernel(const uint32_t* __restrict__ ks, RowGather rg, int D, int M, int64_t n_tiles, int64_t ready_cap,
-                  const uint2* __restrict__ tile_cnt, const uint4* __restrict__ grp_rec,
+acc_reduce_kernel(RowGather rg, int D, int M, int64_t ready_cap, const uint2* __restrict__ plan_totals, const uint4* __restrict__ grp_rec,
                   const uint32_t* __restrict__ blk_first, const uint32_t* __restrict__ run_end,
                   float* __restrict__ gsum, int32_t* __restrict__ gcnt,
                   int32_t* __restrict__ q_id, float* __restrict__ q_avg, const EmitTarget direct,
                   DevState* __restrict__ state) {
     wait_for_predecessor();
     extern __shared__ float4 ring_mem[];                          // [warps][S][NQ * 32] float4
-    const uint2 totals = tile_cnt[n_tiles];
+    const uint2 totals = *plan_totals;
     const int64_t n_groups = totals.x;
     // Averages go to the ready queue, or (the queue being empty, so that queue slot k is also entry k of the hand-over)
     // straight into the caller's lists, whose capacity the host has checked against the row count.
@@ -496,8 +497,18 @@ cudaError_t launch_accumulate_plan_ahead(const gear_ctx_impl& c, int64_t n, cons
     SortJob sb = c.sort_job(gear_ctx_impl::SORT_IMG);
     cudaError_t e = enqueue_plan(c, sb.keys[c.img_sorted_buf], sb.vals[c.img_sorted_buf], n, src_row, scale, st);
     if (e != cudaSuccess) return e;
-    c.plan_ready = true; c.plan_n = n; c.plan_src_row = src_row; c.plan_scale = scale;
+    note_plan(c, n, src_row, scale);
     return cudaSuccess;
+}
+void note_plan(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale) {
+    c.plan_ready = true; c.plan_n = n; c.plan_src_row = src_row; c.plan_scale = scale;
+}
+PlanArgs plan_args(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale) {
+    int s = 0;
+    while (s < 31 && (1ll << s) < c.cfg.M) ++s;
+    return PlanArgs{c.at<uint2>(c.ws.tile_cnt) + ceil_div(n, AF_TILE), (uint32_t)c.cfg.img_vocab, c.cfg.M, c.buf.dfv_gcnt, c.at<uint4>(c.ws.grp_rec), src_row, scale,
+                    c.at<int2>(c.ws.pmeta), c.at<uint32_t>(c.ws.blk_first), c.at<uint32_t>(c.ws.run_end), c.state(),
+                    (uint32_t)(((1ull << (31 + s)) + c.cfg.M - 1) / c.cfg.M), 31 + s};
 }
 
 // to_caller (optional): the caller's lists; only valid while the ready queue is known to be empty and the lists hold
@@ -510,7 +521,7 @@ static cudaError_t launch_accumulate_to(const gear_ctx_impl& c, const int32_t* i
     const int D = c.cfg.dfv_dim, M = c.cfg.M;
     SortJob sb = c.sort_job(gear_ctx_impl::SORT_IMG);
     DevState* state = c.state();
-    const bool planned = !img_id && c.plan_ready && c.plan_n == n && c.plan_src_row == src_row && c.plan_scale == scale;
+    bool planned = !img_id && c.plan_ready && c.plan_n == n && c.plan_src_row == src_row && c.plan_scale == scale;
     c.plan_ready = false;
     // "the batch of the last gear_forward_backward" after a call with explicit IDs has used the sort buffers: sort again
     const bool resort_batch = !img_id && !c.img_sort_valid;
@@ -526,24 +537,23 @@ static cudaError_t launch_accumulate_to(const gear_ctx_impl& c, const int32_t* i
         batch.job[0].bits = bits_for(vocab);
         cudaError_t se;
         batch.name = "sort_img";
-        cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
+        planned = sort_small_fits(batch);
+        if (planned) { se = launch_sort_small(c, batch, plan_args(c, n, src_row, scale), st); cur = 0; }
+        else cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
         if (se != cudaSuccess) return se;
         c.img_sort_valid = resort_batch;
         if (resort_batch) c.img_sorted_buf = cur;
     }
     const uint32_t* ks = sb.keys[cur];
-    const int64_t n_tiles = ceil_div(n, AF_TILE);
-    uint2* tile_cnt = c.at<uint2>(c.ws.tile_cnt);
     if (!planned) {
         cudaError_t pe = enqueue_plan(c, ks, sb.vals[cur], n, src_row, scale, st);
         if (pe != cudaSuccess) return pe;
     }
     uint4* grp_rec = c.at<uint4>(c.ws.grp_rec);
-    int2* pmeta = c.at<int2>(c.ws.pmeta);
-    RowGather rg{grads, ld, pmeta};
+    RowGather rg{grads, ld, c.at<int2>(c.ws.pmeta)};
     uint32_t* blk_first = c.at<uint32_t>(c.ws.blk_first);
     uint32_t* run_end = c.at<uint32_t>(c.ws.run_end);
-    (void)vocab; (void)state;
+
     const int nq = (int)ceil_div(D / 4, 32);
     const int64_t want = ceil_div(ceil_div(n, ACC_SPAN), 8);
     const int resident = sm_count() * (nq <= 2 ? 3 : 2);          // every block stays resident
@@ -554,7 +564,7 @@ static cudaError_t launch_accumulate_to(const gear_ctx_impl& c, const int32_t* i
         const int smem = 8 * slots * slot_bytes;
         le = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (le != cudaSuccess) return;
-        le = launch_dependent(kernel, dim3(grid), dim3(256), (size_t)smem, st, ks, rg, D, M, n_tiles, c.ws.ready_cap, tile_cnt, grp_rec, blk_first, run_end,
+        le = launch_dependent(kernel, dim3(grid), dim3(256), (size_t)smem, st, rg, D, M, c.ws.ready_cap, c.at<uint2>(c.ws.tile_cnt) + ceil_div(n, AF_TILE), grp_rec, blk_first, run_end,
                                         c.buf.dfv_gsum, c.buf.dfv_gcnt, c.at<int32_t>(c.ws.q_id),
                                         c.at<float>(c.ws.q_avg), to_caller, state);
     };
@@ -693,7 +703,7 @@ cudaError_t launch_accumulate_atomic(const gear_ctx_impl& c, const int32_t* img_
     if (n <= 0) return cudaSuccess;
     DevState* state = c.state();
     int32_t* touched = c.at<int32_t>(c.ws.pmeta);               // the sorted path's scratch is free in this mode
-    cudaError_t e = cudaMemsetAsync(&state->pad[2], 0, sizeof(int64_t), st);
+    cudaError_t e = enqueue_memset(&state->pad[2], sizeof(int64_t), st);
     if (e != cudaSuccess) return e;
     const int64_t want = ceil_div(n, 8);
     const int resident = sm_count() * 8;

@@ -70,6 +70,7 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
     for (int l = 0; l < c.n_hidden; ++l) {
         p->h[l] = take(B * c.hidden[l] * hsz);
         p->da[l] = take(B * c.hidden[l] * hsz);
+        if (c.head_dtype == GEAR_F32) p->xf[l] = take(B * fan * 4);
         p->wb[l] = take((size_t)fan * c.hidden[l] * hsz);
         p->wbt[l] = take((size_t)fan * c.hidden[l] * hsz);
         fan = c.hidden[l];
@@ -105,18 +106,16 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// the ctx's side stream and fork/join events (host-side driver objects, no device memory)
+// the ctx's own streams and the events between them (host-side driver objects, no device memory)
 static void release_host_objects(gear_ctx_impl& c) {
-    if (c.ev_fork) cudaEventDestroy(c.ev_fork);
-    if (c.ev_join) cudaEventDestroy(c.ev_join);
-    if (c.ev_gather) cudaEventDestroy(c.ev_gather);
-    if (c.ev_dx) cudaEventDestroy(c.ev_dx);
-    c.ev_dx = nullptr;
+    for (cudaEvent_t& e : c.ev) { if (e) cudaEventDestroy(e); e = nullptr; }
     if (c.side_stream) cudaStreamDestroy(c.side_stream);
+    if (c.aux_stream) cudaStreamDestroy(c.aux_stream);
+    if (c.h_counts) cudaFreeHost(c.h_counts);
+    c.h_counts = nullptr;
     delete_tma_cache(c.tma);
     c.tma = nullptr;
-    c.ev_fork = c.ev_join = c.ev_gather = nullptr;
-    c.side_stream = nullptr;
+    c.side_stream = c.aux_stream = nullptr;
 }
 
 }  // namespace gear
@@ -124,6 +123,183 @@ static void release_host_objects(gear_ctx_impl& c) {
 using namespace gear;
 
 struct gear_ctx { gear_ctx_impl impl; };
+
+static int check_batch(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o) {
+    if (b.B < 0 || b.B > c.cfg.max_batch) return arg_fail("B outside [0, max_batch]");
+    if (b.nnz < 0 || b.nnz > c.cfg.max_nnz) return arg_fail("nnz outside [0, max_nnz]");
+    if (b.B > 0 && (!b.user_id || !b.url_id || !b.img_off || !b.label)) return arg_fail("NULL batch array");
+    if (b.nnz > 0 && !b.img_id) return arg_fail("NULL img_id");
+    if (b.B > 0 && c.cfg.fast_dim > 0 && (!b.fast || !aligned16(b.fast))) return arg_fail("fast: needed (16-byte aligned) when fast_dim > 0");
+    if (!o.loss || !o.head_grad || !o.dX) return arg_fail("loss, head_grad and dX are required outputs");
+    if ((o.user_grad == nullptr) != (o.url_grad == nullptr)) return arg_fail("user_grad and url_grad: both or neither");
+    if (o.adam) {
+        const gear_adam& a = *o.adam;
+        if (o.user_grad) return arg_fail("adam and user_grad / url_grad exclude each other");
+        if (!o.user_m || !o.user_v || !o.url_m || !o.url_v) return arg_fail("adam needs the four moment tables");
+        if (!aligned16(o.user_m) || !aligned16(o.user_v) || !aligned16(o.url_m) || !aligned16(o.url_v))
+            return arg_fail("moment tables must be 16-byte aligned");
+        if (o.adam_step < 1) return arg_fail("adam_step >= 1");
+        if (!(a.beta1 >= 0.f && a.beta1 < 1.f && a.beta2 >= 0.f && a.beta2 < 1.f && a.eps >= 0.f))
+            return arg_fail("adam: beta1, beta2 in [0, 1), eps >= 0");
+    }
+    if (c.cfg.head_dtype == GEAR_BF16 && (!aligned16(o.head_grad) || !aligned16(c.buf.head_params)))
+        return arg_fail("bf16 head: head_params and head_grad must be 16-byte aligned");
+    if (o.dfv_grad && (!o.row_view || !o.inv_n || !aligned16(o.dfv_grad)))
+        return arg_fail("dfv_grad needs row_view and inv_n and 16-byte alignment");
+    if (!aligned16(o.dX) || (o.x_debug && !aligned16(o.x_debug)) || (o.user_grad && !aligned16(o.user_grad)) ||
+        (o.url_grad && !aligned16(o.url_grad)))
+        return arg_fail("dX, x_debug, user_grad, url_grad must be 16-byte aligned");
+    return GEAR_OK;
+}
+static int check_rows(const gear_ctx_impl& c, const int32_t* img_id, const float* grads, int64_t ld, int64_t n) {
+    if (n < 0 || n > c.cfg.max_nnz) return arg_fail("n outside [0, max_nnz]");
+    if (n == 0) return GEAR_OK;
+    if (!grads) return arg_fail("NULL pointer");
+    if (!img_id && (!c.img_sorted || c.img_sorted_n != n)) {
+        snprintf(g_last_error, sizeof(g_last_error), "img_id == NULL needs a preceding gear_forward_backward whose nnz equals n");
+        return GEAR_ERR_STATE;
+    }
+    if (ld < c.cfg.dfv_dim || ld % 4 || !aligned16(grads)) return arg_fail("grads rows must be 16-byte aligned, ld >= dfv_dim");
+    return GEAR_OK;
+}
+static int check_lists(const int32_t* ids, const int32_t* seq, const float* avg, int64_t cap) {
+    if (cap < 0 || (cap > 0 && (!ids || !seq || !avg))) return arg_fail("NULL output with cap > 0");
+    if (avg && !aligned16(avg)) return arg_fail("avg must be 16-byte aligned");
+    return GEAR_OK;
+}
+
+// Events 1, 3, 4 and, where `lists` is given, 5, 6 and the expiry scan.  Written down with three streams:
+//   the caller's  weight copies, gather, the head's products in the order in which they wait for one another (dA of every
+//                 layer, dX), the accumulate call's reduce pass
+//   side          what depends on the batch's ID arrays alone: the key sort of the three ID arrays (the user and URL orders
+//                 drive the embedding scatter, the image order the accumulate call), then, once the gather has written
+//                 row_view / inv_n, the accumulate call's plan; the embedding scatter as soon as dX exists
+//   aux           the expiry scan (it depends on nothing a training call produces) and, for batches whose products leave SMs
+//                 idle, the weight gradients, which nothing but the caller waits for
+// The caller's stream waits for the other two before the call ends.  With per-kernel timing on, everything stays on the
+// caller's stream so that each kernel is timed alone.
+struct StepLists {
+    int32_t* ids; int32_t* seq; float* avg; int64_t cap; int64_t* d_n;
+    int32_t* expired; int64_t expired_cap; int64_t* d_expired;
+    int64_t now; int restamp; bool scan_beside;
+};
+static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr, const gear_step_out& o, const StepLists* lists, cudaStream_t st) {
+    c.img_sorted = false;
+    c.img_sort_valid = false;
+    c.plan_ready = false;
+    enum { EV_FORK, EV_JOIN, EV_GATHER, EV_DX, EV_PLAN, EV_AUX };
+    const bool apart = !c.prof.on || c.prof.keep_streams;
+    const bool forked = apart && b.B > 0;
+    const bool scan_beside = lists && apart && lists->scan_beside;
+    const bool sorted_mode = c.cfg.accum_mode == GEAR_ACC_SORT;
+    // weight gradients beside the other products while a product of the widest layer does not fill the GPU by itself
+    int widest = c.d_in;
+    for (int l = 0; l < c.cfg.n_hidden; ++l) widest = widest < c.cfg.hidden[l] ? c.cfg.hidden[l] : widest;
+    const bool dw_beside = forked && ceil_div(b.B, 128) * ceil_div(widest, 128) <= sm_count();
+    const cudaStream_t side = forked ? c.side_stream : st, aux = forked || scan_beside ? c.aux_stream : st;
+    cudaError_t e = cudaSuccess;
+#define GEAR_TRY(x) do { e = (x); if (e != cudaSuccess) return e; } while (0)
+    if (forked || scan_beside) {
+        GEAR_TRY(enqueue_record(c.ev[EV_FORK], st));
+        if (forked) GEAR_TRY(enqueue_wait(side, c.ev[EV_FORK]));
+        if (scan_beside) GEAR_TRY(enqueue_wait(aux, c.ev[EV_FORK]));
+    }
+    auto scan = [&](cudaStream_t where) {
+        return launch_collect_expired(c, lists->now, lists->restamp, lists->expired, lists->expired_cap, lists->d_expired, where);
+    };
+    if (scan_beside) GEAR_TRY(scan(aux));
+    // The weights in the form the head's products read: first on the caller's stream, ahead of the gather.  The gather keeps
+    // every SM busy for its whole duration, so a small kernel on another stream would get its blocks placed only when the
+    // gather ends, and the first product of the head would wait for it.
+    GEAR_TRY(launch_round_weights(c, o, st));
+    int sorted_buf = 0;
+    bool small_sort = false;
+    const bool plan = b.nnz > 0 && o.row_view && o.inv_n && sorted_mode;
+    SortBatch batch = c.sort_batch();
+    if (b.B > 0) {
+        batch.job[0] = c.sort_job(gear_ctx_impl::SORT_USER);
+        batch.job[0].ids = b.user_id; batch.job[0].sentinel = (uint32_t)c.cfg.user_vocab;
+        batch.job[0].n_max = b.B; batch.job[0].bits = bits_for(c.cfg.user_vocab);
+        batch.job[1] = c.sort_job(gear_ctx_impl::SORT_URL);
+        batch.job[1].ids = b.url_id; batch.job[1].sentinel = (uint32_t)c.cfg.url_vocab;
+        batch.job[1].n_max = b.B; batch.job[1].bits = bits_for(c.cfg.url_vocab);
+        batch.n_jobs = 2;
+        if (b.nnz > 0 && sorted_mode) {      // the atomic mode takes the image IDs as they come
+            batch.job[2] = c.sort_job(gear_ctx_impl::SORT_IMG);
+            batch.job[2].ids = b.img_id; batch.job[2].sentinel = (uint32_t)c.cfg.img_vocab;
+            batch.job[2].n_max = b.nnz; batch.job[2].bits = bits_for(c.cfg.img_vocab);
+            batch.n_jobs = 3;
+        }
+        batch.name = "sort_ids";
+        small_sort = sort_small_fits(batch);
+        if (!small_sort) sorted_buf = sort_jobs(batch, &c.gbs, side, &c.prof, &e);
+        if (e != cudaSuccess) return e;
+        if (b.nnz > 0) {
+            c.img_sorted = true; c.img_sorted_n = b.nnz; c.img_sorted_buf = sorted_buf; c.last_img_id = b.img_id;
+            c.img_sort_valid = sorted_mode;
+        }
+    }
+    GEAR_TRY(launch_gather(c, b, o.row_view, o.inv_n, o.x_debug, st));
+    if (forked) GEAR_TRY(enqueue_record(c.ev[EV_GATHER], st));
+    // behind the sort: the plan of the accumulate call that usually follows (which rows form which group, where every group's
+    // rows and queue slot are).  It needs the gather's row_view / inv_n.  Small arrays are sorted and planned by one kernel.
+    if (small_sort || (forked && plan)) {
+        if (forked) GEAR_TRY(enqueue_wait(side, c.ev[EV_GATHER]));
+        if (small_sort) {
+            GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, o.row_view, o.inv_n) : PlanArgs{}, side));
+            if (plan) note_plan(c, b.nnz, o.row_view, o.inv_n);
+        } else GEAR_TRY(launch_accumulate_plan_ahead(c, b.nnz, o.row_view, o.inv_n, side));
+    }
+    if (forked && lists) GEAR_TRY(enqueue_record(c.ev[EV_PLAN], side));
+    // the embedding scatter: enqueued by the head as soon as dX is on its way
+    struct Scatter { gear_ctx_impl* c; const gear_step_out* o; int sorted_buf; int32_t B; float lr; cudaStream_t st, side; } sc{&c, &o, sorted_buf, b.B, lr, st, side};
+    auto scatter = [](void* arg) -> cudaError_t {
+        Scatter& k = *static_cast<Scatter*>(arg);
+        gear_ctx_impl& c = *k.c;
+        const gear_step_out& o = *k.o;
+        if (k.side != k.st) {
+            cudaError_t e = enqueue_record(c.ev[EV_DX], k.st);
+            if (e == cudaSuccess) e = enqueue_wait(k.side, c.ev[EV_DX]);
+            if (e != cudaSuccess) return e;
+        }
+        if (o.adam)
+            return launch_emb_adam(c, k.sorted_buf, k.B, o.dX, c.d_in, *o.adam, o.adam_step, o.user_m, o.user_v, o.url_m, o.url_v, k.side);
+        return launch_emb_reduce(c, k.sorted_buf, k.B, o.user_grad ? o.user_grad : c.buf.user_emb, o.url_grad ? o.url_grad : c.buf.url_emb,
+                                 o.dX, c.d_in, o.user_grad ? 1.0f : -k.lr, k.side);
+    };
+    const HeadHooks hooks{scatter, &sc, dw_beside ? aux : st, &c.ev[EV_AUX + 1]};
+    GEAR_TRY(launch_head(c, b, o, st, hooks));
+    if (o.dfv_grad && b.B > 0) GEAR_TRY(launch_dfv_grad_rows(c, o.dX, o.row_view, o.inv_n, b.nnz, o.dfv_grad, st));
+    if (lists) {
+        if (forked) GEAR_TRY(enqueue_wait(st, c.ev[EV_PLAN]));
+        GEAR_TRY(launch_accumulate_collect(c, b.nnz > 0 ? nullptr : b.img_id, o.dX + 2 * c.cfg.emb_dim, c.d_in, o.row_view, o.inv_n, b.nnz,
+                                           lists->ids, lists->seq, lists->avg, lists->cap, lists->d_n, st));
+        if (!scan_beside) GEAR_TRY(scan(st));
+    }
+    if (forked) {
+        GEAR_TRY(enqueue_record(c.ev[EV_JOIN], side));
+        GEAR_TRY(enqueue_wait(st, c.ev[EV_JOIN]));
+    }
+    if (scan_beside || dw_beside) {
+        GEAR_TRY(enqueue_record(c.ev[EV_AUX], aux));
+        GEAR_TRY(enqueue_wait(st, c.ev[EV_AUX]));
+    }
+#undef GEAR_TRY
+    return cudaSuccess;
+}
+
+// Writes a call down, plays it; on a failure the ctx forgets the batch whose order it may have been in the middle of.
+template <typename Fn> static int run_call(gear_ctx_impl& c, const char* where, cudaStream_t st, Fn&& enqueue) {
+    c.last_stream = st;
+    const unsigned long long base = c.gbs.host_base;
+    Recording rec(c.player, st);
+    cudaError_t e = enqueue();
+    if (e != cudaSuccess) c.gbs.host_base = base;            // nothing has been enqueued
+    else e = rec.play(&c.prof);
+    if (e == cudaSuccess) return GEAR_OK;
+    c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
+    return cuda_fail(e, where);
+}
 
 extern "C" {
 
@@ -181,16 +357,19 @@ int gear_init_tables(gear_ctx** out_ctx, const gear_config* cfg, const gear_buff
     c.acc_calls_pending = 0;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c.last_stream = st;
-    c.side_stream = nullptr;
-    c.ev_fork = c.ev_join = c.ev_gather = c.ev_dx = nullptr;
+    c.side_stream = c.aux_stream = nullptr;
+    for (cudaEvent_t& ev : c.ev) ev = nullptr;
     c.plan_ready = false; c.plan_n = 0; c.plan_src_row = nullptr; c.plan_scale = nullptr;
 
-    cudaError_t e = cudaStreamCreateWithFlags(&c.side_stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ev_gather, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ev_join, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c.ev_dx, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMemsetAsync(c.state(), 0, sizeof(DevState), st);
+    c.h_counts = nullptr;
+    cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&c.h_counts), 2 * sizeof(int64_t), cudaHostAllocDefault);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c.side_stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c.aux_stream, cudaStreamNonBlocking);
+    for (cudaEvent_t& ev : c.ev)
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = enqueue_memset(c.state(), sizeof(DevState), st);
+    // the expiry scan's section counts start from zero
+    if (e == cudaSuccess) e = enqueue_memset(c.at<char>(c.ws.exp_cnt), c.ws.total - c.ws.exp_cnt, st);
     if (e == cudaSuccess && fill) {
         const double amp = 0.17320508075688773;   // uniform half-width for standard deviation 0.1
         e = launch_fill_uniform(buf->user_emb, GEAR_F32, cfg->user_vocab * cfg->emb_dim, seed, GEAR_TAG_USER, amp, st);
@@ -199,8 +378,8 @@ int gear_init_tables(gear_ctx** out_ctx, const gear_config* cfg, const gear_buff
         if (e == cudaSuccess)
             e = launch_fill_uniform(buf->dfv, cfg->dfv_dtype, cfg->img_vocab * cfg->dfv_dim, seed, GEAR_TAG_DFV, amp, st);
         if (e == cudaSuccess)
-            e = cudaMemsetAsync(buf->dfv_gsum, 0, sizeof(float) * (size_t)cfg->img_vocab * cfg->dfv_dim, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(buf->dfv_gcnt, 0, sizeof(int32_t) * (size_t)cfg->img_vocab, st);
+            e = enqueue_memset(buf->dfv_gsum, sizeof(float) * (size_t)cfg->img_vocab * cfg->dfv_dim, st);
+        if (e == cudaSuccess) e = enqueue_memset(buf->dfv_gcnt, sizeof(int32_t) * (size_t)cfg->img_vocab, st);
         if (e == cudaSuccess) e = launch_fill_ts(buf->dfv_ts, cfg->img_vocab, seed, cfg->expire, now, st);
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -213,192 +392,69 @@ int gear_forward_backward(gear_ctx* ctx, const gear_batch* batch, float lr, cons
     if (!ctx || !ctx->impl.alive) return GEAR_ERR_STATE;
     if (!batch || !out) return arg_fail("NULL pointer");
     gear_ctx_impl& c = ctx->impl;
-    const gear_batch& b = *batch;
-    const gear_step_out& o = *out;
-    if (b.B < 0 || b.B > c.cfg.max_batch) return arg_fail("B outside [0, max_batch]");
-    if (b.nnz < 0 || b.nnz > c.cfg.max_nnz) return arg_fail("nnz outside [0, max_nnz]");
-    if (b.B > 0 && (!b.user_id || !b.url_id || !b.img_off || !b.label)) return arg_fail("NULL batch array");
-    if (b.nnz > 0 && !b.img_id) return arg_fail("NULL img_id");
-    if (b.B > 0 && c.cfg.fast_dim > 0 && (!b.fast || !aligned16(b.fast))) return arg_fail("fast: needed (16-byte aligned) when fast_dim > 0");
-    if (!o.loss || !o.head_grad || !o.dX) return arg_fail("loss, head_grad and dX are required outputs");
-    if ((o.user_grad == nullptr) != (o.url_grad == nullptr)) return arg_fail("user_grad and url_grad: both or neither");
-    gear_adam adam_cfg = {0.f, 0.f, 0.f, 0.f};
-    if (o.adam) {
-        adam_cfg = *o.adam;
-        if (o.user_grad) return arg_fail("adam and user_grad / url_grad exclude each other");
-        if (!o.user_m || !o.user_v || !o.url_m || !o.url_v) return arg_fail("adam needs the four moment tables");
-        if (!aligned16(o.user_m) || !aligned16(o.user_v) || !aligned16(o.url_m) || !aligned16(o.url_v))
-            return arg_fail("moment tables must be 16-byte aligned");
-        if (o.adam_step < 1) return arg_fail("adam_step >= 1");
-        if (!(adam_cfg.beta1 >= 0.f && adam_cfg.beta1 < 1.f && adam_cfg.beta2 >= 0.f && adam_cfg.beta2 < 1.f && adam_cfg.eps >= 0.f))
-            return arg_fail("adam: beta1, beta2 in [0, 1), eps >= 0");
-    }
-    if (c.cfg.head_dtype == GEAR_BF16 && (!aligned16(o.head_grad) || !aligned16(c.buf.head_params)))
-        return arg_fail("bf16 head: head_params and head_grad must be 16-byte aligned");
-    if (o.dfv_grad && (!o.row_view || !o.inv_n || !aligned16(o.dfv_grad)))
-        return arg_fail("dfv_grad needs row_view and inv_n and 16-byte alignment");
-    if (!aligned16(o.dX) || (o.x_debug && !aligned16(o.x_debug)) || (o.user_grad && !aligned16(o.user_grad)) ||
-        (o.url_grad && !aligned16(o.url_grad)))
-        return arg_fail("dX, x_debug, user_grad, url_grad must be 16-byte aligned");
+    if (int rc = check_batch(c, *batch, *out)) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    c.last_stream = st;
-
-    // What depends on the batch's ID arrays and on head_params alone runs on the ctx's side stream, beside the gather
-    // and the head: the bf16 copies of the weights, the key sort of the three ID arrays (the user and URL orders drive
-    // the embedding scatter, the image order is kept for gear_accumulate_dfv_grad with img_id == NULL) and, once the
-    // gather has written row_view / inv_n, the plan of that accumulate call.  The embedding scatter itself joins them
-    // there as soon as dX exists, beside the last weight-gradient product; the caller's stream waits for the side
-    // stream before the call returns.  With per-kernel timing on, everything stays on the caller's stream so that each
-    // kernel is timed alone.
-    c.img_sorted = false;
-    c.img_sort_valid = false;
-    c.plan_ready = false;
-    const bool forked = (!c.prof.on || c.prof.keep_streams) && b.B > 0;
-    bool join_pending = false;          // the side stream holds work the caller's stream has not waited for
-    cudaStream_t side = forked ? c.side_stream : st;
-    // A failure between the fork and the join must not leave the side stream unjoined or the sorted order marked as
-    // usable: the caller's stream waits for whatever the side stream was given, and the ctx forgets the batch.
-    auto abandon = [&](cudaError_t err, const char* where) {
-        if (join_pending) {
-            if (cudaEventRecord(c.ev_join, c.side_stream) != cudaSuccess || cudaStreamWaitEvent(st, c.ev_join, 0) != cudaSuccess)
-                cudaStreamSynchronize(c.side_stream);
-        }
-        c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
-        return cuda_fail(err, where);
-    };
-    cudaError_t e = cudaSuccess;
-    if (forked) {
-        e = cudaEventRecord(c.ev_fork, st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(c.side_stream, c.ev_fork, 0);
-        if (e != cudaSuccess) return cuda_fail(e, "fork");
-        join_pending = true;
-    }
-    // The weights in the form the head's products read: first on the caller's stream, ahead of the gather.  The gather keeps
-    // every SM busy for its whole duration, so a small kernel on another stream would get its blocks placed only when the
-    // gather ends, and the first product of the head would wait for it.
-    if (b.B > 0) {
-        e = launch_round_weights(c, st);
-        if (e != cudaSuccess) return abandon(e, "weight copies");
-    }
-    int sorted_buf = 0;
-    if (b.B > 0) {
-        SortBatch batch = c.sort_batch();
-        batch.job[0] = c.sort_job(gear_ctx_impl::SORT_USER);
-        batch.job[0].ids = b.user_id; batch.job[0].sentinel = (uint32_t)c.cfg.user_vocab;
-        batch.job[0].n_max = b.B; batch.job[0].bits = bits_for(c.cfg.user_vocab);
-        batch.job[1] = c.sort_job(gear_ctx_impl::SORT_URL);
-        batch.job[1].ids = b.url_id; batch.job[1].sentinel = (uint32_t)c.cfg.url_vocab;
-        batch.job[1].n_max = b.B; batch.job[1].bits = bits_for(c.cfg.url_vocab);
-        batch.n_jobs = 2;
-        if (b.nnz > 0 && c.cfg.accum_mode == GEAR_ACC_SORT) {      // the atomic mode takes the image IDs as they come
-            batch.job[2] = c.sort_job(gear_ctx_impl::SORT_IMG);
-            batch.job[2].ids = b.img_id; batch.job[2].sentinel = (uint32_t)c.cfg.img_vocab;
-            batch.job[2].n_max = b.nnz; batch.job[2].bits = bits_for(c.cfg.img_vocab);
-            batch.n_jobs = 3;
-        }
-        cudaError_t se = cudaSuccess;
-        batch.name = "sort_ids";
-        sorted_buf = sort_jobs(batch, &c.gbs, side, &c.prof, &se);
-        if (se != cudaSuccess) return abandon(se, "id sort");
-        if (b.nnz > 0) {
-            c.img_sorted = true; c.img_sorted_n = b.nnz; c.img_sorted_buf = sorted_buf; c.last_img_id = b.img_id;
-            c.img_sort_valid = c.cfg.accum_mode == GEAR_ACC_SORT;
-        }
-    }
-    e = launch_gather(c, b, o.row_view, o.inv_n, o.x_debug, st);
-    if (e != cudaSuccess) return abandon(e, "gather");
-    if (forked && b.nnz > 0 && o.row_view && o.inv_n && c.cfg.accum_mode == GEAR_ACC_SORT) {
-        // behind the sort: the plan of the accumulate call that usually follows (which rows form which group, where every
-        // group's rows and queue slot are).  It needs the gather's row_view / inv_n.
-        e = cudaEventRecord(c.ev_gather, st);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(c.side_stream, c.ev_gather, 0);
-        if (e == cudaSuccess) e = launch_accumulate_plan_ahead(c, b.nnz, o.row_view, o.inv_n, c.side_stream);
-        if (e != cudaSuccess) return abandon(e, "accumulate plan");
-    }
-    // the embedding scatter: enqueued by the head as soon as dX is on its way
-    struct Scatter {
-        gear_ctx_impl* c; const gear_step_out* o; int sorted_buf; int32_t B; float lr; cudaStream_t st; bool forked;
-        const gear_adam* adam;
-    } sc{&c, &o, sorted_buf, b.B, lr, st, forked, o.adam ? &adam_cfg : nullptr};
-    auto scatter = [](void* arg) -> cudaError_t {
-        Scatter& k = *static_cast<Scatter*>(arg);
-        gear_ctx_impl& c = *k.c;
-        float* ut = k.o->user_grad ? k.o->user_grad : c.buf.user_emb;
-        float* ht = k.o->url_grad ? k.o->url_grad : c.buf.url_emb;
-        const float alpha = k.o->user_grad ? 1.0f : -k.lr;
-        cudaStream_t where = k.st;
-        if (k.forked) {
-            cudaError_t e = cudaEventRecord(c.ev_dx, k.st);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(c.side_stream, c.ev_dx, 0);
-            if (e != cudaSuccess) return e;
-            where = c.side_stream;
-        }
-        if (k.adam)
-            return launch_emb_adam(c, k.sorted_buf, k.B, k.o->dX, c.d_in, *k.adam, k.o->adam_step, k.o->user_m, k.o->user_v,
-                                   k.o->url_m, k.o->url_v, where);
-        return launch_emb_reduce(c, k.sorted_buf, k.B, ut, ht, k.o->dX, c.d_in, alpha, where);
-    };
-    const HeadHooks hooks{scatter, &sc};
-    e = launch_head(c, b, o, st, hooks);
-    if (e != cudaSuccess) return abandon(e, "head");
-    if (o.dfv_grad && b.B > 0) {
-        e = launch_dfv_grad_rows(c, o.dX, o.row_view, o.inv_n, b.nnz, o.dfv_grad, st);
-        if (e != cudaSuccess) return abandon(e, "gradient rows");
-    }
-    if (forked) {
-        e = cudaEventRecord(c.ev_join, c.side_stream);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, c.ev_join, 0);
-        if (e != cudaSuccess) return abandon(e, "join");
-        join_pending = false;
-    }
-    return GEAR_OK;
+    return run_call(c, "forward_backward", st, [&] { return enqueue_step(c, *batch, lr, *out, nullptr, st); });
 }
 
 int gear_accumulate_dfv_grad(gear_ctx* ctx, const int32_t* img_id, const float* grads, int64_t ld,
                              const int32_t* src_row, const float* scale, int64_t n, void* stream) {
     if (!ctx || !ctx->impl.alive) return GEAR_ERR_STATE;
     gear_ctx_impl& c = ctx->impl;
-    if (n < 0 || n > c.cfg.max_nnz) return arg_fail("n outside [0, max_nnz]");
+    if (int rc = check_rows(c, img_id, grads, ld, n)) return rc;
     if (n == 0) return GEAR_OK;
-    if (!grads) return arg_fail("NULL pointer");
-    if (!img_id && (!c.img_sorted || c.img_sorted_n != n)) {
-        snprintf(g_last_error, sizeof(g_last_error),
-                 "img_id == NULL needs a preceding gear_forward_backward whose nnz equals n");
-        return GEAR_ERR_STATE;
-    }
-    if (ld < c.cfg.dfv_dim || ld % 4 || !aligned16(grads)) return arg_fail("grads rows must be 16-byte aligned, ld >= dfv_dim");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    c.last_stream = st;
-    cudaError_t e = c.cfg.accum_mode == GEAR_ACC_ATOMIC
-                        ? launch_accumulate_atomic(c, img_id ? img_id : c.last_img_id, grads, ld, src_row, scale, n, st)
-                        : launch_accumulate(c, img_id, grads, ld, src_row, scale, n, st);
-    return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "accumulate");
+    return run_call(c, "accumulate", st, [&] {
+        return c.cfg.accum_mode == GEAR_ACC_ATOMIC ? launch_accumulate_atomic(c, img_id ? img_id : c.last_img_id, grads, ld, src_row, scale, n, st)
+                                                   : launch_accumulate(c, img_id, grads, ld, src_row, scale, n, st);
+    });
 }
 
 static int finish_count(gear_ctx_impl& c, const int64_t* d_src, int64_t cap, int64_t* h_n, cudaStream_t st);
+static int check_capacity(int64_t cap, int64_t n) {
+    if (n <= cap) return GEAR_OK;
+    snprintf(g_last_error, sizeof(g_last_error), "capacity %lld too small, %lld entries waiting", (long long)cap, (long long)n);
+    return GEAR_ERR_CAPACITY;
+}
 
 int gear_accumulate_collect(gear_ctx* ctx, const int32_t* img_id, const float* grads, int64_t ld, const int32_t* src_row,
                             const float* scale, int64_t n, int32_t* ids, int32_t* seq, float* avg, int64_t cap,
                             int64_t* d_n, int64_t* h_n, void* stream) {
     if (!ctx || !ctx->impl.alive) return GEAR_ERR_STATE;
     gear_ctx_impl& c = ctx->impl;
-    if (n < 0 || n > c.cfg.max_nnz) return arg_fail("n outside [0, max_nnz]");
-    if (n > 0 && !grads) return arg_fail("NULL pointer");
-    if (n > 0 && !img_id && (!c.img_sorted || c.img_sorted_n != n)) {
-        snprintf(g_last_error, sizeof(g_last_error),
-                 "img_id == NULL needs a preceding gear_forward_backward whose nnz equals n");
-        return GEAR_ERR_STATE;
-    }
-    if (n > 0 && (ld < c.cfg.dfv_dim || ld % 4 || !aligned16(grads)))
-        return arg_fail("grads rows must be 16-byte aligned, ld >= dfv_dim");
-    if (cap < 0 || (cap > 0 && (!ids || !seq || !avg))) return arg_fail("NULL output with cap > 0");
-    if (avg && !aligned16(avg)) return arg_fail("avg must be 16-byte aligned");
+    if (int rc = check_rows(c, img_id, grads, ld, n)) return rc;
+    if (int rc = check_lists(ids, seq, avg, cap)) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    c.last_stream = st;
     int64_t* d_cnt = d_n ? d_n : &c.state()->pad[0];
-    cudaError_t e = launch_accumulate_collect(c, img_id, grads, ld, src_row, scale, n, ids, seq, avg, cap, d_cnt, st);
-    if (e != cudaSuccess) return cuda_fail(e, "accumulate_collect");
+    if (int rc = run_call(c, "accumulate_collect", st, [&] {
+            return launch_accumulate_collect(c, img_id, grads, ld, src_row, scale, n, ids, seq, avg, cap, d_cnt, st); }))
+        return rc;
     return finish_count(c, d_cnt, cap, h_n, st);
+}
+
+int gear_step(gear_ctx* ctx, const gear_batch* batch, float lr, const gear_step_out* out, const gear_step_lists* lists,
+              int64_t now, int restamp, int scan_beside, int64_t* h_n, void* stream) {
+    if (!ctx || !ctx->impl.alive) return GEAR_ERR_STATE;
+    if (!batch || !out || !lists) return arg_fail("NULL pointer");
+    gear_ctx_impl& c = ctx->impl;
+    if (int rc = check_batch(c, *batch, *out)) return rc;
+    if (!out->row_view || !out->inv_n) return arg_fail("gear_step needs row_view and inv_n");
+    if (int rc = check_lists(lists->ids, lists->seq, lists->avg, lists->cap)) return rc;
+    if (lists->expired_cap < 0 || (lists->expired_cap > 0 && !lists->expired)) return arg_fail("NULL output with cap > 0");
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const StepLists l{lists->ids, lists->seq, lists->avg, lists->cap, lists->d_n ? lists->d_n : &c.state()->pad[0],
+                      lists->expired, lists->expired_cap, lists->d_expired ? lists->d_expired : &c.state()->pad[1],
+                      now, restamp, scan_beside != 0};
+    if (int rc = run_call(c, "step", st, [&] { return enqueue_step(c, *batch, lr, *out, &l, st); })) return rc;
+    if (!h_n) return GEAR_OK;
+    // both counts with one wait
+    cudaError_t e = cudaMemcpyAsync(c.h_counts, l.d_n, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c.h_counts + 1, l.d_expired, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "read counts");
+    h_n[0] = c.h_counts[0]; h_n[1] = c.h_counts[1];
+    if (int rc = check_capacity(l.cap, h_n[0])) return rc;
+    return check_capacity(l.expired_cap, h_n[1]);
 }
 
 // Waits for everything the ctx has enqueued: the stream of the training calls and, if the expiry scan went to a
@@ -412,29 +468,22 @@ static cudaError_t sync_streams(const gear_ctx_impl& c) {
 
 static int finish_count(gear_ctx_impl& c, const int64_t* d_src, int64_t cap, int64_t* h_n, cudaStream_t st) {
     if (!h_n) return GEAR_OK;
-    cudaError_t e = cudaMemcpyAsync(h_n, d_src, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaMemcpyAsync(c.h_counts, d_src, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "read count");
-    if (*h_n > cap) {
-        snprintf(g_last_error, sizeof(g_last_error), "capacity %lld too small, %lld entries waiting", (long long)cap,
-                 (long long)*h_n);
-        return GEAR_ERR_CAPACITY;
-    }
-    return GEAR_OK;
+    *h_n = c.h_counts[0];
+    return check_capacity(cap, *h_n);
 }
 
 int gear_collect_ready(gear_ctx* ctx, int32_t* ids, int32_t* seq, float* avg, int64_t cap, int64_t* d_n, int64_t* h_n,
                        void* stream) {
     if (!ctx || !ctx->impl.alive) return GEAR_ERR_STATE;
     gear_ctx_impl& c = ctx->impl;
-    if (cap < 0 || (cap > 0 && (!ids || !seq || !avg))) return arg_fail("NULL output with cap > 0");
-    if (avg && !aligned16(avg)) return arg_fail("avg must be 16-byte aligned");
+    if (int rc = check_lists(ids, seq, avg, cap)) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    c.last_stream = st;
     // the count is staged in the device state so that h_n can be served even when d_n is NULL
     int64_t* d_cnt = d_n ? d_n : &c.state()->pad[0];
-    cudaError_t e = launch_collect_ready(c, ids, seq, avg, cap, d_cnt, st);
-    if (e != cudaSuccess) return cuda_fail(e, "collect_ready");
+    if (int rc = run_call(c, "collect_ready", st, [&] { return launch_collect_ready(c, ids, seq, avg, cap, d_cnt, st); })) return rc;
     return finish_count(c, d_cnt, cap, h_n, st);
 }
 
@@ -488,9 +537,7 @@ int gear_apply_emb_grad(gear_ctx* ctx, int32_t which, const int32_t* ids, const 
     if (n == 0) return GEAR_OK;
     if (!ids || !rows || !aligned16(rows) || ld < c.cfg.emb_dim || (ld & 3)) return arg_fail("rows: 16-byte aligned, ld >= emb_dim, multiple of 4");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    c.last_stream = st;
-    cudaError_t e = launch_apply_emb_grad(c, which, ids, rows, ld, n, -lr, st);
-    return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "apply_emb_grad");
+    return run_call(c, "apply_emb_grad", st, [&] { return launch_apply_emb_grad(c, which, ids, rows, ld, n, -lr, st); });
 }
 
 int gear_dense_forward(gear_ctx* ctx, const float* raw, int32_t raw_dim, const float* Wd, const int32_t* ids, int64_t n,
@@ -573,6 +620,7 @@ int gear_profile_timeline(gear_ctx* ctx, char* names, float* start_ms, float* st
     gear_ctx_impl& c = ctx->impl;
     cudaError_t e = sync_streams(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c.side_stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c.aux_stream);
     if (e != cudaSuccess) return cuda_fail(e, "gear_profile_timeline");
     int n = 0;
     for (const auto& r : c.prof.recs) {
@@ -633,6 +681,7 @@ int gear_destroy(gear_ctx* ctx) {
                                                      // ctx is freed memory and must not be passed in again
     sync_streams(ctx->impl);
     cudaStreamSynchronize(ctx->impl.side_stream);
+    cudaStreamSynchronize(ctx->impl.aux_stream);
     release_host_objects(ctx->impl);
     ctx->impl.alive = false;
     delete ctx;

@@ -5,9 +5,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
 #include <vector>
 
 #include "../../include/gear.h"
+#include "enqueue.cuh"
 
 namespace gear {
 
@@ -22,7 +24,7 @@ struct DevState {
     int64_t direct_done;   // accumulate + collect as one call: 1 while the hand-over pass that follows has nothing to do
                            // (the reduce pass wrote the averages straight into the caller's lists)
     int64_t n_complete;    // accumulate: groups of this call that reached M
-    int64_t exp_total;     // expiry scan: entries found
+    int64_t pad0;
     int64_t collect_n;     // collect_ready: entries moved by the running call
     unsigned long long grid_barrier;   // arrival counter of the cooperative sort's grid barrier
     unsigned int colsum_ticket;        // blocks of head_out_kernel that have delivered their partial loss (wraps to 0)
@@ -155,20 +157,23 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                                    Args&&... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+inline cudaError_t launch_as(Op::Attr attr, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    OpList local;
+    OpList& l = t_ops ? *t_ops : local;
+    l.kernel(reinterpret_cast<const void*>(kernel), grid, block, smem, attr, st);
+    auto push = [&l](const auto& v) { l.arg(&v, sizeof(v)); return 0; };
+    (push(static_cast<const KArgs&>(KArgs(args))), ...);
+    return t_ops ? cudaSuccess : launch_list_kernel(l.ops.back(), l, st);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
+    return launch_as(Op::DEPENDENT, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
 // ---------------------------------------------------------------- launch accounting / per-kernel timing
-// Every kernel launch of the library goes through a KernelScope: it counts the launch and, when profiling
-// is on, brackets it with a pair of CUDA events on the caller's stream (read back by gear_profile_read).
+// Every kernel launch of the library goes through a KernelScope: it counts the launch and, when profiling is on, has it
+// bracketed with a pair of CUDA events on its stream (read back by gear_profile_read): by the player where the
+// launch is being written down, by the scope itself otherwise.
 struct Profiler {
     struct Rec { const char* name; cudaEvent_t start, stop; };
     bool on = false;
@@ -197,7 +202,8 @@ struct KernelScope {
     KernelScope(Profiler* prof, const char* name, cudaStream_t s) : p(prof), st(s) {
         if (!p) return;
         ++p->launches;
-        if (p->on) {
+        if (t_ops) t_ops->next_name = name;
+        else if (p->on) {
             Profiler::Rec r{name, p->get(), p->get()};
             stop = r.stop;
             cudaEventRecord(r.start, st);

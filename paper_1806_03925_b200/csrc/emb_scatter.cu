@@ -123,8 +123,8 @@ cudaError_t launch_emb_adam(const gear_ctx_impl& c, int cur, int32_t B, const fl
     const int E = c.cfg.emb_dim, n_chunks = E / 4;
     float* gu = c.at<float>(c.ws.emb_gsum[0]);
     float* gh = c.at<float>(c.ws.emb_gsum[1]);
-    cudaError_t e = cudaMemsetAsync(gu, 0, sizeof(float) * (size_t)B * E, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(gh, 0, sizeof(float) * (size_t)B * E, st);
+    cudaError_t e = enqueue_memset(gu, sizeof(float) * (size_t)B * E, st);
+    if (e == cudaSuccess) e = enqueue_memset(gh, sizeof(float) * (size_t)B * E, st);
     if (e != cudaSuccess) return e;
     int lpr = 1;
     while (lpr < n_chunks && lpr < 32) lpr <<= 1;
@@ -167,7 +167,9 @@ cudaError_t launch_apply_emb_grad(const gear_ctx_impl& c, int which, const int32
     batch.job[0].n_max = n; batch.job[0].bits = bits_for(vocab);
     batch.name = "sort_emb";
     cudaError_t se;
-    const int cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
+    int cur = 0;
+    if (sort_small_fits(batch)) se = launch_sort_small(c, batch, PlanArgs{}, st);
+    else cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
     if (se != cudaSuccess) return se;
     const int E = c.cfg.emb_dim, n_chunks = E / 4;
     int lpr = 1;

@@ -1,13 +1,15 @@
 // Inference-expired time (Section 1, second point; Section 3: the workers drop expired inference
 // results continuously): list every image whose cached DFV is older than the expiry time.
 //
-// Three launches, none waits on another block:
+// Two launches, none waits on another block:
 //   mark   streams the int64 timestamp table once (the only HBM-sized traffic: 8 bytes per image),
-//          evaluates now - ts >= expire, packs the predicate 32 entries to a word with a warp ballot and
-//          counts per 2048-entry tile;
-//   scan   one block scans the tile counts;
-//   write  checks the caller's capacity, re-reads only the bitmap (1 bit per image), ranks the set bits
-//          with popc + block scan and writes the ascending ID list; listed entries are restamped on request.
+//          evaluates now - ts >= expire, packs the predicate 32 entries to a word with a warp ballot and counts per
+//          2048-entry tile and, with one atomic per tile, per section of 64 tiles;
+//   write  every block adds up the sections and tiles before its own, checks the caller's capacity against the total,
+//          re-reads only the bitmap (1 bit per image), ranks the set bits with popc + block scan and writes the ascending ID
+//          list; listed entries are restamped on request.
+// (A scan kernel between the two took 7 us for 20 M images, and one kernel that keeps the bits in shared memory and waits for
+// the counts of the blocks before it read the table at 2.8 TB/s instead of 5.7: too few loads in flight.)
 #include "common.cuh"
 #include "internal.h"
 
@@ -18,11 +20,18 @@ constexpr int EXP_MARK_ITEMS = EXP_MARK_TILE / EXP_THREADS;
 static_assert(EXP_TILE == EXP_THREADS * 32, "one bitmap word per thread in the write pass");
 static_assert(EXP_MARK_TILE % (EXP_THREADS * 1) == 0 && EXP_TILE % EXP_MARK_TILE == 0, "mark tiles nest in write tiles");
 
+// Per-tile counts, then the sections' counts twice over: a scan adds to one set and clears the other for the next scan.
+struct ExpiryCounts {
+    uint32_t* tile; uint32_t* section; uint32_t* section_next;
+    int64_t n_tiles;
+};
+constexpr int EXP_SECTION = 64;           // mark tiles per section
+
 // One block per EXP_MARK_TILE timestamps.  All of a thread's loads are issued before the first ballot, so a
 // block keeps its whole 16 KB tile in flight; the small tiles leave the balancing to the block scheduler.
 __global__ void __launch_bounds__(EXP_THREADS)
 expiry_mark_kernel(const int64_t* __restrict__ ts, int64_t vocab, int64_t now, int64_t expire,
-                   uint32_t* __restrict__ bits, uint2* __restrict__ tile_cnt) {
+                   uint32_t* __restrict__ bits, const ExpiryCounts cnt) {
     wait_for_predecessor();
     __shared__ uint32_t warp_cnt[EXP_THREADS / 32];
     const int64_t tile0 = (int64_t)blockIdx.x * EXP_MARK_TILE;
@@ -51,29 +60,41 @@ expiry_mark_kernel(const int64_t* __restrict__ ts, int64_t vocab, int64_t now, i
         uint32_t total = 0;
 #pragma unroll
         for (int w = 0; w < EXP_THREADS / 32; ++w) total += warp_cnt[w];
-        tile_cnt[blockIdx.x] = make_uint2(total, 0u);
+        cnt.tile[blockIdx.x] = total;
+        if (total) atomicAdd(cnt.section + blockIdx.x / EXP_SECTION, total);
+        if (blockIdx.x % EXP_SECTION == 0) cnt.section_next[blockIdx.x / EXP_SECTION] = 0u;
     }
 }
 
 // One block per EXP_TILE entries: re-reads the bitmap only.  Every block compares the total with the
 // caller's capacity itself; block 0 reports the count and raises the status bit.
 __global__ void __launch_bounds__(EXP_THREADS)
-expiry_write_kernel(const uint32_t* __restrict__ bits, int64_t vocab, const uint2* __restrict__ tile_cnt,
-                    int64_t n_mark_tiles, int64_t cap, int64_t* __restrict__ d_n, DevState* __restrict__ state,
-                    int64_t now, int restamp, int64_t* __restrict__ ts, int32_t* __restrict__ ids) {
+expiry_write_kernel(const uint32_t* __restrict__ bits, int64_t vocab, const ExpiryCounts cnt, int64_t cap,
+                    int64_t* __restrict__ d_n, DevState* __restrict__ state, int64_t now, int restamp, int64_t* __restrict__ ts,
+                    int32_t* __restrict__ ids) {
     wait_for_predecessor();
     __shared__ uint32_t scratch[33];
-    const int64_t total = tile_cnt[n_mark_tiles].x;
+    const int64_t w = (int64_t)blockIdx.x * EXP_THREADS + threadIdx.x;
+    uint32_t word = (w * 32 < vocab) ? bits[w] : 0u;
+    const int64_t my_tile = (int64_t)blockIdx.x * (EXP_TILE / EXP_MARK_TILE), my_section = my_tile / EXP_SECTION;
+    const int64_t sections = ceil_div(cnt.n_tiles, EXP_SECTION);
+    uint32_t before = 0, after = 0;                         // this thread's share
+    for (int64_t s = threadIdx.x; s < sections; s += EXP_THREADS) {
+        const uint32_t v = cnt.section[s];
+        if (s < my_section) before += v; else after += v;
+    }
+    const int64_t t = my_section * EXP_SECTION + threadIdx.x;
+    if (threadIdx.x < EXP_SECTION && t < my_tile) { const uint32_t v = cnt.tile[t]; before += v; after -= v; }
+    uint32_t n_before, n_after;
+    block_exclusive_scan(before, scratch, &n_before);
+    block_exclusive_scan(after, scratch, &n_after);
+    const int64_t total = (int64_t)(n_before + n_after);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (d_n) *d_n = total;
-        state->exp_total = total > cap ? -1 : total;
         if (total > cap) atomicOr(&state->status, GEAR_DEV_OUT_CAPACITY);
     }
     if (total > cap) return;                                // capacity too small: nothing listed, nothing restamped
-    const int64_t w = (int64_t)blockIdx.x * EXP_THREADS + threadIdx.x;
-    uint32_t word = (w * 32 < vocab) ? bits[w] : 0u;
-    const uint32_t ex = block_exclusive_scan(__popc(word), scratch, nullptr);
-    int64_t out = (int64_t)tile_cnt[(int64_t)blockIdx.x * (EXP_TILE / EXP_MARK_TILE)].x + ex;
+    int64_t out = (int64_t)n_before + block_exclusive_scan(__popc(word), scratch, nullptr);
     while (word) {
         const int bit = __ffs(word) - 1;
         word &= word - 1;
@@ -83,24 +104,31 @@ expiry_write_kernel(const uint32_t* __restrict__ bits, int64_t vocab, const uint
     }
 }
 
-// The three launches of one scan over scratch (bits, tile_cnt, state).  prof may be null.
+// The two launches of one scan over scratch (bits, counts, state).  prof may be null.
 static cudaError_t enqueue_expiry_scan(int64_t* ts, int64_t vocab, int64_t expire, int64_t now, int restamp,
-                                       int32_t* ids, int64_t cap, int64_t* d_n, uint32_t* bits, uint2* tile_cnt,
+                                       int32_t* ids, int64_t cap, int64_t* d_n, uint32_t* bits, const ExpiryCounts& cnt,
                                        DevState* state, Profiler* prof, cudaStream_t st) {
-    const int64_t n_mark = ceil_div(vocab, EXP_MARK_TILE), n_write = ceil_div(vocab, EXP_TILE);
+    const int64_t n_write = ceil_div(vocab, EXP_TILE);
+    cudaError_t e;
     { KernelScope k(prof, "expiry_mark", st);
-    launch_dependent(expiry_mark_kernel, dim3((unsigned)n_mark), dim3(EXP_THREADS), 0, st, ts, vocab, now, expire, bits, tile_cnt); }
-    scan_pairs(tile_cnt, n_mark, tile_cnt + n_mark, st, prof);
-    { KernelScope k(prof, "expiry_write", st);
-    launch_dependent(expiry_write_kernel, dim3((unsigned)n_write), dim3(EXP_THREADS), 0, st, bits, vocab, tile_cnt, n_mark, cap, d_n, state, now,
-                                                                  restamp, ts, ids); }
-    return cudaGetLastError();
+    e = launch_dependent(expiry_mark_kernel, dim3((unsigned)cnt.n_tiles), dim3(EXP_THREADS), 0, st, ts, vocab, now, expire, bits, cnt); }
+    if (e != cudaSuccess) return e;
+    KernelScope k(prof, "expiry_write", st);
+    return launch_dependent(expiry_write_kernel, dim3((unsigned)n_write), dim3(EXP_THREADS), 0, st, bits, vocab, cnt, cap, d_n, state, now,
+                            restamp, ts, ids);
+}
+
+// counts: [n_tiles] tile counts, then two sets of section counts; the sections of `set` are zero before the scan
+static ExpiryCounts expiry_counts(uint32_t* counts, int64_t vocab, int set) {
+    const int64_t n = ceil_div(vocab, EXP_MARK_TILE), sections = ceil_div(n, EXP_SECTION);
+    return ExpiryCounts{counts, counts + n + set * sections, counts + n + (set ^ 1) * sections, n};
 }
 
 cudaError_t launch_collect_expired(const gear_ctx_impl& c, int64_t now, int restamp, int32_t* ids, int64_t cap,
                                    int64_t* d_n, cudaStream_t st) {
-    return enqueue_expiry_scan(c.buf.dfv_ts, c.cfg.img_vocab, c.cfg.expire, now, restamp, ids, cap, d_n,
-                               c.at<uint32_t>(c.ws.exp_bits), c.at<uint2>(c.ws.exp_cnt), c.state(), &c.prof, st);
+    c.expiry_set ^= 1;
+    return enqueue_expiry_scan(c.buf.dfv_ts, c.cfg.img_vocab, c.cfg.expire, now, restamp, ids, cap, d_n, c.at<uint32_t>(c.ws.exp_bits),
+                               expiry_counts(c.at<uint32_t>(c.ws.exp_cnt), c.cfg.img_vocab, c.expiry_set), c.state(), &c.prof, st);
 }
 
 }  // namespace gear
@@ -123,7 +151,7 @@ namespace gear {
 constexpr int64_t STATIC_MAX_VOCAB = GEAR_STATIC_EXPIRY_MAX_VOCAB;
 constexpr size_t STATIC_STATE_BYTES = 256;
 constexpr size_t STATIC_BITS_BYTES = (size_t)(STATIC_MAX_VOCAB / 32) * 4;
-constexpr size_t STATIC_CNT_BYTES = ((size_t)(STATIC_MAX_VOCAB / EXP_MARK_TILE) + 1) * sizeof(uint2);
+constexpr size_t STATIC_CNT_BYTES = ((size_t)(STATIC_MAX_VOCAB / EXP_MARK_TILE) + 1) * 8;     // tile and section counts
 constexpr size_t STATIC_SCRATCH_BYTES = STATIC_STATE_BYTES + STATIC_BITS_BYTES + ((STATIC_CNT_BYTES + 255) / 256) * 256;
 static_assert(sizeof(DevState) <= STATIC_STATE_BYTES, "state block");
 static_assert(STATIC_SCRATCH_BYTES == GEAR_STATIC_EXPIRY_SCRATCH_BYTES, "the header states the size of the array");
@@ -164,13 +192,15 @@ extern "C" int gear_collect_expired_static(int64_t* dfv_ts, int64_t img_vocab, i
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     DevState* state = reinterpret_cast<DevState*>(base);
     uint32_t* bits = reinterpret_cast<uint32_t*>(base + STATIC_STATE_BYTES);
-    uint2* tile_cnt = reinterpret_cast<uint2*>(base + STATIC_STATE_BYTES + STATIC_BITS_BYTES);
+    uint32_t* counts = reinterpret_cast<uint32_t*>(base + STATIC_STATE_BYTES + STATIC_BITS_BYTES);
 
-    // the array keeps what the previous call left: the state block has to start from zero, the bitmap words
-    // and tile counts of this table size are all rewritten by the mark pass
-    if (cudaMemsetAsync(state, 0, STATIC_STATE_BYTES, st) != cudaSuccess) return GEAR_ERR_CUDA;
+    // the array keeps what the previous call left: the state block and the section counts have to start from zero, the
+    // bitmap words and tile counts of this table size are all rewritten by the mark pass
+    const ExpiryCounts cnt = expiry_counts(counts, img_vocab, 0);
+    if (enqueue_memset(state, STATIC_STATE_BYTES, st) != cudaSuccess) return GEAR_ERR_CUDA;
+    if (enqueue_memset(cnt.section, sizeof(uint32_t) * (size_t)ceil_div(cnt.n_tiles, EXP_SECTION), st) != cudaSuccess) return GEAR_ERR_CUDA;
     int64_t* d_cnt = d_n ? d_n : &state->pad[1];
-    if (enqueue_expiry_scan(dfv_ts, img_vocab, expire, now, restamp, ids, cap, d_cnt, bits, tile_cnt, state, nullptr, st) !=
+    if (enqueue_expiry_scan(dfv_ts, img_vocab, expire, now, restamp, ids, cap, d_cnt, bits, cnt, state, nullptr, st) !=
         cudaSuccess)
         return GEAR_ERR_CUDA;
     if (h_n) {

@@ -38,8 +38,8 @@ template <> struct Chunk<__nv_bfloat16> {
 };
 
 // N (4 or 8) values of a row of the head input at X + off: rounded to bf16 (HB: bf16 heads) or as three bf16 planes,
-// `stride` apart; and, if asked for, a copy of them at xd + off, in bf16 or fp32.
-template <bool HB, int N> __device__ __forceinline__ void store_x(__nv_bfloat16* X, int64_t stride, void* xd, int64_t off, const float* v) {
+// `stride` apart, and in fp32 at Xf + off (fp32 heads); and, if asked for, a copy of them at xd + off, in bf16 or fp32.
+template <bool HB, int N> __device__ __forceinline__ void store_x(__nv_bfloat16* X, int64_t stride, float* Xf, void* xd, int64_t off, const float* v) {
     constexpr int PLANES = HB ? 1 : 3;
     uint32_t w[3][N / 2];
 #pragma unroll
@@ -55,6 +55,10 @@ template <bool HB, int N> __device__ __forceinline__ void store_x(__nv_bfloat16*
     };
 #pragma unroll
     for (int p = 0; p < PLANES; ++p) put(X + p * stride + off, w[p]);
+    if constexpr (!HB) {
+#pragma unroll
+        for (int k = 0; k < N; k += 4) st_f4(Xf + off + k, make_float4(v[k], v[k + 1], v[k + 2], v[k + 3]));
+    }
     if (xd) {
         if constexpr (HB) put(static_cast<__nv_bfloat16*>(xd) + off, w[0]);
         else {
@@ -81,7 +85,7 @@ struct GatherArgs {
     const float* fast;          // [B][F] the views' own dense input (F > 0)
     int64_t nnz;
     const int32_t* user_id; const int32_t* url_id; const int32_t* img_off; const int32_t* img_id;
-    __nv_bfloat16* X; int64_t x_stride; void* x_debug;      // X: bf16, or three planes x_stride apart
+    __nv_bfloat16* X; int64_t x_stride; float* Xf; void* x_debug;      // X: bf16, or three planes x_stride apart and fp32 at Xf
     int32_t* row_view; float* inv_n;
     DevState* state;
 };
@@ -237,7 +241,7 @@ gather_pool_kernel(const GatherArgs a) {
         // ---- write the row of X
         if (lane < 2 * ce) {
             const float f[4] = {emb.x, emb.y, emb.z, emb.w};
-            store_x<HB, 4>(a.X, a.x_stride, a.x_debug, x0 + lane * 4, f);
+            store_x<HB, 4>(a.X, a.x_stride, a.Xf, a.x_debug, x0 + lane * 4, f);
         }
         for (int c = 32 + lane; c < 2 * ce; c += 32) {             // embedding rows wider than 32 chunks in total
             const bool is_url = c >= ce;
@@ -246,7 +250,7 @@ gather_pool_kernel(const GatherArgs a) {
             float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
             if (id >= 0) t = __ldg(reinterpret_cast<const float4*>(table + (int64_t)id * a.E + (is_url ? c - ce : c) * 4));
             const float f[4] = {t.x, t.y, t.z, t.w};
-            store_x<HB, 4>(a.X, a.x_stride, a.x_debug, x0 + c * 4, f);
+            store_x<HB, 4>(a.X, a.x_stride, a.Xf, a.x_debug, x0 + c * 4, f);
         }
         const float nf = (float)n, rinv = n > 0 ? 1.0f / nf : 0.f;
 #pragma unroll
@@ -256,7 +260,7 @@ gather_pool_kernel(const GatherArgs a) {
                 float o[PER];
 #pragma unroll
                 for (int k = 0; k < PER; ++k) o[k] = n > 0 ? div_by_count(acc[q][k], nf, rinv) : 0.f;
-                store_x<HB, PER>(a.X, a.x_stride, a.x_debug, x0 + 2 * a.E + ch * PER, o);
+                store_x<HB, PER>(a.X, a.x_stride, a.Xf, a.x_debug, x0 + 2 * a.E + ch * PER, o);
             }
         }
         if (a.inv_n && lane == 0) a.inv_n[b] = rinv;
@@ -264,7 +268,7 @@ gather_pool_kernel(const GatherArgs a) {
         for (int c = lane * 8; c < a.F; c += 256) {
             const float4 f0 = ld_stream_f4(a.fast + (int64_t)b * a.F + c), f1 = ld_stream_f4(a.fast + (int64_t)b * a.F + c + 4);
             const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-            store_x<HB, 8>(a.X, a.x_stride, a.x_debug, x0 + 2 * a.E + a.D + c, f);
+            store_x<HB, 8>(a.X, a.x_stride, a.Xf, a.x_debug, x0 + 2 * a.E + a.D + c, f);
         }
 
         cur = nxt; nxt = nxt2; ids_cur = ids_nxt;
@@ -302,7 +306,7 @@ cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* 
     a.user_vocab = c.cfg.user_vocab; a.url_vocab = c.cfg.url_vocab; a.img_vocab = c.cfg.img_vocab;
     a.E = c.cfg.emb_dim; a.D = c.cfg.dfv_dim; a.B = b.B; a.nnz = b.nnz; a.F = c.cfg.fast_dim; a.fast = b.fast;
     a.user_id = b.user_id; a.url_id = b.url_id; a.img_off = b.img_off; a.img_id = b.img_id;
-    a.X = c.at<__nv_bfloat16>(c.ws.x); a.x_stride = (int64_t)c.cfg.max_batch * c.d_in; a.x_debug = x_debug; a.row_view = row_view; a.inv_n = inv_n;
+    a.X = c.at<__nv_bfloat16>(c.ws.x); a.x_stride = (int64_t)c.cfg.max_batch * c.d_in; a.Xf = c.cfg.head_dtype == GEAR_F32 ? c.at<float>(c.ws.xf[0]) : nullptr; a.x_debug = x_debug; a.row_view = row_view; a.inv_n = inv_n;
     a.state = c.state();
     const bool dbf = c.cfg.dfv_dtype == GEAR_BF16, xbf = c.cfg.head_dtype == GEAR_BF16;
     if (dbf && xbf) return dispatch_nq<__nv_bfloat16, true>(a, st, &c.prof);

@@ -4,7 +4,7 @@
 //   input gradient dH_{l-1} = (dA_l W_l^T) masked by H_{l-1} > 0
 //   weight gradient dW_l  = H_{l-1}^T dA_l           (reduction over the batch, split over blocks)
 // GEAR_BF16 heads: operands rounded to bf16 (head_tc.cu).  GEAR_F32 heads: every fp32 matrix is held as three bf16 planes
-// whose sum it is (head_tc3.cu); no precision is given up.
+// whose sum it is for the backward products on the tensor cores (head_tc3.cu), and in fp32 for the forward ones (head_fwd.cu).
 #include <type_traits>
 
 #include "common.cuh"
@@ -219,12 +219,20 @@ struct RoundArgs {
     const float* W[MAX_LAYERS];
     __nv_bfloat16* wb[MAX_LAYERS];
     __nv_bfloat16* wbt[MAX_LAYERS];
+    float* grad; int64_t n_grad;                // the parameters' gradient, cleared by the same launch
+    float* loss;                                // empty batch only: its loss (0)
 };
 // 32 x 32 tiles through shared memory, so that both copies are written with coalesced rows
 template <int PLANES>
 __global__ void __launch_bounds__(256)
 round_weights_kernel(const RoundArgs a) {
     wait_for_predecessor();
+    {
+        const int64_t blk = blockIdx.x + (int64_t)gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
+        const int64_t threads = (int64_t)gridDim.x * gridDim.y * gridDim.z * blockDim.x;
+        for (int64_t i = blk * blockDim.x + threadIdx.x; i < a.n_grad; i += threads) a.grad[i] = 0.f;
+        if (a.loss && blk == 0 && threadIdx.x == 0) *a.loss = 0.f;
+    }
     __shared__ __nv_bfloat16 tile[PLANES][32][33];
     const int l = blockIdx.z;
     const int fan_in = a.fan_in[l], fan_out = a.fan_out[l];
@@ -279,11 +287,18 @@ static HeadParams split_params(const gear_ctx_impl& c, float* grad) {
     return p;
 }
 
+// Where the parameters' gradient is put together.  The copy engine adds the weight gradients to it in 16-byte pieces; an fp32
+// head may be handed a less aligned array: its gradient is then put together in the workspace and copied.
+static float* grad_array(const gear_ctx_impl& c, const gear_step_out& o) {
+    return (reinterpret_cast<uintptr_t>(o.head_grad) & 15u) == 0 ? o.head_grad : c.at<float>(c.ws.head_grad);
+}
+
 // bf16 copies or planes of the hidden layers' weights in both orientations (what the tensor-core products read).  Depends
-// on head_params only, so a step runs it ahead of the gather.
-cudaError_t launch_round_weights(const gear_ctx_impl& c, cudaStream_t st) {
+// on head_params only, so a step runs it ahead of the gather.  Clears head_grad on the way.
+cudaError_t launch_round_weights(const gear_ctx_impl& c, const gear_step_out& o, cudaStream_t st) {
     const int L = c.cfg.n_hidden;
     RoundArgs ra;
+    ra.grad = grad_array(c, o); ra.n_grad = c.n_params; ra.loss = o.loss;     // the loss of a batch is written after this
     int max_in = 0, max_out = 0, fan = c.d_in;
     int64_t pos = 0;
     for (int l = 0; l < L; ++l) {
@@ -308,20 +323,13 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
                             const HeadHooks& hooks) {
     constexpr bool BF = std::is_same<TX, __nv_bfloat16>::value;
     const int L = c.cfg.n_hidden, B = bt.B;
-    // the copy engine adds the weight gradients to head_grad in 16-byte pieces; an fp32 head may hand over a less aligned
-    // array: its gradient is then put together in the workspace and copied
-    const bool staged = !BF && (reinterpret_cast<uintptr_t>(o.head_grad) & 15u) != 0;
-    float* grad = staged ? c.at<float>(c.ws.head_grad) : o.head_grad;
-    HeadParams p = split_params(c, grad);
-    cudaError_t err = cudaMemsetAsync(grad, 0, sizeof(float) * c.n_params, st);
-    if (err != cudaSuccess) return err;
+    float* grad = grad_array(c, o);
+    const HeadParams p = split_params(c, grad);
     auto finish = [&]() -> cudaError_t {
-        return staged ? cudaMemcpyAsync(o.head_grad, grad, sizeof(float) * c.n_params, cudaMemcpyDeviceToDevice, st) : cudaSuccess;
+        return grad != o.head_grad ? enqueue_copy(o.head_grad, grad, sizeof(float) * c.n_params, st) : cudaSuccess;
     };
-    if (B <= 0) {
-        err = cudaMemsetAsync(o.loss, 0, sizeof(float), st);
-        return err == cudaSuccess ? finish() : err;
-    }
+    if (B <= 0) return finish();
+    cudaError_t err = cudaSuccess;
 
     const int64_t max_b = c.cfg.max_batch;
     Planes H[MAX_LAYERS + 1], dA[MAX_LAYERS + 1] = {}, W[MAX_LAYERS], Wt[MAX_LAYERS];      // Wt: [out][in]
@@ -341,7 +349,7 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
         if constexpr (BF)
             err = tc_gemm_kmajor(c, "tc_gemm_fwd", B, N, K, H[l].p, K, Wt[l].p, K, 0, H[l + 1].p, N, p.b[l], nullptr, 0, nullptr, st);
         else
-            err = tc3_gemm_kmajor(c, "tc3_gemm_fwd", B, N, K, H[l], K, Wt[l], K, 0, H[l + 1], nullptr, N, p.b[l], nullptr, 0, nullptr, st);
+            err = launch_fwd_f32(c, B, N, K, c.at<float>(c.ws.xf[l]), p.W[l], p.b[l], H[l + 1], l + 1 < L ? c.at<float>(c.ws.xf[l + 1]) : nullptr, st);
         if (err != cudaSuccess) return err;
     }
     const int HT = p.fan[L];
@@ -363,28 +371,35 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
 #undef GEAR_HEAD_OUT
         if (err != cudaSuccess) return err;
     }
+    // dW_l = H_l^T dA_{l+1}, on the stream the hooks name
+    const bool beside = hooks.dw_stream != st;
+    auto weight_grad = [&](int l) -> cudaError_t {
+        const int K = p.fan[l], N = p.fan[l + 1];
+        if (beside) {
+            err = enqueue_record(hooks.dw_ev[l], st);
+            if (err == cudaSuccess) err = enqueue_wait(hooks.dw_stream, hooks.dw_ev[l]);
+            if (err != cudaSuccess) return err;
+        }
+        if constexpr (BF) return tc_gemm_mnmajor(c, "tc_gemm_dw", K, N, B, H[l].p, K, dA[l + 1].p, N, p.gW[l], N, hooks.dw_stream);
+        else return tc3_gemm_mnmajor(c, "tc3_gemm_dw", K, N, B, H[l], K, dA[l + 1], N, p.gW[l], N, hooks.dw_stream);
+    };
     // backward.  Per layer the gradient that the layers below wait for (dA_l, at the bottom dX) comes first, its weight
-    // gradient after it: once dX exists the caller's hook may start the embedding scatter on another stream, beside the
-    // last weight-gradient product.  The bias gradient of a lower layer is summed in the epilogue of the product that
-    // makes its dA (the top layer's came out of head_out_kernel).
+    // gradient after it (or, on a stream of its own, as soon as dA_{l+1} exists): once dX exists the caller's hook may start
+    // the embedding scatter on another stream.  The bias gradient of a lower layer is summed in the epilogue of the product
+    // that makes its dA (the top layer's came out of head_out_kernel).
     for (int l = L - 1; l >= 0; --l) {
         const int K = p.fan[l], N = p.fan[l + 1];
+        if (beside && (err = weight_grad(l)) != cudaSuccess) return err;
         if constexpr (BF) {
             if (l > 0) err = tc_gemm_kmajor(c, "tc_gemm_dh", B, K, N, dA[l + 1].p, N, W[l].p, N, 1, dA[l].p, K, nullptr, H[l].p, K, p.gb[l - 1], st);
             else err = tc_gemm_kmajor(c, "tc_gemm_dx", B, K, N, dA[l + 1].p, N, W[l].p, N, 2, o.dX, K, nullptr, nullptr, 0, nullptr, st);
         } else {
-            if (l > 0) err = tc3_gemm_kmajor(c, "tc3_gemm_dh", B, K, N, dA[l + 1], N, W[l], N, 1, dA[l], nullptr, K, nullptr, H[l].p, K, p.gb[l - 1], st);
-            else err = tc3_gemm_kmajor(c, "tc3_gemm_dx", B, K, N, dA[l + 1], N, W[l], N, 2, Planes{}, o.dX, K, nullptr, nullptr, 0, nullptr, st);
+            if (l > 0) err = tc3_gemm_kmajor(c, "tc3_gemm_dh", B, K, N, dA[l + 1], N, W[l], N, dA[l], nullptr, K, H[l].p, K, p.gb[l - 1], st);
+            else err = tc3_gemm_kmajor(c, "tc3_gemm_dx", B, K, N, dA[l + 1], N, W[l], N, Planes{}, o.dX, K, nullptr, 0, nullptr, st);
         }
         if (err != cudaSuccess) return err;
-        if (l == 0 && hooks.after_dx) {
-            err = hooks.after_dx(hooks.arg);
-            if (err != cudaSuccess) return err;
-        }
-        // dW_l = H_l^T dA_{l+1}
-        if constexpr (BF) err = tc_gemm_mnmajor(c, "tc_gemm_dw", K, N, B, H[l].p, K, dA[l + 1].p, N, p.gW[l], N, st);
-        else err = tc3_gemm_mnmajor(c, "tc3_gemm_dw", K, N, B, H[l], K, dA[l + 1], N, p.gW[l], N, st);
-        if (err != cudaSuccess) return err;
+        if (l == 0 && hooks.after_dx && (err = hooks.after_dx(hooks.arg)) != cudaSuccess) return err;
+        if (!beside && (err = weight_grad(l)) != cudaSuccess) return err;
     }
     return finish();
 }

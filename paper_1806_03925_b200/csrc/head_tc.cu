@@ -108,7 +108,6 @@ __device__ __forceinline__ void epilogue_tile(const TcArgs& g, const CUtensorMap
     constexpr int CHUNKS = COLS / 32;                     // 32-column chunks per warp and tile
     static_assert(EPI == TC_EPI_F32 || EPI == TC_EPI_RED || CHUNKS % 2 == 0, "bf16 output leaves in blocks of 64 columns");
     const int m0 = mt * TC_BM + quarter * 32;         // first row of this warp's block
-    const int m = m0 + lane;
     const int rows = min(32, max(0, g.M - m0));
     const int col0 = nt * BN + part * COLS;
     const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * BN + part * COLS);

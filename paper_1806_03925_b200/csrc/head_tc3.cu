@@ -1,4 +1,4 @@
-// fp32 matrix products of the head (GEAR_F32) on the 5th-generation tensor cores.
+// Backward matrix products of fp32 heads (GEAR_F32) on the 5th-generation tensor cores.
 //
 // Every fp32 operand is held as three bf16 matrices ("planes"): a = a0 + a1 + a2 with a0 = bf16(a), a1 = bf16(a - a0),
 // a2 = bf16(a - a0 - a1), each rounded to nearest.  The three hold 24 significant bits, so the sum is the fp32 value itself
@@ -14,9 +14,8 @@
 // One persistent kernel, one CTA per SM, the same roles as the bf16 products (head_tc.cu): warp 0 streams operand tiles
 // with TMA (all three planes of a 128 x 32 or BN x 32 box in one copy), warp 1 issues tcgen05.mma, warps 2-9 drain one pair
 // of accumulators while the next tile fills the other.  Tiles are 32 deep so that three stages of two operands with three
-// planes each (48 KB) fit beside the output blocks.  Epilogues: bias + ReLU or ReLU mask, split into planes again
-// (activations stay in planes between the products; masked outputs also sum their columns, the bias gradient of
-// the layer below); plain fp32 (dX); fp32 added to memory by the copy engine (weight gradients, reduction over the batch
+// planes each (48 KB) fit beside the output blocks.  Epilogues: ReLU mask, split into planes again (matrices stay in planes
+// between the products; masked outputs also sum their columns, the bias gradient of the layer below); plain fp32 (dX); fp32 added to memory by the copy engine (weight gradients, reduction over the batch
 // split across CTAs).  Every wait is bounded.
 #include "common.cuh"
 #include "internal.h"
@@ -29,16 +28,16 @@ constexpr int T3_EW = 8;                  // epilogue warps
 constexpr int T3_THREADS = 64 + 32 * T3_EW;
 constexpr int T3_MAX_N = 1024;
 
-enum { T3_BIAS_RELU = 0, T3_MASK = 1, T3_F32 = 2, T3_RED = 3 };
+enum { T3_MASK = 1, T3_F32 = 2, T3_RED = 3 };
 
 template <int BN, int EPI> struct T3Cfg {
-    static constexpr bool PLANES_OUT = EPI == T3_BIAS_RELU || EPI == T3_MASK;
+    static constexpr bool PLANES_OUT = EPI == T3_MASK;
     static constexpr int A_PLANE = TC_BM * T3_BK * 2, A_BYTES = 3 * A_PLANE;
     static constexpr int B_PLANE = BN * T3_BK * 2, B_BYTES = 3 * B_PLANE;
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
     static constexpr int OUT_BLOCK = PLANES_OUT ? 3 * 32 * 64 : 32 * 128;     // a warp's 32 x 32 block on its way out
     static constexpr int OUT_BYTES = T3_EW * OUT_BLOCK;
-    static constexpr int VEC_BYTES = PLANES_OUT ? T3_MAX_N * 4 : 0;           // bias, or the CTA's column sums
+    static constexpr int VEC_BYTES = PLANES_OUT ? T3_MAX_N * 4 : 0;           // the CTA's column sums
     static constexpr int FIXED = 1024 /*alignment slack*/ + 256 /*barriers*/ + VEC_BYTES + OUT_BYTES;
     static constexpr int ROOM = (227 * 1024 - FIXED) / STAGE_BYTES;
     static constexpr int STAGES = ROOM > 6 ? 6 : ROOM;
@@ -51,7 +50,6 @@ template <int BN, int EPI> struct T3Cfg {
 struct T3Args {
     int M, N, K;
     int m_tiles, n_tiles, k_splits, kb_per_split;   // kb = blocks of T3_BK along K
-    const float* bias;                              // T3_BIAS_RELU
     const __nv_bfloat16* mask; int64_t ldm;         // T3_MASK: leading plane of the activations (positive where they are)
     float* colsum;                                  // T3_MASK: colsum[n] += column sums of the masked output (may be null)
     int32_t* err;
@@ -71,14 +69,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, uint32_t sr
 template <int EPI>
 __device__ __forceinline__ void t3_emit(const T3Args& g, const CUtensorMap* map_out, float (&v)[32], const uint4 (&mk)[4], int m0,
                                         int n0, int lane, float* s_vec, uint32_t out_buf, uint64_t keep_policy) {
-    if (EPI == T3_BIAS_RELU) {
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float4 b = *reinterpret_cast<const float4*>(s_vec + n0 + 4 * j);      // zeros past N
-            v[4 * j] = fmaxf(v[4 * j] + b.x, 0.f); v[4 * j + 1] = fmaxf(v[4 * j + 1] + b.y, 0.f);
-            v[4 * j + 2] = fmaxf(v[4 * j + 2] + b.z, 0.f); v[4 * j + 3] = fmaxf(v[4 * j + 3] + b.w, 0.f);
-        }
-    }
     if (EPI == T3_MASK) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -92,7 +82,7 @@ __device__ __forceinline__ void t3_emit(const T3Args& g, const CUtensorMap* map_
     }
     if (lane == 0) tma_store_wait_read<0>();                    // the block's previous contents have left
     __syncwarp();
-    if (EPI == T3_BIAS_RELU || EPI == T3_MASK) {
+    if (EPI == T3_MASK) {
         const uint32_t row_addr = out_buf + (uint32_t)lane * 64u, swz = ((uint32_t)lane >> 1) & 3u;
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
@@ -187,18 +177,13 @@ t3_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                      :: "r"(tmem_word), "r"((uint32_t)Cfg::TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    // the bias belongs to the caller's parameters, which no kernel of the library writes: it may be read ahead of the wait only
-    // if no other kernel of the stream does either, so it is read behind it
+    if (EPI == T3_MASK)
+        for (int n = threadIdx.x; n < T3_MAX_N; n += T3_THREADS) s_vec[n] = 0.f;
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_word_ptr;
     wait_for_predecessor();
-    if (Cfg::PLANES_OUT) {
-        for (int n = threadIdx.x; n < T3_MAX_N; n += T3_THREADS)
-            s_vec[n] = (EPI == T3_BIAS_RELU && n < g.N) ? __ldg(g.bias + n) : 0.f;
-        __syncthreads();
-    }
 
     if (warp == 0) {
         // ---------------- TMA producer
@@ -386,26 +371,25 @@ static int t3_bn(const T3Args& g) {
 }
 
 cudaError_t tc3_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,
-                            const Planes& W, int64_t ldw, int epi, const Planes& out_planes, float* out_f32, int64_t ldo,
-                            const float* bias, const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st) {
+                            const Planes& W, int64_t ldw, const Planes& out_planes, float* out_f32, int64_t ldo,
+                            const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     T3Args g{};
     g.M = M; g.N = N; g.K = K;
     const int bn = t3_bn(g);
     g.m_tiles = (int)ceil_div(M, TC_BM); g.n_tiles = (int)ceil_div(N, bn);
     g.k_splits = 1; g.kb_per_split = (int)ceil_div(K, T3_BK);
-    g.bias = bias; g.mask = mask; g.ldm = ldm; g.colsum = colsum; g.err = &c.state()->tc_error;
-    if (N > T3_MAX_N && epi != T3_F32) return cudaErrorInvalidValue;
+    g.mask = mask; g.ldm = ldm; g.colsum = colsum; g.err = &c.state()->tc_error;
+    if (N > T3_MAX_N && mask) return cudaErrorInvalidValue;
     CUtensorMap ma, mb, mo;
     if (!c.tma->get(&ma, TmaSpec{A.p, M, K, lda, A.stride, 3, TC_BM, T3_BK, 0, 64}) ||
         !c.tma->get(&mb, TmaSpec{W.p, N, K, ldw, W.stride, 3, bn, T3_BK, 0, 64}) ||
-        !c.tma->get(&mo, epi == T3_F32 ? TmaSpec{out_f32, M, N, ldo, 0, 1, 32, 32, 1, 128}
-                                       : TmaSpec{out_planes.p, M, N, ldo, out_planes.stride, 3, 32, 32, 0, 64}))
+        !c.tma->get(&mo, mask ? TmaSpec{out_planes.p, M, N, ldo, out_planes.stride, 3, 32, 32, 0, 64}
+                              : TmaSpec{out_f32, M, N, ldo, 0, 1, 32, 32, 1, 128}))
         return cudaErrorInvalidValue;
     KernelScope ks(&c.prof, name, st);
-#define GEAR_T3(EPI) (bn == 128 ? t3_launch<128, false, EPI>(ma, mb, mo, g, st) : t3_launch<64, false, EPI>(ma, mb, mo, g, st))
-    return epi == T3_BIAS_RELU ? GEAR_T3(T3_BIAS_RELU) : epi == T3_MASK ? GEAR_T3(T3_MASK) : GEAR_T3(T3_F32);
-#undef GEAR_T3
+    if (mask) return bn == 128 ? t3_launch<128, false, T3_MASK>(ma, mb, mo, g, st) : t3_launch<64, false, T3_MASK>(ma, mb, mo, g, st);
+    return bn == 128 ? t3_launch<128, false, T3_F32>(ma, mb, mo, g, st) : t3_launch<64, false, T3_F32>(ma, mb, mo, g, st);
 }
 
 cudaError_t tc3_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,

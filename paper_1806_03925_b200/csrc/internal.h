@@ -21,6 +21,7 @@ struct WsPlan {
     size_t x;                           // [max_batch][d_in]      head input
     size_t h[MAX_LAYERS];               // [max_batch][hidden[l]] post-ReLU activations
     size_t da[MAX_LAYERS];              // [max_batch][hidden[l]] gradient at the pre-activation
+    size_t xf[MAX_LAYERS];              // fp32 head: the inputs of its layers (head input, lower hidden activations) in fp32
     size_t dz;                          // [max_batch] fp32
     size_t loss_part;                   // [loss_blocks] fp32 per-block partial losses
     size_t head_grad;                   // fp32 head: the parameters' gradient, when the caller's array is not 16-byte aligned
@@ -30,7 +31,7 @@ struct WsPlan {
     size_t sort_keys[4][2], sort_vals[4][2];
     size_t sort_hist[4], sort_tot[4];
     int64_t sort_n[4];
-    size_t tile_cnt;                    // [sort tiles + 1] uint2 per-tile (groups, complete) counts
+    size_t tile_cnt;                    // [plan tiles + 1] uint2 per-tile (groups, complete) counts, then their totals
     size_t grp_rec;                     // [max_nnz] uint4 group records (start | first flag, image ID, queue slot, held rows)
     size_t blk_first;                   // [ceil(max_nnz / 16) + 2] uint32: first group that starts in each span of sorted positions
     size_t run_end;                     // [max_nnz] uint32: at the first position of an image's run, one past its last
@@ -40,7 +41,7 @@ struct WsPlan {
     size_t emb_gsum[2];                 // [max_batch][emb_dim] fp32 per table: summed gradient of every distinct ID of the
                                         // batch, in the row of the sorted position where the ID's run starts (Adam only)
     size_t exp_bits;                    // [ceil(img_vocab / 32)] uint32 expired bitmap
-    size_t exp_cnt;                     // [expiry mark tiles + 1] uint2
+    size_t exp_cnt;                     // [expiry mark tiles + 1][2] words: tile counts, two sets of section counts
     size_t total;
     int64_t ready_cap;
     int loss_blocks;
@@ -72,9 +73,13 @@ struct gear_ctx_impl {
     bool alive;
     TmaCache* tma;      // tensor maps of the head's products (tc_ptx.cuh)
     cudaStream_t side_stream;          // runs the ID sort of a step beside the gather and the head
-    cudaEvent_t ev_fork, ev_join;
+    cudaStream_t aux_stream;           // runs the expiry scan and, for small batches, the weight gradients
+    cudaEvent_t ev[8];                 // between the streams of a step (enqueue_step in api.cu)
+    int64_t* h_counts;                 // two counts on their way to the caller (pinned)
+    Player player;                     // plays what a call has written down
     mutable Profiler prof;
     mutable GridBarrierState gbs;
+    mutable int expiry_set = 0;             // which set of section counts the last expiry scan used
     // image IDs of the last gear_forward_backward batch, already sorted (reused by gear_accumulate_dfv_grad)
     const int32_t* last_img_id;         // img_id array of that batch (the atomic mode reads it unsorted)
     bool img_sorted;
@@ -87,8 +92,6 @@ struct gear_ctx_impl {
     mutable int64_t plan_n;
     mutable const int32_t* plan_src_row;
     mutable const float* plan_scale;
-    cudaEvent_t ev_gather;              // the gather's outputs (row_view, inv_n) exist
-    cudaEvent_t ev_dx;                  // dX exists: the embedding scatter may start on the side stream
     mutable int acc_calls_pending;      // accumulate calls enqueued since a collect that was sure to drain the queue
 
     template <typename T> T* at(size_t off) const { return reinterpret_cast<T*>(static_cast<char*>(buf.workspace) + off); }
@@ -112,6 +115,17 @@ struct gear_ctx_impl {
     }
 };
 
+// sort_small.cu: one block per array (raw IDs, at most 16384 of them), sorted into the first buffer pair of each job; the block
+// of the last job also plans the accumulate call where plan.totals is set.
+// What a plan is made from and where it goes (plan.cuh).
+struct PlanArgs {
+    uint2* totals; uint32_t vocab; int M; const int32_t* cnt; uint4* grp_rec; const int32_t* src_row; const float* scale;
+    int2* pmeta; uint32_t* blk_first; uint32_t* run_end; DevState* state;
+    uint32_t div_factor; int div_shift;         // division by M (plan.cuh)
+};
+bool sort_small_fits(const SortBatch& batch);
+cudaError_t launch_sort_small(const gear_ctx_impl& c, const SortBatch& batch, const PlanArgs& plan, cudaStream_t st);
+
 // fill.cu
 cudaError_t launch_fill_uniform(void* dst, int dtype, int64_t n_elems, uint64_t seed, uint64_t tag, double amp,
                                 cudaStream_t st);
@@ -121,11 +135,13 @@ cudaError_t launch_fill_ts(int64_t* ts, int64_t n, uint64_t seed, int64_t expire
 cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* row_view, float* inv_n,
                           void* x_debug, cudaStream_t st);
 
-// head.cu: forward + backward of the head.  The weights' copies must have been made earlier on the same stream
-// (launch_round_weights).  after_dx(arg) is called once dX has been enqueued, before the last weight-gradient product.
-struct HeadHooks { cudaError_t (*after_dx)(void*); void* arg; };
+// head.cu: forward + backward of the head.  The weights' copies must have been made and head_grad cleared earlier on the same
+// stream (launch_round_weights).  after_dx(arg) is called once dX has been enqueued.  dw_stream: where the weight gradients go;
+// if it is not the head's own stream, it is made to wait for what they read (one event of dw_ev per layer).
+struct HeadHooks { cudaError_t (*after_dx)(void*); void* arg; cudaStream_t dw_stream; cudaEvent_t* dw_ev; };
 cudaError_t launch_head(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o, cudaStream_t st, const HeadHooks& hooks);
-cudaError_t launch_round_weights(const gear_ctx_impl& c, cudaStream_t st);
+// the weights as the products read them; clears head_grad (all of it, also for an empty batch)
+cudaError_t launch_round_weights(const gear_ctx_impl& c, const gear_step_out& o, cudaStream_t st);
 
 // head_tc.cu: bf16 products on tcgen05 tensor cores.  epi: 0 bias+ReLU -> bf16, 1 ReLU mask -> bf16, 2 plain fp32.
 // colsum (epi 1 only, may be null): colsum[n] += sum over the rows of the stored (rounded) output.
@@ -136,11 +152,15 @@ cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int 
 cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
                             const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo, cudaStream_t st);
 
-// head_tc3.cu: the same products of fp32 matrices held as three bf16 planes.  epi 0 and 1 write planes, 2 plain fp32; the mask
-// is the leading plane of the activations.
+// head_fwd.cu: H = ReLU(A W + bias), A [M][K], W [K][N] fp32; H in planes and, if Hf is given, in fp32
+cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
+                           const Planes& H, float* Hf, cudaStream_t st);
+
+// head_tc3.cu: the backward products of fp32 matrices held as three bf16 planes.  With a mask (the leading plane of the
+// activations) the output goes to planes, masked, and colsum[n] += its column sums; without, to out_f32.
 cudaError_t tc3_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,
-                            const Planes& W, int64_t ldw, int epi, const Planes& out_planes, float* out_f32, int64_t ldo,
-                            const float* bias, const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st);
+                            const Planes& W, int64_t ldw, const Planes& out_planes, float* out_f32, int64_t ldo,
+                            const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st);
 cudaError_t tc3_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,
                              const Planes& Bm, int64_t ldb, float* out, int64_t ldo, cudaStream_t st);
 
@@ -182,6 +202,9 @@ cudaError_t launch_accumulate_atomic(const gear_ctx_impl& c, const int32_t* img_
 // steps 2-4 of the sorted accumulate for the batch just sorted by gear_forward_backward, ahead of the accumulate call
 cudaError_t launch_accumulate_plan_ahead(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale,
                                          cudaStream_t st);
+// what the plan for n rows needs; note_plan: it has been made (for the image IDs of the last batch)
+PlanArgs plan_args(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale);
+void note_plan(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale);
 cudaError_t launch_collect_ready(const gear_ctx_impl& c, int32_t* ids, int32_t* seq, float* avg, int64_t cap,
                                  int64_t* d_n, cudaStream_t st);
 // accumulate followed by the hand-over; averages bypass the queue when the host knows it to be empty and cap >= n

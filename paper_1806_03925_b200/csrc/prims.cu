@@ -22,7 +22,6 @@
 // earlier launch contributes).  The kernel is launched cooperatively, so all blocks are resident and a tile's
 // predecessors are always being worked on; the spins (barrier and look-back) are bounded all the same, and a block
 // that gives up records an error and makes every later wait of the launch fall through.
-#include <cstdlib>
 #include "common.cuh"
 
 namespace gear {
@@ -340,7 +339,6 @@ static int coop_grid_limit() {
         if (sms <= 0) sms = 148;
         if (per_sm <= 0) per_sm = 1;
         if (per_sm > 3) per_sm = 3;
-        if (getenv("GEAR_SORT_PER_SM")) per_sm = atoi(getenv("GEAR_SORT_PER_SM"));
         limit = sms * per_sm;
     }
     return limit;
@@ -359,7 +357,7 @@ int sort_jobs(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st, Profiler
         job.n_tiles = (int)sort_tiles(job.n_max);
         total_tiles += job.n_tiles;
         // the per-pass digit histograms start from zero
-        *err_out = cudaMemsetAsync(job.tot, 0, sizeof(uint32_t) * RS_MAX_PASSES * RS_BUCKETS, st);
+        *err_out = enqueue_memset(job.tot, sizeof(uint32_t) * RS_MAX_PASSES * RS_BUCKETS, st);
         if (*err_out != cudaSuccess) return 0;
     }
     batch.passes = passes;
@@ -370,8 +368,7 @@ int sort_jobs(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st, Profiler
     batch.barrier_base = gbs->host_base;
     gbs->host_base += (unsigned long long)grid * (unsigned long long)batch.n_barriers;
     KernelScope k(prof, batch.name ? batch.name : "coop_sort", st);
-    void* args[] = {&batch};
-    *err_out = cudaLaunchCooperativeKernel((const void*)coop_sort_kernel, dim3(grid), dim3(RS_THREADS), args, RS_STAGE_BYTES, st);
+    *err_out = launch_as(Op::COOPERATIVE, coop_sort_kernel, dim3(grid), dim3(RS_THREADS), RS_STAGE_BYTES, st, batch);
     return passes & 1;
 }
 

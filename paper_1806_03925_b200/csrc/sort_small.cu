@@ -1,0 +1,188 @@
+// Key sort of small ID arrays (at most 32768 entries each), and the accumulate call's plan for the image array behind it.
+//
+// A cluster of eight blocks (one block for arrays of one tile) per array: the pairs stay in registers and shared memory over
+// all passes of a stable radix sort (digits of up to 10 bits, so that a vocabulary of a million takes two passes).  A block
+// owns a tile of consecutive entries, a warp 32 * ITEMS of them; it finds equal digits with match_any, sums the warps' digit
+// counts column by column, reads the other blocks' counts through distributed shared memory and writes its pairs straight
+// into the shared memory of the block that owns their new place.  Two cluster barriers per pass instead of grid barriers and
+// trips through the L2.  Bound: latency of the barriers, and instructions: about 500 per 32 entries, which is why the
+// work is spread over eight SMs (one block of 1024 threads took 75 us for 12 k entries).
+//
+// The cluster that sorts the image IDs goes on to plan the accumulate call (plan.cuh) from the keys it holds.
+#include <cooperative_groups.h>
+
+#include "common.cuh"
+#include "internal.h"
+#include "plan.cuh"
+
+namespace gear {
+
+namespace cg = cooperative_groups;
+
+constexpr int SS_THREADS = 512;
+constexpr int SS_WARPS = SS_THREADS / 32;
+constexpr int SS_MAX_BITS = 10;
+constexpr int SS_RADIX = 1 << SS_MAX_BITS;
+constexpr int SS_CLUSTER = 8;
+
+template <int ITEMS> constexpr int ss_smem() { return SS_THREADS * ITEMS * 8 + 2 * SS_RADIX * 4 + SS_WARPS * SS_RADIX * 2; }
+
+template <int ITEMS, int CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(SS_THREADS)
+sort_small_kernel(const SortBatch batch, const PlanArgs plan) {
+    wait_for_predecessor();
+    extern __shared__ uint32_t dyn[];
+    constexpr int TILE = SS_THREADS * ITEMS;
+    uint32_t* skey = dyn;                                                   // the block's tile of the current order
+    uint32_t* sval = dyn + TILE;
+    uint32_t* tot = dyn + 2 * TILE;                                         // [RADIX] the tile's digit counts (read by the cluster)
+    uint32_t* base = tot + SS_RADIX;                                        // [RADIX] where the tile's entries of a digit go
+    uint16_t* wcnt = reinterpret_cast<uint16_t*>(base + SS_RADIX);          // [SS_WARPS][RADIX]
+    __shared__ uint32_t scratch[2 * SS_WARPS + 2];
+    __shared__ int xchg[4];                                                 // plan: last run head; groups, complete groups
+    cg::cluster_group cluster = cg::this_cluster();
+    const int cr = CL == 1 ? 0 : (int)cluster.block_rank();
+    auto sync_cluster = [&]() { if constexpr (CL == 1) __syncthreads(); else cluster.sync(); };
+    auto peer = [&](auto* p, int r) { if constexpr (CL == 1) return p; else return cluster.map_shared_rank(p, r); };
+    const int job = (int)blockIdx.x / CL;
+    const SortJob& j = batch.job[job];
+    const int lane = (int)lane_id(), warp = (int)(threadIdx.x >> 5);
+    const int n = (int)j.n_max;
+    const int tile0 = cr * TILE, seg0 = tile0 + warp * 32 * ITEMS;
+    const int passes = (j.bits + SS_MAX_BITS - 1) / SS_MAX_BITS, width = (j.bits + passes - 1) / passes;
+    const uint32_t mask = (1u << width) - 1u, lt = (1u << lane) - 1u;
+    uint32_t key[ITEMS], val[ITEMS];
+    bool bad = false;
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+        const int i = seg0 + it * 32 + lane;
+        key[it] = 0u; val[it] = (uint32_t)i;
+        if (i < n) {
+            const int32_t id = __ldg(j.ids + i);
+            const bool ok = id >= 0 && (uint32_t)id < j.sentinel;
+            bad |= !ok;
+            key[it] = ok ? (uint32_t)id : j.sentinel;
+        }
+    }
+    if (bad && j.status) atomicOr(j.status, GEAR_DEV_BAD_ID);
+    for (int pass = 0; pass < passes; ++pass) {
+        const int shift = pass * width;
+        for (int q = threadIdx.x; q < SS_WARPS * SS_RADIX / 8; q += SS_THREADS) reinterpret_cast<uint4*>(wcnt)[q] = make_uint4(0u, 0u, 0u, 0u);
+        __syncthreads();
+        uint16_t* mine = wcnt + warp * SS_RADIX;
+        uint32_t rank[ITEMS];
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            rank[it] = 0;
+            if (seg0 + it * 32 < n) {                                       // warp-uniform
+                const bool valid = seg0 + it * 32 + lane < n;
+                const uint32_t d = valid ? (key[it] >> shift) & mask : 0xffffu;
+                const uint32_t peers = __match_any_sync(0xffffffffu, d);
+                const int leader = __ffs(peers) - 1;
+                uint32_t old = 0;
+                if (valid && lane == leader) {
+                    old = mine[d];
+                    mine[d] = (uint16_t)(old + __popc(peers));
+                }
+                rank[it] = __shfl_sync(0xffffffffu, old, leader) + __popc(peers & lt);
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        for (int d = threadIdx.x; d < SS_RADIX; d += SS_THREADS) {
+            uint32_t total = 0;
+            if (d <= (int)mask) {
+                uint32_t c[SS_WARPS];
+#pragma unroll
+                for (int w = 0; w < SS_WARPS; ++w) c[w] = wcnt[w * SS_RADIX + d];
+#pragma unroll
+                for (int w = 0; w < SS_WARPS; ++w) { wcnt[w * SS_RADIX + d] = (uint16_t)total; total += c[w]; }
+            }
+            tot[d] = total;
+        }
+        sync_cluster();                                                     // every tile's counts are there; every tile is in registers
+        {
+            // a thread owns two adjacent digits
+            uint32_t all[2] = {0u, 0u}, before[2] = {0u, 0u};
+            if (2 * (int)threadIdx.x <= (int)mask) {
+#pragma unroll
+                for (int r = 0; r < CL; ++r) {
+                    const uint2 t = *reinterpret_cast<const uint2*>(peer(tot, r) + 2 * threadIdx.x);
+                    all[0] += t.x; all[1] += t.y;
+                    if (r < cr) { before[0] += t.x; before[1] += t.y; }
+                }
+            }
+            const uint32_t start = block_exclusive_scan(all[0] + all[1], scratch, nullptr);
+            base[2 * threadIdx.x] = start + before[0];
+            base[2 * threadIdx.x + 1] = start + all[0] + before[1];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+            if (seg0 + it * 32 + lane < n) {
+                const uint32_t d = (key[it] >> shift) & mask;
+                const uint32_t pos = base[d] + mine[d] + rank[it];
+                const int r = CL == 1 ? 0 : (int)(pos / TILE);
+                const uint32_t at = pos - (uint32_t)r * TILE;
+                peer(skey, r)[at] = key[it];
+                peer(sval, r)[at] = val[it];
+            }
+        }
+        sync_cluster();
+        if (pass + 1 < passes) {
+#pragma unroll
+            for (int it = 0; it < ITEMS; ++it) {
+                const int i = seg0 + it * 32 + lane;
+                if (i < n) { key[it] = skey[i - tile0]; val[it] = sval[i - tile0]; }
+            }
+        }
+    }
+    const int live = min(max(n - tile0, 0), TILE);
+    for (int i = threadIdx.x; i < live; i += SS_THREADS) { j.keys[0][tile0 + i] = skey[i]; j.vals[0][tile0 + i] = sval[i]; }
+    if (plan.totals && job == batch.n_jobs - 1) {
+        auto key_at = [&](int i) -> uint32_t {
+            if (CL == 1 || (unsigned)(i - tile0) < (unsigned)TILE) return skey[i - tile0];
+            return peer(skey, i / TILE)[i % TILE];
+        };
+        plan_tile<ITEMS, SS_WARPS>(plan, n, tile0, key_at, [&](int i) { return sval[i - tile0]; }, reinterpret_cast<int*>(scratch),
+            [&](int last_head) -> int {                                     // run heads of the tiles before this one
+                if (CL == 1) return -1;
+                if (threadIdx.x == 0) xchg[0] = last_head;
+                sync_cluster();
+                int run0 = -1;
+                for (int r = 0; r < cr; ++r) run0 = max(run0, *peer(xchg, r));
+                return run0;
+            },
+            [&](uint32_t g, uint32_t f, uint32_t& g0, uint32_t& f0) {       // groups in the tiles before this one
+                g0 = f0 = 0;
+                if (threadIdx.x == 0) { xchg[1] = (int)g; xchg[2] = (int)f; }
+                sync_cluster();
+                for (int r = 0; r < cr; ++r) { const int* x = peer(xchg, r); g0 += (uint32_t)x[1]; f0 += (uint32_t)x[2]; }
+                if (cr == CL - 1 && threadIdx.x == 0) *plan.totals = make_uint2(g0 + g, f0 + f);
+            });
+        sync_cluster();                                                     // nobody leaves while its keys may still be read
+    }
+}
+
+bool sort_small_fits(const SortBatch& batch) {
+    for (int j = 0; j < batch.n_jobs; ++j)
+        if (batch.job[j].n_max > SS_CLUSTER * SS_THREADS * 8 || !batch.job[j].ids || batch.job[j].n_dev) return false;
+    return true;
+}
+
+// Sorts every job of the batch into its first buffer pair; plan (totals not null): the last job's accumulate plan.
+cudaError_t launch_sort_small(const gear_ctx_impl& c, const SortBatch& batch, const PlanArgs& plan, cudaStream_t st) {
+    int64_t n = 0;
+    for (int j = 0; j < batch.n_jobs; ++j) n = batch.job[j].n_max > n ? batch.job[j].n_max : n;
+    KernelScope k(&c.prof, batch.name, st);
+    auto launch = [&](auto kernel, int smem, int cl) -> cudaError_t {
+        cudaError_t e = smem > 48 * 1024 ? cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) : cudaSuccess;
+        return e == cudaSuccess ? launch_dependent(kernel, dim3(batch.n_jobs * cl), dim3(SS_THREADS), smem, st, batch, plan) : e;
+    };
+    // one block while a tile holds the longest array (no cluster barriers); tiles of 2048 entries, then of 4096
+    if (n <= SS_THREADS * 4) return launch(sort_small_kernel<4, 1>, ss_smem<4>(), 1);
+    if (n <= SS_CLUSTER * SS_THREADS * 4) return launch(sort_small_kernel<4, SS_CLUSTER>, ss_smem<4>(), SS_CLUSTER);
+    return launch(sort_small_kernel<8, SS_CLUSTER>, ss_smem<8>(), SS_CLUSTER);
+}
+
+}  // namespace gear

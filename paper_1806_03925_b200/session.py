@@ -113,25 +113,36 @@ class GearSession:
         self._expired_ids_g = torch.full((self.expired_cap + 1,), self.GUARD_I, dtype=torch.int32, device=dev)
         self.expired_ids = self._expired_ids_g[:self.expired_cap]
         self.d_counts = self.scalars[1:3]
-        self._expiry_stream = None
-        self._step_out = None
+        self._step_out = self._step_lists = None
 
     # ---- the four calls of a step ---------------------------------------------------------------
     def forward_backward(self, b: DeviceBatch, lr: Optional[float] = None):
-        # the output struct never changes and a batch's struct only in its counts: both are made once
-        if self._step_out is None:
-            self._step_out = gb.make_step_out(self.loss, self.head_grad, self.dX, prob=self.prob, row_view=self.row_view,
+        o = self._step_out or self._make_step_out()
+        if self.adam is not None:
+            self.adam_step += 1
+            o.adam_step = self.adam_step
+        return gb.gear_forward_backward_structs(self.ctx, self._c_batch(b), self.p.lr if lr is None else lr, o)
+
+    # the structs of the outputs never change and a batch's struct only in its counts: all are made once
+    def _make_step_out(self):
+        self._step_out = gb.make_step_out(self.loss, self.head_grad, self.dX, prob=self.prob, row_view=self.row_view,
                                               inv_n=self.inv_n, x_debug=self.x_debug, user_grad=self.user_grad,
                                               url_grad=self.url_grad, dfv_grad=self.dfv_grad, adam=self.adam, user_m=self.user_m,
                                               user_v=self.user_v, url_m=self.url_m, url_v=self.url_v)
-        if self.adam is not None:
-            self.adam_step += 1
-            self._step_out.adam_step = self.adam_step
-        bt = b.__dict__.get("_c_batch")
+        return self._step_out
+
+    def _make_step_lists(self):
+        self._step_lists = gb.make_step_lists(self.ready_ids, self.ready_seq, self.ready_avg, self.ready_cap, self.expired_ids,
+                                              self.expired_cap, d_n=self.d_counts[0:1], d_expired=self.d_counts[1:2])
+        return self._step_lists
+
+    @staticmethod
+    def _c_batch(b: DeviceBatch):
+        bt = b.__dict__.get("_c_struct")
         if bt is None:
-            bt = b.__dict__["_c_batch"] = gb.make_batch(b.user_id, b.url_id, b.img_off, b.img_id, b.label, fast=b.fast)
+            bt = b.__dict__["_c_struct"] = gb.make_batch(b.user_id, b.url_id, b.img_off, b.img_id, b.label, fast=b.fast)
         bt.B, bt.nnz = b.B, b.nnz
-        return gb.gear_forward_backward_structs(self.ctx, bt, self.p.lr if lr is None else lr, self._step_out)
+        return bt
 
     def accumulate_from_step(self, b: DeviceBatch, reuse_sorted_ids: bool = True):
         """Event 5 in its indirect form: row r of the batch is dX[row_view[r], 2E:] * inv_n[row_view[r]].
@@ -182,30 +193,14 @@ class GearSession:
         return gb.gear_dense_backward(self.ctx, raw, self.ready_ids, self.ready_avg, n, Wd_grad, d_n=d_n)
 
     def step(self, b: DeviceBatch, now: int, sync: bool = False, expiry_beside: Optional[bool] = None):
-        """One pass of the whole hot path over one batch.  The expiry scan depends on nothing the training calls
-        produce: with expiry_beside it goes to a stream of its own, starts when the step starts and is joined
-        at the step's end, so that it runs beside the gather and the head.  Default: beside for tables of 4M images
-        or more (the fork and join cost the host more than a scan of a small table takes on the device)."""
-        if expiry_beside is None:
-            expiry_beside = self.p.img_vocab >= (1 << 22)
-        if not expiry_beside:
-            self.forward_backward(b)
-            n_ready = self.accumulate_collect_from_step(b, sync=sync)
-            n_exp = self.collect_expired(now, restamp=True, sync=sync)
-            return n_ready, n_exp
-        main = torch.cuda.current_stream()
-        if self._expiry_stream is None:
-            self._expiry_stream = torch.cuda.Stream()
-            self._ev_fork, self._ev_join = torch.cuda.Event(), torch.cuda.Event()
-        self._ev_fork.record(main)
-        self._expiry_stream.wait_event(self._ev_fork)      # earlier readers of expired_ids and the count are done
-        with torch.cuda.stream(self._expiry_stream):
-            n_exp = self.collect_expired(now, restamp=True, sync=sync)
-            self._ev_join.record(self._expiry_stream)
-        self.forward_backward(b)
-        n_ready = self.accumulate_collect_from_step(b, sync=sync)
-        main.wait_event(self._ev_join)
-        return n_ready, n_exp
+        """One pass of the whole hot path over one batch (gear_step).  The expiry scan depends on nothing the training
+        calls produce and runs beside them (expiry_beside=False: behind them)."""
+        beside = True if expiry_beside is None else expiry_beside
+        o, lists = self._step_out or self._make_step_out(), self._step_lists or self._make_step_lists()
+        if self.adam is not None:
+            self.adam_step += 1
+            o.adam_step = self.adam_step
+        return gb.gear_step_structs(self.ctx, self._c_batch(b), self.p.lr, o, lists, now, True, beside, sync)
 
     def status(self):
         return gb.gear_status(self.ctx)
