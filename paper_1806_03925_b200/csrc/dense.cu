@@ -8,9 +8,9 @@
 //   Adam            Section 4: the optimiser of the paper's experiments, for dense parameter vectors (head, Wd) and for
 //                   the rows of an embedding table that received a gradient in this step.
 //
-// The two products are fp32 FMA products with one operand gathered by Image ID (the tolerance is 1e-5; reductions of
-// a few dozen to a few hundred terms).  64 x 64 x 16 tiles through shared memory, 4 x 4 outputs per thread.
+// The two products are fp32 FMA products with one operand gathered by Image ID (the tolerance is 1e-5).
 #include "common.cuh"
+#include "f32_chain.cuh"
 #include "internal.h"
 
 namespace gear {
@@ -19,64 +19,47 @@ constexpr int DT = 64;     // tile edge
 constexpr int DK = 16;     // tile depth
 
 // rows[k][c] = sum_r raw[ids[k]][r] * Wd[r][c],  k < min(n, *d_n),  c < D.  An ID outside [0, vocab) gives a zero row.
-__global__ void __launch_bounds__(256)
+// A chain of R multiply-adds per output cannot be cut, so small tiles spread the live rows over the SMs (2500 rows of 1536
+// values, 64 columns: 40 blocks of 64 x 64 took 242 us), and blocks walk the tiles so that a capacity far above the live
+// count costs nothing.  AVEC / BVEC: raw rows / Wd rows may be read 16 bytes at a time.
+template <bool AVEC, bool BVEC>
+__global__ void __launch_bounds__(128)
 dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const float* __restrict__ Wd, int D,
                      const int32_t* __restrict__ ids, int64_t n, const int64_t* __restrict__ d_n,
                      float* __restrict__ rows, int64_t ld, DevState* __restrict__ state) {
     wait_for_predecessor();
+    constexpr int BM = 16, BN = 64, TM = 2, TN = 4;
+    using T = ChainTile<BM, BN, TM, TN, 32>;
+    __shared__ __align__(16) typename T::Smem smem;
+    __shared__ int64_t row_of[BM];
     if (d_n) { const int64_t live = *d_n; n = live < n ? (live < 0 ? 0 : live) : n; }
-    const int64_t m0 = (int64_t)blockIdx.x * DT;           // row tiles along x: an expiry list can hold millions of IDs
-    if (m0 >= n) return;
-    __shared__ float As[DK][DT + 4];
-    __shared__ float Bs[DK][DT + 4];
-    __shared__ int64_t row_of[DT];
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int n0 = blockIdx.y * DT;
-    if (tid < DT) {
-        int64_t id = -1;
-        if (m0 + tid < n) {
-            id = ids[m0 + tid];
-            if (id < 0 || id >= vocab) { id = -1; atomicOr(&state->status, GEAR_DEV_BAD_ID); }
-        }
-        row_of[tid] = id;
-    }
-    __syncthreads();
-    float acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-    for (int k0 = 0; k0 < R; k0 += DK) {
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int idx = tid + r * 256;
-            const int m = idx >> 4, k = idx & 15;                  // A: the reduction index is the fast one
-            const int64_t id = row_of[m];
-            As[k][m] = (id >= 0 && k0 + k < R) ? __ldg(raw + id * R + k0 + k) : 0.f;
-            const int kb = idx >> 6, c = idx & 63;                 // B: the column is the fast one
-            Bs[kb][c] = (k0 + kb < R && n0 + c < D) ? __ldg(Wd + (int64_t)(k0 + kb) * D + n0 + c) : 0.f;
+    const int n0 = blockIdx.y * BN;
+    for (int64_t m0 = (int64_t)blockIdx.x * BM; m0 < n; m0 += (int64_t)gridDim.x * BM) {
+        __syncthreads();                                          // the tile before this one has been read
+        if (threadIdx.x < BM) {
+            int64_t id = -1;
+            if (m0 + threadIdx.x < n) {
+                id = ids[m0 + threadIdx.x];
+                if (id < 0 || id >= vocab) { id = -1; atomicOr(&state->status, GEAR_DEV_BAD_ID); }
+            }
+            row_of[threadIdx.x] = id;
         }
         __syncthreads();
+        f32x2 acc[TM][TN / 2];
 #pragma unroll
-        for (int k = 0; k < DK; ++k) {
-            const float4 a4 = *reinterpret_cast<const float4*>(&As[k][ty * 4]);
-            const float4 b4 = *reinterpret_cast<const float4*>(&Bs[k][tx * 4]);
-            const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+        for (int i = 0; i < TM; ++i)
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+        T::product(acc, R, smem, [&](int r, int k) { const int64_t id = row_of[r]; return load4<AVEC>(raw + id * R + k, id >= 0 ? R - k : 0); },
+                   [&](int k, int c) { return load4<BVEC>(Wd + (int64_t)k * D + n0 + c, k < R ? D - (n0 + c) : 0); });
 #pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int64_t m = m0 + ty * 4 + i;
-        if (m >= n) continue;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = n0 + tx * 4 + j;
-            if (c < D) rows[m * ld + c] = acc[i][j];
+        for (int i = 0; i < TM; ++i) {
+            const int64_t m = m0 + T::row(i);
+            const int c = n0 + T::col(0);
+            if (m >= n || c >= D) continue;                       // D is a multiple of 8: whole strips
+            const float2 lo = unpack2(acc[i][0]), hi = unpack2(acc[i][1]);
+            float* dst = rows + m * ld + c;
+            dst[0] = lo.x; dst[1] = lo.y; dst[2] = hi.x; dst[3] = hi.y;
         }
     }
 }
@@ -145,19 +128,23 @@ cudaError_t launch_dense_forward(const gear_ctx_impl& c, const float* raw, int R
                                  int64_t n, const int64_t* d_n, float* rows, int64_t ld, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     KernelScope k(&c.prof, "dense_forward", st);
-    const dim3 grid((unsigned)ceil_div(n, DT), (unsigned)ceil_div(c.cfg.dfv_dim, DT));
-    return launch_dependent(dense_forward_kernel, grid, dim3(256), 0, st, raw, c.cfg.img_vocab, R, Wd, c.cfg.dfv_dim, ids, n, d_n,
-                            rows, ld, c.state());
+    const int64_t want = ceil_div(n, 16), cap = (int64_t)sm_count() * 8;
+    const dim3 grid((unsigned)(want < cap ? want : cap), (unsigned)ceil_div(c.cfg.dfv_dim, 64));
+    const bool avec = (R & 3) == 0 && (reinterpret_cast<uintptr_t>(raw) & 15u) == 0, bvec = (reinterpret_cast<uintptr_t>(Wd) & 15u) == 0;
+#define GEAR_DF(A, B) launch_dependent(dense_forward_kernel<A, B>, grid, dim3(128), 0, st, raw, c.cfg.img_vocab, R, Wd, c.cfg.dfv_dim, ids, n, d_n, rows, ld, c.state())
+    return avec ? (bvec ? GEAR_DF(true, true) : GEAR_DF(true, false)) : (bvec ? GEAR_DF(false, true) : GEAR_DF(false, false));
+#undef GEAR_DF
 }
 
 cudaError_t launch_dense_backward(const gear_ctx_impl& c, const float* raw, int R, const int32_t* ids, const float* avg,
                                   int64_t ld_avg, int64_t n, const int64_t* d_n, float* G, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     KernelScope k(&c.prof, "dense_backward", st);
-    // slices of the emission list: enough of them to fill the GPU a few times over, each at least 256 emissions long
+    // slices of the emission list: enough of them to fill the GPU a few times over, each at least 64 emissions long (the list's
+    // live count is usually far below n: 256 of 1024 emissions were one slice of 24 blocks, 32 us)
     const int64_t tiles = ceil_div(c.cfg.dfv_dim, DT) * ceil_div(R, DT);
     int64_t slices = ceil_div((int64_t)sm_count() * 8, tiles);
-    const int64_t max_slices = ceil_div(n, 256);
+    const int64_t max_slices = ceil_div(n, 64);
     if (slices > max_slices) slices = max_slices;
     if (slices < 1) slices = 1;
     if (slices > 65535) slices = 65535;

@@ -1,0 +1,115 @@
+// Products of fp32 matrices with one ascending chain of multiply-adds per output (head_fwd.cu, dense.cu).
+//
+// Multiply-adds are issued in pairs (fma.rn.f32x2: two independent fp32 multiply-adds, each rounded like fmaf), which
+// leaves issue slots for the shared-memory reads.  Bound: the fp32 lanes (128 multiply-adds per SM and cycle) for large
+// products, the length of the chain for small ones.
+#pragma once
+
+#include "common.cuh"
+
+namespace gear {
+
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 dup2(float a) { f32x2 r; asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a)); return r; }
+__device__ __forceinline__ void fma2(f32x2& d, f32x2 a, f32x2 b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
+__device__ __forceinline__ float2 unpack2(f32x2 v) { float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
+
+// 4 consecutive values of a row; VEC: one 16-byte load, else one by one, `left` of them within the row
+template <bool VEC> __device__ __forceinline__ float4 load4(const float* __restrict__ p, int left) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (left <= 0) return v;
+    if (VEC) return __ldg(reinterpret_cast<const float4*>(p));
+    v.x = __ldg(p);
+    if (left > 1) v.y = __ldg(p + 1);
+    if (left > 2) v.z = __ldg(p + 2);
+    if (left > 3) v.w = __ldg(p + 3);
+    return v;
+}
+
+// A block of (BM / TM) * (BN / TN) threads computes BM x BN outputs, a thread TM x TN of them: rows in strips of
+// ChainTile::RS, BM / (TM / RS) apart, columns in strips of four, BN / (TN / 4) apart, so that shared-memory reads are wide
+// and free of bank conflicts.  Operand tiles are fetched one step ahead into registers and pass through two shared-memory
+// buffers.  The A tile is transposed on its way in: neighbouring lanes fetch a row's BK values, and the row index is XORed so
+// that the 32 stores of a warp hit 32 banks.
+template <int BM, int BN, int TM, int TN, int BK> struct ChainTile {
+    static constexpr int THREADS = (BM / TM) * (BN / TN), TX = BN / TN, KQ = BK / 4;
+    static constexpr int A_PIECES = BM * KQ / THREADS, B_PIECES = BK * (BN / 4) / THREADS;      // 4-value pieces per thread
+    static constexpr int RS = TM < 4 ? TM : 4;
+    static constexpr int SW = 32 / KQ < 4 ? 4 : 32 / KQ;             // the XOR's unit: rows a warp's store covers per k
+    static_assert(A_PIECES >= 1 && B_PIECES >= 1 && A_PIECES * THREADS == BM * KQ && B_PIECES * THREADS == BK * (BN / 4), "whole pieces");
+    static_assert(TM % RS == 0 && (RS == 2 || RS == 4) && TN % 4 == 0 && BM % 16 == 0 && (KQ == 2 || KQ == 4 || KQ == 8), "strips");
+    struct Smem { float a[2][BK][BM]; float b[2][BK][BN]; };
+    static __device__ __forceinline__ int swizzle(int kq) { return (kq * SW) % BM; }
+    // row / first column of the tile that output (i, 4 j) of this thread stands for
+    static __device__ __forceinline__ int row(int i) { return (i / RS) * (BM / (TM / RS)) + (int)(threadIdx.x / TX) * RS + i % RS; }
+    static __device__ __forceinline__ int col(int j) { return j * (BN / (TN / 4)) + (int)(threadIdx.x % TX) * 4; }
+
+    // acc += A . B over k < K; load_a(row of the tile, k), load_b(k, column of the tile): four consecutive values (along k / the
+    // columns), zeros where there are none
+    template <typename LoadA, typename LoadB>
+    static __device__ __forceinline__ void product(f32x2 (&acc)[TM][TN / 2], int K, Smem& s, LoadA load_a, LoadB load_b) {
+        const int tid = threadIdx.x;
+        float4 ra[A_PIECES], rb[B_PIECES];
+        auto fetch = [&](int k0) {
+#pragma unroll
+            for (int q = 0; q < A_PIECES; ++q) { const int p = tid + q * THREADS; ra[q] = load_a(p / KQ, k0 + 4 * (p % KQ)); }
+#pragma unroll
+            for (int q = 0; q < B_PIECES; ++q) { const int p = tid + q * THREADS; rb[q] = load_b(k0 + p / (BN / 4), 4 * (p % (BN / 4))); }
+        };
+        auto stash = [&](int buf) {
+#pragma unroll
+            for (int q = 0; q < A_PIECES; ++q) {
+                const int p = tid + q * THREADS, kq = p % KQ, m = (p / KQ) ^ swizzle(kq);
+                s.a[buf][4 * kq][m] = ra[q].x; s.a[buf][4 * kq + 1][m] = ra[q].y;
+                s.a[buf][4 * kq + 2][m] = ra[q].z; s.a[buf][4 * kq + 3][m] = ra[q].w;
+            }
+#pragma unroll
+            for (int q = 0; q < B_PIECES; ++q) {
+                const int p = tid + q * THREADS;
+                st_f4(&s.b[buf][p / (BN / 4)][4 * (p % (BN / 4))], rb[q]);
+            }
+        };
+        fetch(0);
+        stash(0);
+        __syncthreads();
+        int buf = 0;
+        for (int k0 = 0; k0 < K; k0 += BK) {
+            const bool more = k0 + BK < K;
+            if (more) fetch(k0 + BK);
+#pragma unroll
+            for (int k = 0; k < BK; ++k) {
+                float a[TM];
+                f32x2 b[TN / 2];
+#pragma unroll
+                for (int i = 0; i < TM / RS; ++i) {
+                    const float* p = &s.a[buf][k][row(i * RS) ^ swizzle(k / 4)];
+                    if constexpr (RS == 4) {
+                        const float4 t = ld_f4(p);
+                        a[4 * i] = t.x; a[4 * i + 1] = t.y; a[4 * i + 2] = t.z; a[4 * i + 3] = t.w;
+                    } else {
+                        const float2 t = *reinterpret_cast<const float2*>(p);
+                        a[2 * i] = t.x; a[2 * i + 1] = t.y;
+                    }
+                }
+#pragma unroll
+                for (int j = 0; j < TN / 4; ++j) {
+                    const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(&s.b[buf][k][col(j)]);
+                    b[2 * j] = t.x; b[2 * j + 1] = t.y;
+                }
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    const f32x2 aa = dup2(a[i]);
+#pragma unroll
+                    for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], aa, b[j]);
+                }
+            }
+            if (more) {
+                stash(buf ^ 1);                                     // the other buffer: nobody reads it during this step
+                __syncthreads();
+                buf ^= 1;
+            }
+        }
+    }
+};
+
+}  // namespace gear
