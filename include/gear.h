@@ -311,6 +311,32 @@ int gear_apply_emb_grad(gear_ctx* ctx, int32_t which, const int32_t* ids, const 
                         float lr, void* stream);
 
 /*
+ * The same exchange when the shards of all ranks are memory of this device (any number of ranks up to
+ * GEAR_MAX_LOCAL_RANKS): no rows travel through send and receive buffers.  All lists are the workers' lists one behind the
+ * other, sender by sender; start[s] is where sender s's entries begin, start[world] their number (host array, [3][world + 1],
+ * tables in the order user, URL, images).
+ *
+ * gear_shard_fetch     events 1 to 3: row k of sender s gets row (id div world) of the table shard of owner (id mod world), for
+ *                      all three tables: out[t] + (s * out_stride[t] + k) rows.  An ID outside its owner's shard gives a zero
+ *                      row and raises GEAR_DEV_BAD_ID at the owner.
+ * gear_shard_route     picks every owner's arrivals out of the lists, in arrival order (sender by sender, each in its own row
+ *                      order): local[t][owner][.] = id div world, src[t][owner][.] = s * src_stride[t] + k;
+ *                      both arrays are [world][start[world]] per table.  counts (device, [3][world]): their numbers.
+ * gear_owner_step      what one owner does with its arrivals: the same results as gear_apply_emb_grad on both tables,
+ *                      gear_accumulate_collect and gear_collect_expired.  The gradient row of entry k of a list is row
+ *                      src[k]: of emb_rows (user gradient in columns 0 .. emb_dim, URL gradient behind it), and of img_rows.
+ */
+enum { GEAR_MAX_LOCAL_RANKS = 8 };
+typedef struct { const int32_t* ids; const int32_t* src; int64_t n; } gear_arrivals;
+int gear_shard_fetch(gear_ctx* const* owners, int32_t world, const int32_t* const* ids, const int32_t* start, void* const* out,
+                     const int64_t* out_stride, void* stream);
+int gear_shard_route(int32_t world, const int32_t* const* ids, const int32_t* start, const int64_t* src_stride,
+                     int32_t* const* local, int32_t* const* src, int32_t* counts, void* stream);
+int gear_owner_step(gear_ctx* ctx, const gear_arrivals* user, const gear_arrivals* url, const gear_arrivals* img,
+                    const float* emb_rows, int64_t emb_ld, const float* img_rows, int64_t img_ld, float lr,
+                    const gear_step_lists* lists, int64_t now, int restamp, void* stream);
+
+/*
  * The smallest Dense Part there is, for closing the loop on one device: DFV[id] = raw[id] . Wd, with raw
  * [img_vocab][raw_dim] the images' raw feature rows and Wd [raw_dim][dfv_dim] the Dense Part's weights (fp32, device,
  * row-major).

@@ -216,7 +216,10 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     bool small_sort = false;
     const bool plan = b.nnz > 0 && o.row_view && o.inv_n && sorted_mode;
     SortBatch batch = c.sort_batch();
-    if (b.B > 0) {
+    // a learning rate of zero moves no embedding row: nothing to sort for, nothing to scatter (a worker whose tables are
+    // copies of rows that live elsewhere passes it)
+    const bool scatters = lr != 0.f || o.adam || o.user_grad;
+    if (b.B > 0 && scatters) {
         batch.job[0] = c.sort_job(gear_ctx_impl::SORT_USER);
         batch.job[0].ids = b.user_id; batch.job[0].sentinel = (uint32_t)c.cfg.user_vocab;
         batch.job[0].n_max = b.B; batch.job[0].bits = bits_for(c.cfg.user_vocab);
@@ -224,15 +227,17 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
         batch.job[1].ids = b.url_id; batch.job[1].sentinel = (uint32_t)c.cfg.url_vocab;
         batch.job[1].n_max = b.B; batch.job[1].bits = bits_for(c.cfg.url_vocab);
         batch.n_jobs = 2;
+    }
+    if (b.B > 0) {
         if (b.nnz > 0 && sorted_mode) {      // the atomic mode takes the image IDs as they come
-            batch.job[2] = c.sort_job(gear_ctx_impl::SORT_IMG);
-            batch.job[2].ids = b.img_id; batch.job[2].sentinel = (uint32_t)c.cfg.img_vocab;
-            batch.job[2].n_max = b.nnz; batch.job[2].bits = bits_for(c.cfg.img_vocab);
-            batch.n_jobs = 3;
+            SortJob& j = batch.job[batch.n_jobs++];
+            j = c.sort_job(gear_ctx_impl::SORT_IMG);
+            j.ids = b.img_id; j.sentinel = (uint32_t)c.cfg.img_vocab;
+            j.n_max = b.nnz; j.bits = bits_for(c.cfg.img_vocab);
         }
         batch.name = "sort_ids";
-        small_sort = sort_small_fits(batch);
-        if (!small_sort) sorted_buf = sort_jobs(batch, &c.gbs, side, &c.prof, &e);
+        small_sort = batch.n_jobs > 0 && sort_small_fits(batch);
+        if (batch.n_jobs > 0 && !small_sort) sorted_buf = sort_jobs(batch, &c.gbs, side, &c.prof, &e);
         if (e != cudaSuccess) return e;
         if (b.nnz > 0) {
             c.img_sorted = true; c.img_sorted_n = b.nnz; c.img_sorted_buf = sorted_buf; c.last_img_id = b.img_id;
@@ -267,7 +272,7 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
         return launch_emb_reduce(c, k.sorted_buf, k.B, o.user_grad ? o.user_grad : c.buf.user_emb, o.url_grad ? o.url_grad : c.buf.url_emb,
                                  o.dX, c.d_in, o.user_grad ? 1.0f : -k.lr, k.side);
     };
-    const HeadHooks hooks{scatter, &sc, dw_beside ? aux : st, &c.ev[EV_AUX + 1]};
+    const HeadHooks hooks{scatters ? +scatter : nullptr, &sc, dw_beside ? aux : st, &c.ev[EV_AUX + 1]};
     GEAR_TRY(launch_head(c, b, o, st, hooks));
     if (o.dfv_grad && b.B > 0) GEAR_TRY(launch_dfv_grad_rows(c, o.dX, o.row_view, o.inv_n, b.nnz, o.dfv_grad, st));
     if (lists) {
@@ -538,6 +543,128 @@ int gear_apply_emb_grad(gear_ctx* ctx, int32_t which, const int32_t* ids, const 
     if (!ids || !rows || !aligned16(rows) || ld < c.cfg.emb_dim || (ld & 3)) return arg_fail("rows: 16-byte aligned, ld >= emb_dim, multiple of 4");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     return run_call(c, "apply_emb_grad", st, [&] { return launch_apply_emb_grad(c, which, ids, rows, ld, n, -lr, st); });
+}
+
+int gear_shard_fetch(gear_ctx* const* owners, int32_t world, const int32_t* const* ids, const int32_t* start, void* const* out,
+                     const int64_t* out_stride, void* stream) {
+    if (!owners || !ids || !start || !out || !out_stride || world < 1 || world > GEAR_MAX_LOCAL_RANKS) return arg_fail("gear_shard_fetch");
+    ShardFetch f{};
+    f.world = world;
+    for (int r = 0; r < world; ++r) {
+        if (!owners[r] || !owners[r]->impl.alive) return GEAR_ERR_STATE;
+        const gear_ctx_impl& c = owners[r]->impl;
+        const gear_config &g = c.cfg, &g0 = owners[0]->impl.cfg;
+        if (g.emb_dim != g0.emb_dim || g.dfv_dim != g0.dfv_dim || g.dfv_dtype != g0.dfv_dtype) return arg_fail("the shards' rows differ");
+        f.state[r] = c.state();
+        const void* shard[3] = {c.buf.user_emb, c.buf.url_emb, c.buf.dfv};
+        const int64_t rows[3] = {g.user_vocab, g.url_vocab, g.img_vocab};
+        for (int t = 0; t < 3; ++t) { f.table[t].shard[r] = static_cast<const uint4*>(shard[t]); f.table[t].rows[r] = rows[t]; }
+    }
+    const gear_config& g = owners[0]->impl.cfg;
+    bool any = false;
+    for (int t = 0; t < 3; ++t) {
+        ShardFetch::Table& x = f.table[t];
+        x.chunks = t < 2 ? g.emb_dim / 4 : g.dfv_dim / (g.dfv_dtype == GEAR_BF16 ? 8 : 4);
+        x.ids = ids[t]; x.out = static_cast<uint4*>(out[t]); x.out_stride = out_stride[t];
+        for (int r = 0; r <= world; ++r) x.start[r] = start[t * (world + 1) + r];
+        if (x.start[world] > 0 && (!ids[t] || !out[t] || !aligned16(out[t]))) return arg_fail("NULL or misaligned pointer");
+        any = any || x.start[world] > 0;
+    }
+    if (!any) return GEAR_OK;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    for (int r = 0; r < world; ++r) owners[r]->impl.note_stream(st);
+    cudaError_t e = launch_shard_fetch(&owners[0]->impl.prof, f, st);
+    return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "shard_fetch");
+}
+
+int gear_shard_route(int32_t world, const int32_t* const* ids, const int32_t* start, const int64_t* src_stride, int32_t* const* local,
+                     int32_t* const* src, int32_t* counts, void* stream) {
+    if (!ids || !start || !src_stride || !local || !src || !counts || world < 1 || world > GEAR_MAX_LOCAL_RANKS) return arg_fail("gear_shard_route");
+    ShardRoute r{};
+    r.world = world; r.counts = counts;
+    for (int t = 0; t < 3; ++t) {
+        ShardRoute::Table& x = r.table[t];
+        x.ids = ids[t]; x.local = local[t]; x.src = src[t]; x.src_stride = src_stride[t];
+        for (int k = 0; k <= world; ++k) x.start[k] = start[t * (world + 1) + k];
+        if (x.start[world] > 0 && (!ids[t] || !local[t] || !src[t])) return arg_fail("NULL pointer");
+    }
+    cudaError_t e = launch_shard_route(nullptr, r, static_cast<cudaStream_t>(stream));
+    return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "shard_route");
+}
+
+int gear_owner_step(gear_ctx* ctx, const gear_arrivals* user, const gear_arrivals* url, const gear_arrivals* img, const float* emb_rows,
+                    int64_t emb_ld, const float* img_rows, int64_t img_ld, float lr, const gear_step_lists* lists, int64_t now,
+                    int restamp, void* stream) {
+    if (!ctx || !ctx->impl.alive) return GEAR_ERR_STATE;
+    if (!user || !url || !img || !lists) return arg_fail("NULL pointer");
+    gear_ctx_impl& c = ctx->impl;
+    if (user->n < 0 || user->n > c.cfg.max_batch || url->n < 0 || url->n > c.cfg.max_batch) return arg_fail("n outside [0, max_batch]");
+    if (img->n < 0 || img->n > c.cfg.max_nnz) return arg_fail("n outside [0, max_nnz]");
+    if ((user->n || url->n) && (!emb_rows || !aligned16(emb_rows) || emb_ld < 2 * c.cfg.emb_dim || (emb_ld & 3)))
+        return arg_fail("emb_rows: 16-byte aligned, ld >= 2 emb_dim, multiple of 4");
+    if (img->n && (!img_rows || !aligned16(img_rows) || img_ld < c.cfg.dfv_dim || (img_ld & 3)))
+        return arg_fail("img_rows: 16-byte aligned, ld >= dfv_dim, multiple of 4");
+    for (const gear_arrivals* a : {user, url, img})
+        if (a->n > 0 && (!a->ids || !a->src)) return arg_fail("NULL list");
+    if (int rc = check_lists(lists->ids, lists->seq, lists->avg, lists->cap)) return rc;
+    if (lists->expired_cap < 0 || (lists->expired_cap > 0 && !lists->expired)) return arg_fail("NULL output with cap > 0");
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    int64_t* d_n = lists->d_n ? lists->d_n : &c.state()->pad[0];
+    int64_t* d_expired = lists->d_expired ? lists->d_expired : &c.state()->pad[1];
+    return run_call(c, "owner_step", st, [&]() -> cudaError_t {
+#define GEAR_TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return e_; } while (0)
+        const bool apart = !c.prof.on || c.prof.keep_streams, sorted_mode = c.cfg.accum_mode == GEAR_ACC_SORT;
+        const cudaStream_t side = apart ? c.side_stream : st, aux = apart ? c.aux_stream : st;
+        if (apart) {
+            GEAR_TRY(enqueue_record(c.ev[0], st));
+            GEAR_TRY(enqueue_wait(aux, c.ev[0]));
+        }
+        GEAR_TRY(launch_collect_expired(c, now, restamp, lists->expired, lists->expired_cap, d_expired, aux));
+        SortBatch batch = c.sort_batch();
+        batch.name = "sort_ids";
+        auto add = [&](const gear_arrivals& a, int which, int64_t vocab) {
+            if (a.n == 0) return;
+            SortJob& j = batch.job[batch.n_jobs++];
+            j = c.sort_job(which);
+            j.ids = a.ids; j.src = a.src; j.sentinel = (uint32_t)vocab; j.n_max = a.n; j.bits = bits_for(vocab);
+        };
+        c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
+        add(*user, gear_ctx_impl::SORT_USER, c.cfg.user_vocab);
+        add(*url, gear_ctx_impl::SORT_URL, c.cfg.url_vocab);
+        if (sorted_mode) add(*img, gear_ctx_impl::SORT_IMG, c.cfg.img_vocab);
+        const bool plan = sorted_mode && img->n > 0;
+        int cur = 0;
+        if (batch.n_jobs > 0) {
+            if (sort_small_fits(batch)) GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, img->n, nullptr, nullptr) : PlanArgs{}, st));
+            else {
+                cudaError_t se;
+                cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
+                if (se != cudaSuccess) return se;
+            }
+        }
+        if (apart) {
+            GEAR_TRY(enqueue_record(c.ev[1], st));
+            GEAR_TRY(enqueue_wait(side, c.ev[1]));
+        }
+        GEAR_TRY(launch_emb_arrivals(c, cur, user->n, url->n, c.buf.user_emb, c.buf.url_emb, emb_rows, emb_ld, -lr, side));
+        if (plan) {
+            c.img_sorted = true; c.img_sorted_n = img->n; c.img_sorted_buf = cur; c.img_sort_valid = true; c.last_img_id = img->ids;
+            if (sort_small_fits(batch)) note_plan(c, img->n, nullptr, nullptr);
+            else GEAR_TRY(launch_accumulate_plan_ahead(c, img->n, nullptr, nullptr, st));
+        }
+        // (the sorted values are the source rows, so the accumulate call itself has no row indirection left)
+        GEAR_TRY(launch_accumulate_collect(c, plan ? nullptr : img->ids, img_rows, img_ld, plan ? nullptr : img->src, nullptr, img->n, lists->ids,
+                                           lists->seq, lists->avg, lists->cap, d_n, st));
+        c.img_sorted = false; c.img_sort_valid = false;
+        if (apart) {
+            GEAR_TRY(enqueue_record(c.ev[2], side));
+            GEAR_TRY(enqueue_wait(st, c.ev[2]));
+            GEAR_TRY(enqueue_record(c.ev[3], aux));
+            GEAR_TRY(enqueue_wait(st, c.ev[3]));
+        }
+#undef GEAR_TRY
+        return cudaSuccess;
+    });
 }
 
 int gear_dense_forward(gear_ctx* ctx, const float* raw, int32_t raw_dim, const float* Wd, const int32_t* ids, int64_t n,

@@ -240,6 +240,7 @@ struct SortJob {
     const int64_t* n_dev;   // optional device-resident count, capped at n_max
     int bits;
     int identity_vals;
+    const int32_t* src;     // with identity_vals: the value of element i is src[i] instead, if set
     int width, n_tiles;     // filled in by sort_jobs
 };
 

@@ -15,21 +15,23 @@ constexpr int ES_SEG = 8;    // sorted positions walked by one lane group
 
 // LPR lanes share a row: lane c of the group owns the float4 chunks c, c + LPR, ... (NQ of them)
 // One of the two tables of a launch (blockIdx.y picks it).
-struct EmbTable { const uint32_t* ks; const uint32_t* perm; uint32_t vocab; int col0; float* table; };
+// n sorted (ID, row) pairs; row r of its gradient rows starts at rows + r * ld
+struct EmbTable { const uint32_t* ks; const uint32_t* perm; uint32_t vocab; int n; const float* rows; int64_t ld; float* table; };
 
 // COMPACT: the sums do not go to the table but to a buffer with one row per sorted position: an ID's sum lands in the
 // row of the position at which its run starts (table then points to that buffer, alpha is 1).  The optimiser's row
 // kernel (dense.cu) picks the sums up from there: a non-linear update needs an ID's whole sum before it can start.
 template <int NQ, bool COMPACT>
 __global__ void __launch_bounds__(256)
-emb_reduce_kernel(const EmbTable t0, const EmbTable t1, int n, int E, int lpr, const float* __restrict__ dX, int64_t ldx,
-                  float alpha) {
+emb_reduce_kernel(const EmbTable t0, const EmbTable t1, int E, int lpr, float alpha) {
     wait_for_predecessor();
     const EmbTable& t = blockIdx.y == 0 ? t0 : t1;
     const uint32_t* __restrict__ ks = t.ks;
     const uint32_t* __restrict__ perm = t.perm;
     const uint32_t vocab = t.vocab;
-    const int col0 = t.col0;
+    const int n = t.n;
+    const float* __restrict__ rows = t.rows;
+    const int64_t ld = t.ld;
     float* __restrict__ table = t.table;
     const int64_t gthread = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t group = gthread / lpr;
@@ -51,7 +53,7 @@ emb_reduce_kernel(const EmbTable t0, const EmbTable t1, int n, int E, int lpr, c
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
             const int ch = c + q * lpr;
-            v[t][q] = (key[t] < vocab && ch < n_chunks) ? ld_f4(dX + (int64_t)row[t] * ldx + col0 + ch * 4)
+            v[t][q] = (key[t] < vocab && ch < n_chunks) ? ld_f4(rows + (int64_t)row[t] * ld + ch * 4)
                                                         : make_float4(0.f, 0.f, 0.f, 0.f);
         }
     float4 acc[NQ];
@@ -91,27 +93,36 @@ emb_reduce_kernel(const EmbTable t0, const EmbTable t1, int n, int E, int lpr, c
     }
 }
 
-// both tables of a step in one launch: user rows (columns 0 .. E) and URL-hash rows (columns E .. 2E) of dX
-cudaError_t launch_emb_reduce(const gear_ctx_impl& c, int cur, int32_t B, float* user_table, float* url_table,
-                              const float* dX, int ldx, float alpha, cudaStream_t st) {
-    if (B <= 0) return cudaSuccess;
-    SortJob su = c.sort_job(gear_ctx_impl::SORT_USER), sh = c.sort_job(gear_ctx_impl::SORT_URL);
+// both tables in one launch
+template <bool COMPACT>
+static cudaError_t launch_emb_tables(const gear_ctx_impl& c, const EmbTable& t0, const EmbTable& t1, float alpha, cudaStream_t st) {
+    const int n = t0.n > t1.n ? t0.n : t1.n;
+    if (n <= 0) return cudaSuccess;
     const int E = c.cfg.emb_dim, n_chunks = E / 4;
     int lpr = 1;
     while (lpr < n_chunks && lpr < 32) lpr <<= 1;
     const int nq = (int)ceil_div(n_chunks, lpr);
-    const int64_t groups = ceil_div(B, ES_SEG);
-    const dim3 grid((unsigned)ceil_div(groups * lpr, 256), 2);
-    const EmbTable t0{su.keys[cur], su.vals[cur], (uint32_t)c.cfg.user_vocab, 0, user_table};
-    const EmbTable t1{sh.keys[cur], sh.vals[cur], (uint32_t)c.cfg.url_vocab, E, url_table};
-#define GEAR_ES_LAUNCH(NQ) launch_dependent(emb_reduce_kernel<NQ, false>, grid, dim3(256), 0, st, t0, t1, B, E, lpr, dX, (int64_t)ldx, alpha)
+    const dim3 grid((unsigned)ceil_div(ceil_div(n, ES_SEG) * lpr, 256), 2);
+#define GEAR_ES_LAUNCH(NQ) launch_dependent(emb_reduce_kernel<NQ, COMPACT>, grid, dim3(256), 0, st, t0, t1, E, lpr, alpha)
     KernelScope ks(&c.prof, "emb_reduce", st);
-    if (nq <= 1) GEAR_ES_LAUNCH(1);
-    else if (nq <= 2) GEAR_ES_LAUNCH(2);
-    else if (nq <= 4) GEAR_ES_LAUNCH(4);
-    else GEAR_ES_LAUNCH(8);
+    if (nq <= 1) return GEAR_ES_LAUNCH(1);
+    if (nq <= 2) return GEAR_ES_LAUNCH(2);
+    if (nq <= 4) return GEAR_ES_LAUNCH(4);
+    return GEAR_ES_LAUNCH(8);
 #undef GEAR_ES_LAUNCH
-    return cudaGetLastError();
+}
+
+// user rows (columns 0 .. E) and URL-hash rows (columns E .. 2E) of dX
+cudaError_t launch_emb_reduce(const gear_ctx_impl& c, int cur, int32_t B, float* user_table, float* url_table,
+                              const float* dX, int ldx, float alpha, cudaStream_t st) {
+    return launch_emb_arrivals(c, cur, B, B, user_table, url_table, dX, ldx, alpha, st);
+}
+cudaError_t launch_emb_arrivals(const gear_ctx_impl& c, int cur, int64_t n_user, int64_t n_url, float* user_table, float* url_table,
+                                const float* rows, int64_t ld, float alpha, cudaStream_t st) {
+    SortJob su = c.sort_job(gear_ctx_impl::SORT_USER), sh = c.sort_job(gear_ctx_impl::SORT_URL);
+    return launch_emb_tables<false>(c, EmbTable{su.keys[cur], su.vals[cur], (uint32_t)c.cfg.user_vocab, (int)n_user, rows, ld, user_table},
+                                    EmbTable{sh.keys[cur], sh.vals[cur], (uint32_t)c.cfg.url_vocab, (int)n_url, rows + c.cfg.emb_dim, ld, url_table},
+                                    alpha, st);
 }
 
 // Section 4's optimiser on the rows of both embedding tables that the batch touched: the per-ID sums go to the compact
@@ -120,29 +131,14 @@ cudaError_t launch_emb_adam(const gear_ctx_impl& c, int cur, int32_t B, const fl
                             int64_t t, float* user_m, float* user_v, float* url_m, float* url_v, cudaStream_t st) {
     if (B <= 0) return cudaSuccess;
     SortJob su = c.sort_job(gear_ctx_impl::SORT_USER), sh = c.sort_job(gear_ctx_impl::SORT_URL);
-    const int E = c.cfg.emb_dim, n_chunks = E / 4;
+    const int E = c.cfg.emb_dim;
     float* gu = c.at<float>(c.ws.emb_gsum[0]);
     float* gh = c.at<float>(c.ws.emb_gsum[1]);
     cudaError_t e = enqueue_memset(gu, sizeof(float) * (size_t)B * E, st);
     if (e == cudaSuccess) e = enqueue_memset(gh, sizeof(float) * (size_t)B * E, st);
     if (e != cudaSuccess) return e;
-    int lpr = 1;
-    while (lpr < n_chunks && lpr < 32) lpr <<= 1;
-    const int nq = (int)ceil_div(n_chunks, lpr);
-    const int64_t groups = ceil_div(B, ES_SEG);
-    const dim3 grid((unsigned)ceil_div(groups * lpr, 256), 2);
-    const EmbTable t0{su.keys[cur], su.vals[cur], (uint32_t)c.cfg.user_vocab, 0, gu};
-    const EmbTable t1{sh.keys[cur], sh.vals[cur], (uint32_t)c.cfg.url_vocab, E, gh};
-    {
-#define GEAR_ES_LAUNCH(NQ) launch_dependent(emb_reduce_kernel<NQ, true>, grid, dim3(256), 0, st, t0, t1, B, E, lpr, dX, (int64_t)ldx, 1.0f)
-        KernelScope ks(&c.prof, "emb_reduce", st);
-        if (nq <= 1) GEAR_ES_LAUNCH(1);
-        else if (nq <= 2) GEAR_ES_LAUNCH(2);
-        else if (nq <= 4) GEAR_ES_LAUNCH(4);
-        else GEAR_ES_LAUNCH(8);
-#undef GEAR_ES_LAUNCH
-    }
-    e = cudaGetLastError();
+    e = launch_emb_tables<true>(c, EmbTable{su.keys[cur], su.vals[cur], (uint32_t)c.cfg.user_vocab, B, dX, ldx, gu},
+                                EmbTable{sh.keys[cur], sh.vals[cur], (uint32_t)c.cfg.url_vocab, B, dX + E, ldx, gh}, 1.0f, st);
     if (e != cudaSuccess) return e;
     const EmbAdamTable a0{su.keys[cur], (uint32_t)c.cfg.user_vocab, c.buf.user_emb, user_m, user_v, gu};
     const EmbAdamTable a1{sh.keys[cur], (uint32_t)c.cfg.url_vocab, c.buf.url_emb, url_m, url_v, gh};
@@ -171,21 +167,10 @@ cudaError_t launch_apply_emb_grad(const gear_ctx_impl& c, int which, const int32
     if (sort_small_fits(batch)) se = launch_sort_small(c, batch, PlanArgs{}, st);
     else cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
     if (se != cudaSuccess) return se;
-    const int E = c.cfg.emb_dim, n_chunks = E / 4;
-    int lpr = 1;
-    while (lpr < n_chunks && lpr < 32) lpr <<= 1;
-    const int nq = (int)ceil_div(n_chunks, lpr);
-    const int64_t groups = ceil_div(n, ES_SEG);
-    const dim3 grid((unsigned)ceil_div(groups * lpr, 256), 1);
-    const EmbTable t0{batch.job[0].keys[cur], batch.job[0].vals[cur], (uint32_t)vocab, 0, user ? c.buf.user_emb : c.buf.url_emb};
-#define GEAR_ES_LAUNCH(NQ) launch_dependent(emb_reduce_kernel<NQ, false>, grid, dim3(256), 0, st, t0, t0, (int)n, E, lpr, rows, ld, alpha)
-    KernelScope ks(&c.prof, "emb_reduce", st);
-    if (nq <= 1) GEAR_ES_LAUNCH(1);
-    else if (nq <= 2) GEAR_ES_LAUNCH(2);
-    else if (nq <= 4) GEAR_ES_LAUNCH(4);
-    else GEAR_ES_LAUNCH(8);
-#undef GEAR_ES_LAUNCH
-    return cudaGetLastError();
+    const EmbTable t{batch.job[0].keys[cur], batch.job[0].vals[cur], (uint32_t)vocab, (int)n, rows, ld, user ? c.buf.user_emb : c.buf.url_emb};
+    EmbTable none = t;
+    none.n = 0;
+    return launch_emb_tables<false>(c, t, none, alpha, st);
 }
 
 }  // namespace gear

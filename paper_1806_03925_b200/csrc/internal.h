@@ -170,6 +170,10 @@ cudaError_t tc3_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, in
 cudaError_t launch_emb_reduce(const gear_ctx_impl& c, int buf, int32_t B, float* user_table, float* url_table,
                               const float* dX, int ldx, float alpha, cudaStream_t st);
 
+// the same for arrivals: rows [.][ld], user gradients in columns 0 .. emb_dim, URL gradients behind them
+cudaError_t launch_emb_arrivals(const gear_ctx_impl& c, int buf, int64_t n_user, int64_t n_url, float* user_table, float* url_table,
+                                const float* rows, int64_t ld, float alpha, cudaStream_t st);
+
 // dense.cu: a linear Dense Part (DFV = raw row . Wd) and Adam
 struct EmbAdamTable { const uint32_t* ks; uint32_t vocab; float* table; float* m; float* v; const float* gsum; };
 cudaError_t launch_dense_forward(const gear_ctx_impl& c, const float* raw, int R, const float* Wd, const int32_t* ids,
@@ -188,6 +192,27 @@ cudaError_t launch_emb_adam(const gear_ctx_impl& c, int buf, int32_t B, const fl
 cudaError_t launch_fetch_rows(const gear_ctx_impl& c, int which, const int32_t* ids, int64_t n, void* out, cudaStream_t st);
 cudaError_t launch_dfv_grad_rows(const gear_ctx_impl& c, const float* dX, const int32_t* row_view, const float* inv_n,
                                  int64_t nnz, float* out, cudaStream_t st);
+// the exchange of a step with all ranks' shards on this device: table 0 user, 1 URL, 2 images; start[s]: where sender s's IDs
+// begin in the concatenated list, start[world] = its length
+struct ShardFetch {
+    struct Table {
+        const int32_t* ids; int32_t start[GEAR_MAX_LOCAL_RANKS + 1];
+        const uint4* shard[GEAR_MAX_LOCAL_RANKS]; int64_t rows[GEAR_MAX_LOCAL_RANKS]; int chunks;      // 16-byte chunks of a row
+        uint4* out; int64_t out_stride;                                      // sender s's rows start at row s * out_stride
+    } table[3];
+    int world;
+    DevState* state[GEAR_MAX_LOCAL_RANKS];
+};
+struct ShardRoute {
+    struct Table {
+        const int32_t* ids; int32_t start[GEAR_MAX_LOCAL_RANKS + 1];
+        int32_t* local; int32_t* src; int64_t src_stride;                    // [world][start[world]]
+    } table[3];
+    int world;
+    int32_t* counts;                                                         // [3][world]
+};
+cudaError_t launch_shard_fetch(Profiler* prof, const ShardFetch& f, cudaStream_t st);
+cudaError_t launch_shard_route(Profiler* prof, const ShardRoute& r, cudaStream_t st);
 // emb_scatter.cu: table[id] += alpha * (sum of the rows with that id), ids given explicitly (sorted here)
 cudaError_t launch_apply_emb_grad(const gear_ctx_impl& c, int which, const int32_t* ids, const float* rows, int64_t ld,
                                   int64_t n, float alpha, cudaStream_t st);

@@ -207,7 +207,7 @@ coop_sort_kernel(const SortBatch batch) {
             for (int it = 0; it < RS_ITEMS; ++it) {                 // keys and values of the tile: one trip to memory
                 const int64_t i = seg0 + it * 32 + lane;
                 key[it] = i < n ? load_key(j, pass, i, src) : 0u;
-                val[it] = identity ? (uint32_t)i : (i < n ? __ldcg(j.vals[src] + i) : 0u);
+                val[it] = identity ? (j.src && i < n ? (uint32_t)__ldcg(j.src + i) : (uint32_t)i) : (i < n ? __ldcg(j.vals[src] + i) : 0u);
             }
 #pragma unroll
             for (int it = 0; it < RS_ITEMS; ++it) {

@@ -90,4 +90,104 @@ cudaError_t launch_dfv_grad_rows(const gear_ctx_impl& c, const float* dX, const 
                             2 * c.cfg.emb_dim, c.cfg.dfv_dim, row_view, inv_n, nnz, out);
 }
 
+// ---------------------------------------------------------------- all ranks' shards on this device
+// The exchange of a step when every owner's shard is memory of this device: a worker's rows are read straight from the owner's
+// table (row id div world of shard id mod world), and the arrivals of every owner are picked out of the workers' ID lists on
+// the device.  Both work on the concatenation of the workers' lists, sender by sender.
+
+__device__ __forceinline__ void split_id(int32_t id, int world, int& owner, int& local) {
+    local = id / world;
+    owner = id - local * world;
+    if (owner < 0) { owner += world; --local; }               // floor: a negative ID stays negative and is refused by its owner
+}
+__device__ __forceinline__ int sender_of(const int32_t* start, int world, int p) {
+    int s = 0;
+    while (s + 1 < world && p >= start[s + 1]) ++s;
+    return s;
+}
+
+// blockIdx.y: table.  A warp takes SH_ROWS consecutive entries of the concatenated list per pass.
+__global__ void __launch_bounds__(256)
+shard_fetch_kernel(const ShardFetch f) {
+    wait_for_predecessor();
+    const ShardFetch::Table& t = f.table[blockIdx.y];
+    const int lane = (int)lane_id(), n = t.start[f.world];
+    const int warps = (int)(gridDim.x * (blockDim.x >> 5));
+    for (int k0 = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * SH_ROWS; k0 < n; k0 += warps * SH_ROWS) {
+        const uint4* row[SH_ROWS];
+        int64_t to[SH_ROWS];
+#pragma unroll
+        for (int q = 0; q < SH_ROWS; ++q) {
+            const int k = k0 + q;
+            row[q] = nullptr; to[q] = -1;
+            if (k < n) {
+                const int s = sender_of(t.start, f.world, k);
+                int owner, local;
+                split_id(__ldg(t.ids + k), f.world, owner, local);
+                to[q] = s * t.out_stride + (k - t.start[s]);
+                if (local >= 0 && local < t.rows[owner]) row[q] = t.shard[owner] + (int64_t)local * t.chunks;
+                else if (lane == 0) atomicOr(&f.state[owner]->status, GEAR_DEV_BAD_ID);       // a zero row is written
+            }
+        }
+        for (int ch = lane; ch < t.chunks; ch += 32) {
+            uint4 v[SH_ROWS];
+#pragma unroll
+            for (int q = 0; q < SH_ROWS; ++q) v[q] = row[q] ? __ldg(row[q] + ch) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int q = 0; q < SH_ROWS; ++q) if (to[q] >= 0) t.out[to[q] * t.chunks + ch] = v[q];
+        }
+    }
+}
+
+// blockIdx.x: owner, blockIdx.y: table.  One block compacts the owner's entries in order: a warp counts the matches of its
+// stretch of the list, the counts are scanned, the warp goes over its stretch again (it is in the L1) and writes.
+__global__ void __launch_bounds__(1024)
+shard_route_kernel(const ShardRoute r) {
+    wait_for_predecessor();
+    __shared__ int s_cnt[32];
+    const ShardRoute::Table& t = r.table[blockIdx.y];
+    const int owner = (int)blockIdx.x, lane = (int)lane_id(), warp = (int)(threadIdx.x >> 5);
+    const int n = t.start[r.world], per = (int)ceil_div(ceil_div(n, 32), 32) * 32;       // a warp's stretch: whole words of 32
+    const int p0 = warp * per, p1 = min(n, p0 + per);
+    int count = 0;
+#pragma unroll 4
+    for (int p = p0; p < p1; p += 32) {
+        int o = -1, local;
+        if (p + lane < p1) split_id(__ldg(t.ids + p + lane), r.world, o, local);
+        count += __popc(__ballot_sync(0xffffffffu, o == owner));
+    }
+    if (lane == 0) s_cnt[warp] = count;
+    __syncthreads();
+    const int mine = s_cnt[lane];
+    int at = __reduce_add_sync(0xffffffffu, lane < warp ? mine : 0);
+    int32_t* __restrict__ out_local = t.local + (int64_t)owner * n;
+    int32_t* __restrict__ out_src = t.src + (int64_t)owner * n;
+#pragma unroll 4
+    for (int p = p0; p < p1; p += 32) {
+        int o = -1, local = 0;
+        if (p + lane < p1) split_id(__ldg(t.ids + p + lane), r.world, o, local);
+        const uint32_t hit = __ballot_sync(0xffffffffu, o == owner);
+        if (o == owner) {
+            const int s = sender_of(t.start, r.world, p + lane);
+            const int to = at + __popc(hit & ((1u << lane) - 1u));
+            out_local[to] = local;
+            out_src[to] = (int32_t)(s * t.src_stride + (p + lane - t.start[s]));
+        }
+        at += __popc(hit);
+    }
+    if (warp == 31 && lane == 0) r.counts[blockIdx.y * r.world + owner] = at;
+}
+
+cudaError_t launch_shard_fetch(Profiler* prof, const ShardFetch& f, cudaStream_t st) {
+    int n = 1;
+    for (int t = 0; t < 3; ++t) n = f.table[t].start[f.world] > n ? f.table[t].start[f.world] : n;
+    const int64_t want = ceil_div(n, 8 * SH_ROWS), cap = (int64_t)sm_count() * 8;
+    KernelScope k(prof, "shard_fetch", st);
+    return launch_dependent(shard_fetch_kernel, dim3((unsigned)(want < cap ? want : cap), 3), dim3(256), 0, st, f);
+}
+cudaError_t launch_shard_route(Profiler* prof, const ShardRoute& r, cudaStream_t st) {
+    KernelScope k(prof, "shard_route", st);
+    return launch_dependent(shard_route_kernel, dim3((unsigned)r.world, 3), dim3(1024), 0, st, r);
+}
+
 }  // namespace gear

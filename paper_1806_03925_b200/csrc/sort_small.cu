@@ -62,6 +62,7 @@ sort_small_kernel(const SortBatch batch, const PlanArgs plan) {
             const bool ok = id >= 0 && (uint32_t)id < j.sentinel;
             bad |= !ok;
             key[it] = ok ? (uint32_t)id : j.sentinel;
+            if (j.src) val[it] = (uint32_t)__ldg(j.src + i);
         }
     }
     if (bad && j.status) atomicOr(j.status, GEAR_DEV_BAD_ID);

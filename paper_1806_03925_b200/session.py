@@ -42,7 +42,10 @@ class GearSession:
                  max_nnz: Optional[int] = None, seed: int = 0, fill: bool = True, now: int = 0,
                  tables: Optional[Dict[str, np.ndarray]] = None, ready_cap: int = 0, device: str = "cuda",
                  want_emb_grad: bool = False, want_debug: bool = False, expired_cap: Optional[int] = None,
-                 accum_mode: int = gb.GEAR_ACC_SORT, adam: Optional["gb.gear_adam"] = None):
+                 accum_mode: int = gb.GEAR_ACC_SORT, adam: Optional["gb.gear_adam"] = None,
+                 scalars: Optional[torch.Tensor] = None):
+        """tables: initial contents of user_emb, url_emb, dfv (bf16 as uint16) and ts; a device tensor is used as it is.
+        scalars: where the loss and the two counts go (3 x int64), e.g. a part of a larger buffer."""
         gb.load()
         self.p = p
         self.dev = torch.device(device)
@@ -63,15 +66,16 @@ class GearSession:
             self.dfv_ts = torch.zeros(p.img_vocab, dtype=torch.int64, device=dev)
         else:
             fill = False
-            self.user_emb = torch.from_numpy(tables["user_emb"]).to(dev)
-            self.url_emb = torch.from_numpy(tables["url_emb"]).to(dev)
+            own = lambda t: t if torch.is_tensor(t) else torch.from_numpy(t).to(dev)
+            self.user_emb = own(tables["user_emb"])
+            self.url_emb = own(tables["url_emb"])
             dfv = tables["dfv"]
             if dfv.dtype == np.uint16:
                 self.dfv = torch.from_numpy(dfv.view(np.int16)).to(dev).view(torch.bfloat16)
             else:
-                self.dfv = torch.from_numpy(dfv).to(dev)
+                self.dfv = own(dfv)
             assert self.dfv.dtype == dfv_t
-            self.dfv_ts = torch.from_numpy(tables["ts"]).to(dev)
+            self.dfv_ts = own(tables["ts"])
         self.dfv_gsum = torch.zeros((p.img_vocab, p.dfv_dim), dtype=torch.float32, device=dev)
         self.dfv_gcnt = torch.zeros(p.img_vocab, dtype=torch.int32, device=dev)
         self.head_params = torch.from_numpy(np.ascontiguousarray(head_params, dtype=np.float32)).to(dev)
@@ -81,7 +85,7 @@ class GearSession:
                                        self.dfv_ts, self.head_params, self.workspace, seed=seed, fill=fill, now=now)
         B, nnz = self.max_batch, self.max_nnz
         # loss and the two counts share one small buffer, so that a caller can read them back with a single copy
-        self.scalars = torch.zeros(3, dtype=torch.int64, device=dev)
+        self.scalars = torch.zeros(3, dtype=torch.int64, device=dev) if scalars is None else scalars
         self.loss = self.scalars[0:1].view(torch.float32)[0:1]
         self.prob = torch.zeros(B, dtype=torch.float32, device=dev)
         self.head_grad = torch.zeros(p.n_params, dtype=torch.float32, device=dev)

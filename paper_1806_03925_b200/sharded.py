@@ -20,7 +20,7 @@ is a valid one; this one is reproducible).  The workers do not rescale their gra
 in the paper, every worker's batch is a batch of its own.
 
 Nothing here computes anything of the method: routing by ID (remainder, quotient, a stable partition by owner),
-copies and collectives.  `Exchange` has two forms with the same interface: `DistExchange` runs one rank per process
+copies and collectives.  With all ranks in one process the step takes a shorter way to the same results (_InProcessStep).  `Exchange` has two forms with the same interface: `DistExchange` runs one rank per process
 over torch.distributed (NCCL on GPUs, gloo on CPU tensors); `LoopbackExchange` holds all ranks in one process and
 moves the pieces by indexing, so that the whole sharded step can be run and checked on a single GPU, rank after rank,
 with no kernel of one rank waiting on another's.
@@ -183,9 +183,19 @@ class ShardedGear:
         """tables (optional): the WHOLE tables as host arrays (user_emb, url_emb, dfv, ts), of which every owner takes
         its rows (rank, rank + world, ...); without them every shard gets its own procedural fill."""
         self.p, self.ex, self.world = p, ex, ex.world
-        W = self.world
+        W, n = self.world, len(ex.local_ranks)
         self.owners: List[GearSession] = []
         self.workers: List[GearSession] = []
+        # the local workers' row buffers and gradient rows one behind the other: worker i's start at row i * max_*_local
+        dev = torch.device(device)
+        self.max_batch_local, self.max_nnz_local = max_batch_local, max_nnz_local
+        zeros = lambda *shape, dtype=torch.float32: torch.zeros(shape, dtype=dtype, device=dev)
+        self._user_rows, self._url_rows = zeros(n * max_batch_local, p.emb_dim), zeros(n * max_batch_local, p.emb_dim)
+        self._dfv_rows = zeros(n * max_nnz_local, p.dfv_dim, dtype=torch.bfloat16 if p.dfv_dtype == BF16 else torch.float32)
+        self._dX, self._dfv_grad = zeros(n * max_batch_local, p.d_in), zeros(n * max_nnz_local, p.dfv_dim)
+        # head gradients: rows of a matrix, each on a 16-byte boundary
+        self._head_grads = zeros(n, (p.n_params + 3) // 4 * 4)[:, :p.n_params]
+        self._scalars = zeros(3 * n, dtype=torch.int64)        # loss and the two counts of every owner
         for r in ex.local_ranks:
             sp = replace(p, user_vocab=shard_rows(p.user_vocab, r, W), url_vocab=shard_rows(p.url_vocab, r, W),
                          img_vocab=shard_rows(p.img_vocab, r, W))
@@ -193,24 +203,31 @@ class ShardedGear:
             if tables is not None:
                 mine = {k: np.ascontiguousarray(v[r::W]) for k, v in tables.items()}
             self.owners.append(GearSession(sp, head_params, max_batch=max_batch_local * W, max_nnz=max_nnz_local * W,
-                                           seed=seed + r, fill=True, now=now, tables=mine, device=device))
+                                           seed=seed + r, fill=True, now=now, tables=mine, device=device,
+                                           scalars=self._scalars[3 * len(self.owners):3 * len(self.owners) + 3]))
             wp = replace(p, user_vocab=max_batch_local, url_vocab=max_batch_local, img_vocab=max_nnz_local)
-            dfv_np = np.uint16 if p.dfv_dtype == BF16 else np.float32
-            blank = dict(user_emb=np.zeros((max_batch_local, p.emb_dim), np.float32),
-                         url_emb=np.zeros((max_batch_local, p.emb_dim), np.float32),
-                         dfv=np.zeros((max_nnz_local, p.dfv_dim), dfv_np), ts=np.zeros(max_nnz_local, np.int64))
+            i = len(self.workers)
+            rows = slice(i * max_batch_local, (i + 1) * max_batch_local), slice(i * max_nnz_local, (i + 1) * max_nnz_local)
+            blank = dict(user_emb=self._user_rows[rows[0]], url_emb=self._url_rows[rows[0]], dfv=self._dfv_rows[rows[1]],
+                         ts=torch.zeros(max_nnz_local, dtype=torch.int64, device=dev))
+            # a worker keeps no gradient store (GEAR_ACC_ATOMIC: its image IDs are not sorted)
             wk = GearSession(wp, head_params, max_batch=max_batch_local, max_nnz=max_nnz_local, tables=blank,
-                             expired_cap=1, ready_cap=1, device=device)
-            wk.dfv_grad = torch.zeros((max_nnz_local, p.dfv_dim), dtype=torch.float32, device=device)
+                             expired_cap=1, ready_cap=1, device=device, accum_mode=gb.GEAR_ACC_ATOMIC)
+            wk.dX, wk.dfv_grad, wk.head_grad = self._dX[rows[0]], self._dfv_grad[rows[1]], self._head_grads[i]
             wk._step_out = None
             self.workers.append(wk)
         self._iota = torch.arange(max(max_batch_local, max_nnz_local), dtype=torch.int32, device=device)
+        self._in_process = None
 
     def step(self, batches: Sequence[Batch], now: int, lr: Optional[float] = None, mean_head_grad: bool = True):
         """One step of every local rank.  batches[i]: the page views of local rank i (host arrays).  Returns per local
         rank (averages handed over by its owner, IDs its owner's scan listed)."""
         p, ex = self.p, self.ex
         lr = p.lr if lr is None else lr
+        if isinstance(ex, LoopbackExchange) and self.world <= gb.GEAR_MAX_LOCAL_RANKS:
+            if self._in_process is None:
+                self._in_process = _InProcessStep(self)
+            return self._in_process.step(batches, now, lr, mean_head_grad)
         E = p.emb_dim
         dev = self.workers[0].dev
         ids = {k: [torch.from_numpy(np.ascontiguousarray(getattr(b, k))).to(dev) for b in batches]
@@ -252,3 +269,95 @@ class ShardedGear:
     def close(self):
         for s in self.owners + self.workers:
             s.close()
+
+
+class _InProcessStep:
+    """The step when all shards are memory of one device: the same results as the exchange-by-exchange form, without send
+    and receive buffers.  The batches travel to the device in one copy; workers read their rows straight from the owners'
+    shards (gear_shard_fetch); a kernel picks every owner's arrivals out of the ID lists (gear_shard_route) while the workers
+    run; an owner takes its arrivals in one call (gear_owner_step), reading the gradient rows where the workers left them.
+    The host waits twice: for the numbers of arrivals (beside the workers' kernels) and for the counts it returns."""
+
+    def __init__(self, sg: ShardedGear):
+        self.sg = sg
+        p, W = sg.p, sg.world
+        mb, mn, dev = sg.max_batch_local, sg.max_nnz_local, sg.workers[0].dev
+        # one pinned host buffer and its device twin: user, URL and image IDs, offsets, labels, each list sender by sender
+        caps = (W * mb, W * mb, W * mn, W * (mb + 1), W * mb)
+        self.at, total = [], 0
+        for c in caps:
+            self.at.append(total)
+            total += (c + 3) // 4 * 4
+        self.host = torch.zeros(total, dtype=torch.int32).pin_memory()
+        self.np_i, self.np_f = self.host.numpy(), self.host.numpy().view(np.float32)
+        self.dev = torch.zeros(total, dtype=torch.int32, device=dev)
+        self.base = self.dev.data_ptr()
+        VP = gb.C.c_void_p
+        ptrs = lambda *a: (VP * len(a))(*a)
+        self.owners = ptrs(*(o.ctx.value for o in sg.owners))
+        self.ids = ptrs(*(self.base + 4 * self.at[t] for t in range(3)))
+        self.out = ptrs(sg._user_rows.data_ptr(), sg._url_rows.data_ptr(), sg._dfv_rows.data_ptr())
+        self.start = (gb.C.c_int32 * (3 * (W + 1)))()
+        self.stride = (gb.C.c_int64 * 3)(mb, mb, mn)
+        # arrivals of every owner: [table][local / src][world * entries]
+        self.lists = [[torch.zeros(W * c, dtype=torch.int32, device=dev) for _ in range(2)] for c in caps[:3]]
+        self.local, self.src = (ptrs(*(l[k].data_ptr() for l in self.lists)) for k in range(2))
+        self.counts = torch.zeros(3 * W, dtype=torch.int32, device=dev)
+        self.host_counts = torch.zeros(3 * W, dtype=torch.int32).pin_memory()
+        self.host_scalars = torch.zeros(3 * W, dtype=torch.int64).pin_memory()
+        self.routed, self.done = torch.cuda.Event(), torch.cuda.Event()
+        self.arrivals = [gb.gear_arrivals() for _ in range(3)]
+        self.batch = []
+        for wk in sg.workers:
+            bt = gb.gear_batch()
+            bt.user_id = bt.url_id = bt.img_id = sg._iota.data_ptr()
+            self.batch.append((bt, wk._make_step_out()))
+
+    def step(self, batches: Sequence[Batch], now: int, lr: float, mean_head_grad: bool):
+        sg = self.sg
+        p, W = sg.p, sg.world
+        # ---- the batches, one copy
+        pos = list(self.at)
+        for s, b in enumerate(batches):
+            for t, a in enumerate((b.user_id, b.url_id, b.img_id)):
+                self.start[t * (W + 1) + s] = pos[t] - self.at[t]
+                self.np_i[pos[t]:pos[t] + len(a)] = a
+                pos[t] += len(a)
+            bt = self.batch[s][0]
+            bt.B, bt.nnz = b.B, b.nnz
+            bt.img_off, bt.label = self.base + 4 * pos[3], self.base + 4 * pos[4]
+            self.np_i[pos[3]:pos[3] + b.B + 1] = b.img_off
+            self.np_f[pos[4]:pos[4] + b.B] = b.label
+            pos[3] += b.B + 1
+            pos[4] += b.B
+        for t in range(3):
+            self.start[t * (W + 1) + W] = pos[t] - self.at[t]
+        used = pos[4]
+        self.dev[:used].copy_(self.host[:used], non_blocking=True)
+        # ---- events 1-4 on the workers; the owners' arrivals
+        gb.gear_shard_route(W, self.ids, self.start, self.stride, self.local, self.src, self.counts)
+        self.host_counts.copy_(self.counts, non_blocking=True)
+        self.routed.record()
+        gb.gear_shard_fetch(self.owners, W, self.ids, self.start, self.out, self.stride)
+        for wk, (bt, o) in zip(sg.workers, self.batch):
+            gb.gear_forward_backward_structs(wk.ctx, bt, 0.0, o)      # the worker's copies of the rows are scratch: nothing to update
+        if mean_head_grad:
+            sg._head_grads.copy_(sg._head_grads.mean(0, keepdim=True).expand_as(sg._head_grads))
+        # ---- events 4 (push), 5 and 6 at the owners
+        self.routed.synchronize()
+        counts = self.host_counts.tolist()
+        emb_rows, img_rows = sg._dX.data_ptr(), sg._dfv_grad.data_ptr()
+        for i, ow in enumerate(sg.owners):
+            for t, a in enumerate(self.arrivals):
+                first = 4 * i * self.start[t * (W + 1) + W]
+                a.ids, a.src, a.n = self.local[t] + first, self.src[t] + first, counts[t * W + i]
+            gb.gear_owner_step(ow.ctx, *self.arrivals, emb_rows, p.d_in, img_rows, p.dfv_dim, lr, ow._step_lists or ow._make_step_lists(), now)
+        self.host_scalars.copy_(sg._scalars, non_blocking=True)
+        self.done.record()
+        self.done.synchronize()
+        v = self.host_scalars.tolist()
+        out = [(v[3 * i + 1], v[3 * i + 2]) for i in range(W)]
+        for ow, (n_ready, n_expired) in zip(sg.owners, out):
+            if n_ready > ow.ready_cap or n_expired > ow.expired_cap:
+                raise gb.GearError(gb.GEAR_ERR_CAPACITY, "gear_owner_step")
+        return out
