@@ -86,13 +86,13 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
             p->sort_keys[s][i] = take((size_t)p->sort_n[s] * 4);
             p->sort_vals[s][i] = take((size_t)p->sort_n[s] * 4);
         }
-        p->sort_hist[s] = take((size_t)RS_MAX_PASSES * RS_BUCKETS * sort_tiles(p->sort_n[s]) * 4);
-        p->sort_tot[s] = take((size_t)RS_MAX_PASSES * RS_BUCKETS * 4);
+        p->sort_hist[s] = take((size_t)RS_BUCKETS * sort_max_blocks(p->sort_n[s]) * 4);
+        p->sort_tot[s] = take((size_t)RS_BUCKETS * 4);
     }
     p->tile_cnt = take((size_t)(ceil_div(c.max_nnz, 1024) + 1) * sizeof(uint2));
     p->grp_rec = take((size_t)c.max_nnz * 16);
     p->pmeta = take((size_t)c.max_nnz * 8);
-    p->blk_first = take((size_t)(ceil_div(c.max_nnz, ACC_SPAN) + 2) * 4);
+    p->blk_first = take((size_t)acc_max_spans(c.max_nnz) * 4);
     p->run_end = take((size_t)c.max_nnz * 4);
     p->q_id = take((size_t)p->ready_cap * 4);
     p->q_avg = take((size_t)p->ready_cap * c.dfv_dim * 4);
@@ -207,11 +207,14 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     auto scan = [&](cudaStream_t where) {
         return launch_collect_expired(c, lists->now, lists->restamp, lists->expired, lists->expired_cap, lists->d_expired, where);
     };
-    if (scan_beside) GEAR_TRY(scan(aux));
     // The weights in the form the head's products read: first on the caller's stream, ahead of the gather.  The gather keeps
     // every SM busy for its whole duration, so a small kernel on another stream would get its blocks placed only when the
     // gather ends, and the first product of the head would wait for it.
-    GEAR_TRY(launch_round_weights(c, o, st));
+    // (Small batches leave SMs free: there the copies run beside the gather.)
+    if (dw_beside && !scan_beside) GEAR_TRY(enqueue_wait(aux, c.ev[EV_FORK]));
+    GEAR_TRY(launch_round_weights(c, o, dw_beside ? aux : st));
+    if (dw_beside) GEAR_TRY(enqueue_record(c.ev[EV_AUX], aux));
+    if (scan_beside) GEAR_TRY(scan(aux));
     int sorted_buf = 0;
     bool small_sort = false;
     const bool plan = b.nnz > 0 && o.row_view && o.inv_n && sorted_mode;
@@ -246,6 +249,7 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     }
     GEAR_TRY(launch_gather(c, b, o.row_view, o.inv_n, o.x_debug, st));
     if (forked) GEAR_TRY(enqueue_record(c.ev[EV_GATHER], st));
+    if (dw_beside) GEAR_TRY(enqueue_wait(st, c.ev[EV_AUX]));
     // behind the sort: the plan of the accumulate call that usually follows (which rows form which group, where every group's
     // rows and queue slot are).  It needs the gather's row_view / inv_n.  Small arrays are sorted and planned by one kernel.
     if (small_sort || (forked && plan)) {

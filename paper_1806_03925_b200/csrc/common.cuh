@@ -213,18 +213,48 @@ struct KernelScope {
     ~KernelScope() { if (stop) cudaEventRecord(stop, st); }
 };
 
-// sorted positions per unit of work of the accumulate's reduce pass (at most 32); the workspace holds one word per span
+// Sorted positions per unit of work (span) of the accumulate's reduce pass: 16, or as few as 2 while longer spans would leave
+// warps idle (12 k rows in spans of 16 kept 768 of 3552 warps busy, each with a serial chain of 16 rows).  The workspace
+// holds one word per span.
 constexpr int ACC_SPAN = 16;
+constexpr int64_t ACC_WARPS = 3552;        // warps of a full reduce grid: 148 SMs x 3 blocks x 8
+inline int acc_span_log2(int64_t n) {
+    int s = 4;
+    while (s > 1 && (n >> s) < ACC_WARPS) --s;
+    return s;
+}
+// words of the span table for any n up to n_max
+inline int64_t acc_max_spans(int64_t n_max) {
+    const int64_t small = n_max < (ACC_WARPS << 5) ? n_max : (ACC_WARPS << 5);
+    const int64_t a = ceil_div(n_max, ACC_SPAN), b = ceil_div(small, 2);
+    return (a > b ? a : b) + 2;
+}
+
+// x / M for x < M + 2^30: a multiplication and a shift (division by an invariant integer, Granlund and Montgomery, PLDI 1994:
+// exact for x < 2^31 with the factor ceil(2^(31 + s) / M), s = ceil(log2 M)); from M = 2^30 on the quotient is 0 or 1.
+struct DivM {
+    int M; uint32_t factor; int shift;
+    __host__ __device__ __forceinline__ uint32_t operator()(uint32_t x) const {
+        return M >= (1 << 30) ? (uint32_t)(x >= (uint32_t)M) : (uint32_t)(((uint64_t)x * factor) >> shift);
+    }
+};
+inline DivM make_div(int M) {
+    int s = 0;
+    while (s < 31 && (1ll << s) < M) ++s;
+    return DivM{M, (uint32_t)(((1ull << (31 + s)) + M - 1) / M), 31 + s};
+}
 
 // ---------------------------------------------------------------- radix sort / scans (prims.cu)
 constexpr int RS_THREADS = 256;
-constexpr int RS_ITEMS = 16;
-constexpr int RS_TILE = RS_THREADS * RS_ITEMS;
 constexpr int RS_RADIX_BITS = 9;
 constexpr int RS_BUCKETS = 1 << RS_RADIX_BITS;
-constexpr int RS_MAX_PASSES = 4;          // 32-bit keys in digits of 9 bits
+constexpr int RS_MAX_BLOCKS = 512;        // of the sort's grid (three per SM)
 
-inline int64_t sort_tiles(int64_t n_max) { return n_max > 0 ? ceil_div(n_max, RS_TILE) : 1; }
+// most blocks a job can get: one per tile of RS_THREADS * 8 entries
+inline int64_t sort_max_blocks(int64_t n_max) {
+    const int64_t tiles = ceil_div(n_max, RS_THREADS * 8);
+    return tiles < 1 ? 1 : tiles < RS_MAX_BLOCKS ? tiles : RS_MAX_BLOCKS;
+}
 
 // One array to sort: (key, value) pairs ordered by the low `bits` bits of the key, equal keys in input order.
 struct SortJob {
@@ -233,15 +263,14 @@ struct SortJob {
     int32_t* status;        // device status word that gets GEAR_DEV_BAD_ID when a sentinel key is met (may be null)
     uint32_t* keys[2];      // without ids the input keys are keys[0]
     uint32_t* vals[2];      // with identity_vals the value of element i is i, else vals[0][i]
-    uint32_t* hist;         // [RS_MAX_PASSES][n_tiles][RS_BUCKETS] tile descriptors: per pass and tile, how many of the
-                            // tile's elements (or of all tiles up to it) carry each digit; top two bits say which
-    uint32_t* tot;          // [RS_MAX_PASSES][RS_BUCKETS] digit histogram of every pass
+    uint32_t* hist;         // [RS_BUCKETS][blocks of the job] digit counts of the blocks' chunks
+    uint32_t* tot;          // [RS_BUCKETS] digit counts of the array
     int64_t n_max;          // element count (or its upper bound when n_dev is given)
     const int64_t* n_dev;   // optional device-resident count, capped at n_max
     int bits;
     int identity_vals;
     const int32_t* src;     // with identity_vals: the value of element i is src[i] instead, if set
-    int width, n_tiles;     // filled in by sort_jobs
+    int width, block0, n_blocks;     // filled in by sort_jobs
 };
 
 struct SortBatch {

@@ -45,6 +45,12 @@ dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const 
             row_of[threadIdx.x] = id;
         }
         __syncthreads();
+        // the tile's rows are random lines of a large table: all of them on their way at once, so that the steps of the chain wait
+        // for the L2 only
+        for (int q = threadIdx.x; q < BM * (int)ceil_div(R, 32); q += 128) {
+            const int64_t id = row_of[q % BM];
+            if (id >= 0) asm volatile("prefetch.global.L2 [%0];" :: "l"(raw + id * R + 32 * (q / BM)));
+        }
         f32x2 acc[TM][TN / 2];
 #pragma unroll
         for (int i = 0; i < TM; ++i)

@@ -33,7 +33,7 @@ struct WsPlan {
     int64_t sort_n[4];
     size_t tile_cnt;                    // [plan tiles + 1] uint2 per-tile (groups, complete) counts, then their totals
     size_t grp_rec;                     // [max_nnz] uint4 group records (start | first flag, image ID, queue slot, held rows)
-    size_t blk_first;                   // [ceil(max_nnz / 16) + 2] uint32: first group that starts in each span of sorted positions
+    size_t blk_first;                   // [acc_max_spans] uint32: first group that starts in each span of sorted positions
     size_t run_end;                     // [max_nnz] uint32: at the first position of an image's run, one past its last
     size_t pmeta;                       // [max_nnz] int2: source row and scale (fp32 bits) of every sorted position
     size_t q_id;                        // [ready_cap] int32
@@ -119,11 +119,14 @@ struct gear_ctx_impl {
 // of the last job also plans the accumulate call where plan.totals is set.
 // What a plan is made from and where it goes (plan.cuh).
 struct PlanArgs {
-    uint2* totals; uint32_t vocab; int M; const int32_t* cnt; uint4* grp_rec; const int32_t* src_row; const float* scale;
+    uint2* totals; uint32_t vocab; const int32_t* cnt; uint4* grp_rec; const int32_t* src_row; const float* scale;
     int2* pmeta; uint32_t* blk_first; uint32_t* run_end; DevState* state;
-    uint32_t div_factor; int div_shift;         // division by M (plan.cuh)
+    DivM div; int span;                         // log2 of the positions per span
 };
 bool sort_small_fits(const SortBatch& batch);
+int64_t sort_small_max();
+// the first launch of a hand-over that may have to sort the queue: count, capacity check, sort of up to sort_small_max() entries
+cudaError_t launch_collect_sort(const gear_ctx_impl& c, const SortJob& job, int64_t cap, int64_t* d_n, cudaStream_t st);
 cudaError_t launch_sort_small(const gear_ctx_impl& c, const SortBatch& batch, const PlanArgs& plan, cudaStream_t st);
 
 // fill.cu

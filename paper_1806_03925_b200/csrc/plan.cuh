@@ -13,12 +13,6 @@ namespace gear {
 //                           covers tile0 starts, if it starts before tile0
 //   base(g, f, g0, f0)      g groups start in the tile, f of them complete; sets how many there are in the tiles before it
 // s_warp: 2 * WARPS words of shared memory.  Every thread of the block must call this.
-// x / M for x < M + 2^30: a multiplication and a shift (division by an invariant integer, Granlund and Montgomery, PLDI 1994:
-// exact for x < 2^31 with the factor ceil(2^(31 + s) / M), s = ceil(log2 M)); from M = 2^30 on the quotient is 0 or 1.
-__device__ __forceinline__ uint32_t div_m(const PlanArgs& p, uint32_t x) {
-    return p.M >= (1 << 30) ? (uint32_t)(x >= (uint32_t)p.M) : (uint32_t)(((uint64_t)x * p.div_factor) >> p.div_shift);
-}
-
 template <int ITEMS, int WARPS, typename KeyAt, typename PermAt, typename RunBefore, typename Base>
 __device__ __forceinline__ void plan_tile(const PlanArgs& p, int n, int tile0, KeyAt key_at, PermAt perm_at, int* s_warp, RunBefore run_before, Base base) {
     const int lane = (int)lane_id(), warp = (int)(threadIdx.x >> 5);
@@ -55,10 +49,10 @@ __device__ __forceinline__ void plan_tile(const PlanArgs& p, int n, int tile0, K
         rank[it] = i - start;
         bool head = false, complete = false;
         if (key < p.vocab) {
-            const uint32_t x = (uint32_t)c0[it] + (uint32_t)rank[it], rem = x - div_m(p, x) * (uint32_t)p.M;
+            const uint32_t x = (uint32_t)c0[it] + (uint32_t)rank[it], rem = x - p.div(x) * (uint32_t)p.div.M;
             head = rank[it] == 0 || rem == 0;
             if (head) {
-                const int64_t last = (int64_t)i + (p.M - (int64_t)rem) - 1;          // the row that brings the count to M
+                const int64_t last = (int64_t)i + (p.div.M - (int64_t)rem) - 1;          // the row that brings the count to M
                 complete = last < n && key_at((int)last) == key;
             }
             const uint32_t after = i + 1 < n ? key_at(i + 1) : p.vocab;
@@ -107,8 +101,8 @@ __device__ __forceinline__ void plan_tile(const PlanArgs& p, int n, int tile0, K
         const uint32_t key = i < n ? key_at(i) : p.vocab;
         if (key < p.vocab) {
             const uint32_t g = gi + __popc(hb & lt);
-            // the reduce pass hands out spans of ACC_SPAN sorted positions: index of the first group that starts in each
-            if ((i % ACC_SPAN) == 0) p.blk_first[i / ACC_SPAN] = g;
+            // the reduce pass hands out spans of 2^span sorted positions: index of the first group that starts in each
+            if ((i & ((1 << p.span) - 1)) == 0) p.blk_first[i >> p.span] = g;
             if (head) {
                 // one 16-byte record per group: start position (top bit: first group of its image in this call), image ID,
                 // ready-queue slot (-1: the group stays open), and for the image's first group the rows the image already held,
@@ -116,7 +110,7 @@ __device__ __forceinline__ void plan_tile(const PlanArgs& p, int n, int tile0, K
                 const bool first = rank[it] == 0;
                 p.grp_rec[g] = make_uint4((uint32_t)i | (first ? 0x80000000u : 0u), key,
                                           (uint32_t)(complete ? (int32_t)(q_base + ci + __popc(fb & lt)) : -1),
-                                          first ? (uint32_t)c0[it] : div_m(p, (uint32_t)c0[it] + (uint32_t)rank[it]));
+                                          first ? (uint32_t)c0[it] : p.div((uint32_t)c0[it] + (uint32_t)rank[it]));
             }
         }
         gi += __popc(hb);
