@@ -11,7 +11,7 @@
 //   2. flag pass: position i of the sorted array starts a group if it is the first row of its image or if
 //      (c0 + rank within image) is a multiple of M; a group is complete if the image has enough further
 //      rows to reach the next multiple.  Per-tile counts of (groups, complete groups).
-//   3. one-block scan of the tile counts.
+//   3. every block of the plan pass adds up the counts before its tile (sections of 64 tiles, then tiles).
 //   4. plan pass: the flags again, now with their global prefix: group g starts at grp_start[g]; complete
 //      groups get consecutive ready-queue slots (a counter-threshold stream compaction: ballot-free block
 //      scan of the "count reaches M" predicate).
@@ -44,6 +44,18 @@ __device__ __forceinline__ uint32_t warp_inclusive_max(uint32_t v) {
     return v;
 }
 
+// The AF_ITEMS consecutive words a thread owns (a 16-byte load away from the array's end).
+__device__ __forceinline__ void load_items(uint32_t (&v)[AF_ITEMS], const uint32_t* __restrict__ p, int64_t i0, int64_t n, uint32_t pad) {
+    static_assert(AF_ITEMS == 4, "one 16-byte load");
+    if (i0 + AF_ITEMS <= n) {
+        const uint4 q = __ldg(reinterpret_cast<const uint4*>(p + i0));
+        v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+        return;
+    }
+#pragma unroll
+    for (int t = 0; t < AF_ITEMS; ++t) v[t] = i0 + t < n ? p[i0 + t] : pad;
+}
+
 // Flags of the AF_ITEMS consecutive sorted positions a thread owns.
 struct TileFlags {
     uint32_t key[AF_ITEMS];
@@ -64,8 +76,7 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
     f.i0 = tile0 + (int64_t)threadIdx.x * AF_ITEMS;
     uint32_t prev = vocab;   // key just before this thread's first position
     if (f.i0 < n && f.i0 > 0) prev = ks[f.i0 - 1];
-#pragma unroll
-    for (int t = 0; t < AF_ITEMS; ++t) f.key[t] = (f.i0 + t < n) ? ks[f.i0 + t] : vocab;
+    load_items(f.key, ks, f.i0, n, vocab);
 
     // start of the image's run that covers the tile's first position (the run may begin in an earlier tile).  Warp 0
     // searches backwards with all its lanes at once: first one round of probes at distances 1, 2, 4, ... brackets the
@@ -132,7 +143,7 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
         uint32_t rs = max(run_start[t], before_thread);
         const int64_t start = rs ? (int64_t)rs - 1 : (int64_t)carry;
         const int64_t j = i - start;                 // rank of this row among the call's rows of its image
-        const int c0 = cnt[f.key[t]];
+        const int c0 = t > 0 && f.key[t] == f.key[t > 0 ? t - 1 : 0] ? f.c0[t > 0 ? t - 1 : 0] : cnt[f.key[t]];
         f.c0[t] = c0;
         const uint32_t x = (uint32_t)c0 + (uint32_t)j, full = div(x);
         const int rem = (int)(x - full * (uint32_t)div.M);
@@ -154,9 +165,13 @@ struct RowSource {
     const uint32_t* perm; const float* grads; int64_t ld; const int32_t* src_row; const float* scale;
 };
 
+// Counts of (groups, complete groups, in the upper word): per tile, and per section of AF_SECTION tiles (zero before a plan).
+struct PlanCounts { uint2* tile; unsigned long long* section; };
+constexpr int AF_SECTION = 64;
+
 __global__ void __launch_bounds__(AF_THREADS)
 acc_flag_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, const DivM div, const int32_t* __restrict__ cnt,
-                uint2* __restrict__ tile_cnt, DevState* __restrict__ state) {
+                const PlanCounts counts, DevState* __restrict__ state) {
     wait_for_predecessor();
     __shared__ uint32_t smem[34];
     TileFlags f;
@@ -167,12 +182,15 @@ acc_flag_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, cons
     uint32_t tg, tc;
     block_exclusive_scan(g, smem, &tg);
     block_exclusive_scan(c, smem, &tc);
-    if (threadIdx.x == 0) tile_cnt[blockIdx.x] = make_uint2(tg, tc);
+    if (threadIdx.x == 0) {
+        counts.tile[blockIdx.x] = make_uint2(tg, tc);
+        if (tg) atomicAdd(counts.section + blockIdx.x / AF_SECTION, (unsigned long long)tg | ((unsigned long long)tc << 32));
+    }
 }
 
 __global__ void __launch_bounds__(AF_THREADS)
 acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, const DivM div, const int32_t* __restrict__ cnt,
-                const uint2* __restrict__ tile_cnt, uint4* __restrict__ grp_rec, RowSource rs,
+                const PlanCounts counts, uint2* __restrict__ totals, uint4* __restrict__ grp_rec, RowSource rs,
                 int2* __restrict__ pmeta, uint32_t* __restrict__ blk_first, uint32_t* __restrict__ run_end,
                 int span, DevState* __restrict__ state) {
     wait_for_predecessor();
@@ -182,9 +200,18 @@ acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, cons
     uint32_t g = 0, c = 0;
 #pragma unroll
     for (int t = 0; t < AF_ITEMS; ++t) { g += f.head[t]; c += f.complete[t]; }
-    const uint2 tile_base = tile_cnt[blockIdx.x];
-    uint32_t gi = tile_base.x + block_exclusive_scan(g, smem, nullptr);
-    uint32_t ci = tile_base.y + block_exclusive_scan(c, smem, nullptr);
+    // groups in the sections and tiles before this one: a thread's share of both counts in one word (each stays below 2^30)
+    const int section = (int)blockIdx.x / AF_SECTION;
+    unsigned long long before = 0;
+    for (int q = threadIdx.x; q < section; q += AF_THREADS) before += counts.section[q];
+    const int q = section * AF_SECTION + (int)threadIdx.x;
+    if (threadIdx.x < AF_SECTION && q < (int)blockIdx.x) { const uint2 v = counts.tile[q]; before += (unsigned long long)v.x | ((unsigned long long)v.y << 32); }
+    uint32_t g0, c0, g_tile, c_tile;
+    block_exclusive_scan((uint32_t)before, smem, &g0);
+    block_exclusive_scan((uint32_t)(before >> 32), smem, &c0);
+    uint32_t gi = g0 + block_exclusive_scan(g, smem, &g_tile);
+    uint32_t ci = c0 + block_exclusive_scan(c, smem, &c_tile);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *totals = make_uint2(g0 + g_tile, c0 + c_tile);
     const int64_t q_base = state->q_count;
 #pragma unroll
     for (int t = 0; t < AF_ITEMS; ++t) {
@@ -202,13 +229,22 @@ acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, cons
     }
     // where the gradient row of every sorted position lives and what it is scaled by (one 8-byte record), resolved
     // through the sort permutation once, so that the reduce pass reads both with one coalesced load
+    uint32_t src[AF_ITEMS];
+    float scale[AF_ITEMS];
+    load_items(src, rs.perm, f.i0, n, 0u);
+    if (rs.src_row)
 #pragma unroll
-    for (int t = 0; t < AF_ITEMS; ++t) {
-        const int64_t i = f.i0 + t;
-        if (i >= n || f.key[t] >= vocab) continue;
-        const uint32_t r = rs.perm[i];
-        const int32_t src = rs.src_row ? rs.src_row[r] : (int32_t)r;
-        pmeta[i] = make_int2(src, __float_as_int(rs.scale ? rs.scale[src] : 1.f));
+        for (int t = 0; t < AF_ITEMS; ++t) src[t] = f.i0 + t < n && f.key[t] < vocab ? (uint32_t)__ldg(rs.src_row + src[t]) : 0u;
+#pragma unroll
+    for (int t = 0; t < AF_ITEMS; ++t) scale[t] = rs.scale && f.i0 + t < n && f.key[t] < vocab ? __ldg(rs.scale + src[t]) : 1.f;
+    if (f.i0 + AF_ITEMS <= n) {                                     // (records of rows without a valid image are never read)
+        int4* dst = reinterpret_cast<int4*>(pmeta + f.i0);
+        dst[0] = make_int4((int)src[0], __float_as_int(scale[0]), (int)src[1], __float_as_int(scale[1]));
+        dst[1] = make_int4((int)src[2], __float_as_int(scale[2]), (int)src[3], __float_as_int(scale[3]));
+    } else {
+#pragma unroll
+        for (int t = 0; t < AF_ITEMS; ++t)
+            if (f.i0 + t < n) pmeta[f.i0 + t] = make_int2((int)src[t], __float_as_int(scale[t]));
     }
 }
 
@@ -257,8 +293,10 @@ acc_reduce_kernel(RowGather rg, int D, const DivM div, int span_log2, int64_t re
                   const uint32_t* __restrict__ blk_first, const uint32_t* __restrict__ run_end,
                   float* __restrict__ gsum, int32_t* __restrict__ gcnt,
                   int32_t* __restrict__ q_id, float* __restrict__ q_avg, const EmitTarget direct,
-                  DevState* __restrict__ state) {
+                  unsigned long long* __restrict__ sections, int n_sections, DevState* __restrict__ state) {
     wait_for_predecessor();
+    // the plan's section counts are not needed any more: zero for the next plan
+    for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < n_sections; i += (int)(gridDim.x * blockDim.x)) sections[i] = 0ull;
     extern __shared__ float4 ring_mem[];                          // [warps][S][NQ * 32] float4
     const uint2 totals = *plan_totals;
     const int64_t n_groups = totals.x;
@@ -477,15 +515,22 @@ static cudaError_t enqueue_plan(const gear_ctx_impl& c, const uint32_t* ks, cons
     DevState* state = c.state();
     const int64_t n_tiles = ceil_div(n, AF_TILE);
     uint2* tile_cnt = c.at<uint2>(c.ws.tile_cnt);
+    const PlanCounts counts{tile_cnt, c.at<unsigned long long>(c.ws.plan_sections)};
+    // the reduce pass puts the sections back to zero; a plan that never got there left them
+    if (c.plan_sections_dirty) {
+        cudaError_t me = enqueue_memset(counts.section, sizeof(unsigned long long) * (size_t)c.plan_sections_dirty, st);
+        if (me != cudaSuccess) return me;
+    }
+    c.plan_sections_dirty = (int)ceil_div(n_tiles, AF_SECTION);
+    cudaError_t e;
     { KernelScope k(&c.prof, "acc_flag", st);
-    launch_dependent(acc_flag_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, n, (uint32_t)vocab, div, c.buf.dfv_gcnt, tile_cnt, state); }
-    scan_pairs(tile_cnt, n_tiles, tile_cnt + n_tiles, st, &c.prof);
+    e = launch_dependent(acc_flag_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, n, (uint32_t)vocab, div, c.buf.dfv_gcnt, counts, state); }
+    if (e != cudaSuccess) return e;
     RowSource rs{perm, nullptr, 0, src_row, scale};
-    { KernelScope k(&c.prof, "acc_plan", st);
-    launch_dependent(acc_plan_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, n, (uint32_t)vocab, div, c.buf.dfv_gcnt, tile_cnt,
-                     c.at<uint4>(c.ws.grp_rec), rs, c.at<int2>(c.ws.pmeta), c.at<uint32_t>(c.ws.blk_first),
-                     c.at<uint32_t>(c.ws.run_end), acc_span_log2(n), state); }
-    return cudaGetLastError();
+    KernelScope k(&c.prof, "acc_plan", st);
+    return launch_dependent(acc_plan_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, n, (uint32_t)vocab, div, c.buf.dfv_gcnt, counts, tile_cnt + n_tiles,
+                            c.at<uint4>(c.ws.grp_rec), rs, c.at<int2>(c.ws.pmeta), c.at<uint32_t>(c.ws.blk_first),
+                            c.at<uint32_t>(c.ws.run_end), acc_span_log2(n), state);
 }
 
 // The plan for the image occurrences of the batch gear_forward_backward has just sorted, enqueued ahead of the
@@ -566,7 +611,7 @@ static cudaError_t launch_accumulate_to(const gear_ctx_impl& c, const int32_t* i
         if (le != cudaSuccess) return;
         le = launch_dependent(kernel, dim3(grid), dim3(256), (size_t)smem, st, rg, D, make_div(M), span, c.ws.ready_cap, c.at<uint2>(c.ws.tile_cnt) + ceil_div(n, AF_TILE), grp_rec, blk_first, run_end,
                                         c.buf.dfv_gsum, c.buf.dfv_gcnt, c.at<int32_t>(c.ws.q_id),
-                                        c.at<float>(c.ws.q_avg), to_caller, state);
+                                        c.at<float>(c.ws.q_avg), to_caller, c.at<unsigned long long>(c.ws.plan_sections), c.plan_sections_dirty, state);
     };
     // ring depth: as many row slots as about 96 KB per block (two blocks per SM) allow, at most 8.
     // FULL only when a row fills the instantiated width exactly (D == NQ * 128): every lane then owns a chunk of every
@@ -580,6 +625,7 @@ static cudaError_t launch_accumulate_to(const gear_ctx_impl& c, const int32_t* i
 #undef GEAR_ACC_LAUNCH
     }
     if (le != cudaSuccess) return le;
+    c.plan_sections_dirty = 0;
     if (!to_caller.avg) ++c.acc_calls_pending;                    // a call that bypasses the queue leaves it empty (a call
                                                                   // that may or may not bypass it: see launch_accumulate_collect)
     return cudaGetLastError();

@@ -90,6 +90,7 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
         p->sort_tot[s] = take((size_t)RS_BUCKETS * 4);
     }
     p->tile_cnt = take((size_t)(ceil_div(c.max_nnz, 1024) + 1) * sizeof(uint2));
+    p->plan_sections = take((size_t)(ceil_div(ceil_div(c.max_nnz, 1024), 64) + 1) * 8);
     p->grp_rec = take((size_t)c.max_nnz * 16);
     p->pmeta = take((size_t)c.max_nnz * 8);
     p->blk_first = take((size_t)acc_max_spans(c.max_nnz) * 4);
@@ -307,6 +308,7 @@ template <typename Fn> static int run_call(gear_ctx_impl& c, const char* where, 
     else e = rec.play(&c.prof);
     if (e == cudaSuccess) return GEAR_OK;
     c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
+    c.plan_sections_dirty = (int)((c.ws.grp_rec - c.ws.plan_sections) / 8);
     return cuda_fail(e, where);
 }
 
@@ -377,7 +379,8 @@ int gear_init_tables(gear_ctx** out_ctx, const gear_config* cfg, const gear_buff
     for (cudaEvent_t& ev : c.ev)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
     if (e == cudaSuccess) e = enqueue_memset(c.state(), sizeof(DevState), st);
-    // the expiry scan's section counts start from zero
+    // section counts start from zero
+    if (e == cudaSuccess) e = enqueue_memset(c.at<char>(c.ws.plan_sections), c.ws.grp_rec - c.ws.plan_sections, st);
     if (e == cudaSuccess) e = enqueue_memset(c.at<char>(c.ws.exp_cnt), c.ws.total - c.ws.exp_cnt, st);
     if (e == cudaSuccess && fill) {
         const double amp = 0.17320508075688773;   // uniform half-width for standard deviation 0.1

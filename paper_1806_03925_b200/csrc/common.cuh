@@ -245,14 +245,14 @@ inline DivM make_div(int M) {
 }
 
 // ---------------------------------------------------------------- radix sort / scans (prims.cu)
-constexpr int RS_THREADS = 256;
+constexpr int RS_THREADS = 512;
 constexpr int RS_RADIX_BITS = 9;
 constexpr int RS_BUCKETS = 1 << RS_RADIX_BITS;
-constexpr int RS_MAX_BLOCKS = 512;        // of the sort's grid (three per SM)
+constexpr int RS_MAX_BLOCKS = 512;        // of the sort's grid (two per SM)
 
-// most blocks a job can get: one per tile of RS_THREADS * 8 entries
+// most blocks a job can get: one per tile of RS_THREADS * 4 entries
 inline int64_t sort_max_blocks(int64_t n_max) {
-    const int64_t tiles = ceil_div(n_max, RS_THREADS * 8);
+    const int64_t tiles = ceil_div(n_max, RS_THREADS * 4);
     return tiles < 1 ? 1 : tiles < RS_MAX_BLOCKS ? tiles : RS_MAX_BLOCKS;
 }
 
@@ -292,9 +292,6 @@ struct GridBarrierState {
 // Sorts every job of the batch in one cooperative launch.  Returns the index (0 or 1) of the keys/vals
 // buffer pair that holds the sorted result of every job.
 int sort_jobs(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st, Profiler* prof, cudaError_t* err_out);
-
-// In-place exclusive scan of m (a, b) counter pairs by one block; the totals go to total[0..1].
-void scan_pairs(uint2* data, int64_t m, uint2* total, cudaStream_t st, Profiler* prof);
 
 inline int bits_for(int64_t max_key_inclusive) {
     int b = 1;

@@ -32,6 +32,7 @@ struct WsPlan {
     size_t sort_hist[4], sort_tot[4];
     int64_t sort_n[4];
     size_t tile_cnt;                    // [plan tiles + 1] uint2 per-tile (groups, complete) counts, then their totals
+    size_t plan_sections;               // 64-bit counts per section of the accumulate plan
     size_t grp_rec;                     // [max_nnz] uint4 group records (start | first flag, image ID, queue slot, held rows)
     size_t blk_first;                   // [acc_max_spans] uint32: first group that starts in each span of sorted positions
     size_t run_end;                     // [max_nnz] uint32: at the first position of an image's run, one past its last
@@ -79,6 +80,7 @@ struct gear_ctx_impl {
     Player player;                     // plays what a call has written down
     mutable Profiler prof;
     mutable GridBarrierState gbs;
+    mutable int plan_sections_dirty = 0;    // section counts a plan has added to and no reduce pass has cleared yet
     mutable int expiry_set = 0;             // which set of section counts the last expiry scan used
     // image IDs of the last gear_forward_backward batch, already sorted (reused by gear_accumulate_dfv_grad)
     const int32_t* last_img_id;         // img_id array of that batch (the atomic mode reads it unsorted)
