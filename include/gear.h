@@ -311,30 +311,38 @@ int gear_apply_emb_grad(gear_ctx* ctx, int32_t which, const int32_t* ids, const 
                         float lr, void* stream);
 
 /*
- * The same exchange when the shards of all ranks are memory of this device (any number of ranks up to
- * GEAR_MAX_LOCAL_RANKS): no rows travel through send and receive buffers.  All lists are the workers' lists one behind the
- * other, sender by sender; start[s] is where sender s's entries begin, start[world] their number (host array, [3][world + 1],
- * tables in the order user, URL, images).
- *
- * gear_shard_fetch     events 1 to 3: row k of sender s gets row (id div world) of the table shard of owner (id mod world), for
- *                      all three tables: out[t] + (s * out_stride[t] + k) rows.  An ID outside its owner's shard gives a zero
- *                      row and raises GEAR_DEV_BAD_ID at the owner.
- * gear_shard_route     picks every owner's arrivals out of the lists, in arrival order (sender by sender, each in its own row
- *                      order): local[t][owner][.] = id div world, src[t][owner][.] = s * src_stride[t] + k;
- *                      both arrays are [world][start[world]] per table.  counts (device, [3][world]): their numbers.
- * gear_owner_step      what one owner does with its arrivals: the same results as gear_apply_emb_grad on both tables,
- *                      gear_accumulate_collect and gear_collect_expired.  The gradient row of entry k of a list is row
- *                      src[k]: of emb_rows (user gradient in columns 0 .. emb_dim, URL gradient behind it), and of img_rows.
+ * A whole step of a job whose tables are partitioned by ID over `world` ranks when all ranks' shards are memory of this
+ * device: the same results as the exchange above, without send and receive buffers, in one call.  Owner o holds row
+ * (id div world) of every ID with id mod world = o; rank s is also a worker with a batch of its own.
+ *   - the batches (host arrays) travel in one copy;
+ *   - a worker's rows are read straight from the owners' tables into the worker's own tables (rows 0, 1, 2, ... in the order of
+ *     its ID lists; an ID outside its owner's shard gives a zero row and raises GEAR_DEV_BAD_ID at the owner);
+ *   - gear_forward_backward on every worker with learning rate 0, side by side;
+ *   - mean_head_grad: every worker's head_grad becomes the mean over the workers;
+ *   - every owner takes its arrivals, sender by sender, each in its own row order: gear_apply_emb_grad on both embedding tables
+ *     (rate lr), gear_accumulate_collect, gear_collect_expired with restamp, with the lists of its own.
+ * counts (host, [world][2]): averages handed over and images listed per owner.  The call returns when they are known;
+ * GEAR_ERR_CAPACITY if a list was too small (see the calls named).
  */
 enum { GEAR_MAX_LOCAL_RANKS = 8 };
-typedef struct { const int32_t* ids; const int32_t* src; int64_t n; } gear_arrivals;
-int gear_shard_fetch(gear_ctx* const* owners, int32_t world, const int32_t* const* ids, const int32_t* start, void* const* out,
-                     const int64_t* out_stride, void* stream);
-int gear_shard_route(int32_t world, const int32_t* const* ids, const int32_t* start, const int64_t* src_stride,
-                     int32_t* const* local, int32_t* const* src, int32_t* counts, void* stream);
-int gear_owner_step(gear_ctx* ctx, const gear_arrivals* user, const gear_arrivals* url, const gear_arrivals* img,
-                    const float* emb_rows, int64_t emb_ld, const float* img_rows, int64_t img_ld, float lr,
-                    const gear_step_lists* lists, int64_t now, int restamp, void* stream);
+typedef struct {
+    int32_t world;
+    int32_t max_batch; int64_t max_nnz;      /* per worker (the workers' own max_batch and max_nnz are at least these) */
+    gear_ctx* const* owners;                 /* [world] */
+    gear_ctx* const* workers;                /* [world] tables of max_batch / max_batch / max_nnz rows */
+    int32_t* host_stage; int32_t* stage;     /* pinned host memory and device memory of gear_shard_stage_words words each */
+    const int32_t* iota;                     /* device: 0, 1, 2, ... max(max_batch, max_nnz) - 1 */
+    const gear_step_out* out;                /* [world] workers' outputs (host array).  dX of worker s starts s * max_batch rows behind
+                                                that of worker 0, dfv_grad s * max_nnz rows; prob optional as always */
+    const gear_step_lists* lists;            /* [world] owners' lists (host array) */
+} gear_shard_plan;
+typedef struct {                             /* host arrays of one worker's batch, as in gear_batch */
+    int32_t B; int64_t nnz;
+    const int32_t* user_id; const int32_t* url_id; const int32_t* img_off; const int32_t* img_id; const float* label;
+} gear_host_batch;
+int gear_shard_stage_words(int32_t world, int32_t max_batch, int64_t max_nnz, int64_t* words);
+int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches, float lr, int64_t now, int mean_head_grad,
+                    int64_t* counts, void* stream);
 
 /*
  * The smallest Dense Part there is, for closing the loop on one device: DFV[id] = raw[id] . Wd, with raw

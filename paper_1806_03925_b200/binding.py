@@ -28,7 +28,7 @@ EXPORTS = ("gear_workspace_bytes", "gear_init_tables", "gear_forward_backward", 
            "gear_last_error", "gear_profile_enable", "gear_profile_read", "gear_launch_count",
            "gear_collect_expired_static", "gear_refresh_dfv", "gear_accumulate_collect", "gear_dense_forward",
            "gear_dense_backward", "gear_adam_dense", "gear_fetch_rows", "gear_apply_emb_grad", "gear_profile_timeline", "gear_step",
-           "gear_shard_fetch", "gear_shard_route", "gear_owner_step")
+           "gear_shard_stage_words", "gear_shard_step")
 GEAR_STATIC_EXPIRY_MAX_VOCAB = 16777216
 GEAR_MAX_LOCAL_RANKS = 8
 
@@ -75,8 +75,15 @@ class gear_step_lists(C.Structure):
                 ("expired", C.c_void_p), ("expired_cap", C.c_int64), ("d_expired", C.c_void_p)]
 
 
-class gear_arrivals(C.Structure):
-    _fields_ = [("ids", C.c_void_p), ("src", C.c_void_p), ("n", C.c_int64)]
+class gear_shard_plan(C.Structure):
+    _fields_ = [("world", C.c_int32), ("max_batch", C.c_int32), ("max_nnz", C.c_int64), ("owners", C.POINTER(C.c_void_p)),
+                ("workers", C.POINTER(C.c_void_p)), ("host_stage", C.c_void_p), ("stage", C.c_void_p), ("iota", C.c_void_p),
+                ("out", C.POINTER(gear_step_out)), ("lists", C.POINTER(gear_step_lists))]
+
+
+class gear_host_batch(C.Structure):
+    _fields_ = [("B", C.c_int32), ("nnz", C.c_int64), ("user_id", C.c_void_p), ("url_id", C.c_void_p), ("img_off", C.c_void_p),
+                ("img_id", C.c_void_p), ("label", C.c_void_p)]
 
 
 _lib = None
@@ -108,14 +115,10 @@ def load() -> C.CDLL:
     L.gear_step.restype = C.c_int
     L.gear_step.argtypes = [vp, C.POINTER(gear_batch), C.c_float, C.POINTER(gear_step_out), C.POINTER(gear_step_lists), i64, C.c_int,
                             C.c_int, C.POINTER(i64), vp]
-    pvp, pi32, pi64 = C.POINTER(vp), C.POINTER(i32), C.POINTER(i64)
-    L.gear_shard_fetch.restype = C.c_int
-    L.gear_shard_fetch.argtypes = [pvp, i32, pvp, pi32, pvp, pi64, vp]
-    L.gear_shard_route.restype = C.c_int
-    L.gear_shard_route.argtypes = [i32, pvp, pi32, pi64, pvp, pvp, vp, vp]
-    L.gear_owner_step.restype = C.c_int
-    L.gear_owner_step.argtypes = [vp, C.POINTER(gear_arrivals), C.POINTER(gear_arrivals), C.POINTER(gear_arrivals), vp, i64, vp, i64,
-                                  C.c_float, C.POINTER(gear_step_lists), i64, C.c_int, vp]
+    L.gear_shard_stage_words.restype = C.c_int
+    L.gear_shard_stage_words.argtypes = [i32, i32, i64, C.POINTER(i64)]
+    L.gear_shard_step.restype = C.c_int
+    L.gear_shard_step.argtypes = [C.POINTER(gear_shard_plan), C.POINTER(gear_host_batch), C.c_float, i64, C.c_int, C.POINTER(i64), vp]
     L.gear_fetch_rows.restype = C.c_int
     L.gear_fetch_rows.argtypes = [vp, i32, vp, i64, vp, vp]
     L.gear_apply_emb_grad.restype = C.c_int
@@ -313,20 +316,15 @@ def gear_step_structs(ctx, bt: gear_batch, lr: float, o: gear_step_out, lists: g
     return (h[0], h[1]) if sync else (None, None)
 
 
-def gear_shard_fetch(owners, world: int, ids, start, out, out_stride, stream=None):
-    """owners, ids, out: ctypes arrays of pointers; start: c_int32 [3 * (world + 1)]; out_stride: c_int64 [3]."""
-    _check((_lib or load()).gear_shard_fetch(owners, world, ids, start, out, out_stride, _raw_stream(stream)), "gear_shard_fetch")
+def gear_shard_stage_words(world: int, max_batch: int, max_nnz: int) -> int:
+    n = C.c_int64(0)
+    _check(load().gear_shard_stage_words(world, max_batch, max_nnz, C.byref(n)), "gear_shard_stage_words")
+    return n.value
 
 
-def gear_shard_route(world: int, ids, start, src_stride, local, src, counts, stream=None):
-    _check((_lib or load()).gear_shard_route(world, ids, start, src_stride, local, src, _p(counts), _raw_stream(stream)), "gear_shard_route")
-
-
-def gear_owner_step(ctx, user: gear_arrivals, url: gear_arrivals, img: gear_arrivals, emb_rows, emb_ld: int, img_rows, img_ld: int,
-                    lr: float, lists: gear_step_lists, now: int, restamp: bool = True, stream=None):
-    """emb_rows, img_rows: device addresses."""
-    _check((_lib or load()).gear_owner_step(ctx, user, url, img, emb_rows, emb_ld, img_rows, img_ld, lr, lists, now, 1 if restamp else 0,
-                                            _raw_stream(stream)), "gear_owner_step")
+def gear_shard_step(plan: gear_shard_plan, batches, lr: float, now: int, mean_head_grad: bool, counts, stream=None):
+    """batches: ctypes array of gear_host_batch [world]; counts: c_int64 [2 * world], filled in."""
+    _check((_lib or load()).gear_shard_step(plan, batches, lr, now, 1 if mean_head_grad else 0, counts, _raw_stream(stream)), "gear_shard_step")
 
 
 def gear_collect_expired(ctx, now: int, restamp: bool, ids, cap: int, d_n=None, sync: bool = True,

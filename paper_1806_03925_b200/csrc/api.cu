@@ -112,6 +112,8 @@ static void release_host_objects(gear_ctx_impl& c) {
     for (cudaEvent_t& e : c.ev) { if (e) cudaEventDestroy(e); e = nullptr; }
     if (c.side_stream) cudaStreamDestroy(c.side_stream);
     if (c.aux_stream) cudaStreamDestroy(c.aux_stream);
+    if (c.rank_stream) cudaStreamDestroy(c.rank_stream);
+    c.rank_stream = nullptr;
     if (c.h_counts) cudaFreeHost(c.h_counts);
     c.h_counts = nullptr;
     delete_tma_cache(c.tma);
@@ -298,7 +300,101 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     return cudaSuccess;
 }
 
-// Writes a call down, plays it; on a failure the ctx forgets the batch whose order it may have been in the middle of.
+static int check_capacity(int64_t cap, int64_t n) {
+    if (n <= cap) return GEAR_OK;
+    snprintf(g_last_error, sizeof(g_last_error), "capacity %lld too small, %lld entries waiting", (long long)cap, (long long)n);
+    return GEAR_ERR_CAPACITY;
+}
+
+// Where things lie in the staging buffer of a partitioned job (words): the five lists of the batches, the numbers of arrivals, and
+// on the device each owner's arrivals per table.
+struct ShardStage {
+    int64_t list[5], counts, local[3], src[3], words = 0;
+    ShardStage(int W, int64_t max_batch, int64_t max_nnz) {
+        auto take = [&](int64_t n) { const int64_t at = words; words += (n + 3) / 4 * 4; return at; };
+        const int64_t cap[5] = {W * max_batch, W * max_batch, W * max_nnz, W * (max_batch + 1), W * max_batch};
+        for (int t = 0; t < 5; ++t) list[t] = take(cap[t]);
+        counts = take(3 * W);
+        for (int t = 0; t < 3; ++t) { local[t] = take(W * cap[t]); src[t] = take(W * cap[t]); }
+    }
+};
+
+// both counts of a step to the ctx's pinned words (one copy where they lie side by side)
+static cudaError_t enqueue_counts(gear_ctx_impl& c, const int64_t* d_n, const int64_t* d_expired, cudaStream_t st) {
+    if (d_expired == d_n + 1) return enqueue_copy(c.h_counts, d_n, 2 * sizeof(int64_t), st);
+    cudaError_t e = enqueue_copy(c.h_counts, d_n, sizeof(int64_t), st);
+    return e == cudaSuccess ? enqueue_copy(c.h_counts + 1, d_expired, sizeof(int64_t), st) : e;
+}
+
+// What one owner of a partitioned job does with its arrivals: the sort of their IDs (the sorted values are the rows' places, so no
+// indirection is left behind it), embedding rows, gradient store and hand-over; the expiry scan beside them.
+struct Arrivals { const int32_t* ids; const int32_t* src; int64_t n; };
+static cudaError_t enqueue_owner(gear_ctx_impl& c, const Arrivals& user, const Arrivals& url, const Arrivals& img, const float* emb_rows,
+                                 int64_t emb_ld, const float* img_rows, int64_t img_ld, float lr, const gear_step_lists& lists, int64_t now,
+                                 cudaStream_t st) {
+    int64_t* d_n = lists.d_n ? lists.d_n : &c.state()->pad[0];
+    int64_t* d_expired = lists.d_expired ? lists.d_expired : &c.state()->pad[1];
+#define GEAR_TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return e_; } while (0)
+    const bool apart = !c.prof.on || c.prof.keep_streams, sorted_mode = c.cfg.accum_mode == GEAR_ACC_SORT;
+    const cudaStream_t side = apart ? c.side_stream : st, aux = apart ? c.aux_stream : st;
+    if (apart) {
+        GEAR_TRY(enqueue_record(c.ev[0], st));
+        GEAR_TRY(enqueue_wait(aux, c.ev[0]));
+    }
+    GEAR_TRY(launch_collect_expired(c, now, 1, lists.expired, lists.expired_cap, d_expired, aux));
+    SortBatch batch = c.sort_batch();
+    batch.name = "sort_ids";
+    auto add = [&](const Arrivals& a, int which, int64_t vocab) {
+        if (a.n == 0) return;
+        SortJob& j = batch.job[batch.n_jobs++];
+        j = c.sort_job(which);
+        j.ids = a.ids; j.src = a.src; j.sentinel = (uint32_t)vocab; j.n_max = a.n; j.bits = bits_for(vocab);
+    };
+    c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
+    add(user, gear_ctx_impl::SORT_USER, c.cfg.user_vocab);
+    add(url, gear_ctx_impl::SORT_URL, c.cfg.url_vocab);
+    if (sorted_mode) add(img, gear_ctx_impl::SORT_IMG, c.cfg.img_vocab);
+    const bool plan = sorted_mode && img.n > 0;
+    int cur = 0;
+    if (batch.n_jobs > 0) {
+        if (sort_small_fits(batch)) GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, img.n, nullptr, nullptr) : PlanArgs{}, st));
+        else {
+            cudaError_t se;
+            cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
+            if (se != cudaSuccess) return se;
+        }
+    }
+    if (apart) {
+        GEAR_TRY(enqueue_record(c.ev[1], st));
+        GEAR_TRY(enqueue_wait(side, c.ev[1]));
+    }
+    GEAR_TRY(launch_emb_arrivals(c, cur, user.n, url.n, c.buf.user_emb, c.buf.url_emb, emb_rows, emb_ld, -lr, side));
+    if (plan) {
+        c.img_sorted = true; c.img_sorted_n = img.n; c.img_sorted_buf = cur; c.img_sort_valid = true; c.last_img_id = img.ids;
+        if (sort_small_fits(batch)) note_plan(c, img.n, nullptr, nullptr);
+        else GEAR_TRY(launch_accumulate_plan_ahead(c, img.n, nullptr, nullptr, st));
+    }
+    // (the sorted values are the source rows, so the accumulate call itself has no row indirection left)
+    GEAR_TRY(launch_accumulate_collect(c, plan ? nullptr : img.ids, img_rows, img_ld, plan ? nullptr : img.src, nullptr, img.n, lists.ids,
+                                       lists.seq, lists.avg, lists.cap, d_n, st));
+    c.img_sorted = false; c.img_sort_valid = false;
+    if (apart) {
+        GEAR_TRY(enqueue_record(c.ev[2], side));
+        GEAR_TRY(enqueue_wait(st, c.ev[2]));
+        GEAR_TRY(enqueue_record(c.ev[3], aux));
+        GEAR_TRY(enqueue_wait(st, c.ev[3]));
+    }
+    return enqueue_counts(c, d_n, d_expired, st);
+#undef GEAR_TRY
+}
+
+// The ctx forgets the batch whose order it may have been in the middle of.
+static void forget_batch(gear_ctx_impl& c) {
+    c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
+    c.plan_sections_dirty = (int)((c.ws.grp_rec - c.ws.plan_sections) / 8);
+}
+
+// Writes a call down and plays it.
 template <typename Fn> static int run_call(gear_ctx_impl& c, const char* where, cudaStream_t st, Fn&& enqueue) {
     c.last_stream = st;
     const unsigned long long base = c.gbs.host_base;
@@ -307,8 +403,7 @@ template <typename Fn> static int run_call(gear_ctx_impl& c, const char* where, 
     if (e != cudaSuccess) c.gbs.host_base = base;            // nothing has been enqueued
     else e = rec.play(&c.prof);
     if (e == cudaSuccess) return GEAR_OK;
-    c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
-    c.plan_sections_dirty = (int)((c.ws.grp_rec - c.ws.plan_sections) / 8);
+    forget_batch(c);
     return cuda_fail(e, where);
 }
 
@@ -423,11 +518,6 @@ int gear_accumulate_dfv_grad(gear_ctx* ctx, const int32_t* img_id, const float* 
 }
 
 static int finish_count(gear_ctx_impl& c, const int64_t* d_src, int64_t cap, int64_t* h_n, cudaStream_t st);
-static int check_capacity(int64_t cap, int64_t n) {
-    if (n <= cap) return GEAR_OK;
-    snprintf(g_last_error, sizeof(g_last_error), "capacity %lld too small, %lld entries waiting", (long long)cap, (long long)n);
-    return GEAR_ERR_CAPACITY;
-}
 
 int gear_accumulate_collect(gear_ctx* ctx, const int32_t* img_id, const float* grads, int64_t ld, const int32_t* src_row,
                             const float* scale, int64_t n, int32_t* ids, int32_t* seq, float* avg, int64_t cap,
@@ -457,12 +547,13 @@ int gear_step(gear_ctx* ctx, const gear_batch* batch, float lr, const gear_step_
     const StepLists l{lists->ids, lists->seq, lists->avg, lists->cap, lists->d_n ? lists->d_n : &c.state()->pad[0],
                       lists->expired, lists->expired_cap, lists->d_expired ? lists->d_expired : &c.state()->pad[1],
                       now, restamp, scan_beside != 0};
-    if (int rc = run_call(c, "step", st, [&] { return enqueue_step(c, *batch, lr, *out, &l, st); })) return rc;
+    if (int rc = run_call(c, "step", st, [&]() -> cudaError_t {
+            cudaError_t e = enqueue_step(c, *batch, lr, *out, &l, st);
+            return e == cudaSuccess && h_n ? enqueue_counts(c, l.d_n, l.d_expired, st) : e;
+        }))
+        return rc;
     if (!h_n) return GEAR_OK;
-    // both counts with one wait
-    cudaError_t e = cudaMemcpyAsync(c.h_counts, l.d_n, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c.h_counts + 1, l.d_expired, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    cudaError_t e = cudaStreamSynchronize(st);               // both counts with one wait
     if (e != cudaSuccess) return cuda_fail(e, "read counts");
     h_n[0] = c.h_counts[0]; h_n[1] = c.h_counts[1];
     if (int rc = check_capacity(l.cap, h_n[0])) return rc;
@@ -552,126 +643,171 @@ int gear_apply_emb_grad(gear_ctx* ctx, int32_t which, const int32_t* ids, const 
     return run_call(c, "apply_emb_grad", st, [&] { return launch_apply_emb_grad(c, which, ids, rows, ld, n, -lr, st); });
 }
 
-int gear_shard_fetch(gear_ctx* const* owners, int32_t world, const int32_t* const* ids, const int32_t* start, void* const* out,
-                     const int64_t* out_stride, void* stream) {
-    if (!owners || !ids || !start || !out || !out_stride || world < 1 || world > GEAR_MAX_LOCAL_RANKS) return arg_fail("gear_shard_fetch");
+int gear_shard_stage_words(int32_t world, int32_t max_batch, int64_t max_nnz, int64_t* words) {
+    if (!words || world < 1 || world > GEAR_MAX_LOCAL_RANKS || max_batch < 1 || max_nnz < 1) return arg_fail("gear_shard_stage_words");
+    *words = ShardStage(world, max_batch, max_nnz).words;
+    return GEAR_OK;
+}
+
+int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches, float lr, int64_t now, int mean_head_grad, int64_t* counts,
+                    void* stream) {
+    if (!plan || !batches || !counts) return arg_fail("NULL pointer");
+    const gear_shard_plan& p = *plan;
+    const int W = p.world;
+    if (W < 1 || W > GEAR_MAX_LOCAL_RANKS || p.max_batch < 1 || p.max_nnz < 1 || !p.owners || !p.workers || !p.host_stage || !p.stage ||
+        !p.iota || !p.out || !p.lists)
+        return arg_fail("gear_shard_plan");
+    // ---- what the call will read and write
+    gear_batch bt[GEAR_MAX_LOCAL_RANKS] = {};
+    const gear_config* g0 = nullptr;
+    for (int s = 0; s < W; ++s) {
+        if (!p.owners[s] || !p.owners[s]->impl.alive || !p.workers[s] || !p.workers[s]->impl.alive) return GEAR_ERR_STATE;
+        const gear_ctx_impl &o = p.owners[s]->impl, &w = p.workers[s]->impl;
+        if (!g0) g0 = &o.cfg;
+        for (const gear_config* g : {&o.cfg, &w.cfg})
+            if (g->emb_dim != g0->emb_dim || g->dfv_dim != g0->dfv_dim || g->dfv_dtype != g0->dfv_dtype || g->fast_dim != 0)
+                return arg_fail("the ranks' tables differ, or have a dense input of their own");
+        if (w.d_in != p.workers[0]->impl.d_in || w.n_params != p.workers[0]->impl.n_params) return arg_fail("the ranks' heads differ");
+        if (w.cfg.user_vocab < p.max_batch || w.cfg.url_vocab < p.max_batch || w.cfg.img_vocab < p.max_nnz) return arg_fail("a worker's tables are too small");
+        const gear_host_batch& b = batches[s];
+        if (b.B < 0 || b.B > p.max_batch || b.nnz < 0 || b.nnz > p.max_nnz) return arg_fail("a batch is larger than the plan's");
+        if ((b.B > 0 && (!b.user_id || !b.url_id || !b.img_off || !b.label)) || (b.nnz > 0 && !b.img_id)) return arg_fail("NULL batch array");
+        const gear_step_out& out = p.out[s];
+        if (!out.dfv_grad || out.dX != p.out[0].dX + (int64_t)s * p.max_batch * w.d_in ||
+            out.dfv_grad != p.out[0].dfv_grad + (int64_t)s * p.max_nnz * g0->dfv_dim)
+            return arg_fail("the workers' gradient rows do not lie one behind the other");
+        bt[s].B = b.B; bt[s].nnz = b.nnz;
+        bt[s].user_id = bt[s].url_id = bt[s].img_id = p.iota;
+        bt[s].img_off = bt[s].img_id; bt[s].label = reinterpret_cast<const float*>(p.iota);      // (set below)
+        if (int rc = check_batch(w, bt[s], out)) return rc;
+        const gear_step_lists& l = p.lists[s];
+        if (int rc = check_lists(l.ids, l.seq, l.avg, l.cap)) return rc;
+        if (l.expired_cap < 0 || (l.expired_cap > 0 && !l.expired)) return arg_fail("NULL output with cap > 0");
+        if ((int64_t)W * p.max_batch > o.cfg.max_batch || (int64_t)W * p.max_nnz > o.cfg.max_nnz) return arg_fail("an owner's max_batch or max_nnz is too small");
+    }
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    cudaError_t e = cudaSuccess;
+    for (int s = 1; s < W && e == cudaSuccess; ++s)
+        if (!p.owners[s]->impl.rank_stream) e = cudaStreamCreateWithFlags(&p.owners[s]->impl.rank_stream, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return cuda_fail(e, "shard_step");
+    // ---- the batches: lists sender by sender in the staging buffer, one copy
+    const ShardStage at(W, p.max_batch, p.max_nnz);
     ShardFetch f{};
-    f.world = world;
-    for (int r = 0; r < world; ++r) {
-        if (!owners[r] || !owners[r]->impl.alive) return GEAR_ERR_STATE;
-        const gear_ctx_impl& c = owners[r]->impl;
-        const gear_config &g = c.cfg, &g0 = owners[0]->impl.cfg;
-        if (g.emb_dim != g0.emb_dim || g.dfv_dim != g0.dfv_dim || g.dfv_dtype != g0.dfv_dtype) return arg_fail("the shards' rows differ");
-        f.state[r] = c.state();
-        const void* shard[3] = {c.buf.user_emb, c.buf.url_emb, c.buf.dfv};
-        const int64_t rows[3] = {g.user_vocab, g.url_vocab, g.img_vocab};
-        for (int t = 0; t < 3; ++t) { f.table[t].shard[r] = static_cast<const uint4*>(shard[t]); f.table[t].rows[r] = rows[t]; }
-    }
-    const gear_config& g = owners[0]->impl.cfg;
-    bool any = false;
-    for (int t = 0; t < 3; ++t) {
-        ShardFetch::Table& x = f.table[t];
-        x.chunks = t < 2 ? g.emb_dim / 4 : g.dfv_dim / (g.dfv_dtype == GEAR_BF16 ? 8 : 4);
-        x.ids = ids[t]; x.out = static_cast<uint4*>(out[t]); x.out_stride = out_stride[t];
-        for (int r = 0; r <= world; ++r) x.start[r] = start[t * (world + 1) + r];
-        if (x.start[world] > 0 && (!ids[t] || !out[t] || !aligned16(out[t]))) return arg_fail("NULL or misaligned pointer");
-        any = any || x.start[world] > 0;
-    }
-    if (!any) return GEAR_OK;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    for (int r = 0; r < world; ++r) owners[r]->impl.note_stream(st);
-    cudaError_t e = launch_shard_fetch(&owners[0]->impl.prof, f, st);
-    return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "shard_fetch");
-}
-
-int gear_shard_route(int32_t world, const int32_t* const* ids, const int32_t* start, const int64_t* src_stride, int32_t* const* local,
-                     int32_t* const* src, int32_t* counts, void* stream) {
-    if (!ids || !start || !src_stride || !local || !src || !counts || world < 1 || world > GEAR_MAX_LOCAL_RANKS) return arg_fail("gear_shard_route");
     ShardRoute r{};
-    r.world = world; r.counts = counts;
-    for (int t = 0; t < 3; ++t) {
-        ShardRoute::Table& x = r.table[t];
-        x.ids = ids[t]; x.local = local[t]; x.src = src[t]; x.src_stride = src_stride[t];
-        for (int k = 0; k <= world; ++k) x.start[k] = start[t * (world + 1) + k];
-        if (x.start[world] > 0 && (!ids[t] || !local[t] || !src[t])) return arg_fail("NULL pointer");
+    f.world = r.world = W;
+    r.counts = p.stage + at.counts;
+    int64_t pos[5];
+    for (int t = 0; t < 5; ++t) pos[t] = at.list[t];
+    for (int s = 0; s < W; ++s) {
+        const gear_host_batch& b = batches[s];
+        const void* src[5] = {b.user_id, b.url_id, b.img_id, b.img_off, b.label};
+        const int64_t n[5] = {b.B, b.B, b.nnz, b.B > 0 ? b.B + 1 : 0, b.B};
+        bt[s].img_off = p.stage + pos[3];
+        bt[s].label = reinterpret_cast<const float*>(p.stage + pos[4]);
+        for (int t = 0; t < 5; ++t) {
+            if (t < 3) f.table[t].start[s] = r.table[t].start[s] = (int32_t)(pos[t] - at.list[t]);
+            if (n[t]) memcpy(p.host_stage + pos[t], src[t], (size_t)n[t] * 4);
+            pos[t] += n[t];
+        }
+        const gear_ctx_impl &o = p.owners[s]->impl, &w = p.workers[s]->impl;
+        f.state[s] = o.state();
+        const void* shard[3] = {o.buf.user_emb, o.buf.url_emb, o.buf.dfv};
+        void* rows[3] = {w.buf.user_emb, w.buf.url_emb, w.buf.dfv};
+        const int64_t n_rows[3] = {o.cfg.user_vocab, o.cfg.url_vocab, o.cfg.img_vocab};
+        for (int t = 0; t < 3; ++t) {
+            f.table[t].shard[s] = static_cast<const uint4*>(shard[t]); f.table[t].rows[s] = n_rows[t];
+            f.table[t].out[s] = static_cast<uint4*>(rows[t]);
+        }
     }
-    cudaError_t e = launch_shard_route(nullptr, r, static_cast<cudaStream_t>(stream));
-    return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "shard_route");
-}
-
-int gear_owner_step(gear_ctx* ctx, const gear_arrivals* user, const gear_arrivals* url, const gear_arrivals* img, const float* emb_rows,
-                    int64_t emb_ld, const float* img_rows, int64_t img_ld, float lr, const gear_step_lists* lists, int64_t now,
-                    int restamp, void* stream) {
-    if (!ctx || !ctx->impl.alive) return GEAR_ERR_STATE;
-    if (!user || !url || !img || !lists) return arg_fail("NULL pointer");
-    gear_ctx_impl& c = ctx->impl;
-    if (user->n < 0 || user->n > c.cfg.max_batch || url->n < 0 || url->n > c.cfg.max_batch) return arg_fail("n outside [0, max_batch]");
-    if (img->n < 0 || img->n > c.cfg.max_nnz) return arg_fail("n outside [0, max_nnz]");
-    if ((user->n || url->n) && (!emb_rows || !aligned16(emb_rows) || emb_ld < 2 * c.cfg.emb_dim || (emb_ld & 3)))
-        return arg_fail("emb_rows: 16-byte aligned, ld >= 2 emb_dim, multiple of 4");
-    if (img->n && (!img_rows || !aligned16(img_rows) || img_ld < c.cfg.dfv_dim || (img_ld & 3)))
-        return arg_fail("img_rows: 16-byte aligned, ld >= dfv_dim, multiple of 4");
-    for (const gear_arrivals* a : {user, url, img})
-        if (a->n > 0 && (!a->ids || !a->src)) return arg_fail("NULL list");
-    if (int rc = check_lists(lists->ids, lists->seq, lists->avg, lists->cap)) return rc;
-    if (lists->expired_cap < 0 || (lists->expired_cap > 0 && !lists->expired)) return arg_fail("NULL output with cap > 0");
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    int64_t* d_n = lists->d_n ? lists->d_n : &c.state()->pad[0];
-    int64_t* d_expired = lists->d_expired ? lists->d_expired : &c.state()->pad[1];
-    return run_call(c, "owner_step", st, [&]() -> cudaError_t {
+    int64_t total[3];
+    for (int t = 0; t < 3; ++t) {
+        total[t] = pos[t] - at.list[t];
+        f.table[t].ids = r.table[t].ids = p.stage + at.list[t];
+        f.table[t].start[W] = r.table[t].start[W] = (int32_t)total[t];
+        f.table[t].chunks = t < 2 ? g0->emb_dim / 4 : g0->dfv_dim / (g0->dfv_dtype == GEAR_BF16 ? 8 : 4);
+        r.table[t].local = p.stage + at.local[t]; r.table[t].src = p.stage + at.src[t];
+        r.table[t].src_stride = t < 2 ? p.max_batch : p.max_nnz;
+    }
+    gear_ctx_impl &w0 = p.workers[0]->impl, &o0 = p.owners[0]->impl;
+    unsigned long long base[2 * GEAR_MAX_LOCAL_RANKS];
+    for (int s = 0; s < W; ++s) {
+        base[2 * s] = p.workers[s]->impl.gbs.host_base; base[2 * s + 1] = p.owners[s]->impl.gbs.host_base;
+        p.workers[s]->impl.last_stream = p.owners[s]->impl.last_stream = st;
+    }
+    auto fail = [&](cudaError_t err, bool enqueued) {
+        for (int s = 0; s < W; ++s) {
+            if (!enqueued) { p.workers[s]->impl.gbs.host_base = base[2 * s]; p.owners[s]->impl.gbs.host_base = base[2 * s + 1]; }
+            for (gear_ctx_impl* c : {&p.workers[s]->impl, &p.owners[s]->impl}) forget_batch(*c);
+        }
+        return cuda_fail(err, "shard_step");
+    };
+    enum { EV_RANKS = 8, EV_ROUTED = 9 };
+    e = cudaMemcpyAsync(p.stage, p.host_stage, (size_t)pos[4] * 4, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess && total[0] + total[1] + total[2] > 0) e = launch_shard_route(&w0.prof, r, st);
+    else if (e == cudaSuccess) e = cudaMemsetAsync(r.counts, 0, sizeof(int32_t) * 3 * W, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(p.host_stage + at.counts, r.counts, sizeof(int32_t) * 3 * W, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaEventRecord(w0.ev[EV_ROUTED], st);
+    if (e != cudaSuccess) return fail(e, true);
+    auto stream_of = [&](int s) { return s == 0 ? st : p.owners[s]->impl.rank_stream; };
 #define GEAR_TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return e_; } while (0)
-        const bool apart = !c.prof.on || c.prof.keep_streams, sorted_mode = c.cfg.accum_mode == GEAR_ACC_SORT;
-        const cudaStream_t side = apart ? c.side_stream : st, aux = apart ? c.aux_stream : st;
-        if (apart) {
-            GEAR_TRY(enqueue_record(c.ev[0], st));
-            GEAR_TRY(enqueue_wait(aux, c.ev[0]));
-        }
-        GEAR_TRY(launch_collect_expired(c, now, restamp, lists->expired, lists->expired_cap, d_expired, aux));
-        SortBatch batch = c.sort_batch();
-        batch.name = "sort_ids";
-        auto add = [&](const gear_arrivals& a, int which, int64_t vocab) {
-            if (a.n == 0) return;
-            SortJob& j = batch.job[batch.n_jobs++];
-            j = c.sort_job(which);
-            j.ids = a.ids; j.src = a.src; j.sentinel = (uint32_t)vocab; j.n_max = a.n; j.bits = bits_for(vocab);
-        };
-        c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
-        add(*user, gear_ctx_impl::SORT_USER, c.cfg.user_vocab);
-        add(*url, gear_ctx_impl::SORT_URL, c.cfg.url_vocab);
-        if (sorted_mode) add(*img, gear_ctx_impl::SORT_IMG, c.cfg.img_vocab);
-        const bool plan = sorted_mode && img->n > 0;
-        int cur = 0;
-        if (batch.n_jobs > 0) {
-            if (sort_small_fits(batch)) GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, img->n, nullptr, nullptr) : PlanArgs{}, st));
-            else {
-                cudaError_t se;
-                cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
-                if (se != cudaSuccess) return se;
+    // ---- events 1 to 4 on the workers, side by side
+    {
+        Recording rec(w0.player, st);
+        e = [&]() -> cudaError_t {
+            if (total[0] + total[1] + total[2] > 0) GEAR_TRY(launch_shard_fetch(&w0.prof, f, st));
+            if (W > 1) GEAR_TRY(enqueue_record(w0.ev[EV_RANKS], st));
+            for (int s = 1; s < W; ++s) GEAR_TRY(enqueue_wait(stream_of(s), w0.ev[EV_RANKS]));
+            for (int s = 0; s < W; ++s) GEAR_TRY(enqueue_step(p.workers[s]->impl, bt[s], 0.f, p.out[s], nullptr, stream_of(s)));
+            for (int s = 1; s < W; ++s) {
+                GEAR_TRY(enqueue_record(p.workers[s]->impl.ev[EV_RANKS], stream_of(s)));
+                GEAR_TRY(enqueue_wait(st, p.workers[s]->impl.ev[EV_RANKS]));
             }
-        }
-        if (apart) {
-            GEAR_TRY(enqueue_record(c.ev[1], st));
-            GEAR_TRY(enqueue_wait(side, c.ev[1]));
-        }
-        GEAR_TRY(launch_emb_arrivals(c, cur, user->n, url->n, c.buf.user_emb, c.buf.url_emb, emb_rows, emb_ld, -lr, side));
-        if (plan) {
-            c.img_sorted = true; c.img_sorted_n = img->n; c.img_sorted_buf = cur; c.img_sort_valid = true; c.last_img_id = img->ids;
-            if (sort_small_fits(batch)) note_plan(c, img->n, nullptr, nullptr);
-            else GEAR_TRY(launch_accumulate_plan_ahead(c, img->n, nullptr, nullptr, st));
-        }
-        // (the sorted values are the source rows, so the accumulate call itself has no row indirection left)
-        GEAR_TRY(launch_accumulate_collect(c, plan ? nullptr : img->ids, img_rows, img_ld, plan ? nullptr : img->src, nullptr, img->n, lists->ids,
-                                           lists->seq, lists->avg, lists->cap, d_n, st));
-        c.img_sorted = false; c.img_sort_valid = false;
-        if (apart) {
-            GEAR_TRY(enqueue_record(c.ev[2], side));
-            GEAR_TRY(enqueue_wait(st, c.ev[2]));
-            GEAR_TRY(enqueue_record(c.ev[3], aux));
-            GEAR_TRY(enqueue_wait(st, c.ev[3]));
-        }
+            if (mean_head_grad && W > 1) {
+                ShardMean m{};
+                m.world = W; m.n = w0.n_params;
+                for (int s = 0; s < W; ++s) m.p[s] = p.out[s].head_grad;
+                GEAR_TRY(launch_shard_mean(&w0.prof, m, st));
+            }
+            return cudaSuccess;
+        }();
+        if (e != cudaSuccess) return fail(e, false);
+        e = rec.play(&w0.prof);
+    }
+    if (e == cudaSuccess) e = cudaEventSynchronize(w0.ev[EV_ROUTED]);
+    if (e != cudaSuccess) return fail(e, true);
+    // ---- events 4 (push), 5 and 6 at the owners, side by side
+    {
+        Recording rec(o0.player, st);
+        e = [&]() -> cudaError_t {
+            if (W > 1) GEAR_TRY(enqueue_record(o0.ev[EV_RANKS], st));
+            for (int s = 0; s < W; ++s) {
+                gear_ctx_impl& c = p.owners[s]->impl;
+                Arrivals a[3];
+                for (int t = 0; t < 3; ++t)
+                    a[t] = Arrivals{r.table[t].local + s * total[t], r.table[t].src + s * total[t], (int64_t)p.host_stage[at.counts + t * W + s]};
+                if (s > 0) GEAR_TRY(enqueue_wait(stream_of(s), o0.ev[EV_RANKS]));
+                GEAR_TRY(enqueue_owner(c, a[0], a[1], a[2], p.out[0].dX, w0.d_in, p.out[0].dfv_grad, g0->dfv_dim, lr, p.lists[s], now, stream_of(s)));
+                if (s > 0) {
+                    GEAR_TRY(enqueue_record(c.ev[EV_ROUTED], stream_of(s)));
+                    GEAR_TRY(enqueue_wait(st, c.ev[EV_ROUTED]));
+                }
+            }
+            return cudaSuccess;
+        }();
+        if (e != cudaSuccess) return fail(e, true);
+        e = rec.play(&o0.prof);
+    }
 #undef GEAR_TRY
-        return cudaSuccess;
-    });
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return fail(e, true);
+    int rc = GEAR_OK;
+    for (int s = 0; s < W; ++s) {
+        const gear_ctx_impl& c = p.owners[s]->impl;
+        counts[2 * s] = c.h_counts[0]; counts[2 * s + 1] = c.h_counts[1];
+        for (int q = 0; q < 2; ++q)
+            if (int bad = check_capacity(q ? p.lists[s].expired_cap : p.lists[s].cap, counts[2 * s + q])) rc = bad;
+    }
+    return rc;
 }
 
 int gear_dense_forward(gear_ctx* ctx, const float* raw, int32_t raw_dim, const float* Wd, const int32_t* ids, int64_t n,

@@ -14,6 +14,8 @@
 
 #include <vector>
 
+#include "../../include/gear.h"
+
 namespace gear {
 
 struct Profiler;
@@ -38,7 +40,7 @@ struct Op {
 
 class OpList {
 public:
-    static constexpr int MAX_STREAMS = 4;
+    static constexpr int MAX_STREAMS = 3 * GEAR_MAX_LOCAL_RANKS + 1;
     cudaStream_t streams[MAX_STREAMS] = {};      // [0] the caller's stream
     int n_streams = 0;
     int n_kernels = 0;

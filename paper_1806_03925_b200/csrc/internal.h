@@ -75,7 +75,8 @@ struct gear_ctx_impl {
     TmaCache* tma;      // tensor maps of the head's products (tc_ptx.cuh)
     cudaStream_t side_stream;          // runs the ID sort of a step beside the gather and the head
     cudaStream_t aux_stream;           // runs the expiry scan and, for small batches, the weight gradients
-    cudaEvent_t ev[8];                 // between the streams of a step (enqueue_step in api.cu)
+    cudaStream_t rank_stream = nullptr;  // a partitioned job's rank other than the first (made on demand)
+    cudaEvent_t ev[10];                // between the streams of a step (enqueue_step, gear_shard_step in api.cu)
     int64_t* h_counts;                 // two counts on their way to the caller (pinned)
     Player player;                     // plays what a call has written down
     mutable Profiler prof;
@@ -203,7 +204,7 @@ struct ShardFetch {
     struct Table {
         const int32_t* ids; int32_t start[GEAR_MAX_LOCAL_RANKS + 1];
         const uint4* shard[GEAR_MAX_LOCAL_RANKS]; int64_t rows[GEAR_MAX_LOCAL_RANKS]; int chunks;      // 16-byte chunks of a row
-        uint4* out; int64_t out_stride;                                      // sender s's rows start at row s * out_stride
+        uint4* out[GEAR_MAX_LOCAL_RANKS];                                    // where sender s's rows go
     } table[3];
     int world;
     DevState* state[GEAR_MAX_LOCAL_RANKS];
@@ -218,6 +219,9 @@ struct ShardRoute {
 };
 cudaError_t launch_shard_fetch(Profiler* prof, const ShardFetch& f, cudaStream_t st);
 cudaError_t launch_shard_route(Profiler* prof, const ShardRoute& r, cudaStream_t st);
+// every array becomes the mean of them all
+struct ShardMean { float* p[GEAR_MAX_LOCAL_RANKS]; int world; int64_t n; };
+cudaError_t launch_shard_mean(Profiler* prof, const ShardMean& m, cudaStream_t st);
 // emb_scatter.cu: table[id] += alpha * (sum of the rows with that id), ids given explicitly (sorted here)
 cudaError_t launch_apply_emb_grad(const gear_ctx_impl& c, int which, const int32_t* ids, const float* rows, int64_t ld,
                                   int64_t n, float alpha, cudaStream_t st);

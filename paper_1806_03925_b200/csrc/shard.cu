@@ -115,16 +115,16 @@ shard_fetch_kernel(const ShardFetch f) {
     const int warps = (int)(gridDim.x * (blockDim.x >> 5));
     for (int k0 = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * SH_ROWS; k0 < n; k0 += warps * SH_ROWS) {
         const uint4* row[SH_ROWS];
-        int64_t to[SH_ROWS];
+        uint4* to[SH_ROWS];
 #pragma unroll
         for (int q = 0; q < SH_ROWS; ++q) {
             const int k = k0 + q;
-            row[q] = nullptr; to[q] = -1;
+            row[q] = nullptr; to[q] = nullptr;
             if (k < n) {
                 const int s = sender_of(t.start, f.world, k);
                 int owner, local;
                 split_id(__ldg(t.ids + k), f.world, owner, local);
-                to[q] = s * t.out_stride + (k - t.start[s]);
+                to[q] = t.out[s] + (int64_t)(k - t.start[s]) * t.chunks;
                 if (local >= 0 && local < t.rows[owner]) row[q] = t.shard[owner] + (int64_t)local * t.chunks;
                 else if (lane == 0) atomicOr(&f.state[owner]->status, GEAR_DEV_BAD_ID);       // a zero row is written
             }
@@ -134,7 +134,7 @@ shard_fetch_kernel(const ShardFetch f) {
 #pragma unroll
             for (int q = 0; q < SH_ROWS; ++q) v[q] = row[q] ? __ldg(row[q] + ch) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
-            for (int q = 0; q < SH_ROWS; ++q) if (to[q] >= 0) t.out[to[q] * t.chunks + ch] = v[q];
+            for (int q = 0; q < SH_ROWS; ++q) if (to[q]) to[q][ch] = v[q];
         }
     }
 }
@@ -188,6 +188,23 @@ cudaError_t launch_shard_fetch(Profiler* prof, const ShardFetch& f, cudaStream_t
 cudaError_t launch_shard_route(Profiler* prof, const ShardRoute& r, cudaStream_t st) {
     KernelScope k(prof, "shard_route", st);
     return launch_dependent(shard_route_kernel, dim3((unsigned)r.world, 3), dim3(1024), 0, st, r);
+}
+
+
+__global__ void __launch_bounds__(256)
+shard_mean_kernel(const ShardMean m) {
+    wait_for_predecessor();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m.n; i += (int64_t)gridDim.x * blockDim.x) {
+        float s = 0.f;
+        for (int r = 0; r < m.world; ++r) s += m.p[r][i];
+        s /= (float)m.world;
+        for (int r = 0; r < m.world; ++r) m.p[r][i] = s;
+    }
+}
+cudaError_t launch_shard_mean(Profiler* prof, const ShardMean& m, cudaStream_t st) {
+    const int64_t want = ceil_div(m.n, 256), cap = (int64_t)sm_count() * 8;
+    KernelScope k(prof, "shard_mean", st);
+    return launch_dependent(shard_mean_kernel, dim3((unsigned)(want < cap ? want : cap)), dim3(256), 0, st, m);
 }
 
 }  // namespace gear

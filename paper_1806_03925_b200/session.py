@@ -27,9 +27,25 @@ class DeviceBatch:
 
     @staticmethod
     def from_host(b: Batch, device="cuda") -> "DeviceBatch":
-        f = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(device)
-        return DeviceBatch(f(b.user_id), f(b.url_id), f(b.img_off), f(b.img_id), f(b.label), b.B, b.nnz,
-                           None if b.fast is None else f(b.fast))
+        """The batch's arrays on the device: put side by side in pinned memory (torch's pool of it), one asynchronous copy,
+        and slices of what arrives.  (Five copies from pageable memory, each a synchronisation, took 80 us for 4096 views.)"""
+        arrays = [b.user_id, b.url_id, b.img_off, b.img_id, b.label]
+        if b.fast is not None:
+            arrays.insert(0, b.fast)                  # first: its rows are read 16 bytes at a time
+        if torch.device(device).type != "cuda" or any(a.dtype.itemsize != 4 for a in arrays):
+            f = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(device)
+            return DeviceBatch(f(b.user_id), f(b.url_id), f(b.img_off), f(b.img_id), f(b.label), b.B, b.nnz,
+                               None if b.fast is None else f(b.fast))
+        sizes = [a.size for a in arrays]
+        host = torch.empty(sum(sizes), dtype=torch.int32, pin_memory=True)
+        view, at = host.numpy(), 0
+        for a, n in zip(arrays, sizes):
+            view[at:at + n] = a.reshape(-1).view(np.int32) if a.flags.c_contiguous else np.ascontiguousarray(a).reshape(-1).view(np.int32)
+            at += n
+        parts = [t if a.dtype == np.int32 else t.view(getattr(torch, a.dtype.name))
+                 for a, t in zip(arrays, host.to(device, non_blocking=True).split(sizes))]
+        fast = parts.pop(0).view(b.fast.shape) if b.fast is not None else None
+        return DeviceBatch(*parts, b.B, b.nnz, fast)
 
 
 class GearSession:

@@ -272,92 +272,32 @@ class ShardedGear:
 
 
 class _InProcessStep:
-    """The step when all shards are memory of one device: the same results as the exchange-by-exchange form, without send
-    and receive buffers.  The batches travel to the device in one copy; workers read their rows straight from the owners'
-    shards (gear_shard_fetch); a kernel picks every owner's arrivals out of the ID lists (gear_shard_route) while the workers
-    run; an owner takes its arrivals in one call (gear_owner_step), reading the gradient rows where the workers left them.
-    The host waits twice: for the numbers of arrivals (beside the workers' kernels) and for the counts it returns."""
+    """The step when all shards are memory of one device (gear_shard_step): the same results as the exchange-by-exchange
+    form, without send and receive buffers."""
 
     def __init__(self, sg: ShardedGear):
         self.sg = sg
-        p, W = sg.p, sg.world
-        mb, mn, dev = sg.max_batch_local, sg.max_nnz_local, sg.workers[0].dev
-        # one pinned host buffer and its device twin: user, URL and image IDs, offsets, labels, each list sender by sender
-        caps = (W * mb, W * mb, W * mn, W * (mb + 1), W * mb)
-        self.at, total = [], 0
-        for c in caps:
-            self.at.append(total)
-            total += (c + 3) // 4 * 4
-        self.host = torch.zeros(total, dtype=torch.int32).pin_memory()
-        self.np_i, self.np_f = self.host.numpy(), self.host.numpy().view(np.float32)
-        self.dev = torch.zeros(total, dtype=torch.int32, device=dev)
-        self.base = self.dev.data_ptr()
-        VP = gb.C.c_void_p
-        ptrs = lambda *a: (VP * len(a))(*a)
-        self.owners = ptrs(*(o.ctx.value for o in sg.owners))
-        self.ids = ptrs(*(self.base + 4 * self.at[t] for t in range(3)))
-        self.out = ptrs(sg._user_rows.data_ptr(), sg._url_rows.data_ptr(), sg._dfv_rows.data_ptr())
-        self.start = (gb.C.c_int32 * (3 * (W + 1)))()
-        self.stride = (gb.C.c_int64 * 3)(mb, mb, mn)
-        # arrivals of every owner: [table][local / src][world * entries]
-        self.lists = [[torch.zeros(W * c, dtype=torch.int32, device=dev) for _ in range(2)] for c in caps[:3]]
-        self.local, self.src = (ptrs(*(l[k].data_ptr() for l in self.lists)) for k in range(2))
-        self.counts = torch.zeros(3 * W, dtype=torch.int32, device=dev)
-        self.host_counts = torch.zeros(3 * W, dtype=torch.int32).pin_memory()
-        self.host_scalars = torch.zeros(3 * W, dtype=torch.int64).pin_memory()
-        self.routed, self.done = torch.cuda.Event(), torch.cuda.Event()
-        self.arrivals = [gb.gear_arrivals() for _ in range(3)]
-        self.batch = []
-        for wk in sg.workers:
-            bt = gb.gear_batch()
-            bt.user_id = bt.url_id = bt.img_id = sg._iota.data_ptr()
-            self.batch.append((bt, wk._make_step_out()))
+        W, C = sg.world, gb.C
+        words = gb.gear_shard_stage_words(W, sg.max_batch_local, sg.max_nnz_local)
+        self.host, self.dev = torch.zeros(words, dtype=torch.int32).pin_memory(), torch.zeros(words, dtype=torch.int32, device=sg.workers[0].dev)
+        self.ctxs = [(C.c_void_p * W)(*(s.ctx.value for s in side)) for side in (sg.owners, sg.workers)]
+        self.out = (gb.gear_step_out * W)(*(w._make_step_out() for w in sg.workers))
+        self.lists = (gb.gear_step_lists * W)(*(o._make_step_lists() for o in sg.owners))
+        self.plan = gb.gear_shard_plan(W, sg.max_batch_local, sg.max_nnz_local, self.ctxs[0], self.ctxs[1], self.host.data_ptr(),
+                                       self.dev.data_ptr(), sg._iota.data_ptr(), self.out, self.lists)
+        self.batches, self.counts = (gb.gear_host_batch * W)(), (C.c_int64 * (2 * W))()
 
     def step(self, batches: Sequence[Batch], now: int, lr: float, mean_head_grad: bool):
-        sg = self.sg
-        p, W = sg.p, sg.world
-        # ---- the batches, one copy
-        pos = list(self.at)
-        for s, b in enumerate(batches):
-            for t, a in enumerate((b.user_id, b.url_id, b.img_id)):
-                self.start[t * (W + 1) + s] = pos[t] - self.at[t]
-                self.np_i[pos[t]:pos[t] + len(a)] = a
-                pos[t] += len(a)
-            bt = self.batch[s][0]
-            bt.B, bt.nnz = b.B, b.nnz
-            bt.img_off, bt.label = self.base + 4 * pos[3], self.base + 4 * pos[4]
-            self.np_i[pos[3]:pos[3] + b.B + 1] = b.img_off
-            self.np_f[pos[4]:pos[4] + b.B] = b.label
-            pos[3] += b.B + 1
-            pos[4] += b.B
-        for t in range(3):
-            self.start[t * (W + 1) + W] = pos[t] - self.at[t]
-        used = pos[4]
-        self.dev[:used].copy_(self.host[:used], non_blocking=True)
-        # ---- events 1-4 on the workers; the owners' arrivals
-        gb.gear_shard_route(W, self.ids, self.start, self.stride, self.local, self.src, self.counts)
-        self.host_counts.copy_(self.counts, non_blocking=True)
-        self.routed.record()
-        gb.gear_shard_fetch(self.owners, W, self.ids, self.start, self.out, self.stride)
-        for wk, (bt, o) in zip(sg.workers, self.batch):
-            gb.gear_forward_backward_structs(wk.ctx, bt, 0.0, o)      # the worker's copies of the rows are scratch: nothing to update
-        if mean_head_grad:
-            sg._head_grads.copy_(sg._head_grads.mean(0, keepdim=True).expand_as(sg._head_grads))
-        # ---- events 4 (push), 5 and 6 at the owners
-        self.routed.synchronize()
-        counts = self.host_counts.tolist()
-        emb_rows, img_rows = sg._dX.data_ptr(), sg._dfv_grad.data_ptr()
-        for i, ow in enumerate(sg.owners):
-            for t, a in enumerate(self.arrivals):
-                first = 4 * i * self.start[t * (W + 1) + W]
-                a.ids, a.src, a.n = self.local[t] + first, self.src[t] + first, counts[t * W + i]
-            gb.gear_owner_step(ow.ctx, *self.arrivals, emb_rows, p.d_in, img_rows, p.dfv_dim, lr, ow._step_lists or ow._make_step_lists(), now)
-        self.host_scalars.copy_(sg._scalars, non_blocking=True)
-        self.done.record()
-        self.done.synchronize()
-        v = self.host_scalars.tolist()
-        out = [(v[3 * i + 1], v[3 * i + 2]) for i in range(W)]
-        for ow, (n_ready, n_expired) in zip(sg.owners, out):
-            if n_ready > ow.ready_cap or n_expired > ow.expired_cap:
-                raise gb.GearError(gb.GEAR_ERR_CAPACITY, "gear_owner_step")
-        return out
+        keep = []                                    # converted arrays live until the call has copied them
+
+        def at(a, dtype):
+            a = np.ascontiguousarray(a, dtype)
+            keep.append(a)
+            return a.__array_interface__["data"][0]
+        for c, b in zip(self.batches, batches):
+            c.B, c.nnz = b.B, b.nnz
+            c.user_id, c.url_id, c.img_off = at(b.user_id, np.int32), at(b.url_id, np.int32), at(b.img_off, np.int32)
+            c.img_id, c.label = at(b.img_id, np.int32), at(b.label, np.float32)
+        gb.gear_shard_step(self.plan, self.batches, lr, now, mean_head_grad, self.counts)
+        v = list(self.counts)
+        return list(zip(v[0::2], v[1::2]))
