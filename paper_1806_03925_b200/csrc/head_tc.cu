@@ -106,7 +106,10 @@ __device__ __forceinline__ void epilogue_tile(const TcArgs& g, const CUtensorMap
     const int part = (warp - 2) >> 2;
     constexpr int COLS = BN / (EW / 4);                   // columns per warp and tile
     constexpr int CHUNKS = COLS / 32;                     // 32-column chunks per warp and tile
-    static_assert(EPI == TC_EPI_F32 || EPI == TC_EPI_RED || CHUNKS % 2 == 0, "bf16 output leaves in blocks of 64 columns");
+    // bf16 output leaves in blocks of 64 columns (chunks 2k and 2k+1), or, where a warp has one chunk only, of 32 (then a CTA
+    // has one tile: the next tile's mask is not asked for)
+    constexpr bool NARROW = CHUNKS == 1;
+    static_assert(EPI == TC_EPI_F32 || EPI == TC_EPI_RED || NARROW || CHUNKS % 2 == 0, "whole blocks of 64 columns");
     const int m0 = mt * TC_BM + quarter * 32;         // first row of this warp's block
     const int rows = min(32, max(0, g.M - m0));
     const int col0 = nt * BN + part * COLS;
@@ -143,7 +146,7 @@ __device__ __forceinline__ void epilogue_tile(const TcArgs& g, const CUtensorMap
                              : "=r"(mask4[j].x), "=r"(mask4[j].y), "=r"(mask4[j].z), "=r"(mask4[j].w)
                              : "r"(row_addr + ((((uint32_t)j) ^ sw) << 4)) : "memory");
             if (c + 2 < CHUNKS) mask_request(mp, h, n0 + 64, m0, lane);
-            else if (mp.next_m0 >= 0) mask_request(mp, h, mp.next_col0 + (c + 2 - CHUNKS) * 32, mp.next_m0, lane);
+            else if (!NARROW && mp.next_m0 >= 0) mask_request(mp, h, mp.next_col0 + (c + 2 - CHUNKS) * 32, mp.next_m0, lane);
         }
         if (!chunk_ok || rows == 0) continue;
         uint32_t (&acc)[32] = r[c & 1];
@@ -182,17 +185,18 @@ __device__ __forceinline__ void epilogue_tile(const TcArgs& g, const CUtensorMap
             }
             {
                 // chunks 2k and 2k+1 fill the left and right half of one 64-column block
-                const int half = c & 1;
-                const uint32_t row_addr = out_buf + (uint32_t)lane * 128u;
+                const int half = NARROW ? 0 : c & 1;
+                const uint32_t row_addr = out_buf + (uint32_t)lane * (NARROW ? 64u : 128u);
+                const uint32_t sw_out = NARROW ? ((uint32_t)lane >> 1) & 3u : swz;      // 64- or 128-byte swizzle
                 if (half == 0) {
                     if (lane == 0) tma_store_wait_read<0>();          // the block's previous contents have been read
                     __syncwarp();
                 }
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
-                    sts_u4(row_addr + ((((uint32_t)(4 * half + j)) ^ swz) << 4),
+                    sts_u4(row_addr + ((((uint32_t)(4 * half + j)) ^ sw_out) << 4),
                            make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]));
-                if (half == 1 || n0 + 32 >= g.N) {
+                if (NARROW || half == 1 || n0 + 32 >= g.N) {
                     fence_async_smem();
                     __syncwarp();
                     if (lane == 0) tma_store_2d(map_out, out_buf, n0 - 32 * half, m0);
@@ -200,13 +204,16 @@ __device__ __forceinline__ void epilogue_tile(const TcArgs& g, const CUtensorMap
                         // column sums of what was stored (the rounded values), read back from the block: lane l owns
                         // columns 2l and 2l + 1 of the 64, one word per row (rows past M hold zeros: their operand rows
                         // and mask were read as zeros)
-                        const int nb = n0 - 32 * half + 2 * lane;
+                        // (a block of 32 columns has 16 words a row: lanes 16 .. 31 take its lower 16 rows)
+                        const uint32_t word = NARROW ? (uint32_t)lane & 15u : (uint32_t)lane;
+                        const int nb = n0 - 32 * half + 2 * (int)word;
                         float s_lo = 0.f, s_hi = 0.f;
 #pragma unroll
-                        for (int rr = 0; rr < 32; ++rr) {
+                        for (int i = 0; i < (NARROW ? 16 : 32); ++i) {
+                            const int rr = NARROW ? i + (lane & 16) : i;
                             uint32_t wv;
-                            const uint32_t addr = out_buf + (uint32_t)rr * 128u + ((((uint32_t)lane >> 2) ^ (uint32_t)(rr & 7)) << 4) +
-                                                  (((uint32_t)lane & 3u) << 2);
+                            const uint32_t addr = out_buf + (uint32_t)rr * (NARROW ? 64u : 128u) +
+                                                  (((word >> 2) ^ (NARROW ? ((uint32_t)rr >> 1) & 3u : (uint32_t)(rr & 7))) << 4) + ((word & 3u) << 2);
                             asm volatile("ld.shared.b32 %0, [%1];" : "=r"(wv) : "r"(addr) : "memory");
                             s_lo += __uint_as_float(wv << 16);
                             s_hi += __uint_as_float(wv & 0xffff0000u);
@@ -372,7 +379,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
         if (EPI == TC_EPI_MASK && (int)blockIdx.x < total_tiles) {
             // the masks of the first tile's first two blocks (after the wait for the previous kernel, which wrote them)
             mask_request(mp, 0, part_col0(blockIdx.x), part_m0(blockIdx.x), lane);
-            mask_request(mp, 1, part_col0(blockIdx.x) + 32, part_m0(blockIdx.x), lane);
+            if (COLS > 32) mask_request(mp, 1, part_col0(blockIdx.x) + 32, part_m0(blockIdx.x), lane);
         }
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tile_it) {
             const int nt = t % g.n_tiles, mt = (t / g.n_tiles) % g.m_tiles;
@@ -493,8 +500,9 @@ static cudaError_t launch_variant(const CUtensorMap& ma, const CUtensorMap& mb, 
 template <bool MN, int EPI, int EW = 8>
 static cudaError_t launch_bn(int bn, const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mo, const CUtensorMap& mm,
                              const TcArgs& g, cudaStream_t st) {
-    return bn == 256 ? launch_variant<256, MN, EPI, EW>(ma, mb, mo, mm, g, st)
-                     : launch_variant<128, MN, EPI, EW>(ma, mb, mo, mm, g, st);
+    return bn == 256   ? launch_variant<256, MN, EPI, EW>(ma, mb, mo, mm, g, st)
+           : bn == 128 ? launch_variant<128, MN, EPI, EW>(ma, mb, mo, mm, g, st)
+                       : launch_variant<64, MN, EPI, EW>(ma, mb, mo, mm, g, st);
 }
 
 cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
@@ -504,13 +512,21 @@ cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int 
     // column tiles of 256 or 128; the fp32 output (dX) also has 192, which fits a width like 384 without a half-empty tile
     int bn = N > 128 ? 256 : 128;
     if (epi == TC_EPI_F32 && N > 128 && ceil_div(N, 192) * 192 < ceil_div(N, 256) * 256) bn = 192;
+    // Where narrower tiles still are no more than the SMs, a tile's epilogue is what a product waits for: a warp then has one
+    // block of 32 columns instead of four (4096 x 256 x 192: 10.7 -> 9.1 us a launch).
+    const int64_t m_tiles = ceil_div(M, TC_BM);
+    if (m_tiles * ceil_div(N, 64) <= sm_count()) bn = 64;
+    else if (m_tiles * ceil_div(N, 128) <= sm_count()) bn = 128;
     CUtensorMap ma, mb, mo;
     if (!make_map(c, &ma, A, M, K, lda, TC_BM) || !make_map(c, &mb, W, N, K, ldw, bn)) return cudaErrorInvalidValue;
-    // the output leaves in boxes of 32 rows x 128 bytes
-    if (!(epi == TC_EPI_F32 ? make_map_f32(c, &mo, out, M, N, ldo) : make_map(c, &mo, out, M, N, ldo, 32))) return cudaErrorInvalidValue;
+    // the output leaves in boxes of 32 rows x 128 bytes (bf16 output of 64-column tiles: 64 bytes)
+    if (!(epi == TC_EPI_F32 ? make_map_f32(c, &mo, out, M, N, ldo)
+          : bn == 64        ? make_map_mask(c, &mo, out, M, N, ldo)
+                            : make_map(c, &mo, out, M, N, ldo, 32)))
+        return cudaErrorInvalidValue;
     TcArgs g;
     g.M = M; g.N = N; g.K = K;
-    g.m_tiles = (int)ceil_div(M, TC_BM); g.n_tiles = (int)ceil_div(N, bn); g.k_splits = 1;
+    g.m_tiles = (int)m_tiles; g.n_tiles = (int)ceil_div(N, bn); g.k_splits = 1;
     g.kb_per_split = (int)ceil_div(K, TC_BK);
     g.out = out; g.ldo = ldo; g.bias = bias; g.mask = mask; g.ldm = ldm; g.err = &c.state()->tc_error;
     g.colsum = (epi == TC_EPI_MASK && N <= TC_MAX_N) ? colsum : nullptr;
@@ -533,18 +549,28 @@ cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int
                             const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo,
                             cudaStream_t st) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
-    const int bn = N > 128 ? 256 : 128;
+    const int total_kb = (int)ceil_div(K, TC_BK);
+    // Tile width and number of slices, by what a CTA's time is made of (in clocks): its operand loads (50 bytes a clock), its
+    // epilogue, and the copy engines' additions of all slices to the matrix (1500 bytes a clock for the whole GPU).  Long
+    // reductions take wide tiles, whose operands are read fewer times (65536 rows, 384 x 512: 24 slices of 256 columns, 30 us),
+    // short ones few slices of narrow tiles (4096 rows, 192 x 256: 11.2 -> 10.0 us a launch against 64 slices of 256 columns).
+    int bn = 256, splits = 1;
+    double best = 1e30;
+    for (int w = N > 128 ? 256 : 128; w >= 64; w >>= 1) {
+        const int tiles = (int)(ceil_div(M, TC_BM) * ceil_div(N, w));
+        // as many slices of the reduction as fit in one wave of CTAs (one more would leave a second, nearly empty wave)
+        for (int s = sm_count() / tiles > 1 ? sm_count() / tiles : 1; s >= 1; s >>= 1) {
+            const int kb = (int)ceil_div(total_kb, s < total_kb ? s : total_kb), n = (int)ceil_div(total_kb, kb);
+            const double t = ceil_div((int64_t)tiles * n, sm_count()) * (kb * (TC_BM + w) * 2.56 + w * 8.0) + (double)n * M * N * 4 / 1500.0;
+            if (t < best) { best = t; bn = w; splits = n; }
+        }
+    }
     CUtensorMap ma, mb, mo;
     if (!make_map(c, &ma, A, K, M, lda, 64) || !make_map(c, &mb, Bm, K, N, ldb, 64) || !make_map_f32(c, &mo, out, M, N, ldo))
         return cudaErrorInvalidValue;
     TcArgs g;
     g.M = M; g.N = N; g.K = K;
     g.m_tiles = (int)ceil_div(M, TC_BM); g.n_tiles = (int)ceil_div(N, bn);
-    const int total_kb = (int)ceil_div(K, TC_BK);
-    // as many slices of the reduction as fit in one wave of CTAs (one more would leave a second, nearly empty wave)
-    int splits = sm_count() / (g.m_tiles * g.n_tiles);
-    if (splits > total_kb) splits = total_kb;
-    if (splits < 1) splits = 1;
     g.kb_per_split = (int)ceil_div(total_kb, splits);
     g.k_splits = (int)ceil_div(total_kb, g.kb_per_split);
     g.out = out; g.ldo = ldo; g.bias = nullptr; g.mask = nullptr; g.ldm = 0; g.colsum = nullptr; g.err = &c.state()->tc_error;
