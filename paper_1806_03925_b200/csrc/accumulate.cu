@@ -547,6 +547,21 @@ cudaError_t launch_accumulate_plan_ahead(const gear_ctx_impl& c, int64_t n, cons
     note_plan(c, n, src_row, scale);
     return cudaSuccess;
 }
+// A record then holds the row's place among the caller's rows; one thread per record.
+__global__ void __launch_bounds__(256)
+plan_resolve_kernel(int n, const DevState* __restrict__ state, const int32_t* __restrict__ src_row, const float* __restrict__ scale,
+                    int2* __restrict__ pmeta) {
+    wait_for_predecessor();
+    const int i = (int)(blockIdx.x * 256 + threadIdx.x);
+    if (i >= min(n, (int)state->n_valid)) return;          // rows without a valid image have no record
+    const int src = __ldg(src_row + pmeta[i].x);
+    pmeta[i] = make_int2(src, __float_as_int(__ldg(scale + src)));
+}
+cudaError_t launch_plan_resolve(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale, cudaStream_t st) {
+    KernelScope k(&c.prof, "plan_resolve", st);
+    return launch_dependent(plan_resolve_kernel, dim3((unsigned)ceil_div(n, 256)), dim3(256), 0, st, (int)n, (const DevState*)c.state(),
+                            src_row, scale, c.at<int2>(c.ws.pmeta));
+}
 void note_plan(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale) {
     c.plan_ready = true; c.plan_n = n; c.plan_src_row = src_row; c.plan_scale = scale;
 }

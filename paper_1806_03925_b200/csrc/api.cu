@@ -195,7 +195,9 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     const bool forked = apart && b.B > 0;
     const bool scan_beside = lists && apart && lists->scan_beside;
     const bool sorted_mode = c.cfg.accum_mode == GEAR_ACC_SORT;
-    // weight gradients beside the other products while a product of the widest layer does not fill the GPU by itself
+    // Weight gradients go to a stream of their own: beside the other products while a product of the widest layer does not fill
+    // the GPU by itself, else after dX, beside the store, which waits for memory where they wait for the tensor cores (65 k
+    // views: step 386 -> 376 us, 32 k views fp32: 329 -> 327).
     int widest = c.d_in;
     for (int l = 0; l < c.cfg.n_hidden; ++l) widest = widest < c.cfg.hidden[l] ? c.cfg.hidden[l] : widest;
     const bool dw_beside = forked && ceil_div(b.B, 128) * ceil_div(widest, 128) <= sm_count();
@@ -217,7 +219,11 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     if (dw_beside && !scan_beside) GEAR_TRY(enqueue_wait(aux, c.ev[EV_FORK]));
     GEAR_TRY(launch_round_weights(c, o, dw_beside ? aux : st));
     if (dw_beside) GEAR_TRY(enqueue_record(c.ev[EV_AUX], aux));
-    if (scan_beside) GEAR_TRY(scan(aux));
+    // The expiry scan reads the whole table of time stamps.  Beside the gather it slows that down; a large fp32 head's forward
+    // products wait for the ALUs and leave the memory to it (32 k views: step 327 -> 316 us).  bf16 products do not (65 k views:
+    // 376 us there, 386 behind the gather).
+    const bool scan_late = scan_beside && forked && !dw_beside && c.cfg.head_dtype == GEAR_F32;
+    if (scan_beside && !scan_late) GEAR_TRY(scan(aux));
     int sorted_buf = 0;
     bool small_sort = false;
     const bool plan = b.nnz > 0 && o.row_view && o.inv_n && sorted_mode;
@@ -250,17 +256,24 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
             c.img_sort_valid = sorted_mode;
         }
     }
+    // behind the sort: the plan of the accumulate call that usually follows (which rows form which group, where every group's
+    // rows and queue slot are).  Only where a row's gradient lies and its scale come from the gather (row_view, inv_n): behind a
+    // multi-block sort they are put in by a launch of its own, so that the plan runs beside the gather instead of beside the
+    // head's first products (65 k views: step 387 -> 381 us).  Small arrays are sorted and planned by one kernel behind the
+    // gather: there the extra launch costs more than the earlier start gives (4 k views: 56.6 us against 58.0).
+    if (plan && forked && !small_sort) GEAR_TRY(launch_accumulate_plan_ahead(c, b.nnz, nullptr, nullptr, side));
     GEAR_TRY(launch_gather(c, b, o.row_view, o.inv_n, o.x_debug, st));
     if (forked) GEAR_TRY(enqueue_record(c.ev[EV_GATHER], st));
+    if (scan_late) {
+        GEAR_TRY(enqueue_wait(aux, c.ev[EV_GATHER]));
+        GEAR_TRY(scan(aux));
+    }
     if (dw_beside) GEAR_TRY(enqueue_wait(st, c.ev[EV_AUX]));
-    // behind the sort: the plan of the accumulate call that usually follows (which rows form which group, where every group's
-    // rows and queue slot are).  It needs the gather's row_view / inv_n.  Small arrays are sorted and planned by one kernel.
     if (small_sort || (forked && plan)) {
         if (forked) GEAR_TRY(enqueue_wait(side, c.ev[EV_GATHER]));
-        if (small_sort) {
-            GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, o.row_view, o.inv_n) : PlanArgs{}, side));
-            if (plan) note_plan(c, b.nnz, o.row_view, o.inv_n);
-        } else GEAR_TRY(launch_accumulate_plan_ahead(c, b.nnz, o.row_view, o.inv_n, side));
+        GEAR_TRY(small_sort ? launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, o.row_view, o.inv_n) : PlanArgs{}, side)
+                            : launch_plan_resolve(c, b.nnz, o.row_view, o.inv_n, side));
+        if (plan) note_plan(c, b.nnz, o.row_view, o.inv_n);
     }
     if (forked && lists) GEAR_TRY(enqueue_record(c.ev[EV_PLAN], side));
     // the embedding scatter: enqueued by the head as soon as dX is on its way
@@ -279,7 +292,7 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
         return launch_emb_reduce(c, k.sorted_buf, k.B, o.user_grad ? o.user_grad : c.buf.user_emb, o.url_grad ? o.url_grad : c.buf.url_emb,
                                  o.dX, c.d_in, o.user_grad ? 1.0f : -k.lr, k.side);
     };
-    const HeadHooks hooks{scatters ? +scatter : nullptr, &sc, dw_beside ? aux : st, &c.ev[EV_AUX + 1]};
+    const HeadHooks hooks{scatters ? +scatter : nullptr, &sc, forked ? aux : st, &c.ev[EV_AUX + 1], !dw_beside};
     GEAR_TRY(launch_head(c, b, o, st, hooks));
     if (o.dfv_grad && b.B > 0) GEAR_TRY(launch_dfv_grad_rows(c, o.dX, o.row_view, o.inv_n, b.nnz, o.dfv_grad, st));
     if (lists) {
@@ -292,7 +305,7 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
         GEAR_TRY(enqueue_record(c.ev[EV_JOIN], side));
         GEAR_TRY(enqueue_wait(st, c.ev[EV_JOIN]));
     }
-    if (scan_beside || dw_beside) {
+    if (scan_beside || forked) {
         GEAR_TRY(enqueue_record(c.ev[EV_AUX], aux));
         GEAR_TRY(enqueue_wait(st, c.ev[EV_AUX]));
     }

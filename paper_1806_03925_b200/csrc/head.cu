@@ -326,7 +326,7 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
     float* grad = grad_array(c, o);
     const HeadParams p = split_params(c, grad);
     auto finish = [&]() -> cudaError_t {
-        return grad != o.head_grad ? enqueue_copy(o.head_grad, grad, sizeof(float) * c.n_params, st) : cudaSuccess;
+        return grad != o.head_grad ? enqueue_copy(o.head_grad, grad, sizeof(float) * c.n_params, hooks.dw_stream) : cudaSuccess;
     };
     if (B <= 0) return finish();
     cudaError_t err = cudaSuccess;
@@ -383,13 +383,13 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
         if constexpr (BF) return tc_gemm_mnmajor(c, "tc_gemm_dw", K, N, B, H[l].p, K, dA[l + 1].p, N, p.gW[l], N, hooks.dw_stream);
         else return tc3_gemm_mnmajor(c, "tc3_gemm_dw", K, N, B, H[l], K, dA[l + 1], N, p.gW[l], N, hooks.dw_stream);
     };
-    // backward.  Per layer the gradient that the layers below wait for (dA_l, at the bottom dX) comes first, its weight
-    // gradient after it (or, on a stream of its own, as soon as dA_{l+1} exists): once dX exists the caller's hook may start
-    // the embedding scatter on another stream.  The bias gradient of a lower layer is summed in the epilogue of the product
+    // backward.  The weight gradients run on a stream of their own, where the caller has one: as soon as dA_{l+1} exists, or after
+    // dX, beside what the caller does with dX.  On one stream the gradient that the layers below wait for (dA_l, at the bottom
+    // dX) comes first: once dX exists the caller's hook may start the embedding scatter on another stream.  The bias gradient of a lower layer is summed in the epilogue of the product
     // that makes its dA (the top layer's came out of head_out_kernel).
     for (int l = L - 1; l >= 0; --l) {
         const int K = p.fan[l], N = p.fan[l + 1];
-        if (beside && (err = weight_grad(l)) != cudaSuccess) return err;
+        if (beside && !hooks.dw_last && (err = weight_grad(l)) != cudaSuccess) return err;
         if constexpr (BF) {
             if (l > 0) err = tc_gemm_kmajor(c, "tc_gemm_dh", B, K, N, dA[l + 1].p, N, W[l].p, N, 1, dA[l].p, K, nullptr, H[l].p, K, p.gb[l - 1], st);
             else err = tc_gemm_kmajor(c, "tc_gemm_dx", B, K, N, dA[l + 1].p, N, W[l].p, N, 2, o.dX, K, nullptr, nullptr, 0, nullptr, st);
@@ -401,6 +401,8 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
         if (l == 0 && hooks.after_dx && (err = hooks.after_dx(hooks.arg)) != cudaSuccess) return err;
         if (!beside && (err = weight_grad(l)) != cudaSuccess) return err;
     }
+    for (int l = 0; beside && hooks.dw_last && l < L; ++l)
+        if ((err = weight_grad(l)) != cudaSuccess) return err;
     return finish();
 }
 

@@ -144,7 +144,9 @@ cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* 
 // head.cu: forward + backward of the head.  The weights' copies must have been made and head_grad cleared earlier on the same
 // stream (launch_round_weights).  after_dx(arg) is called once dX has been enqueued.  dw_stream: where the weight gradients go;
 // if it is not the head's own stream, it is made to wait for what they read (one event of dw_ev per layer).
-struct HeadHooks { cudaError_t (*after_dx)(void*); void* arg; cudaStream_t dw_stream; cudaEvent_t* dw_ev; };
+// after_dx: called once dX is on its way.  The weight gradients go to dw_stream (dw_ev: an event per layer, if that is not the
+// head's own stream), each as soon as its operands exist or, dw_last, all of them after dX.
+struct HeadHooks { cudaError_t (*after_dx)(void*); void* arg; cudaStream_t dw_stream; cudaEvent_t* dw_ev; bool dw_last; };
 cudaError_t launch_head(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o, cudaStream_t st, const HeadHooks& hooks);
 // the weights as the products read them; clears head_grad (all of it, also for an empty batch)
 cudaError_t launch_round_weights(const gear_ctx_impl& c, const gear_step_out& o, cudaStream_t st);
@@ -236,6 +238,8 @@ cudaError_t launch_accumulate_atomic(const gear_ctx_impl& c, const int32_t* img_
 // steps 2-4 of the sorted accumulate for the batch just sorted by gear_forward_backward, ahead of the accumulate call
 cudaError_t launch_accumulate_plan_ahead(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale,
                                          cudaStream_t st);
+// a plan made without them gets its rows' views and their scales
+cudaError_t launch_plan_resolve(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale, cudaStream_t st);
 // what the plan for n rows needs; note_plan: it has been made (for the image IDs of the last batch)
 PlanArgs plan_args(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale);
 void note_plan(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale);
