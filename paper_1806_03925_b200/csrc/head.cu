@@ -344,16 +344,21 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
     float* loss_part = c.at<float>(c.ws.loss_part);
 
     // forward
+    const int HT = p.fan[L];
+    // a bf16 top layer whose columns are one tile of its product takes the output unit along
+    const bool top_fused = BF && HT <= TC_TOP_N;
     for (int l = 0; l < L; ++l) {
         const int K = p.fan[l], N = p.fan[l + 1];
-        if constexpr (BF)
+        if (top_fused && l + 1 == L)
+            err = tc_gemm_top(c, "tc_gemm_top", B, N, K, H[l].p, K, Wt[l].p, K, p.b[l], dA[L].p,
+                              TopArgs{p.w_out, p.b_out, bt.label, o.prob, loss_part, p.gw_out, p.gb[l], p.gb_out, &c.state()->colsum_ticket, o.loss}, st);
+        else if constexpr (BF)
             err = tc_gemm_kmajor(c, "tc_gemm_fwd", B, N, K, H[l].p, K, Wt[l].p, K, 0, H[l + 1].p, N, p.b[l], nullptr, 0, nullptr, st);
         else
             err = launch_fwd_f32(c, B, N, K, c.at<float>(c.ws.xf[l]), p.W[l], p.b[l], H[l + 1], l + 1 < L ? c.at<float>(c.ws.xf[l + 1]) : nullptr, st);
         if (err != cudaSuccess) return err;
     }
-    const int HT = p.fan[L];
-    {
+    if (!top_fused) {
         KernelScope ks(&c.prof, "head_out", st);
         const int nq = (int)ceil_div(HT, 256);
         // rows per warp and pass: as many as the registers hold (8 chunks of bf16, 4 of fp32)

@@ -37,17 +37,27 @@ constexpr int tc_threads(int ew) { return 64 + 32 * ew; }
 constexpr int TC_MAX_N = 1024;            // widest output the column-sum partials cover
 constexpr int TC_MASK_BLOCK = 32 * 64;    // a warp's ReLU-mask block for 32 columns: 32 rows of 64 bytes (two per warp)
 
-enum { TC_EPI_BIAS_RELU = 0, TC_EPI_MASK = 1, TC_EPI_F32 = 2, TC_EPI_RED = 3 };
+enum { TC_EPI_BIAS_RELU = 0, TC_EPI_MASK = 1, TC_EPI_F32 = 2, TC_EPI_RED = 3, TC_EPI_TOP = 4 };
 
 constexpr int TC_OUT_BLOCK = 32 * 128;   // a warp's output block on its way to a TMA store: 32 rows of 128 bytes
+
+struct TopSmem {                          // the top hidden layer's epilogue
+    float w[TC_TOP_N], bias[TC_TOP_N], gw[TC_TOP_N], gb[TC_TOP_N];     // output weights, the layer's bias; column sums
+    float z[2][2][TC_BM];                 // [tile parity][column half] a row's part of the dot product
+    float g[8][32];                       // per epilogue warp: dz of its rows
+    float part[2][8];                     // per epilogue warp: loss, sum of dz
+    int is_last;
+};
 
 template <int BN, int EW, int EPI> struct TcCfg {
     static constexpr int A_BYTES = TC_BM * TC_BK * 2;            // 16 KB
     static constexpr int B_BYTES = BN * TC_BK * 2;               // 32 KB or 16 KB
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    static constexpr int OUT_BYTES = EW * TC_OUT_BLOCK;       // one output block per epilogue warp
+    // one output block per epilogue warp; the top layer's epilogue holds a warp's whole part of the tile
+    static constexpr int OUT_BYTES = EW * TC_OUT_BLOCK * (EPI == TC_EPI_TOP ? BN / (EW / 4) / 64 : 1);
     static constexpr int MASK_BYTES = EPI == TC_EPI_MASK ? EW * 2 * TC_MASK_BLOCK : 0;
-    static constexpr int COLSUM_BYTES = EPI == TC_EPI_MASK ? TC_MAX_N * 4 : 0;     // per-CTA column sums of the masked product
+    // per-CTA column sums of the masked product; the top layer's vectors and sums
+    static constexpr int COLSUM_BYTES = EPI == TC_EPI_MASK ? TC_MAX_N * 4 : EPI == TC_EPI_TOP ? (int)sizeof(TopSmem) : 0;
     static constexpr int FIXED = 1024 /*alignment slack*/ + 512 /*barriers*/ + COLSUM_BYTES + OUT_BYTES + MASK_BYTES;
     static constexpr int ROOM = (227 * 1024 - FIXED) / STAGE_BYTES;
     static constexpr int STAGES = ROOM > (BN == 256 ? 4 : 6) ? (BN == 256 ? 4 : 6) : ROOM;
@@ -66,6 +76,7 @@ struct TcArgs {
     const __nv_bfloat16* mask; int64_t ldm;
     float* colsum;            // ReLU-mask epilogue: colsum[n] += sum over rows of the stored output (may be null)
     int32_t* err;             // device word that receives a non-zero code on a timeout
+    TopArgs top;              // top layer only
 };
 
 // Epilogue of one finished accumulator buffer `a`, as run by one of the epilogue warps: warp w reads
@@ -243,6 +254,125 @@ __device__ __forceinline__ void epilogue_tile(const TcArgs& g, const CUtensorMap
     }
 }
 
+// The top hidden layer's tile (its columns are one tile of the product) with all that hangs off it:
+//   h = ReLU(acc + bias) rounded to bf16;  z = h . w_out + b_out;  p = sigmoid(z);  BCE in its overflow-safe form;
+//   dz = (p - y) / M;  out[b][j] = dz * w_out[j] where h[b][j] > 0, else 0;  gw_out[j] += sum_b h dz;  gb_top[j] += sum_b out
+// A lane first walks its row of the accumulator (dot product; h to the warp's blocks in shared memory, after which the buffer
+// goes back to the MMA warp); the two warps of a lane quarter add their halves of z; then a lane owns two columns of a block and
+// walks its 32 rows: column sums, h replaced by out in place.  h itself goes nowhere: nothing after this reads it.
+// (Bound by instructions, about 15 per 2 elements in the second walk.  In a launch of its own, which read h and wrote out again,
+// the output unit took 11 us for 4096 x 128 and 23 us for 65536 x 256.)
+template <int BN> struct TopSums { float gw[BN / 128][2], gb[BN / 128][2], loss, dz; };
+
+template <int BN>
+__device__ __forceinline__ void epilogue_top(const TcArgs& g, const CUtensorMap* map_out, uint32_t tmem_base, int a, int mt, int parity,
+                                             int warp, int lane, TopSmem& s, TopSums<BN>& sums, uint32_t out_buf, uint32_t empty_bar) {
+    constexpr int COLS = BN / 2, BLOCKS = COLS / 64;
+    const int quarter = warp & 3, part = (warp - 2) >> 2;
+    const int m0 = mt * TC_BM + quarter * 32, b = m0 + lane;
+    const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(a * BN + part * COLS);
+    const uint32_t swz = (uint32_t)(lane & 7);
+    const float y = b < g.M ? __ldg(g.top.label + b) : 0.f;
+    float z = 0.f;
+    uint32_t r[2][32];
+    tc_ld32(t_row, r[0]);
+    if (lane == 0) tma_store_wait_read<0>();                          // the blocks' previous contents have been read
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < COLS / 32; ++c) {
+        const int n0 = part * COLS + c * 32;
+        tc_wait_ld(r[c & 1]);
+        if (c + 1 < COLS / 32) tc_ld32(t_row + (uint32_t)((c + 1) * 32), r[(c + 1) & 1]);
+        if (n0 >= g.N) continue;                                      // warp-uniform; N is a multiple of 64
+        const uint32_t row_addr = out_buf + (uint32_t)(c >> 1) * TC_OUT_BLOCK + (uint32_t)lane * 128u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            uint32_t pk[4];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float4 bi = *reinterpret_cast<const float4*>(&s.bias[n0 + 8 * j + 4 * k]);
+                const float4 w = *reinterpret_cast<const float4*>(&s.w[n0 + 8 * j + 4 * k]);
+                const uint32_t* acc = &r[c & 1][8 * j + 4 * k];
+                __nv_bfloat162 h01 = __floats2bfloat162_rn(fmaxf(__uint_as_float(acc[0]) + bi.x, 0.f), fmaxf(__uint_as_float(acc[1]) + bi.y, 0.f));
+                __nv_bfloat162 h23 = __floats2bfloat162_rn(fmaxf(__uint_as_float(acc[2]) + bi.z, 0.f), fmaxf(__uint_as_float(acc[3]) + bi.w, 0.f));
+                pk[2 * k] = *reinterpret_cast<uint32_t*>(&h01);
+                pk[2 * k + 1] = *reinterpret_cast<uint32_t*>(&h23);
+                z = fmaf(__uint_as_float(pk[2 * k] << 16), w.x, z);
+                z = fmaf(__uint_as_float(pk[2 * k] & 0xffff0000u), w.y, z);
+                z = fmaf(__uint_as_float(pk[2 * k + 1] << 16), w.z, z);
+                z = fmaf(__uint_as_float(pk[2 * k + 1] & 0xffff0000u), w.w, z);
+            }
+            sts_u4(row_addr + ((((uint32_t)(4 * (c & 1) + j)) ^ swz) << 4), make_uint4(pk[0], pk[1], pk[2], pk[3]));
+        }
+    }
+    tc_fence_before();
+    mbar_arrive_relaxed(empty_bar);                                   // all epilogue threads arrive: the buffer returns to the MMA warp
+    s.z[parity][part][quarter * 32 + lane] = z;
+    // the two warps of the quarter meet; two tiles on, z[parity] is written again only behind the next tile's meeting
+    asm volatile("bar.sync %0, 64;" :: "r"(1 + quarter) : "memory");
+    const float zz = s.z[parity][0][quarter * 32 + lane] + s.z[parity][1][quarter * 32 + lane] + __ldg(g.top.b_out);
+    const float p = 1.0f / (1.0f + expf(-zz));
+    const float dz = b < g.M ? (p - y) / (float)g.M : 0.f;            // rows past the edge add nothing
+    if (part == 0 && b < g.M) {
+        sums.loss += fmaxf(zz, 0.f) - zz * y + log1pf(expf(-fabsf(zz)));
+        sums.dz += dz;
+        if (g.top.prob) g.top.prob[b] = p;
+    }
+    s.g[warp - 2][lane] = dz;
+    __syncwarp();
+    const __nv_bfloat162 zero2 = __floats2bfloat162_rn(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < BLOCKS; ++k) {
+        const int nb = part * COLS + 64 * k;
+        if (nb >= g.N) break;
+        const uint32_t blk = out_buf + (uint32_t)k * TC_OUT_BLOCK + (((uint32_t)lane & 3u) << 2);
+        const float2 w = *reinterpret_cast<const float2*>(&s.w[nb + 2 * lane]);
+#pragma unroll
+        for (int r4 = 0; r4 < 8; ++r4) {
+            const float4 g4 = *reinterpret_cast<const float4*>(&s.g[warp - 2][4 * r4]);
+            const float gr[4] = {g4.x, g4.y, g4.z, g4.w};
+            uint32_t h[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(h[i]) : "r"(blk + (uint32_t)(4 * r4 + i) * 128u + ((((uint32_t)lane >> 2) ^ (uint32_t)((4 * r4 + i) & 7)) << 4)) : "memory");
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                sums.gw[k][0] = fmaf(__uint_as_float(h[i] << 16), gr[i], sums.gw[k][0]);
+                sums.gw[k][1] = fmaf(__uint_as_float(h[i] & 0xffff0000u), gr[i], sums.gw[k][1]);
+                __nv_bfloat162 d2 = __floats2bfloat162_rn(gr[i] * w.x, gr[i] * w.y);
+                const uint32_t dv = *reinterpret_cast<uint32_t*>(&d2) & __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&h[i]), zero2);
+                asm volatile("st.shared.b32 [%0], %1;" :: "r"(blk + (uint32_t)(4 * r4 + i) * 128u + ((((uint32_t)lane >> 2) ^ (uint32_t)((4 * r4 + i) & 7)) << 4)), "r"(dv) : "memory");
+                sums.gb[k][0] += __uint_as_float(dv << 16);
+                sums.gb[k][1] += __uint_as_float(dv & 0xffff0000u);
+            }
+        }
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) tma_store_2d(map_out, out_buf + (uint32_t)k * TC_OUT_BLOCK, nb, m0);
+    }
+}
+
+// After the last tile (all threads of the CTA): sums to memory.  The CTA that delivers its partial loss last adds them all up,
+// always in CTA order (the ticket counts arrivals and wraps back to zero by itself, ready for the next launch).
+__device__ __forceinline__ void finish_top(const TcArgs& g, TopSmem& s) {
+    for (int n = threadIdx.x; n < g.N; n += blockDim.x) { atomicAdd(g.top.gw_out + n, s.gw[n]); atomicAdd(g.top.gb_top + n, s.gb[n]); }
+    if (threadIdx.x == 0) {
+        float l = 0.f, t = 0.f;
+        for (int k = 0; k < 8; ++k) { l += s.part[0][k]; t += s.part[1][k]; }
+        g.top.loss_part[blockIdx.x] = l;
+        atomicAdd(g.top.gb_out, t);
+        __threadfence();
+        s.is_last = atomicInc(g.top.ticket, gridDim.x - 1) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s.is_last || threadIdx.x >= 32) return;
+    __threadfence();
+    float l = 0.f;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) l += __ldcg(g.top.loss_part + i);
+    l = warp_sum(l);
+    if (threadIdx.x == 0) g.top.loss[0] = l / (float)g.M;
+}
+
 // ---------------------------------------------------------------- the kernel
 template <int BN, bool MN_MAJOR, int EPI, int EW>
 __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUtensorMap& map_b, const CUtensorMap& map_out,
@@ -264,6 +394,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
         reinterpret_cast<volatile uint32_t*>(smem_raw + (tmem_word - raw));
     auto mask_bar = [&](int w, int h) { return bars + 8u * (24 + 2 * w + h); };     // two per epilogue warp
     float* s_colsum = reinterpret_cast<float*>(smem_raw + (bars + 512u - raw));     // [TC_MAX_N] per-CTA column sums
+    TopSmem& top = *reinterpret_cast<TopSmem*>(s_colsum);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int total_tiles = g.m_tiles * g.n_tiles * g.k_splits;
@@ -367,7 +498,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
         }
     } else {
         // ---------------- epilogue warps
-        const uint32_t out_buf = out_blocks + (uint32_t)((warp - 2) * TC_OUT_BLOCK);
+        const uint32_t out_buf = out_blocks + (uint32_t)((warp - 2) * (Cfg::OUT_BYTES / EW));
         const uint64_t keep_policy = l2_policy_evict_last();
         uint32_t tile_it = 0;
         bool ok = true;
@@ -381,6 +512,32 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
             mask_request(mp, 0, part_col0(blockIdx.x), part_m0(blockIdx.x), lane);
             if (COLS > 32) mask_request(mp, 1, part_col0(blockIdx.x) + 32, part_m0(blockIdx.x), lane);
         }
+        if constexpr (EPI == TC_EPI_TOP) {
+            TopSums<BN> sums = {};
+            for (int n = threadIdx.x - 64; n < TC_TOP_N; n += 32 * EW) {
+                top.w[n] = n < g.N ? __ldg(g.top.w_out + n) : 0.f;
+                top.bias[n] = n < g.N ? __ldg(g.bias + n) : 0.f;
+                top.gw[n] = 0.f; top.gb[n] = 0.f;
+            }
+            asm volatile("bar.sync 5, %0;" :: "n"(32 * EW) : "memory");
+            // A wait that gave up does not leave the loop (the two warps of a quarter meet in every tile; from then on all waits
+            // return at once): the error word tells the host that the results are void.
+            for (int t = blockIdx.x; t < total_tiles; t += gridDim.x, ++tile_it) {
+                const int a = tile_it & 1;
+                mbar_wait(acc_full(a), (tile_it >> 1) & 1u, g.err, 4);
+                __syncwarp();
+                tc_fence_after();
+                epilogue_top<BN>(g, &map_out, tmem_base, a, t, (int)(tile_it & 1u), warp, lane, top, sums, out_buf, acc_empty(a));
+            }
+#pragma unroll
+            for (int k = 0; k < BN / 128; ++k) {
+                const int n = ((warp - 2) >> 2) * COLS + 64 * k + 2 * lane;
+                atomicAdd(&top.gw[n], sums.gw[k][0]); atomicAdd(&top.gw[n + 1], sums.gw[k][1]);
+                atomicAdd(&top.gb[n], sums.gb[k][0]); atomicAdd(&top.gb[n + 1], sums.gb[k][1]);
+            }
+            const float l = warp_sum(sums.loss), d = warp_sum(sums.dz);
+            if (lane == 0) { top.part[0][warp - 2] = l; top.part[1][warp - 2] = d; }
+        } else
         for (int t = blockIdx.x; t < total_tiles && ok; t += gridDim.x, ++tile_it) {
             const int nt = t % g.n_tiles, mt = (t / g.n_tiles) % g.m_tiles;
             const int a = tile_it & 1;
@@ -412,6 +569,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
             const float v = s_colsum[n];
             if (v != 0.f) atomicAdd(g.colsum + n, v);
         }
+    if constexpr (EPI == TC_EPI_TOP) finish_top(g, top);
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;"
@@ -543,6 +701,22 @@ cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int 
         if (bn == 192) return launch_variant<192, false, TC_EPI_F32, 8>(ma, mb, mo, ma /*unused*/, g, st);
         return launch_bn<false, TC_EPI_F32>(bn, ma, mb, mo, ma /*unused*/, g, st);
     }
+}
+
+cudaError_t tc_gemm_top(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
+                        const __nv_bfloat16* W, int64_t ldw, const float* bias, __nv_bfloat16* dA, const TopArgs& top, cudaStream_t st) {
+    const int bn = N > 128 ? 256 : 128;
+    CUtensorMap ma, mb, mo;
+    if (!make_map(c, &ma, A, M, K, lda, TC_BM) || !make_map(c, &mb, W, N, K, ldw, bn) || !make_map(c, &mo, dA, M, N, N, 32))
+        return cudaErrorInvalidValue;
+    TcArgs g = {};
+    g.M = M; g.N = N; g.K = K;
+    g.m_tiles = (int)ceil_div(M, TC_BM); g.n_tiles = 1; g.k_splits = 1;
+    g.kb_per_split = (int)ceil_div(K, TC_BK);
+    g.bias = bias; g.err = &c.state()->tc_error; g.top = top;
+    KernelScope ks(&c.prof, name, st);
+    return bn == 256 ? launch_variant<256, false, TC_EPI_TOP, 8>(ma, mb, mo, ma /*unused*/, g, st)
+                     : launch_variant<128, false, TC_EPI_TOP, 8>(ma, mb, mo, ma /*unused*/, g, st);
 }
 
 cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,

@@ -156,6 +156,16 @@ cudaError_t launch_round_weights(const gear_ctx_impl& c, const gear_step_out& o,
 cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
                            const __nv_bfloat16* W, int64_t ldw, int epi, void* out, int64_t ldo, const float* bias,
                            const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st);
+// The top hidden layer and the output unit behind it: h = ReLU(A . W^T + bias) stays on the chip, dA gets the gradient with
+// respect to its pre-activations.  N at most TC_TOP_N.
+constexpr int TC_TOP_N = 256;
+struct TopArgs {
+    const float* w_out; const float* b_out; const float* label;
+    float* prob; float* loss_part; float* gw_out; float* gb_top; float* gb_out;
+    unsigned int* ticket; float* loss;
+};
+cudaError_t tc_gemm_top(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
+                        const __nv_bfloat16* W, int64_t ldw, const float* bias, __nv_bfloat16* dA, const TopArgs& top, cudaStream_t st);
 // out[M][N] (fp32) += A[K][M]^T . Bm[K][N]
 cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
                             const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo, cudaStream_t st);
