@@ -161,10 +161,6 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
     if (blockIdx.x == 0 && threadIdx.x == 0 && (n == 0 || ks[0] >= vocab)) state->n_valid = 0;   // no valid row at all
 }
 
-struct RowSource {
-    const uint32_t* perm; const float* grads; int64_t ld; const int32_t* src_row; const float* scale;
-};
-
 // Counts of (groups, complete groups, in the upper word): per tile, and per section of AF_SECTION tiles (zero before a plan).
 struct PlanCounts { uint2* tile; unsigned long long* section; };
 constexpr int AF_SECTION = 64;
@@ -190,8 +186,7 @@ acc_flag_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, cons
 
 __global__ void __launch_bounds__(AF_THREADS)
 acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, const DivM div, const int32_t* __restrict__ cnt,
-                const PlanCounts counts, uint2* __restrict__ totals, uint4* __restrict__ grp_rec, RowSource rs,
-                int2* __restrict__ pmeta, uint32_t* __restrict__ blk_first, uint32_t* __restrict__ run_end,
+                const PlanCounts counts, uint2* __restrict__ totals, uint4* __restrict__ grp_rec, uint32_t* __restrict__ blk_first, uint32_t* __restrict__ run_end,
                 int span, DevState* __restrict__ state) {
     wait_for_predecessor();
     __shared__ uint32_t smem[34];
@@ -227,30 +222,13 @@ acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, cons
         ++gi;
         ci += f.complete[t];
     }
-    // where the gradient row of every sorted position lives and what it is scaled by (one 8-byte record), resolved
-    // through the sort permutation once, so that the reduce pass reads both with one coalesced load
-    uint32_t src[AF_ITEMS];
-    float scale[AF_ITEMS];
-    load_items(src, rs.perm, f.i0, n, 0u);
-    if (rs.src_row)
-#pragma unroll
-        for (int t = 0; t < AF_ITEMS; ++t) src[t] = f.i0 + t < n && f.key[t] < vocab ? (uint32_t)__ldg(rs.src_row + src[t]) : 0u;
-#pragma unroll
-    for (int t = 0; t < AF_ITEMS; ++t) scale[t] = rs.scale && f.i0 + t < n && f.key[t] < vocab ? __ldg(rs.scale + src[t]) : 1.f;
-    if (f.i0 + AF_ITEMS <= n) {                                     // (records of rows without a valid image are never read)
-        int4* dst = reinterpret_cast<int4*>(pmeta + f.i0);
-        dst[0] = make_int4((int)src[0], __float_as_int(scale[0]), (int)src[1], __float_as_int(scale[1]));
-        dst[1] = make_int4((int)src[2], __float_as_int(scale[2]), (int)src[3], __float_as_int(scale[3]));
-    } else {
-#pragma unroll
-        for (int t = 0; t < AF_ITEMS; ++t)
-            if (f.i0 + t < n) pmeta[f.i0 + t] = make_int2((int)src[t], __float_as_int(scale[t]));
-    }
 }
 
+// Where the row of sorted position p lives and what it is scaled by: pmeta[p] = (source row, scale bits); or, where the call
+// names neither source rows nor scales, row perm[p] as it is.
 struct RowGather {
     const float* grads; int64_t ld;
-    const int2* pmeta;             // pmeta[p] = (source row, scale bits) of sorted position p
+    const int2* pmeta; const uint32_t* perm;
 };
 
 // What a lane knows about "its" group of a span: own rows [start, start + len), then zlen rows from zstart.
@@ -286,8 +264,9 @@ struct ItemDesc { uint32_t addr_lo, addr_hi; float scale; int meta; };
 // record fetched by the lane), one batch ahead of the copies; the inner loop only broadcasts a lane's
 // descriptor, copies and adds.  The group records of the next span are requested while the current span
 // streams.  Sums are fp32, in arrival order, starting from the stored partial sum.
-// FULL: a row is exactly NQ * 512 bytes, so no lane is ever idle.
-template <int NQ, int S, bool FULL>
+// FULL: a row is exactly NQ * 512 bytes, so no lane is ever idle.  PLAIN: the caller's rows as they are (a store of 16 M rows
+// then needs no 128 MB of records).
+template <int NQ, int S, bool FULL, bool PLAIN>
 __global__ void __launch_bounds__(256, NQ <= 2 ? 3 : 2)
 acc_reduce_kernel(RowGather rg, int D, const DivM div, int span_log2, int64_t ready_cap, const uint2* __restrict__ plan_totals, const uint4* __restrict__ grp_rec,
                   const uint32_t* __restrict__ blk_first, const uint32_t* __restrict__ run_end,
@@ -398,7 +377,9 @@ acc_reduce_kernel(RowGather rg, int D, const DivM div, int span_log2, int64_t re
                 const bool ok = i < total_items, is_tab = k < tab;
                 const int64_t p = k < own_end ? (int64_t)start_l + (k - tab) : (int64_t)zstart_l + (k - own_end);
                 int2 pm = make_int2(0, __float_as_int(1.f));
-                if (ok && !is_tab) pm = __ldg(rg.pmeta + p);
+                if (ok && !is_tab) {
+                    if constexpr (PLAIN) pm.x = (int)__ldg(rg.perm + p); else pm = __ldg(rg.pmeta + p);
+                }
                 const float* row = (ok && is_tab) ? gsum + (int64_t)key_l * D : rg.grads + (int64_t)pm.x * rg.ld;
                 const uint64_t a = reinterpret_cast<uint64_t>(row) | (ok ? 1ull : 0ull);      // rows are 16-byte aligned
                 ItemDesc d;
@@ -507,9 +488,8 @@ acc_reduce_kernel(RowGather rg, int D, const DivM div, int span_log2, int64_t re
     leave();
 }
 
-// Steps 2-4 of the plan over the sorted keys ks / permutation perm (flag pass, scan, plan pass).
-static cudaError_t enqueue_plan(const gear_ctx_impl& c, const uint32_t* ks, const uint32_t* perm, int64_t n,
-                                const int32_t* src_row, const float* scale, cudaStream_t st) {
+// Steps 2-4 of the plan over the sorted keys ks (flag pass, plan pass).
+static cudaError_t enqueue_plan(const gear_ctx_impl& c, const uint32_t* ks, int64_t n, cudaStream_t st) {
     const int64_t vocab = c.cfg.img_vocab;
     const DivM div = make_div(c.cfg.M);
     DevState* state = c.state();
@@ -526,10 +506,9 @@ static cudaError_t enqueue_plan(const gear_ctx_impl& c, const uint32_t* ks, cons
     { KernelScope k(&c.prof, "acc_flag", st);
     e = launch_dependent(acc_flag_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, n, (uint32_t)vocab, div, c.buf.dfv_gcnt, counts, state); }
     if (e != cudaSuccess) return e;
-    RowSource rs{perm, nullptr, 0, src_row, scale};
     KernelScope k(&c.prof, "acc_plan", st);
     return launch_dependent(acc_plan_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, n, (uint32_t)vocab, div, c.buf.dfv_gcnt, counts, tile_cnt + n_tiles,
-                            c.at<uint4>(c.ws.grp_rec), rs, c.at<int2>(c.ws.pmeta), c.at<uint32_t>(c.ws.blk_first),
+                            c.at<uint4>(c.ws.grp_rec), c.at<uint32_t>(c.ws.blk_first),
                             c.at<uint32_t>(c.ws.run_end), acc_span_log2(n), state);
 }
 
@@ -537,30 +516,36 @@ static cudaError_t enqueue_plan(const gear_ctx_impl& c, const uint32_t* ks, cons
 // accumulate call that will use it (on the side stream, beside the head): it depends on the sorted IDs, the counts in
 // the table and the queue length only, none of which changes before that call unless another accumulate or collect
 // comes first -- those calls drop the plan.
-cudaError_t launch_accumulate_plan_ahead(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale,
-                                         cudaStream_t st) {
+cudaError_t launch_accumulate_plan_ahead(const gear_ctx_impl& c, int64_t n, cudaStream_t st) {
     c.plan_ready = false;
     if (n <= 0 || !c.img_sorted || !c.img_sort_valid || c.cfg.accum_mode != GEAR_ACC_SORT) return cudaSuccess;
     SortJob sb = c.sort_job(gear_ctx_impl::SORT_IMG);
-    cudaError_t e = enqueue_plan(c, sb.keys[c.img_sorted_buf], sb.vals[c.img_sorted_buf], n, src_row, scale, st);
-    if (e != cudaSuccess) return e;
-    note_plan(c, n, src_row, scale);
-    return cudaSuccess;
+    cudaError_t e = enqueue_plan(c, sb.keys[c.img_sorted_buf], n, st);
+    if (e == cudaSuccess) note_plan(c, n, nullptr, nullptr);
+    return e;
 }
-// A record then holds the row's place among the caller's rows; one thread per record.
+// Where every sorted row lives and what it is scaled by, one 8-byte record each, resolved through the sort permutation once, so
+// that the reduce pass reads both with one coalesced load (resolving there, 32 rows ahead of the copies, made it wait: 71 -> 79 us
+// for the store of 65 k views).
 __global__ void __launch_bounds__(256)
-plan_resolve_kernel(int n, const DevState* __restrict__ state, const int32_t* __restrict__ src_row, const float* __restrict__ scale,
-                    int2* __restrict__ pmeta) {
+plan_resolve_kernel(int n, const DevState* __restrict__ state, const uint32_t* __restrict__ perm, const int32_t* __restrict__ src_row,
+                    const float* __restrict__ scale, int2* __restrict__ pmeta) {
     wait_for_predecessor();
     const int i = (int)(blockIdx.x * 256 + threadIdx.x);
     if (i >= min(n, (int)state->n_valid)) return;          // rows without a valid image have no record
-    const int src = __ldg(src_row + pmeta[i].x);
-    pmeta[i] = make_int2(src, __float_as_int(__ldg(scale + src)));
+    int src = (int)__ldg(perm + i);
+    if (src_row) src = __ldg(src_row + src);
+    pmeta[i] = make_int2(src, __float_as_int(scale ? __ldg(scale + src) : 1.f));
 }
-cudaError_t launch_plan_resolve(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale, cudaStream_t st) {
+static cudaError_t launch_plan_resolve(const gear_ctx_impl& c, const uint32_t* perm, int64_t n, const int32_t* src_row, const float* scale, cudaStream_t st) {
     KernelScope k(&c.prof, "plan_resolve", st);
-    return launch_dependent(plan_resolve_kernel, dim3((unsigned)ceil_div(n, 256)), dim3(256), 0, st, (int)n, (const DevState*)c.state(),
+    return launch_dependent(plan_resolve_kernel, dim3((unsigned)ceil_div(n, 256)), dim3(256), 0, st, (int)n, (const DevState*)c.state(), perm,
                             src_row, scale, c.at<int2>(c.ws.pmeta));
+}
+cudaError_t launch_accumulate_resolve_ahead(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale, cudaStream_t st) {
+    if (!c.plan_ready) return cudaSuccess;
+    note_plan(c, n, src_row, scale);
+    return launch_plan_resolve(c, c.sort_job(gear_ctx_impl::SORT_IMG).vals[c.img_sorted_buf], n, src_row, scale, st);
 }
 void note_plan(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale) {
     c.plan_ready = true; c.plan_n = n; c.plan_src_row = src_row; c.plan_scale = scale;
@@ -605,11 +590,13 @@ static cudaError_t launch_accumulate_to(const gear_ctx_impl& c, const int32_t* i
     }
     const uint32_t* ks = sb.keys[cur];
     if (!planned) {
-        cudaError_t pe = enqueue_plan(c, ks, sb.vals[cur], n, src_row, scale, st);
+        cudaError_t pe = enqueue_plan(c, ks, n, st);
+        if (pe == cudaSuccess && (src_row || scale)) pe = launch_plan_resolve(c, sb.vals[cur], n, src_row, scale, st);
         if (pe != cudaSuccess) return pe;
     }
     uint4* grp_rec = c.at<uint4>(c.ws.grp_rec);
-    RowGather rg{grads, ld, c.at<int2>(c.ws.pmeta)};
+    const bool plain = !src_row && !scale;
+    RowGather rg{grads, ld, c.at<int2>(c.ws.pmeta), sb.vals[cur]};
     uint32_t* blk_first = c.at<uint32_t>(c.ws.blk_first);
     uint32_t* run_end = c.at<uint32_t>(c.ws.run_end);
 
@@ -632,7 +619,11 @@ static cudaError_t launch_accumulate_to(const gear_ctx_impl& c, const int32_t* i
     // FULL only when a row fills the instantiated width exactly (D == NQ * 128): every lane then owns a chunk of every
     // row; any other width (also 384, 640, 768, 896, which round up to the next instantiation) keeps the per-chunk guard
 #define GEAR_ACC_LAUNCH(NQ, S) \
-    do { if (D == NQ * 128) launch(acc_reduce_kernel<NQ, S, true>, NQ * 512, S); else launch(acc_reduce_kernel<NQ, S, false>, NQ * 512, S); } while (0)
+    do { \
+        if (D == NQ * 128) { if (plain) launch(acc_reduce_kernel<NQ, S, true, true>, NQ * 512, S); else launch(acc_reduce_kernel<NQ, S, true, false>, NQ * 512, S); } \
+        else if (plain) launch(acc_reduce_kernel<NQ, S, false, true>, NQ * 512, S); \
+        else launch(acc_reduce_kernel<NQ, S, false, false>, NQ * 512, S); \
+    } while (0)
     if (nq <= 1) GEAR_ACC_LAUNCH(1, 8);
     else if (nq <= 2) GEAR_ACC_LAUNCH(2, 8);
     else if (nq <= 4) GEAR_ACC_LAUNCH(4, 5);

@@ -261,7 +261,7 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     // multi-block sort they are put in by a launch of its own, so that the plan runs beside the gather instead of beside the
     // head's first products (65 k views: step 387 -> 381 us).  Small arrays are sorted and planned by one kernel behind the
     // gather: there the extra launch costs more than the earlier start gives (4 k views: 56.6 us against 58.0).
-    if (plan && forked && !small_sort) GEAR_TRY(launch_accumulate_plan_ahead(c, b.nnz, nullptr, nullptr, side));
+    if (plan && forked && !small_sort) GEAR_TRY(launch_accumulate_plan_ahead(c, b.nnz, side));
     GEAR_TRY(launch_gather(c, b, o.row_view, o.inv_n, o.x_debug, st));
     if (forked) GEAR_TRY(enqueue_record(c.ev[EV_GATHER], st));
     if (scan_late) {
@@ -271,9 +271,10 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     if (dw_beside) GEAR_TRY(enqueue_wait(st, c.ev[EV_AUX]));
     if (small_sort || (forked && plan)) {
         if (forked) GEAR_TRY(enqueue_wait(side, c.ev[EV_GATHER]));
-        GEAR_TRY(small_sort ? launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, o.row_view, o.inv_n) : PlanArgs{}, side)
-                            : launch_plan_resolve(c, b.nnz, o.row_view, o.inv_n, side));
-        if (plan) note_plan(c, b.nnz, o.row_view, o.inv_n);
+        if (small_sort) {
+            GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, o.row_view, o.inv_n) : PlanArgs{}, side));
+            if (plan) note_plan(c, b.nnz, o.row_view, o.inv_n);
+        } else GEAR_TRY(launch_accumulate_resolve_ahead(c, b.nnz, o.row_view, o.inv_n, side));
     }
     if (forked && lists) GEAR_TRY(enqueue_record(c.ev[EV_PLAN], side));
     // the embedding scatter: enqueued by the head as soon as dX is on its way
@@ -385,7 +386,7 @@ static cudaError_t enqueue_owner(gear_ctx_impl& c, const Arrivals& user, const A
     if (plan) {
         c.img_sorted = true; c.img_sorted_n = img.n; c.img_sorted_buf = cur; c.img_sort_valid = true; c.last_img_id = img.ids;
         if (sort_small_fits(batch)) note_plan(c, img.n, nullptr, nullptr);
-        else GEAR_TRY(launch_accumulate_plan_ahead(c, img.n, nullptr, nullptr, st));
+        else GEAR_TRY(launch_accumulate_plan_ahead(c, img.n, st));
     }
     // (the sorted values are the source rows, so the accumulate call itself has no row indirection left)
     GEAR_TRY(launch_accumulate_collect(c, plan ? nullptr : img.ids, img_rows, img_ld, plan ? nullptr : img.src, nullptr, img.n, lists.ids,

@@ -246,10 +246,9 @@ cudaError_t launch_accumulate(const gear_ctx_impl& c, const int32_t* img_id, con
 cudaError_t launch_accumulate_atomic(const gear_ctx_impl& c, const int32_t* img_id, const float* grads, int64_t ld,
                                      const int32_t* src_row, const float* scale, int64_t n, cudaStream_t st);
 // steps 2-4 of the sorted accumulate for the batch just sorted by gear_forward_backward, ahead of the accumulate call
-cudaError_t launch_accumulate_plan_ahead(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale,
-                                         cudaStream_t st);
-// a plan made without them gets its rows' views and their scales
-cudaError_t launch_plan_resolve(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale, cudaStream_t st);
+cudaError_t launch_accumulate_plan_ahead(const gear_ctx_impl& c, int64_t n, cudaStream_t st);
+// ... and where its rows live and what they are scaled by, once that is known
+cudaError_t launch_accumulate_resolve_ahead(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale, cudaStream_t st);
 // what the plan for n rows needs; note_plan: it has been made (for the image IDs of the last batch)
 PlanArgs plan_args(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale);
 void note_plan(const gear_ctx_impl& c, int64_t n, const int32_t* src_row, const float* scale);

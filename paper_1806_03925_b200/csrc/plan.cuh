@@ -70,10 +70,9 @@ __device__ __forceinline__ void plan_tile(const PlanArgs& p, int n, int tile0, K
     const int g_warp = lane < WARPS ? s_warp[lane] : 0, f_warp = lane < WARPS ? s_warp[WARPS + lane] : 0;
     uint32_t g0, f0;
     base(__reduce_add_sync(0xffffffffu, (uint32_t)g_warp), __reduce_add_sync(0xffffffffu, (uint32_t)f_warp), g0, f0);
-    // where the gradient row of every sorted position lives and what it is scaled by (one 8-byte record), resolved through
-    // the sort permutation once, so that the reduce pass reads both with one coalesced load; every level of the chain is
-    // requested for all positions at once
-    {
+    // where the gradient row of every sorted position lives and what it is scaled by (one 8-byte record), where the call names
+    // either; every level of the chain is requested for all positions at once
+    if (p.src_row || p.scale) {
         int src[ITEMS];
         float scale[ITEMS];
 #pragma unroll
