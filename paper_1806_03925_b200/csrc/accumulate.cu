@@ -33,6 +33,7 @@ namespace gear {
 constexpr int AF_THREADS = 256;
 constexpr int AF_ITEMS = 4;
 constexpr int AF_TILE = AF_THREADS * AF_ITEMS;
+constexpr int AF_WARPS = AF_THREADS / 32;
 
 __device__ __forceinline__ uint32_t warp_inclusive_max(uint32_t v) {
     const unsigned lane = lane_id();
@@ -67,7 +68,9 @@ struct TileFlags {
     int64_t i0;                // first position owned by this thread
 };
 
-// smem: 34 words.  Every thread of the block must call this.
+// smem: AF_WARPS + 1 words, not to be written again before the block's next barrier.  Every thread of the block must call this.
+// (One barrier here and one in each pass: with a block scan per count, nine and fifteen of them, the passes waited at barriers
+// for half of their time.)
 // run_end (optional): run_end[first position of an image's run] = one past its last position.
 __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab,
                                            const DivM& div, const int32_t* __restrict__ cnt, uint32_t* smem,
@@ -106,8 +109,12 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
             }
             start = hi;
         }
-        if (lane0 == 0) smem[33] = (uint32_t)start;
+        if (lane0 == 0) smem[AF_WARPS] = (uint32_t)start;
     }
+    // rows the images already hold: asked for ahead of the barrier
+#pragma unroll
+    for (int t = 0; t < AF_ITEMS; ++t)
+        f.c0[t] = f.i0 + t < n && f.key[t] < vocab && (t == 0 || f.key[t] != f.key[t > 0 ? t - 1 : 0]) ? __ldg(cnt + f.key[t]) : 0;
     // run start of every position: inclusive max-scan of "index if run head"
     uint32_t local_max = 0;
     uint32_t run_start[AF_ITEMS];
@@ -122,29 +129,22 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
     uint32_t inc = warp_inclusive_max(local_max);
     if (lane == 31) smem[warp] = inc;
     __syncthreads();
-    if (warp == 0) {
-        uint32_t w = lane < (AF_THREADS / 32) ? smem[lane] : 0u;
-        w = warp_inclusive_max(w);
-        smem[lane] = w;
-    }
-    __syncthreads();
     uint32_t before_thread = __shfl_up_sync(0xffffffffu, inc, 1);
     if (lane == 0) before_thread = 0;
-    if (warp > 0) before_thread = max(before_thread, smem[warp - 1]);
-    const uint32_t carry = smem[33];
-    __syncthreads();
+    before_thread = max(before_thread, __reduce_max_sync(0xffffffffu, lane < warp ? smem[lane] : 0u));
+    const uint32_t carry = smem[AF_WARPS];
 
 #pragma unroll
     for (int t = 0; t < AF_ITEMS; ++t) {
         const int64_t i = f.i0 + t;
         f.head[t] = f.first[t] = f.complete[t] = false;
-        f.c0[t] = 0; f.seq[t] = 0;
+        f.seq[t] = 0;
         if (i >= n || f.key[t] >= vocab) continue;
         uint32_t rs = max(run_start[t], before_thread);
         const int64_t start = rs ? (int64_t)rs - 1 : (int64_t)carry;
         const int64_t j = i - start;                 // rank of this row among the call's rows of its image
-        const int c0 = t > 0 && f.key[t] == f.key[t > 0 ? t - 1 : 0] ? f.c0[t > 0 ? t - 1 : 0] : cnt[f.key[t]];
-        f.c0[t] = c0;
+        if (t > 0 && f.key[t] == f.key[t > 0 ? t - 1 : 0]) f.c0[t] = f.c0[t > 0 ? t - 1 : 0];
+        const int c0 = f.c0[t];
         const uint32_t x = (uint32_t)c0 + (uint32_t)j, full = div(x);
         const int rem = (int)(x - full * (uint32_t)div.M);
         if (j == 0 || rem == 0) {
@@ -169,18 +169,23 @@ __global__ void __launch_bounds__(AF_THREADS)
 acc_flag_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, const DivM div, const int32_t* __restrict__ cnt,
                 const PlanCounts counts, DevState* __restrict__ state) {
     wait_for_predecessor();
-    __shared__ uint32_t smem[34];
+    __shared__ uint32_t smem[AF_WARPS + 1], s_cnt[AF_WARPS];
     TileFlags f;
     tile_flags(f, ks, n, vocab, div, cnt, smem, state);
-    uint32_t g = 0, c = 0;
+    uint32_t gc = 0;                                                // groups, complete groups (upper half): at most AF_TILE each
 #pragma unroll
-    for (int t = 0; t < AF_ITEMS; ++t) { g += f.head[t]; c += f.complete[t]; }
-    uint32_t tg, tc;
-    block_exclusive_scan(g, smem, &tg);
-    block_exclusive_scan(c, smem, &tc);
-    if (threadIdx.x == 0) {
-        counts.tile[blockIdx.x] = make_uint2(tg, tc);
-        if (tg) atomicAdd(counts.section + blockIdx.x / AF_SECTION, (unsigned long long)tg | ((unsigned long long)tc << 32));
+    for (int t = 0; t < AF_ITEMS; ++t) gc += (uint32_t)f.head[t] | ((uint32_t)f.complete[t] << 16);
+    gc = __reduce_add_sync(0xffffffffu, gc);
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
+    if (lane == 0) s_cnt[warp] = gc;
+    __syncthreads();
+    if (warp == 0) {
+        gc = __reduce_add_sync(0xffffffffu, lane < AF_WARPS ? s_cnt[lane] : 0u);
+        const uint32_t tg = gc & 0xffffu, tc = gc >> 16;
+        if (lane == 0) {
+            counts.tile[blockIdx.x] = make_uint2(tg, tc);
+            if (tg) atomicAdd(counts.section + blockIdx.x / AF_SECTION, (unsigned long long)tg | ((unsigned long long)tc << 32));
+        }
     }
 }
 
@@ -189,24 +194,28 @@ acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, cons
                 const PlanCounts counts, uint2* __restrict__ totals, uint4* __restrict__ grp_rec, uint32_t* __restrict__ blk_first, uint32_t* __restrict__ run_end,
                 int span, DevState* __restrict__ state) {
     wait_for_predecessor();
-    __shared__ uint32_t smem[34];
-    TileFlags f;
-    tile_flags(f, ks, n, vocab, div, cnt, smem, state, run_end);
-    uint32_t g = 0, c = 0;
-#pragma unroll
-    for (int t = 0; t < AF_ITEMS; ++t) { g += f.head[t]; c += f.complete[t]; }
+    __shared__ uint32_t smem[AF_WARPS + 1], s_cnt[AF_WARPS], s_g[AF_WARPS], s_c[AF_WARPS];
+    const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
     // groups in the sections and tiles before this one: a thread's share of both counts in one word (each stays below 2^30)
     const int section = (int)blockIdx.x / AF_SECTION;
     unsigned long long before = 0;
     for (int q = threadIdx.x; q < section; q += AF_THREADS) before += counts.section[q];
     const int q = section * AF_SECTION + (int)threadIdx.x;
     if (threadIdx.x < AF_SECTION && q < (int)blockIdx.x) { const uint2 v = counts.tile[q]; before += (unsigned long long)v.x | ((unsigned long long)v.y << 32); }
-    uint32_t g0, c0, g_tile, c_tile;
-    block_exclusive_scan((uint32_t)before, smem, &g0);
-    block_exclusive_scan((uint32_t)(before >> 32), smem, &c0);
-    uint32_t gi = g0 + block_exclusive_scan(g, smem, &g_tile);
-    uint32_t ci = c0 + block_exclusive_scan(c, smem, &c_tile);
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *totals = make_uint2(g0 + g_tile, c0 + c_tile);
+    TileFlags f;
+    tile_flags(f, ks, n, vocab, div, cnt, smem, state, run_end);
+    uint32_t gc = 0;                                                // groups, complete groups (upper half): at most AF_TILE each
+#pragma unroll
+    for (int t = 0; t < AF_ITEMS; ++t) gc += (uint32_t)f.head[t] | ((uint32_t)f.complete[t] << 16);
+    const uint32_t inc = warp_inclusive_scan(gc);
+    const uint32_t bg = __reduce_add_sync(0xffffffffu, (uint32_t)before), bc = __reduce_add_sync(0xffffffffu, (uint32_t)(before >> 32));
+    if (lane == 31) { s_cnt[warp] = inc; s_g[warp] = bg; s_c[warp] = bc; }
+    __syncthreads();
+    const uint32_t of_warp = lane < AF_WARPS ? s_cnt[lane] : 0u;
+    const uint32_t g0 = __reduce_add_sync(0xffffffffu, lane < AF_WARPS ? s_g[lane] : 0u), c0 = __reduce_add_sync(0xffffffffu, lane < AF_WARPS ? s_c[lane] : 0u);
+    const uint32_t rank = __reduce_add_sync(0xffffffffu, lane < warp ? of_warp : 0u) + inc - gc, tile = __reduce_add_sync(0xffffffffu, of_warp);
+    uint32_t gi = g0 + (rank & 0xffffu), ci = c0 + (rank >> 16);
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *totals = make_uint2(g0 + (tile & 0xffffu), c0 + (tile >> 16));
     const int64_t q_base = state->q_count;
 #pragma unroll
     for (int t = 0; t < AF_ITEMS; ++t) {
