@@ -17,6 +17,8 @@
 // when the counter reaches base + grid * (k + 1), where the host knows `base` (it adds up what every
 // earlier launch contributes).  The kernel is launched cooperatively, so all blocks are resident; the spin is bounded all
 // the same, and a block that gives up records an error and makes every later wait of the launch fall through.
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace gear {
@@ -61,26 +63,28 @@ __device__ __forceinline__ uint32_t load_key(const SortJob& j, int pass, int64_t
 struct SortSmem {
     uint32_t *skey, *sval;        // [TILE] a tile's pairs in digit order on their way out
     uint32_t *base, *lstart;      // [R] where the next entry of each digit goes; where it starts in the tile's own order
-    uint32_t *wcnt, *peers;       // [WARPS][R] counts per warp; lanes with equal digits (zero between uses)
+    uint32_t *wcnt, *peers;       // [WARPS][R] counts per warp; [WARPS][R][KEYS] lanes with equal digits (zero between uses)
 };
-template <int ITEMS> constexpr int rs_smem_bytes(int width) {
-    return (2 * RS_THREADS * ITEMS + (2 + 2 * (RS_THREADS / 32)) * (1 << width)) * 4;
+template <int ITEMS> constexpr int rs_smem_bytes(int width, int keys) {
+    return (2 * RS_THREADS * ITEMS + (2 + (1 + keys) * (RS_THREADS / 32)) * (1 << width)) * 4;
 }
+// Keys a lane ranks at a time: two, where the words for that leave room for two blocks on an SM.
+constexpr int rs_keys(int width) { return width <= 8 ? 2 : 1; }
 
 // One job, block b of nb.  sync(): barrier over everything that works on the batch; false once it has been abandoned.
-template <int ITEMS, typename Sync>
+template <int ITEMS, int KEYS, typename Sync>
 __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes, int b, int nb, uint32_t* dyn, uint32_t* scratch, Sync sync) {
     constexpr int TILE = RS_THREADS * ITEMS, WARPS = RS_THREADS / 32;
     static_assert(RS_THREADS >= RS_BUCKETS, "a thread per digit");
     const int R = 1 << j.width, tid = (int)threadIdx.x, lane = (int)lane_id(), warp = tid >> 5;
     const uint32_t mask = (uint32_t)R - 1u, lt = (1u << lane) - 1u;
     SortSmem sh;
-    sh.skey = dyn; sh.sval = sh.skey + TILE; sh.base = sh.sval + TILE; sh.lstart = sh.base + R; sh.wcnt = sh.lstart + R; sh.peers = sh.wcnt + WARPS * R;
+    sh.skey = dyn; sh.sval = sh.skey + TILE; sh.base = sh.sval + TILE; sh.lstart = sh.base + R; sh.peers = sh.lstart + R; sh.wcnt = sh.peers + KEYS * WARPS * R;
     uint32_t* my_cnt = sh.wcnt + warp * R;
-    uint32_t* my_peers = sh.peers + warp * R;
+    uint32_t* my_peers = sh.peers + KEYS * warp * R;
     const int64_t tiles = ceil_div(n, TILE), per = ceil_div(tiles, nb);
     const int64_t t0 = b * per, t1 = min(tiles, t0 + per);
-    for (int i = tid; i < WARPS * R; i += RS_THREADS) sh.peers[i] = 0;
+    for (int i = tid; i < KEYS * WARPS * R; i += RS_THREADS) sh.peers[i] = 0;
     for (int pass = 0; pass < passes; ++pass) {
         const int src = pass & 1, dst = src ^ 1, shift = pass * j.width;
         // ---- how many entries of each digit the block's chunk holds
@@ -147,32 +151,59 @@ __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes
             const uint32_t ex = block_exclusive_scan(mine, scratch, nullptr);
             if (tid < R) sh.base[tid] = ex + chunk;
         }
+        // Four barriers per tile: a warp goes on to rank the next tile's keys while others still write this one out, so what it
+        // then touches is its own (its row of counts) or is written behind the next tile's first barrier.
+        for (int i = lane; i < R; i += 32) my_cnt[i] = 0;
+        __syncwarp();
+        uint32_t tot = 0;                                           // the tile's entries of digit tid
         for (int64_t t = t0; t < t1; ++t) {
             const int64_t seg0 = t * TILE + (int64_t)warp * (32 * ITEMS);
-            for (int i = tid; i < WARPS * R; i += RS_THREADS) sh.wcnt[i] = 0;
-            __syncthreads();
             // Lanes with equal digits find one another through a word per warp and digit: every lane sets its bit, then reads
             // the word; the last one puts it back to zero and moves the count on.  (match_any, and a ballot per digit bit, took
-            // three times as long.)
+            // three times as long.)  With two keys per lane at a
+            // time, a word each, half as many trips through shared memory.
             uint32_t rank[ITEMS];
 #pragma unroll
-            for (int it = 0; it < ITEMS; ++it) {
-                const bool valid = seg0 + it * 32 + lane < n;
-                const uint32_t d = (key[it] >> shift) & mask;
-                if (valid) atomicOr(&my_peers[d], 1u << lane);
-                __syncwarp();
-                const uint32_t peers = valid ? my_peers[d] : 0u, old = valid ? my_cnt[d] : 0u;
-                rank[it] = old + __popc(peers & lt);
-                __syncwarp();
-                if (peers >> lane == 1u) {                          // the highest lane of its digit
-                    my_cnt[d] = old + __popc(peers);
-                    my_peers[d] = 0u;
+            for (int it = 0; it < ITEMS; it += KEYS) {
+                const bool va = seg0 + it * 32 + lane < n;
+                const uint32_t da = (key[it] >> shift) & mask;
+                if constexpr (KEYS == 1) {
+                    if (va) atomicOr(&my_peers[da], 1u << lane);
+                    __syncwarp();
+                    const uint32_t peers = va ? my_peers[da] : 0u, old = my_cnt[da];
+                    rank[it] = old + __popc(peers & lt);
+                    __syncwarp();
+                    if (peers >> lane == 1u) {                      // the highest lane of its digit
+                        my_cnt[da] = old + __popc(peers);
+                        my_peers[da] = 0u;
+                    }
+                } else {
+                    const bool vb = seg0 + (it + 1) * 32 + lane < n;
+                    const uint32_t db = (key[it + 1] >> shift) & mask;
+                    if (va) atomicOr(&my_peers[2 * da], 1u << lane);
+                    if (vb) atomicOr(&my_peers[2 * db + 1], 1u << lane);
+                    __syncwarp();
+                    const uint2 pa = va ? *reinterpret_cast<const uint2*>(my_peers + 2 * da) : make_uint2(0u, 0u);
+                    const uint2 pb = vb ? *reinterpret_cast<const uint2*>(my_peers + 2 * db) : make_uint2(0u, 0u);
+                    const uint32_t ca = my_cnt[da], cb = my_cnt[db];
+                    rank[it] = ca + __popc(pa.x & lt);
+                    rank[it + 1] = cb + __popc(pb.x) + __popc(pb.y & lt);
+                    __syncwarp();
+                    if (pa.x >> lane == 1u) {                       // the highest lane of its digit among the first keys
+                        if (pa.y == 0u) my_cnt[da] = ca + __popc(pa.x);
+                        my_peers[2 * da] = 0u;
+                    }
+                    if (pb.y >> lane == 1u) {                       // ... and among the second ones
+                        my_cnt[db] = cb + __popc(pb.x) + __popc(pb.y);
+                        my_peers[2 * db + 1] = 0u;
+                    }
                 }
                 __syncwarp();
             }
             __syncthreads();
             // per digit: the warps' counts become running offsets, the tile's counts are scanned into lstart
-            uint32_t tot = 0;
+            if (tid < R) sh.base[tid] += tot;                       // the previous tile has been written out
+            tot = 0;
             if (tid < R) {
 #pragma unroll
                 for (int w = 0; w < WARPS; ++w) {
@@ -181,10 +212,11 @@ __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes
                     tot += c;
                 }
             }
-            {
-                const uint32_t ex = block_exclusive_scan(tot, scratch, nullptr);
-                if (tid < R) sh.lstart[tid] = ex;
-            }
+            const uint32_t inc = warp_inclusive_scan(tot);
+            if (lane == 31) scratch[warp] = inc;
+            __syncthreads();
+            const uint32_t before = __reduce_add_sync(0xffffffffu, lane < warp ? scratch[lane] : 0u);
+            if (tid < R) sh.lstart[tid] = before + inc - tot;
             __syncthreads();
             // The pairs are first put in digit order inside the tile (shared memory), then written out position by
             // position: neighbouring threads write neighbouring words of a digit's run, so the stores of a warp fall
@@ -199,6 +231,7 @@ __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes
                 }
             }
             __syncthreads();
+            for (int i = lane; i < R; i += 32) my_cnt[i] = 0;
             if (t + 1 < t1) load(t + 1);                            // travels while this tile is written out
             const int in_tile = (int)min((int64_t)TILE, n - t * TILE);
 #pragma unroll 4
@@ -209,15 +242,14 @@ __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes
                 __stcg(j.keys[dst] + pos, k);
                 __stcg(j.vals[dst] + pos, sh.sval[lp]);
             }
-            __syncthreads();
-            if (tid < R) sh.base[tid] += tot;
+            __syncwarp();
         }
         if (pass + 1 < passes && !sync()) return false;
     }
     return true;
 }
 
-template <int ITEMS>
+template <int ITEMS, int KEYS>
 __global__ void __launch_bounds__(RS_THREADS, 2)
 coop_sort_kernel(const SortBatch batch) {
     extern __shared__ uint32_t dyn[];
@@ -234,7 +266,7 @@ coop_sort_kernel(const SortBatch batch) {
         for (int q = 0; q < batch.n_jobs; ++q)
             if (live_n[q] > 0) {
                 __syncthreads();
-                sort_job<ITEMS>(batch.job[q], live_n[q], batch.passes, 0, 1, dyn, scratch, [] { __syncthreads(); return true; });
+                sort_job<ITEMS, KEYS>(batch.job[q], live_n[q], batch.passes, 0, 1, dyn, scratch, [] { __syncthreads(); return true; });
             }
         if (threadIdx.x == 0) {
             // the host has already booked this launch's arrivals: deliver them
@@ -246,27 +278,27 @@ coop_sort_kernel(const SortBatch batch) {
     unsigned long long target = batch.barrier_base;
     int q = 0;
     while (q + 1 < batch.n_jobs && (int)blockIdx.x >= batch.job[q + 1].block0) ++q;
-    sort_job<ITEMS>(batch.job[q], live_n[q], batch.passes, (int)blockIdx.x - batch.job[q].block0, batch.job[q].n_blocks, dyn, scratch, [&]() -> bool {
+    sort_job<ITEMS, KEYS>(batch.job[q], live_n[q], batch.passes, (int)blockIdx.x - batch.job[q].block0, batch.job[q].n_blocks, dyn, scratch, [&]() -> bool {
         target += gridDim.x;
         return grid_barrier(batch.barrier_ctr, target, batch.err);
     });
 }
 
-template <int ITEMS> static int coop_grid_limit() {
+template <int ITEMS, int KEYS> static int coop_grid_limit() {
     static const int limit = [] {
         int per_sm = 0;
-        const int smem = rs_smem_bytes<ITEMS>(RS_RADIX_BITS);
-        cudaFuncSetAttribute(coop_sort_kernel<ITEMS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop_sort_kernel<ITEMS>, RS_THREADS, smem);
+        const int smem = rs_smem_bytes<ITEMS>(KEYS == 2 ? 8 : RS_RADIX_BITS, KEYS);
+        cudaFuncSetAttribute(coop_sort_kernel<ITEMS, KEYS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop_sort_kernel<ITEMS, KEYS>, RS_THREADS, smem);
         const int n = sm_count() * (per_sm < 1 ? 1 : per_sm > 2 ? 2 : per_sm);
         return n < RS_MAX_BLOCKS ? n : RS_MAX_BLOCKS;
     }();
     return limit;
 }
 
-template <int ITEMS> static cudaError_t launch_sort(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st) {
+template <int ITEMS, int KEYS> static cudaError_t launch_sort(SortBatch& batch, int width, GridBarrierState* gbs, cudaStream_t st) {
     // every job gets blocks in proportion to its tiles, at least one and at most one per tile
-    const int limit = coop_grid_limit<ITEMS>();
+    const int limit = coop_grid_limit<ITEMS, KEYS>();
     int64_t tiles[3], total = 0;
     for (int j = 0; j < batch.n_jobs; ++j) {
         tiles[j] = ceil_div(batch.job[j].n_max, RS_THREADS * ITEMS);
@@ -282,13 +314,11 @@ template <int ITEMS> static cudaError_t launch_sort(SortBatch& batch, GridBarrie
     }
     if (grid > limit) { batch.job[big].n_blocks -= grid - limit; grid = limit; }      // (very small jobs beside a very large one)
     for (int j = 0, at = 0; j < batch.n_jobs; ++j) { batch.job[j].block0 = at; at += batch.job[j].n_blocks; }
-    int width = 1;
-    for (int j = 0; j < batch.n_jobs; ++j) width = batch.job[j].width > width ? batch.job[j].width : width;
     batch.n_barriers = 3 * batch.passes - 1;            // per pass: counts, running totals, the next order
     batch.barrier_ctr = gbs->device_counter;
     batch.barrier_base = gbs->host_base;
     gbs->host_base += (unsigned long long)grid * (unsigned long long)batch.n_barriers;
-    return launch_as(Op::COOPERATIVE, coop_sort_kernel<ITEMS>, dim3(grid), dim3(RS_THREADS), rs_smem_bytes<ITEMS>(width), st, batch);
+    return launch_as(Op::COOPERATIVE, coop_sort_kernel<ITEMS, KEYS>, dim3(grid), dim3(RS_THREADS), rs_smem_bytes<ITEMS>(width, KEYS), st, batch);
 }
 
 int sort_jobs(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st, Profiler* prof, cudaError_t* err_out) {
@@ -299,11 +329,19 @@ int sort_jobs(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st, Profiler
         if (p > passes) passes = p;
         n += batch.job[j].n_max;
     }
-    for (int j = 0; j < batch.n_jobs; ++j) batch.job[j].width = (batch.job[j].bits + passes - 1) / passes;
+    int width = 1;
+    for (int j = 0; j < batch.n_jobs; ++j) {
+        batch.job[j].width = (batch.job[j].bits + passes - 1) / passes;
+        width = batch.job[j].width > width ? batch.job[j].width : width;
+    }
     batch.passes = passes;
     KernelScope k(prof, batch.name ? batch.name : "coop_sort", st);
     // smaller tiles while the larger ones would leave blocks idle
-    *err_out = n <= (int64_t)RS_THREADS * 4 * coop_grid_limit<4>() ? launch_sort<4>(batch, gbs, st) : launch_sort<8>(batch, gbs, st);
+    auto launch = [&](auto keys) {
+        constexpr int K = decltype(keys)::value;
+        return n <= (int64_t)RS_THREADS * 4 * coop_grid_limit<4, K>() ? launch_sort<4, K>(batch, width, gbs, st) : launch_sort<8, K>(batch, width, gbs, st);
+    };
+    *err_out = rs_keys(width) == 2 ? launch(std::integral_constant<int, 2>{}) : launch(std::integral_constant<int, 1>{});
     return passes & 1;
 }
 
