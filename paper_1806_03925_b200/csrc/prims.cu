@@ -51,14 +51,6 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long* ctr, unsigned l
     return ok_flag != 0;
 }
 
-__device__ __forceinline__ uint32_t load_key(const SortJob& j, int pass, int64_t i, int src) {
-    if (pass == 0 && j.ids) {
-        const int32_t id = __ldcg(j.ids + i);
-        return (id >= 0 && (uint32_t)id < j.sentinel) ? (uint32_t)id : j.sentinel;
-    }
-    return __ldcg(j.keys[src] + i);
-}
-
 // Dynamic shared memory of a block, in words (R = 2^width buckets in use).
 struct SortSmem {
     uint32_t *skey, *sval;        // [TILE] a tile's pairs in digit order on their way out
@@ -87,6 +79,11 @@ __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes
     for (int i = tid; i < KEYS * WARPS * R; i += RS_THREADS) sh.peers[i] = 0;
     for (int pass = 0; pass < passes; ++pass) {
         const int src = pass & 1, dst = src ^ 1, shift = pass * j.width;
+        // The first pass may read raw IDs: an ID out of range (a negative one is a large unsigned word) becomes the sentinel, when the
+        // key is used and not where it is loaded, where the loads would be waited for (first pass over 16 M IDs: 228 -> 135 us).
+        const bool raw = pass == 0 && j.ids;
+        const uint32_t* __restrict__ from = raw ? reinterpret_cast<const uint32_t*>(j.ids) : j.keys[src];
+        const uint32_t most = raw ? j.sentinel : 0xffffffffu;
         // ---- how many entries of each digit the block's chunk holds
         for (int i = tid; i < WARPS * R; i += RS_THREADS) sh.wcnt[i] = 0;
         __syncthreads();
@@ -96,10 +93,11 @@ __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes
 #pragma unroll
             for (int it = 0; it < ITEMS; ++it) {                    // all loads of the tile in flight before the first is used
                 const int64_t i = t * TILE + it * RS_THREADS + tid;
-                key[it] = i < n ? load_key(j, pass, i, src) : 0u;
+                key[it] = i < n ? __ldcg(from + i) : 0u;
             }
 #pragma unroll
             for (int it = 0; it < ITEMS; ++it) {
+                key[it] = min(key[it], most);
                 if (t * TILE + it * RS_THREADS + tid < n) {
                     bad |= key[it] == j.sentinel;
                     atomicAdd(&my_cnt[(key[it] >> shift) & mask], 1u);
@@ -141,7 +139,7 @@ __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes
 #pragma unroll
             for (int it = 0; it < ITEMS; ++it) {                    // keys and values of the tile: one trip to memory
                 const int64_t i = seg0 + it * 32 + lane;
-                key[it] = i < n ? load_key(j, pass, i, src) : 0u;
+                key[it] = i < n ? __ldcg(from + i) : 0u;
                 val[it] = identity ? (j.src && i < n ? (uint32_t)__ldcg(j.src + i) : (uint32_t)i) : (i < n ? __ldcg(j.vals[src] + i) : 0u);
             }
         };
@@ -163,6 +161,8 @@ __device__ __forceinline__ bool sort_job(const SortJob& j, int64_t n, int passes
             // three times as long.)  With two keys per lane at a
             // time, a word each, half as many trips through shared memory.
             uint32_t rank[ITEMS];
+#pragma unroll
+            for (int it = 0; it < ITEMS; ++it) key[it] = min(key[it], most);
 #pragma unroll
             for (int it = 0; it < ITEMS; it += KEYS) {
                 const bool va = seg0 + it * 32 + lane < n;
