@@ -46,7 +46,7 @@ __device__ __forceinline__ uint32_t warp_inclusive_max(uint32_t v) {
 }
 
 // The AF_ITEMS consecutive words a thread owns (a 16-byte load away from the array's end).
-__device__ __forceinline__ void load_items(uint32_t (&v)[AF_ITEMS], const uint32_t* __restrict__ p, int64_t i0, int64_t n, uint32_t pad) {
+__device__ __forceinline__ void load_items(uint32_t (&v)[AF_ITEMS], const uint32_t* __restrict__ p, uint32_t i0, uint32_t n, uint32_t pad) {
     static_assert(AF_ITEMS == 4, "one 16-byte load");
     if (i0 + AF_ITEMS <= n) {
         const uint4 q = __ldg(reinterpret_cast<const uint4*>(p + i0));
@@ -65,18 +65,18 @@ struct TileFlags {
     bool complete[AF_ITEMS];   // ... and the group reaches M
     int c0[AF_ITEMS];          // rows the image already holds in the table
     int seq[AF_ITEMS];         // group heads: how many groups of the image this call completes before this one
-    int64_t i0;                // first position owned by this thread
+    uint32_t i0;               // first position owned by this thread (positions are below 2^31: 32-bit arithmetic throughout)
 };
 
 // smem: AF_WARPS + 1 words, not to be written again before the block's next barrier.  Every thread of the block must call this.
 // (One barrier here and one in each pass: with a block scan per count, nine and fifteen of them, the passes waited at barriers
 // for half of their time.)
 // run_end (optional): run_end[first position of an image's run] = one past its last position.
-__device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab,
+__device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restrict__ ks, uint32_t n, uint32_t vocab,
                                            const DivM& div, const int32_t* __restrict__ cnt, uint32_t* smem,
                                            DevState* __restrict__ state, uint32_t* __restrict__ run_end = nullptr) {
-    const int64_t tile0 = (int64_t)blockIdx.x * AF_TILE;
-    f.i0 = tile0 + (int64_t)threadIdx.x * AF_ITEMS;
+    const uint32_t tile0 = blockIdx.x * (uint32_t)AF_TILE;
+    f.i0 = tile0 + threadIdx.x * (uint32_t)AF_ITEMS;
     uint32_t prev = vocab;   // key just before this thread's first position
     if (f.i0 < n && f.i0 > 0) prev = ks[f.i0 - 1];
     load_items(f.key, ks, f.i0, n, vocab);
@@ -88,10 +88,10 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
     if (threadIdx.x < 32) {
         const int lane0 = (int)threadIdx.x;
         const uint32_t key0 = __shfl_sync(0xffffffffu, f.key[0], 0);
-        int64_t start = tile0;
+        uint32_t start = tile0;
         const bool spans = tile0 > 0 && tile0 < n && ks[tile0 - 1] == key0;      // the same words for every lane
         if (spans) {
-            int64_t hi = tile0 - 1;                                  // ks[hi] == key0
+            int64_t hi = (int64_t)tile0 - 1;                         // ks[hi] == key0
             const int64_t far = hi - ((int64_t)1 << lane0);
             const bool same = lane0 < 31 && far >= 0 && ks[far] == key0;
             const int k = __popc(__ballot_sync(0xffffffffu, same));  // probes 0 .. k-1 still lie inside the run
@@ -107,9 +107,9 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
                 const int64_t below = hi - step;
                 if (below > lo) lo = below;                          // the first probe that failed (it lies above the old lo)
             }
-            start = hi;
+            start = (uint32_t)hi;
         }
-        if (lane0 == 0) smem[AF_WARPS] = (uint32_t)start;
+        if (lane0 == 0) smem[AF_WARPS] = start;
     }
     // rows the images already hold: asked for ahead of the barrier
 #pragma unroll
@@ -122,7 +122,7 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
     for (int t = 0; t < AF_ITEMS; ++t) {
         const uint32_t before = t == 0 ? prev : f.key[t - 1];
         const bool run_head = (f.i0 + t < n) && (f.i0 + t == 0 || f.key[t] != before);
-        if (run_head) { local_max = (uint32_t)(f.i0 + t) + 1u; }   // +1 so that 0 means "none"
+        if (run_head) { local_max = f.i0 + t + 1u; }   // +1 so that 0 means "none"
         run_start[t] = local_max;
     }
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
@@ -136,27 +136,27 @@ __device__ __forceinline__ void tile_flags(TileFlags& f, const uint32_t* __restr
 
 #pragma unroll
     for (int t = 0; t < AF_ITEMS; ++t) {
-        const int64_t i = f.i0 + t;
+        const uint32_t i = f.i0 + t;
         f.head[t] = f.first[t] = f.complete[t] = false;
         f.seq[t] = 0;
         if (i >= n || f.key[t] >= vocab) continue;
         uint32_t rs = max(run_start[t], before_thread);
-        const int64_t start = rs ? (int64_t)rs - 1 : (int64_t)carry;
-        const int64_t j = i - start;                 // rank of this row among the call's rows of its image
+        const uint32_t start = rs ? rs - 1 : carry;
+        const uint32_t j = i - start;                // rank of this row among the call's rows of its image
         if (t > 0 && f.key[t] == f.key[t > 0 ? t - 1 : 0]) f.c0[t] = f.c0[t > 0 ? t - 1 : 0];
         const int c0 = f.c0[t];
-        const uint32_t x = (uint32_t)c0 + (uint32_t)j, full = div(x);
-        const int rem = (int)(x - full * (uint32_t)div.M);
+        const uint32_t x = (uint32_t)c0 + j, full = div(x);
+        const uint32_t rem = x - full * (uint32_t)div.M;
         if (j == 0 || rem == 0) {
             f.head[t] = true;
             f.first[t] = (j == 0);
             f.seq[t] = (int)full;           // c0 < M: the first group of the image gets 0
-            const int64_t last = i + (div.M - (int64_t)rem) - 1;  // the row that brings the count to M
+            const uint32_t last = i + ((uint32_t)div.M - rem) - 1u;  // the row that brings the count to M
             f.complete[t] = last < n && ks[last] == f.key[t];
         }
         const uint32_t after = i + 1 < n ? ks[i + 1] : vocab;
         if (after >= vocab) state->n_valid = i + 1;                     // exactly one thread sees this
-        if (run_end && after != f.key[t]) run_end[start] = (uint32_t)(i + 1);
+        if (run_end && after != f.key[t]) run_end[start] = i + 1;
     }
     if (blockIdx.x == 0 && threadIdx.x == 0 && (n == 0 || ks[0] >= vocab)) state->n_valid = 0;   // no valid row at all
 }
@@ -166,7 +166,7 @@ struct PlanCounts { uint2* tile; unsigned long long* section; };
 constexpr int AF_SECTION = 64;
 
 __global__ void __launch_bounds__(AF_THREADS)
-acc_flag_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, const DivM div, const int32_t* __restrict__ cnt,
+acc_flag_kernel(const uint32_t* __restrict__ ks, uint32_t n, uint32_t vocab, const DivM div, const int32_t* __restrict__ cnt,
                 const PlanCounts counts, DevState* __restrict__ state) {
     wait_for_predecessor();
     __shared__ uint32_t smem[AF_WARPS + 1], s_cnt[AF_WARPS];
@@ -190,7 +190,7 @@ acc_flag_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, cons
 }
 
 __global__ void __launch_bounds__(AF_THREADS)
-acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, const DivM div, const int32_t* __restrict__ cnt,
+acc_plan_kernel(const uint32_t* __restrict__ ks, uint32_t n, uint32_t vocab, const DivM div, const int32_t* __restrict__ cnt,
                 const PlanCounts counts, uint2* __restrict__ totals, uint4* __restrict__ grp_rec, uint32_t* __restrict__ blk_first, uint32_t* __restrict__ run_end,
                 int span, DevState* __restrict__ state) {
     wait_for_predecessor();
@@ -225,7 +225,7 @@ acc_plan_kernel(const uint32_t* __restrict__ ks, int64_t n, uint32_t vocab, cons
         // one 16-byte record per group: start position (top bit: first group of its image in this call), image ID,
         // ready-queue slot (-1: the group stays open), and for the image's first group the rows the image already held,
         // for a later one its number among the groups of the image that this call completes
-        grp_rec[gi] = make_uint4((uint32_t)(f.i0 + t) | (f.first[t] ? 0x80000000u : 0u), f.key[t],
+        grp_rec[gi] = make_uint4((f.i0 + t) | (f.first[t] ? 0x80000000u : 0u), f.key[t],
                                  (uint32_t)(f.complete[t] ? (int32_t)(q_base + ci) : -1),
                                  (uint32_t)(f.first[t] ? f.c0[t] : f.seq[t]));
         ++gi;
@@ -513,10 +513,10 @@ static cudaError_t enqueue_plan(const gear_ctx_impl& c, const uint32_t* ks, int6
     c.plan_sections_dirty = (int)ceil_div(n_tiles, AF_SECTION);
     cudaError_t e;
     { KernelScope k(&c.prof, "acc_flag", st);
-    e = launch_dependent(acc_flag_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, n, (uint32_t)vocab, div, c.buf.dfv_gcnt, counts, state); }
+    e = launch_dependent(acc_flag_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, (uint32_t)n, (uint32_t)vocab, div, c.buf.dfv_gcnt, counts, state); }
     if (e != cudaSuccess) return e;
     KernelScope k(&c.prof, "acc_plan", st);
-    return launch_dependent(acc_plan_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, n, (uint32_t)vocab, div, c.buf.dfv_gcnt, counts, tile_cnt + n_tiles,
+    return launch_dependent(acc_plan_kernel, dim3((unsigned)n_tiles), dim3(AF_THREADS), 0, st, ks, (uint32_t)n, (uint32_t)vocab, div, c.buf.dfv_gcnt, counts, tile_cnt + n_tiles,
                             c.at<uint4>(c.ws.grp_rec), c.at<uint32_t>(c.ws.blk_first),
                             c.at<uint32_t>(c.ws.run_end), acc_span_log2(n), state);
 }
