@@ -75,7 +75,6 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
         p->wbt[l] = take((size_t)fan * c.hidden[l] * hsz);
         fan = c.hidden[l];
     }
-    p->dz = take(B * 4);
     p->loss_part = take((size_t)p->loss_blocks * 4);
     if (c.head_dtype == GEAR_F32) p->head_grad = take((size_t)param_count(c) * 4);
     p->sort_n[0] = p->sort_n[1] = c.max_batch;

@@ -77,9 +77,8 @@ template <typename TX, int NQ, int ROWS>
 __global__ void __launch_bounds__(256, NQ == 4 ? 1 : 2)
 head_out_kernel(int B, int H, const __nv_bfloat16* __restrict__ h, int64_t stride, const float* __restrict__ w_out,
                 const float* __restrict__ b_out, const float* __restrict__ label, float* __restrict__ prob,
-                float* __restrict__ dz, __nv_bfloat16* __restrict__ dA, float* __restrict__ loss_part,
-                float* __restrict__ gw_out, float* __restrict__ gb_top, float* __restrict__ gb_out,
-                unsigned int* __restrict__ ticket, float* __restrict__ loss) {
+                __nv_bfloat16* __restrict__ dA, float* __restrict__ loss_part,
+                float* __restrict__ gw_out, float* __restrict__ gb_top, float* __restrict__ gb_out) {
     wait_for_predecessor();
     constexpr int LG = ROWS == 8 ? 3 : ROWS == 4 ? 2 : ROWS == 2 ? 1 : 0;
     static_assert((1 << LG) == ROWS, "ROWS is 1, 2, 4 or 8");
@@ -147,7 +146,6 @@ head_out_kernel(int B, int H, const __nv_bfloat16* __restrict__ h, int64_t strid
             local += fmaxf(zz, 0.f) - zz * y + log1pf(expf(-fabsf(zz)));
             gsum += g;
             if (prob) prob[b] = p;
-            dz[b] = g;
         }
 #pragma unroll
         for (int j = 0; j < ROWS; ++j) {
@@ -188,27 +186,6 @@ head_out_kernel(int B, int H, const __nv_bfloat16* __restrict__ h, int64_t strid
         for (int k = 0; k < 8; ++k) { s += part[k]; t += gpart[k]; }
         loss_part[blockIdx.x] = s;
         atomicAdd(gb_out, t);
-    }
-    // The block that delivers its partial loss last adds them all up, always in block order (the ticket counts
-    // arrivals and wraps back to zero by itself, ready for the next launch).
-    __shared__ int is_last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        is_last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    float s = 0.f;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) s += __ldcg(loss_part + i);
-    s = warp_sum(s);
-    __syncthreads();
-    if (lane == 0) part[warp] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.f;
-        for (int k = 0; k < 8; ++k) t += part[k];
-        loss[0] = B > 0 ? t / (float)B : 0.f;
     }
 }
 
@@ -340,20 +317,20 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
         W[l] = matrix_at(c, c.ws.wb[l], (int64_t)p.fan[l] * p.fan[l + 1]);
         Wt[l] = matrix_at(c, c.ws.wbt[l], (int64_t)p.fan[l] * p.fan[l + 1]);
     }
-    float* dz = c.at<float>(c.ws.dz);
     float* loss_part = c.at<float>(c.ws.loss_part);
 
     // forward
     const int HT = p.fan[L];
     // a bf16 top layer whose columns are one tile of its product takes the output unit along
     const bool top_fused = BF && HT <= TC_TOP_N;
+    int n_part = 0;                                       // partial losses it leaves
     for (int l = 0; l < L; ++l) {
         const int K = p.fan[l], N = p.fan[l + 1];
         if (top_fused && l + 1 == L)
             err = tc_gemm_top(c, "tc_gemm_top", B, N, K, H[l].p, K, Wt[l].p, K, p.b[l], dA[L].p,
-                              TopArgs{p.w_out, p.b_out, bt.label, o.prob, loss_part, p.gw_out, p.gb[l], p.gb_out, &c.state()->colsum_ticket, o.loss}, st);
+                              TopArgs{p.w_out, p.b_out, bt.label, o.prob, loss_part, p.gw_out, p.gb[l], p.gb_out}, &n_part, st);
         else if constexpr (BF)
-            err = tc_gemm_kmajor(c, "tc_gemm_fwd", B, N, K, H[l].p, K, Wt[l].p, K, 0, H[l + 1].p, N, p.b[l], nullptr, 0, nullptr, st);
+            err = tc_gemm_kmajor(c, "tc_gemm_fwd", B, N, K, H[l].p, K, Wt[l].p, K, 0, H[l + 1].p, N, p.b[l], nullptr, 0, nullptr, LossSum{}, st);
         else
             err = launch_fwd_f32(c, B, N, K, c.at<float>(c.ws.xf[l]), p.W[l], p.b[l], H[l + 1], l + 1 < L ? c.at<float>(c.ws.xf[l + 1]) : nullptr, st);
         if (err != cudaSuccess) return err;
@@ -367,9 +344,9 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
         // every warp gets the same number of passes where the batch allows it
         const int64_t batches = ceil_div(B, rows);
         const int64_t passes = ceil_div(batches, (int64_t)c.ws.loss_blocks * 8);
-        const int blocks = (int)ceil_div(batches, 8 * passes);
+        const int blocks = n_part = (int)ceil_div(batches, 8 * passes);
 #define GEAR_HEAD_OUT(NQ, ROWS) launch_dependent(head_out_kernel<TX, NQ, ROWS>, dim3(blocks), dim3(256), 0, st, B, HT, H[L].p, H[L].stride, p.w_out, p.b_out, bt.label, \
-        o.prob, dz, dA[L].p, loss_part, p.gw_out, p.gb[L - 1], p.gb_out, &c.state()->colsum_ticket, o.loss)
+        o.prob, dA[L].p, loss_part, p.gw_out, p.gb[L - 1], p.gb_out)
         if (nq <= 1) err = GEAR_HEAD_OUT(1, RMAX);
         else if (nq == 2) err = GEAR_HEAD_OUT(2, RMAX / 4);
         else err = GEAR_HEAD_OUT(4, 1);
@@ -395,12 +372,13 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
     for (int l = L - 1; l >= 0; --l) {
         const int K = p.fan[l], N = p.fan[l + 1];
         if (beside && !hooks.dw_last && (err = weight_grad(l)) != cudaSuccess) return err;
+        const LossSum loss = l == L - 1 ? LossSum{loss_part, n_part, B, o.loss} : LossSum{};      // the product behind the output unit
         if constexpr (BF) {
-            if (l > 0) err = tc_gemm_kmajor(c, "tc_gemm_dh", B, K, N, dA[l + 1].p, N, W[l].p, N, 1, dA[l].p, K, nullptr, H[l].p, K, p.gb[l - 1], st);
-            else err = tc_gemm_kmajor(c, "tc_gemm_dx", B, K, N, dA[l + 1].p, N, W[l].p, N, 2, o.dX, K, nullptr, nullptr, 0, nullptr, st);
+            if (l > 0) err = tc_gemm_kmajor(c, "tc_gemm_dh", B, K, N, dA[l + 1].p, N, W[l].p, N, 1, dA[l].p, K, nullptr, H[l].p, K, p.gb[l - 1], loss, st);
+            else err = tc_gemm_kmajor(c, "tc_gemm_dx", B, K, N, dA[l + 1].p, N, W[l].p, N, 2, o.dX, K, nullptr, nullptr, 0, nullptr, loss, st);
         } else {
-            if (l > 0) err = tc3_gemm_kmajor(c, "tc3_gemm_dh", B, K, N, dA[l + 1], N, W[l], N, dA[l], nullptr, K, H[l].p, K, p.gb[l - 1], st);
-            else err = tc3_gemm_kmajor(c, "tc3_gemm_dx", B, K, N, dA[l + 1], N, W[l], N, Planes{}, o.dX, K, nullptr, 0, nullptr, st);
+            if (l > 0) err = tc3_gemm_kmajor(c, "tc3_gemm_dh", B, K, N, dA[l + 1], N, W[l], N, dA[l], nullptr, K, H[l].p, K, p.gb[l - 1], loss, st);
+            else err = tc3_gemm_kmajor(c, "tc3_gemm_dx", B, K, N, dA[l + 1], N, W[l], N, Planes{}, o.dX, K, nullptr, 0, nullptr, loss, st);
         }
         if (err != cudaSuccess) return err;
         if (l == 0 && hooks.after_dx && (err = hooks.after_dx(hooks.arg)) != cudaSuccess) return err;

@@ -46,7 +46,6 @@ struct TopSmem {                          // the top hidden layer's epilogue
     float z[2][2][TC_BM];                 // [tile parity][column half] a row's part of the dot product
     float g[8][32];                       // per epilogue warp: dz of its rows
     float part[2][8];                     // per epilogue warp: loss, sum of dz
-    int is_last;
 };
 
 template <int BN, int EW, int EPI> struct TcCfg {
@@ -77,6 +76,7 @@ struct TcArgs {
     float* colsum;            // ReLU-mask epilogue: colsum[n] += sum over rows of the stored output (may be null)
     int32_t* err;             // device word that receives a non-zero code on a timeout
     TopArgs top;              // top layer only
+    LossSum loss;             // the loss to finish
 };
 
 // Epilogue of one finished accumulator buffer `a`, as run by one of the epilogue warps: warp w reads
@@ -352,8 +352,7 @@ __device__ __forceinline__ void epilogue_top(const TcArgs& g, const CUtensorMap*
     }
 }
 
-// After the last tile (all threads of the CTA): sums to memory.  The CTA that delivers its partial loss last adds them all up,
-// always in CTA order (the ticket counts arrivals and wraps back to zero by itself, ready for the next launch).
+// After the last tile (all threads of the CTA): sums to memory.
 __device__ __forceinline__ void finish_top(const TcArgs& g, TopSmem& s) {
     for (int n = threadIdx.x; n < g.N; n += blockDim.x) { atomicAdd(g.top.gw_out + n, s.gw[n]); atomicAdd(g.top.gb_top + n, s.gb[n]); }
     if (threadIdx.x == 0) {
@@ -361,16 +360,7 @@ __device__ __forceinline__ void finish_top(const TcArgs& g, TopSmem& s) {
         for (int k = 0; k < 8; ++k) { l += s.part[0][k]; t += s.part[1][k]; }
         g.top.loss_part[blockIdx.x] = l;
         atomicAdd(g.top.gb_out, t);
-        __threadfence();
-        s.is_last = atomicInc(g.top.ticket, gridDim.x - 1) == gridDim.x - 1;
     }
-    __syncthreads();
-    if (!s.is_last || threadIdx.x >= 32) return;
-    __threadfence();
-    float l = 0.f;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += 32) l += __ldcg(g.top.loss_part + i);
-    l = warp_sum(l);
-    if (threadIdx.x == 0) g.top.loss[0] = l / (float)g.M;
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -461,6 +451,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
                         __nanosleep(64);
             }
         }
+        if (blockIdx.x == 0) { __syncwarp(); sum_loss(g.loss, lane); }
     } else if (warp == 1) {
         // ---------------- MMA issuer
         if (lane == 0) {
@@ -665,7 +656,7 @@ static cudaError_t launch_bn(int bn, const CUtensorMap& ma, const CUtensorMap& m
 
 cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
                            const __nv_bfloat16* W, int64_t ldw, int epi, void* out, int64_t ldo, const float* bias,
-                           const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st) {
+                           const __nv_bfloat16* mask, int64_t ldm, float* colsum, const LossSum& loss, cudaStream_t st) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     // column tiles of 256 or 128; the fp32 output (dX) also has 192, which fits a width like 384 without a half-empty tile
     int bn = N > 128 ? 256 : 128;
@@ -682,8 +673,8 @@ cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int 
           : bn == 64        ? make_map_mask(c, &mo, out, M, N, ldo)
                             : make_map(c, &mo, out, M, N, ldo, 32)))
         return cudaErrorInvalidValue;
-    TcArgs g;
-    g.M = M; g.N = N; g.K = K;
+    TcArgs g = {};
+    g.M = M; g.N = N; g.K = K; g.loss = loss;
     g.m_tiles = (int)m_tiles; g.n_tiles = (int)ceil_div(N, bn); g.k_splits = 1;
     g.kb_per_split = (int)ceil_div(K, TC_BK);
     g.out = out; g.ldo = ldo; g.bias = bias; g.mask = mask; g.ldm = ldm; g.err = &c.state()->tc_error;
@@ -704,7 +695,7 @@ cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int 
 }
 
 cudaError_t tc_gemm_top(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
-                        const __nv_bfloat16* W, int64_t ldw, const float* bias, __nv_bfloat16* dA, const TopArgs& top, cudaStream_t st) {
+                        const __nv_bfloat16* W, int64_t ldw, const float* bias, __nv_bfloat16* dA, const TopArgs& top, int* n_part, cudaStream_t st) {
     const int bn = N > 128 ? 256 : 128;
     CUtensorMap ma, mb, mo;
     if (!make_map(c, &ma, A, M, K, lda, TC_BM) || !make_map(c, &mb, W, N, K, ldw, bn) || !make_map(c, &mo, dA, M, N, N, 32))
@@ -714,6 +705,7 @@ cudaError_t tc_gemm_top(const gear_ctx_impl& c, const char* name, int M, int N, 
     g.m_tiles = (int)ceil_div(M, TC_BM); g.n_tiles = 1; g.k_splits = 1;
     g.kb_per_split = (int)ceil_div(K, TC_BK);
     g.bias = bias; g.err = &c.state()->tc_error; g.top = top;
+    *n_part = g.m_tiles < sm_count() ? g.m_tiles : sm_count();          // one per CTA
     KernelScope ks(&c.prof, name, st);
     return bn == 256 ? launch_variant<256, false, TC_EPI_TOP, 8>(ma, mb, mo, ma /*unused*/, g, st)
                      : launch_variant<128, false, TC_EPI_TOP, 8>(ma, mb, mo, ma /*unused*/, g, st);
@@ -742,7 +734,7 @@ cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int
     CUtensorMap ma, mb, mo;
     if (!make_map(c, &ma, A, K, M, lda, 64) || !make_map(c, &mb, Bm, K, N, ldb, 64) || !make_map_f32(c, &mo, out, M, N, ldo))
         return cudaErrorInvalidValue;
-    TcArgs g;
+    TcArgs g = {};
     g.M = M; g.N = N; g.K = K;
     g.m_tiles = (int)ceil_div(M, TC_BM); g.n_tiles = (int)ceil_div(N, bn);
     g.kb_per_split = (int)ceil_div(total_kb, splits);

@@ -53,6 +53,7 @@ struct T3Args {
     const __nv_bfloat16* mask; int64_t ldm;         // T3_MASK: leading plane of the activations (positive where they are)
     float* colsum;                                  // T3_MASK: colsum[n] += column sums of the masked output (may be null)
     int32_t* err;
+    LossSum loss;             // the loss to finish
 };
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
@@ -220,6 +221,7 @@ t3_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                         __nanosleep(64);
             }
         }
+        if (blockIdx.x == 0) { __syncwarp(); sum_loss(g.loss, lane); }
     } else if (warp == 1) {
         // ---------------- MMA issuer
         if (lane == 0) {
@@ -372,10 +374,10 @@ static int t3_bn(const T3Args& g) {
 
 cudaError_t tc3_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,
                             const Planes& W, int64_t ldw, const Planes& out_planes, float* out_f32, int64_t ldo,
-                            const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st) {
+                            const __nv_bfloat16* mask, int64_t ldm, float* colsum, const LossSum& loss, cudaStream_t st) {
     if (M <= 0 || N <= 0 || K <= 0) return cudaSuccess;
     T3Args g{};
-    g.M = M; g.N = N; g.K = K;
+    g.M = M; g.N = N; g.K = K; g.loss = loss;
     const int bn = t3_bn(g);
     g.m_tiles = (int)ceil_div(M, TC_BM); g.n_tiles = (int)ceil_div(N, bn);
     g.k_splits = 1; g.kb_per_split = (int)ceil_div(K, T3_BK);

@@ -22,7 +22,6 @@ struct WsPlan {
     size_t h[MAX_LAYERS];               // [max_batch][hidden[l]] post-ReLU activations
     size_t da[MAX_LAYERS];              // [max_batch][hidden[l]] gradient at the pre-activation
     size_t xf[MAX_LAYERS];              // fp32 head: the inputs of its layers (head input, lower hidden activations) in fp32
-    size_t dz;                          // [max_batch] fp32
     size_t loss_part;                   // [loss_blocks] fp32 per-block partial losses
     size_t head_grad;                   // fp32 head: the parameters' gradient, when the caller's array is not 16-byte aligned
     size_t wb[MAX_LAYERS];              // W_l as [in][out]
@@ -151,21 +150,25 @@ cudaError_t launch_head(const gear_ctx_impl& c, const gear_batch& b, const gear_
 // the weights as the products read them; clears head_grad (all of it, also for an empty batch)
 cudaError_t launch_round_weights(const gear_ctx_impl& c, const gear_step_out& o, cudaStream_t st);
 
+// The blocks' partial losses of the batch, added up in a fixed order by a block of the product that follows the output unit (a
+// block that found itself the last of the output unit's would keep everything behind it waiting for its fence, its ticket and
+// the partials: about 2 us).  loss null: nothing to add up.
+struct LossSum { const float* part; int n; int B; float* loss; };
+
 // head_tc.cu: bf16 products on tcgen05 tensor cores.  epi: 0 bias+ReLU -> bf16, 1 ReLU mask -> bf16, 2 plain fp32.
 // colsum (epi 1 only, may be null): colsum[n] += sum over the rows of the stored (rounded) output.
 cudaError_t tc_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
                            const __nv_bfloat16* W, int64_t ldw, int epi, void* out, int64_t ldo, const float* bias,
-                           const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st);
+                           const __nv_bfloat16* mask, int64_t ldm, float* colsum, const LossSum& loss, cudaStream_t st);
 // The top hidden layer and the output unit behind it: h = ReLU(A . W^T + bias) stays on the chip, dA gets the gradient with
-// respect to its pre-activations.  N at most TC_TOP_N.
+// respect to its pre-activations.  N at most TC_TOP_N.  *n_part: how many partial losses it leaves.
 constexpr int TC_TOP_N = 256;
 struct TopArgs {
     const float* w_out; const float* b_out; const float* label;
     float* prob; float* loss_part; float* gw_out; float* gb_top; float* gb_out;
-    unsigned int* ticket; float* loss;
 };
 cudaError_t tc_gemm_top(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
-                        const __nv_bfloat16* W, int64_t ldw, const float* bias, __nv_bfloat16* dA, const TopArgs& top, cudaStream_t st);
+                        const __nv_bfloat16* W, int64_t ldw, const float* bias, __nv_bfloat16* dA, const TopArgs& top, int* n_part, cudaStream_t st);
 // out[M][N] (fp32) += A[K][M]^T . Bm[K][N]
 cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const __nv_bfloat16* A, int64_t lda,
                             const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo, cudaStream_t st);
@@ -178,7 +181,7 @@ cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const fl
 // activations) the output goes to planes, masked, and colsum[n] += its column sums; without, to out_f32.
 cudaError_t tc3_gemm_kmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,
                             const Planes& W, int64_t ldw, const Planes& out_planes, float* out_f32, int64_t ldo,
-                            const __nv_bfloat16* mask, int64_t ldm, float* colsum, cudaStream_t st);
+                            const __nv_bfloat16* mask, int64_t ldm, float* colsum, const LossSum& loss, cudaStream_t st);
 cudaError_t tc3_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int N, int K, const Planes& A, int64_t lda,
                              const Planes& Bm, int64_t ldb, float* out, int64_t ldo, cudaStream_t st);
 

@@ -152,6 +152,15 @@ __host__ __device__ constexpr uint32_t instr_desc(int bn, bool mn_major) {
            ((uint32_t)(bn >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
 }
 
+// One warp of the grid: the batch's loss from the partial losses the kernel before this one left.
+__device__ __forceinline__ void sum_loss(const LossSum& s, int lane) {
+    if (s.loss == nullptr) return;
+    float t = 0.f;
+    for (int i = lane; i < s.n; i += 32) t += __ldcg(s.part + i);
+    t = warp_sum(t);
+    if (lane == 0) s.loss[0] = t / (float)s.B;
+}
+
 // ---------------------------------------------------------------- host side: tensor maps
 // A row-major matrix [planes][rows][cols] (planes = 1: a plain matrix) read or written in boxes of
 // planes x box_rows x box_cols.  Parts of a box past the edge read as zero and are dropped when written.
