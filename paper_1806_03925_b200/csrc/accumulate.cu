@@ -21,7 +21,7 @@
 //      average to its queue slot or, for the open group, the running sum and count back to the table.  The
 //      warp that owns the first group of an image also settles what the image's last, still open group
 //      leaves in the table, so no two warps touch one table row.
-//   6. commit (by the block of the reduce pass that finishes last): the queue length grows by the number of
+//   6. commit (by the reduce pass): the queue length grows by the number of
 //      complete groups (or the call is dropped whole if the queue would overflow).
 // HBM bound: the reduce pass reads every gradient row once and reads/writes one accumulator row per
 // distinct image; the sort and flag passes move 4-byte keys only.
@@ -215,8 +215,8 @@ acc_plan_kernel(const uint32_t* __restrict__ ks, uint32_t n, uint32_t vocab, con
     const uint32_t g0 = __reduce_add_sync(0xffffffffu, lane < AF_WARPS ? s_g[lane] : 0u), c0 = __reduce_add_sync(0xffffffffu, lane < AF_WARPS ? s_c[lane] : 0u);
     const uint32_t rank = __reduce_add_sync(0xffffffffu, lane < warp ? of_warp : 0u) + inc - gc, tile = __reduce_add_sync(0xffffffffu, of_warp);
     uint32_t gi = g0 + (rank & 0xffffu), ci = c0 + (rank >> 16);
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *totals = make_uint2(g0 + (tile & 0xffffu), c0 + (tile >> 16));
     const int64_t q_base = state->q_count;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) { *totals = make_uint2(g0 + (tile & 0xffffu), c0 + (tile >> 16)); state->plan_base = q_base; }
 #pragma unroll
     for (int t = 0; t < AF_ITEMS; ++t) {
         // the reduce pass hands out spans of 2^span sorted positions: index of the first group that starts in each
@@ -287,31 +287,23 @@ acc_reduce_kernel(RowGather rg, int D, const DivM div, int span_log2, int64_t re
     for (int i = (int)(blockIdx.x * blockDim.x + threadIdx.x); i < n_sections; i += (int)(gridDim.x * blockDim.x)) sections[i] = 0ull;
     extern __shared__ float4 ring_mem[];                          // [warps][S][NQ * 32] float4
     const uint2 totals = *plan_totals;
-    const int64_t n_groups = totals.x;
+    const int64_t n_groups = totals.x, q_base = state->plan_base;
     // Averages go to the ready queue, or (the queue being empty, so that queue slot k is also entry k of the hand-over)
     // straight into the caller's lists, whose capacity the host has checked against the row count.
     const bool to_caller = direct.avg != nullptr &&
-                           (direct.cap < 0 || (state->q_count == 0 && (int64_t)totals.y <= direct.cap));
+                           (direct.cap < 0 || (q_base == 0 && (int64_t)totals.y <= direct.cap));
     int32_t* __restrict__ e_id = to_caller ? direct.ids : q_id;
     float* __restrict__ e_avg = to_caller ? direct.avg : q_avg;
-    // Step 6 of the plan (commit) is done by whichever block finishes last: by then every block has read the queue
-    // length it started from.  Every block, also one of a dropped call, leaves through this.
-    const bool dropped = !to_caller && state->q_count + (int64_t)totals.y > ready_cap;
-    auto leave = [&]() {
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            unsigned int* ticket = reinterpret_cast<unsigned int*>(&state->pad[4]);
-            if (atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1) {
-                state->n_complete = totals.y;
-                state->direct_done = (to_caller && direct.cap >= 0) ? 1 : 0;
-                if (to_caller) { if (direct.d_n) *direct.d_n = totals.y; }
-                else if (dropped) atomicOr(&state->status, GEAR_DEV_READY_OVERFLOW);
-                else if (totals.y > 0) { state->q_count += totals.y; state->q_calls += 1; }
-            }
-        }
-    };
-    if (dropped) { leave(); return; }                                // the whole call is dropped
+    const bool dropped = !to_caller && q_base + (int64_t)totals.y > ready_cap;
+    // Step 6 of the plan (commit), by one thread: every block goes by the queue length that the plan noted.  (The block that
+    // found itself last did it before, behind a fence and a ticket that the call's end waited for.)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        state->direct_done = (to_caller && direct.cap >= 0) ? 1 : 0;
+        if (to_caller) { if (direct.d_n) *direct.d_n = totals.y; }
+        else if (dropped) atomicOr(&state->status, GEAR_DEV_READY_OVERFLOW);
+        else if (totals.y > 0) { state->q_count = q_base + totals.y; state->q_calls += 1; }
+    }
+    if (dropped) return;                                             // the whole call is dropped
     const int64_t n_valid = state->n_valid;
     const int lane = (int)lane_id(), warp = (int)(threadIdx.x >> 5);
     const int n_chunks = D / 4;
@@ -494,7 +486,6 @@ acc_reduce_kernel(RowGather rg, int D, const DivM div, int span_log2, int64_t re
         }
         G = G_nxt; range_nxt = range_nxt2;
     }
-    leave();
 }
 
 // Steps 2-4 of the plan over the sorted keys ks (flag pass, plan pass).

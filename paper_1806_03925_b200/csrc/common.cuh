@@ -23,7 +23,7 @@ struct DevState {
     int64_t n_valid;       // accumulate: rows with an in-range ID (sorted prefix length)
     int64_t direct_done;   // accumulate + collect as one call: 1 while the hand-over pass that follows has nothing to do
                            // (the reduce pass wrote the averages straight into the caller's lists)
-    int64_t n_complete;    // accumulate: groups of this call that reached M
+    int64_t plan_base;     // accumulate: length of the ready queue that the plan goes by
     int64_t pad0;
     int64_t collect_n;     // collect_ready: entries moved by the running call
     unsigned long long grid_barrier;   // arrival counter of the cooperative sort's grid barrier

@@ -176,7 +176,7 @@ sort_small_kernel(const SortBatch batch, const PlanArgs plan) {
                 if (threadIdx.x == 0) { xchg[1] = (int)g; xchg[2] = (int)f; }
                 S::sync_cluster();
                 for (int r = 0; r < cr; ++r) { const int* x = S::peer(xchg, r); g0 += (uint32_t)x[1]; f0 += (uint32_t)x[2]; }
-                if (cr == CL - 1 && threadIdx.x == 0) *plan.totals = make_uint2(g0 + g, f0 + f);
+                if (cr == CL - 1 && threadIdx.x == 0) { *plan.totals = make_uint2(g0 + g, f0 + f); plan.state->plan_base = plan.state->q_count; }
             });
         S::sync_cluster();                                                     // nobody leaves while its keys may still be read
     }
