@@ -371,8 +371,9 @@ def gear_dense_backward(ctx, raw, ids, avg, n: int, Wd_grad, d_n=None, stream=No
 def gear_adam_dense(param, grad, m, v, t: int, cfg: gear_adam, stream=None):
     n = param.numel()
     assert grad.numel() == n and m.numel() == n and v.numel() == n
-    _check(load().gear_adam_dense(_p(param), _p(grad), _p(m), _p(v), n, t, C.byref(cfg), _stream(stream)),
-           "gear_adam_dense")
+    rc = (_lib or load()).gear_adam_dense(_p(param), _p(grad), _p(m), _p(v), n, t, cfg, _raw_stream(stream))
+    if rc != GEAR_OK:
+        _check(rc, "gear_adam_dense")
 
 
 def gear_status(ctx, raise_on_error: bool = False):

@@ -14,6 +14,10 @@ from . import binding as gb
 from .workloads import BF16, Batch, GearPreset
 
 
+_WORD = np.dtype(np.int32)
+_TORCH = {np.dtype(np.int32): torch.int32, np.dtype(np.float32): torch.float32}
+
+
 @dataclass
 class DeviceBatch:
     user_id: torch.Tensor
@@ -38,14 +42,20 @@ class DeviceBatch:
                                None if b.fast is None else f(b.fast))
         sizes = [a.size for a in arrays]
         host = torch.empty(sum(sizes), dtype=torch.int32, pin_memory=True)
-        view, at = host.numpy(), 0
-        for a, n in zip(arrays, sizes):
-            view[at:at + n] = a.reshape(-1).view(np.int32) if a.flags.c_contiguous else np.ascontiguousarray(a).reshape(-1).view(np.int32)
-            at += n
-        parts = [t if a.dtype == np.int32 else t.view(getattr(torch, a.dtype.name))
-                 for a, t in zip(arrays, host.to(device, non_blocking=True).split(sizes))]
+        np.concatenate([(a if a.flags.c_contiguous else np.ascontiguousarray(a)).reshape(-1).view(_WORD) for a in arrays],
+                       out=host.numpy())
+        there = host.to(device, non_blocking=True)
+        parts = [t if a.dtype == _WORD else t.view(_TORCH.get(a.dtype) or getattr(torch, a.dtype.name))
+                 for a, t in zip(arrays, there.split_with_sizes(sizes))]
         fast = parts.pop(0).view(b.fast.shape) if b.fast is not None else None
-        return DeviceBatch(*parts, b.B, b.nnz, fast)
+        out = DeviceBatch(*parts, b.B, b.nnz, fast)
+        # the C struct of the batch: the pointers follow from where the copy went
+        c, at = gb.gear_batch(), there.data_ptr()
+        for name, n in zip(("fast",) * (fast is not None) + ("user_id", "url_id", "img_off", "img_id", "label"), sizes):
+            setattr(c, name, at)
+            at += 4 * n
+        out.__dict__["_c_struct"] = c, (*parts, fast)
+        return out
 
 
 class GearSession:
@@ -158,9 +168,12 @@ class GearSession:
 
     @staticmethod
     def _c_batch(b: DeviceBatch):
-        bt = b.__dict__.get("_c_struct")
-        if bt is None:
-            bt = b.__dict__["_c_struct"] = gb.make_batch(b.user_id, b.url_id, b.img_off, b.img_id, b.label, fast=b.fast)
+        bt, of = b.__dict__.get("_c_struct", (None, None))
+        if bt is None or not (of[0] is b.user_id and of[1] is b.url_id and of[2] is b.img_off and of[3] is b.img_id and
+                              of[4] is b.label and of[5] is b.fast):
+            of = (b.user_id, b.url_id, b.img_off, b.img_id, b.label, b.fast)
+            bt = gb.make_batch(*of[:5], fast=b.fast)
+            b.__dict__["_c_struct"] = bt, of
         bt.B, bt.nnz = b.B, b.nnz
         return bt
 
