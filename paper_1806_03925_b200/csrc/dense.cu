@@ -21,7 +21,7 @@ constexpr int DK = 16;     // tile depth
 // rows[k][c] = sum_r raw[ids[k]][r] * Wd[r][c],  k < min(n, *d_n),  c < D.  An ID outside [0, vocab) gives a zero row.
 // A chain of R multiply-adds per output cannot be cut, so small tiles spread the live rows over the SMs (2500 rows of 1536
 // values, 64 columns: 40 blocks of 64 x 64 took 242 us), and blocks walk the tiles so that a capacity far above the live
-// count costs nothing.  AVEC / BVEC: raw rows / Wd rows may be read 16 bytes at a time.
+// count costs nothing.  Fetching two steps ahead and reading shared memory four rounds early: 70 -> 57 us for those rows.  AVEC / BVEC: raw rows / Wd rows may be read 16 bytes at a time.
 template <bool AVEC, bool BVEC>
 __global__ void __launch_bounds__(128)
 dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const float* __restrict__ Wd, int D,
@@ -29,7 +29,7 @@ dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const 
                      float* __restrict__ rows, int64_t ld, DevState* __restrict__ state) {
     wait_for_predecessor();
     constexpr int BM = 16, BN = 64, TM = 2, TN = 4;
-    using T = ChainTile<BM, BN, TM, TN, 32>;
+    using T = ChainTile<BM, BN, TM, TN, 32, 2, 4>;
     __shared__ __align__(16) typename T::Smem smem;
     __shared__ int64_t row_of[BM];
     if (d_n) { const int64_t live = *d_n; n = live < n ? (live < 0 ? 0 : live) : n; }
@@ -51,11 +51,9 @@ dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const 
             const int64_t id = row_of[q % BM];
             if (id >= 0) asm volatile("prefetch.global.L2 [%0];" :: "l"(raw + id * R + 32 * (q / BM)));
         }
-        f32x2 acc[TM][TN / 2];
+        typename T::Acc acc;
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
-#pragma unroll
-            for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+        for (int i = 0; i < TM * TN / 2; ++i) acc[i] = 0ull;
         T::product(acc, R, smem, [&](int r, int k) { const int64_t id = row_of[r]; return load4<AVEC>(raw + id * R + k, id >= 0 ? R - k : 0); },
                    [&](int k, int c) { return load4<BVEC>(Wd + (int64_t)k * D + n0 + c, k < R ? D - (n0 + c) : 0); });
 #pragma unroll
@@ -63,9 +61,9 @@ dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const 
             const int64_t m = m0 + T::row(i);
             const int c = n0 + T::col(0);
             if (m >= n || c >= D) continue;                       // D is a multiple of 8: whole strips
-            const float2 lo = unpack2(acc[i][0]), hi = unpack2(acc[i][1]);
             float* dst = rows + m * ld + c;
-            dst[0] = lo.x; dst[1] = lo.y; dst[2] = hi.x; dst[3] = hi.y;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) dst[j] = T::value(acc, i, j);
         }
     }
 }

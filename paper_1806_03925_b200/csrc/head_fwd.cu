@@ -14,19 +14,17 @@
 namespace gear {
 
 // WVEC: the weights may be read 16 bytes at a time (the head input and the activations always can).
-template <int BM, int BN, int TM, int TN, int BK, int MIN_BLOCKS, bool WVEC>
+template <int BM, int BN, int TM, int TN, int BK, int DEPTH, int AHEAD, int MIN_BLOCKS, bool WVEC>
 __global__ void __launch_bounds__((BM / TM) * (BN / TN), MIN_BLOCKS)
 fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ bias,
            __nv_bfloat16* __restrict__ H, int64_t h_stride, float* __restrict__ Hf) {
     wait_for_predecessor();
-    using T = ChainTile<BM, BN, TM, TN, BK>;
+    using T = ChainTile<BM, BN, TM, TN, BK, DEPTH, AHEAD>;
     __shared__ __align__(16) typename T::Smem smem;
     const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-    f32x2 acc[TM][TN / 2];
+    typename T::Acc acc;
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+    for (int i = 0; i < TM * TN / 2; ++i) acc[i] = 0ull;
     T::product(acc, K, smem, [&](int r, int k) { return load4<true>(A + (int64_t)(m0 + r) * K + k, m0 + r < M ? K - k : 0); },
                [&](int k, int c) { return load4<WVEC>(W + (int64_t)k * N + n0 + c, k < K ? N - (n0 + c) : 0); });
 #pragma unroll
@@ -38,8 +36,8 @@ fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __rest
         for (int i = 0; i < TM; ++i) {
             const int m = m0 + T::row(i);
             if (m >= M) continue;
-            const float2 lo = unpack2(acc[i][2 * j]), hi = unpack2(acc[i][2 * j + 1]);
-            const float4 h = make_float4(fmaxf(lo.x + b0, 0.f), fmaxf(lo.y + b1, 0.f), fmaxf(hi.x + b2, 0.f), fmaxf(hi.y + b3, 0.f));
+            const float4 h = make_float4(fmaxf(T::value(acc, i, 4 * j) + b0, 0.f), fmaxf(T::value(acc, i, 4 * j + 1) + b1, 0.f),
+                                         fmaxf(T::value(acc, i, 4 * j + 2) + b2, 0.f), fmaxf(T::value(acc, i, 4 * j + 3) + b3, 0.f));
             uint2 p[3];
             split3_pair(h.x, h.y, p[0].x, p[1].x, p[2].x);
             split3_pair(h.z, h.w, p[0].y, p[1].y, p[2].y);
@@ -51,24 +49,27 @@ fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __rest
     }
 }
 
-// The chain over the reduction cannot be split, so a small batch is spread over as many SMs as it has tiles.  Measured (us;
-// 64 x 64 tiles with 8 x 4 outputs per thread | 32 x 64 with 4 x 4 | 32 x 32 with 4 x 4): 32768 x 128 x 256: 53 | 65 | 70;
-// 8192 x 128 x 192: 14.5 | 16.5 | 18.6; 4015 x 184 x 128 (189 | 378 | 756 tiles): 11.0 | 10.4 | 10.4; 1024 x 256 x 1632 (64 | 128
-// | 256 tiles): 70 | 42 | 44; 1024 x 64 x 256 (16 | 32 | 64): 14.5 | 10.4 | 8.4.
+// The chain over the reduction cannot be split, so a small batch is spread over as many SMs as it has tiles, in smaller ones the
+// fewer it has, and the fewer warps an SM gets the further ahead it fetches (kernel time; before: one step ahead, at most 32 x 32
+// tiles with 4 x 4 outputs per thread): 32768 views, 192-256-128: 143 -> 139 us; 1024 views, 1632-256-64: 65 -> 52; 1237 views,
+// 120-136 and 256 views, 96-64: steps 39.1 -> 38.8 and 26.5 -> 24.8.  The large tiles issue multiply-adds in half of the
+// cycles; 8 x 4, 8 x 8 and 16 x 4 outputs per thread, pairs along rows or columns, doubled operands in shared memory (178 us)
+// made no other difference.
 cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
                            const Planes& H, float* Hf, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     KernelScope ks(&c.prof, "f32_gemm_fwd", st);
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     auto tiles = [&](int bm, int bn) { return ceil_div(M, bm) * ceil_div(N, bn); };
-#define GEAR_FWD(BM, BN, TM, TN, BK) \
-    (wvec ? launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, 4, true>, dim3((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM)), \
+#define GEAR_FWD(BM, BN, TM, TN, BK, DEPTH, AH, MB) \
+    (wvec ? launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, true>, dim3((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM)), \
                              dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, A, W, bias, H.p, H.stride, Hf) \
-          : launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, 4, false>, dim3((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM)), \
+          : launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, false>, dim3((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM)), \
                              dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, A, W, bias, H.p, H.stride, Hf))
-    if (2 * tiles(64, 64) >= 3 * sm_count()) return GEAR_FWD(64, 64, 8, 4, 16);
-    if (5 * tiles(32, 64) >= 4 * sm_count()) return GEAR_FWD(32, 64, 4, 4, 32);
-    return GEAR_FWD(32, 32, 4, 4, 32);
+    if (2 * tiles(64, 64) >= 3 * sm_count()) return GEAR_FWD(64, 128, 16, 4, 16, 1, 1, 4);
+    if (5 * tiles(32, 64) >= 4 * sm_count()) return GEAR_FWD(32, 64, 4, 4, 32, 4, 2, 1);
+    if (tiles(16, 32) > sm_count()) return GEAR_FWD(32, 32, 2, 4, 32, 2, 3, 2);
+    return GEAR_FWD(16, 32, 2, 4, 32, 2, 3, 2);
 #undef GEAR_FWD
 }
 
