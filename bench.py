@@ -143,9 +143,12 @@ def kernel_models(p, stats):
     def avg(xs):
         return sum(xs) / max(len(xs), 1)
     layers = range(L)
+    # bf16 top layers of at most 256 columns take the output unit along (a product of its own name)
+    plain = range(L - 1) if p.head_dtype == "bf16" and fan[L] <= 256 else layers
     m["gemm"] = {
-        "fwd": (avg([2 * B * fan[l] * fan[l + 1] for l in layers]),
-                avg([(B * fan[l] + fan[l] * fan[l + 1] + B * fan[l + 1]) * xsz for l in layers])),
+        "fwd": (avg([2 * B * fan[l] * fan[l + 1] for l in plain]),
+                avg([(B * fan[l] + fan[l] * fan[l + 1] + B * fan[l + 1]) * xsz for l in plain])),
+        "top": (2 * B * (fan[L - 1] + 1) * fan[L], (B * fan[L - 1] + fan[L - 1] * fan[L] + B * fan[L]) * xsz + B * 8),
         "dw": (avg([2 * B * fan[l] * fan[l + 1] for l in layers]),
                avg([(B * fan[l] + B * fan[l + 1]) * xsz + fan[l] * fan[l + 1] * 4 for l in layers])),
         "dh": (avg([2 * B * fan[l] * fan[l + 1] for l in layers if l > 0]),
@@ -348,8 +351,6 @@ def run_ours(args):
     stream = torch.cuda.current_stream()
     now = [0]
 
-    expiry_beside_default = p.img_vocab >= (1 << 22)       # GearSession.step's own rule
-
     def one_step(db, expiry_beside=None):
         now[0] += 1
         sess.step(db, now[0], sync=False, expiry_beside=expiry_beside)
@@ -515,9 +516,8 @@ def run_ours(args):
                        "M": p.M, "expire": p.expire, "mean_nnz": round(stats["nnz"], 1),
                        "l2": "tables far exceed the 126 MB L2 and rows are Zipf-random; %d pre-generated batches cycle; "
                              "no explicit flush" % N_BATCHES,
-                       "streams": ("training calls on one stream, the expiry scan of the same step on a second one, "
-                                   "forked at the step's start and joined at its end (inside the timed region)")
-                       if expiry_beside_default else "all calls on one stream",
+                       "streams": "one call per step (gear_step); the library runs the ID sort, the weight gradients and the "
+                                  "expiry scan beside the rest and joins them at the step's end (inside the timed region)",
                        "outputs": "the averaged-gradient list (ids, seq, avg) and the expired-ID list of every step stay in "
                                   "device memory, where a Dense Part on the same GPU would consume them; the end-to-end arm "
                                   "reads back the loss and the two counts (24 bytes)",
