@@ -693,6 +693,7 @@ acc_atomic_add_kernel(const int32_t* __restrict__ img_id, int64_t n, int64_t voc
     const bool drop = state->q_count + n > ready_cap;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         state->pad[3] = drop ? 1 : 0;
+        state->n_copies = 0;
         if (drop) atomicOr(&state->status, GEAR_DEV_READY_OVERFLOW);
     }
     if (drop) return;
@@ -776,10 +777,17 @@ acc_atomic_add_kernel(const int32_t* __restrict__ img_id, int64_t n, int64_t voc
     if (flags) atomicOr(&state->status, flags);
 }
 
-// A warp takes 32 touched images: a lane settles the count of one, the warp together the rows of those that emit.
+// An image may emit one average many times (hot ones: a quarter of a call's rows / M).  The warp that settles it writes the first
+// SETTLE_COPIES; the others are written by a launch of their own, a warp per 32 of them.  (One warp wrote 25 thousand copies of the
+// hottest image's average: M = 1, 99.7 k rows, 569 us for the call.)
+constexpr int SETTLE_COPIES = 32;
+struct CopyList { uint32_t* src; uint32_t* first; uint32_t* count; };      // queue slots [first, first + count) repeat slot src
+
+// A warp takes 4 to 32 touched images, as few as the grid allows: a lane settles the count of one, the warp together the rows of
+// those that emit.
 __global__ void __launch_bounds__(256)
 acc_atomic_settle_kernel(const int32_t* __restrict__ touched, int D, const DivM div, float* __restrict__ gsum,
-                         int32_t* __restrict__ gcnt, int32_t* __restrict__ q_id, float* __restrict__ q_avg,
+                         int32_t* __restrict__ gcnt, int32_t* __restrict__ q_id, float* __restrict__ q_avg, const CopyList copies,
                          DevState* __restrict__ state) {
     wait_for_predecessor();
     if (state->pad[3] != 0) return;                            // the call was dropped
@@ -788,9 +796,10 @@ acc_atomic_settle_kernel(const int32_t* __restrict__ touched, int D, const DivM 
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     if (blockIdx.x == 0 && threadIdx.x == 0)                   // emission order is not ID order: collect has to sort
         atomicAdd(reinterpret_cast<unsigned long long*>(&state->q_calls), 2ull);
-    for (int64_t t0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; t0 < n_touched; t0 += warps * 32) {
+    const int per = (int)min((int64_t)32, max((int64_t)4, (n_touched + warps - 1) / warps));
+    for (int64_t t0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per; t0 < n_touched; t0 += warps * per) {
         int32_t id = 0, k = 0, e = 0, rest = 0;
-        if (t0 + lane < n_touched) {
+        if (lane < per && t0 + lane < n_touched) {
             id = touched[t0 + lane];
             k = gcnt[id] & ~ACC_TOUCHED;
             e = (int32_t)div((uint32_t)k);
@@ -810,14 +819,40 @@ acc_atomic_settle_kernel(const int32_t* __restrict__ touched, int D, const DivM 
             const int32_t id_l = __shfl_sync(0xffffffffu, id, l), e_l = __shfl_sync(0xffffffffu, e, l);
             const unsigned long long slot = slot0 + (__shfl_sync(0xffffffffu, incl, l) - (uint32_t)e_l);
             const float kf = (float)__shfl_sync(0xffffffffu, k, l), rf = (float)__shfl_sync(0xffffffffu, rest, l);
+            const int32_t here = min(e_l, SETTLE_COPIES);
             float* row = gsum + (int64_t)id_l * D;
             for (int ch = lane; ch < D / 4; ch += 32) {
                 const float4 sum = ld_f4(row + ch * 4);
                 const float4 avg = make_float4(sum.x / kf, sum.y / kf, sum.z / kf, sum.w / kf);
-                for (int32_t j = 0; j < e_l; ++j) st_f4(q_avg + (int64_t)(slot + j) * D + ch * 4, avg);
+                for (int32_t j = 0; j < here; ++j) st_f4(q_avg + (int64_t)(slot + j) * D + ch * 4, avg);
                 st_f4(row + ch * 4, make_float4(avg.x * rf, avg.y * rf, avg.z * rf, avg.w * rf));
             }
-            for (int32_t j = lane; j < e_l; j += 32) q_id[slot + j] = id_l;
+            if (lane < here) q_id[slot + lane] = id_l;
+            if (e_l > here) {
+                const uint32_t n_rec = (uint32_t)(e_l - here + 31) / 32u;
+                uint32_t at = 0;
+                if (lane == 0) at = atomicAdd(&state->n_copies, n_rec);
+                at = __shfl_sync(0xffffffffu, at, 0);
+                for (uint32_t r = lane; r < n_rec; r += 32) {
+                    copies.src[at + r] = (uint32_t)slot;
+                    copies.first[at + r] = (uint32_t)slot + (uint32_t)here + 32u * r;
+                    copies.count[at + r] = min(32u, (uint32_t)(e_l - here) - 32u * r);
+                }
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(256)
+acc_atomic_copy_kernel(int D, const CopyList copies, int32_t* __restrict__ q_id, float* __restrict__ q_avg, const DevState* __restrict__ state) {
+    wait_for_predecessor();
+    const uint32_t n = state->n_copies, lane = lane_id();
+    for (uint32_t r = blockIdx.x * 8 + (threadIdx.x >> 5); r < n; r += gridDim.x * 8) {
+        const uint32_t src = copies.src[r], first = copies.first[r], count = copies.count[r];
+        if (lane < count) q_id[first + lane] = q_id[src];
+        for (int ch = (int)lane; ch < D / 4; ch += 32) {
+            const float4 v = ld_f4(q_avg + (int64_t)src * D + ch * 4);
+            for (uint32_t j = 0; j < count; ++j) st_f4(q_avg + (int64_t)(first + j) * D + ch * 4, v);
         }
     }
 }
@@ -828,6 +863,9 @@ cudaError_t launch_accumulate_atomic(const gear_ctx_impl& c, const int32_t* img_
     if (n <= 0) return cudaSuccess;
     DevState* state = c.state();
     int32_t* touched = c.at<int32_t>(c.ws.pmeta);               // the sorted path's scratch is free in this mode
+    // (at most n emissions, so far fewer records than the sort buffers, which this mode does not use, have words)
+    const SortJob free_buffers = c.sort_job(gear_ctx_impl::SORT_IMG);
+    const CopyList copies{free_buffers.keys[0], free_buffers.vals[0], free_buffers.keys[1]};
     cudaError_t e = enqueue_memset(&state->pad[2], sizeof(int64_t), st);
     if (e != cudaSuccess) return e;
     const int resident = sm_count() * 8;
@@ -839,7 +877,13 @@ cudaError_t launch_accumulate_atomic(const gear_ctx_impl& c, const int32_t* img_
     // at most n images are touched; a warp that finds nothing to do costs nothing, so the grid follows n
     { KernelScope k(&c.prof, "acc_atomic_settle", st);
     e = launch_dependent(acc_atomic_settle_kernel, grid(ceil_div(n, 256)), dim3(256), 0, st, touched, c.cfg.dfv_dim, make_div(c.cfg.M), c.buf.dfv_gsum, c.buf.dfv_gcnt,
-                         c.at<int32_t>(c.ws.q_id), c.at<float>(c.ws.q_avg), state); }
+                         c.at<int32_t>(c.ws.q_id), c.at<float>(c.ws.q_avg), copies, state); }
+    if (e != cudaSuccess) return e;
+    if ((n + c.cfg.M - 1) / c.cfg.M > SETTLE_COPIES) {          // else no image can emit more than the settle pass writes
+        KernelScope k(&c.prof, "acc_atomic_copy", st);
+        e = launch_dependent(acc_atomic_copy_kernel, grid(ceil_div(n, (int64_t)c.cfg.M * 256)), dim3(256), 0, st, c.cfg.dfv_dim, copies,
+                             c.at<int32_t>(c.ws.q_id), c.at<float>(c.ws.q_avg), (const DevState*)state);
+    }
     if (e != cudaSuccess) return e;
     c.acc_calls_pending += 2;
     return cudaGetLastError();

@@ -27,7 +27,7 @@ struct DevState {
     int64_t pad0;
     int64_t collect_n;     // collect_ready: entries moved by the running call
     unsigned long long grid_barrier;   // arrival counter of the cooperative sort's grid barrier
-    unsigned int pad1;
+    unsigned int n_copies; // order-free store: records of repeated averages still to be written
     unsigned int pad32;                // blocks of a solo collect_move_kernel that have finished (wraps to 0)
     int64_t q_calls;       // accumulate calls that added to the ready queue since the last collect
     int64_t sort_n;        // collect_ready: entries the queue sort has to order (0: the queue is already in order)
