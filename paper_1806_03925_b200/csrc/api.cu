@@ -563,6 +563,10 @@ int gear_step(gear_ctx* ctx, const gear_batch* batch, float lr, const gear_step_
     gear_ctx_impl& c = ctx->impl;
     if (int rc = check_batch(c, *batch, *out)) return rc;
     if (!out->row_view || !out->inv_n) return arg_fail("gear_step needs row_view and inv_n");
+    if (batch->B == 0 && batch->nnz > 0) {          // as gear_accumulate_collect behind gear_forward_backward: there are no rows to add
+        snprintf(g_last_error, sizeof(g_last_error), "image occurrences without page views");
+        return GEAR_ERR_STATE;
+    }
     if (int rc = check_lists(lists->ids, lists->seq, lists->avg, lists->cap)) return rc;
     if (lists->expired_cap < 0 || (lists->expired_cap > 0 && !lists->expired)) return arg_fail("NULL output with cap > 0");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -694,6 +698,7 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
         const gear_host_batch& b = batches[s];
         if (b.B < 0 || b.B > p.max_batch || b.nnz < 0 || b.nnz > p.max_nnz) return arg_fail("a batch is larger than the plan's");
         if ((b.B > 0 && (!b.user_id || !b.url_id || !b.img_off || !b.label)) || (b.nnz > 0 && !b.img_id)) return arg_fail("NULL batch array");
+        if (b.B == 0 && b.nnz > 0) return arg_fail("image occurrences without page views");
         const gear_step_out& out = p.out[s];
         if (!out.dfv_grad || out.dX != p.out[0].dX + (int64_t)s * p.max_batch * w.d_in ||
             out.dfv_grad != p.out[0].dfv_grad + (int64_t)s * p.max_nnz * g0->dfv_dim)

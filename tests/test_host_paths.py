@@ -1,0 +1,138 @@
+"""Host code of libgear without a GPU: the library's own objects, linked against a stand-in for the CUDA runtime
+(fake_cudart.cpp) that writes down what is enqueued and can make a chosen call fail.  What the kernels compute is not tested here."""
+import ctypes as C
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+STREAM = 0x5000                  # the caller's stream
+
+
+class Host:
+    """The linked library, and contexts on addresses that nothing ever reads."""
+
+    def __init__(self, lib, gb):
+        self.lib, self.gb = lib, gb
+        lib.fake_unfinished.restype = C.c_int
+        lib.fake_calls.restype = lib.fake_live.restype = lib.fake_log.restype = C.c_long
+        lib.fake_fail_at.argtypes = [C.c_long]
+        lib.fake_user_capture.argtypes = [C.c_void_p, C.c_int]
+        self.next = 1 << 40
+        self.keep = []
+
+    def address(self, n=1 << 24):
+        self.next += n
+        return self.next - n
+
+    def log(self):
+        buf = C.create_string_buffer(1 << 20)
+        assert self.lib.fake_log(buf, len(buf)) >= 0
+        return [line.split() for line in buf.value.decode().splitlines()]
+
+    def ctx(self, batch=64, nnz=512, hidden=(64,), head=0, M=4, mode=0, img_vocab=1000, max_batch=None, max_nnz=None):
+        gb = self.gb
+        cfg = gb.make_config(1000, 1000, img_vocab, 16, 64, 0, head, list(hidden), M, 10, max_batch or batch, max_nnz or nnz, 0, mode)
+        words = C.c_size_t()
+        assert self.lib.gear_workspace_bytes(C.byref(cfg), C.byref(words)) == 0
+        b = gb.gear_buffers()
+        for name in ("user_emb", "url_emb", "dfv", "dfv_gsum", "dfv_gcnt", "dfv_ts", "head_params"):
+            setattr(b, name, self.address())
+        b.workspace, b.workspace_bytes = self.address(1 << 34), words.value
+        out = C.c_void_p()
+        assert self.lib.gear_init_tables(C.byref(out), C.byref(cfg), C.byref(b), 0, 0, 0, STREAM) == 0
+        return out
+
+    def out(self, **more):
+        o = self.gb.gear_step_out()
+        for name in ("loss", "prob", "head_grad", "dX", "row_view", "inv_n"):
+            setattr(o, name, self.address())
+        for name, v in more.items():
+            setattr(o, name, v)
+        return o
+
+    def lists(self, cap=512):
+        s = self.gb.gear_step_lists()
+        for name in ("ids", "seq", "avg", "d_n", "expired"):
+            setattr(s, name, self.address())
+        s.d_expired, s.cap, s.expired_cap = s.d_n + 8, cap, 1000
+        return s
+
+    def shard(self, world=2, batch=64, nnz=512, arrivals=100, head=0):
+        """A plan, its batches (host arrays), the contexts; `arrivals` is what every owner finds in the staging buffer's counts."""
+        gb, lib = self.gb, self.lib
+        owners = [self.ctx(batch * world, nnz * world, head=head, img_vocab=100_000) for _ in range(world)]
+        workers = [self.ctx(batch, nnz, head=head, mode=gb.GEAR_ACC_ATOMIC) for _ in range(world)]
+        words = C.c_int64()
+        assert lib.gear_shard_stage_words(world, batch, nnz, C.byref(words)) == 0
+        stage = (C.c_int32 * words.value)(*([arrivals] * words.value))
+        dX, rows = self.address(), self.address(1 << 30)
+        outs = (gb.gear_step_out * world)(*(self.out(dX=dX + 4 * s * batch * 96, dfv_grad=rows + 4 * s * nnz * 64) for s in range(world)))
+        lists = (gb.gear_step_lists * world)(*(self.lists(nnz * world) for _ in range(world)))
+        ctxs = [(C.c_void_p * world)(*(c.value for c in side)) for side in (owners, workers)]
+        plan = gb.gear_shard_plan(world, batch, nnz, ctxs[0], ctxs[1], C.addressof(stage), self.address(1 << 30), self.address(), outs, lists)
+        batches = (gb.gear_host_batch * world)()
+        zeros = (C.c_int32 * (batch + nnz))()
+        for b in batches:
+            b.B, b.nnz = batch, nnz
+            for name in ("user_id", "url_id", "img_off", "img_id", "label"):
+                setattr(b, name, C.addressof(zeros))
+        self.keep += [stage, outs, lists, ctxs, zeros]
+        return plan, batches, owners + workers
+
+    def shard_step(self, plan, batches, now=1, mean=1):
+        counts = (C.c_int64 * (2 * plan.world))()
+        return self.lib.gear_shard_step(C.byref(plan), batches, 0.1, now, mean, counts, STREAM)
+
+    def batch(self, B=64, nnz=200):
+        b = self.gb.gear_batch()
+        for name in ("user_id", "url_id", "img_off", "img_id", "label"):
+            setattr(b, name, self.address())
+        b.B, b.nnz = B, nnz
+        return b
+
+
+@pytest.fixture(scope="module")
+def linked(tmp_path_factory):
+    from paper_1806_03925_b200 import binding, build
+    build.build()
+    d = tmp_path_factory.mktemp("host")
+    so = str(d / "libgear_host.so")
+    objs = [os.path.join(build.BUILD, os.path.basename(s)[:-3] + ".o") for s in build.sources()]
+    cuda = os.path.dirname(os.path.dirname(build._nvcc()))
+    subprocess.check_call(["g++", "-std=c++17", "-O1", "-w", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", os.path.join(cuda, "include"),
+                           os.path.join(ROOT, "tests", "fake_cudart.cpp")] + objs + ["-o", so])
+    lib_path, lib = binding.LIB_PATH, binding._lib
+    try:                                                         # the binding's prototypes, on the linked library
+        binding.LIB_PATH, binding._lib = so, None
+        return binding.load(), binding
+    finally:
+        binding.LIB_PATH, binding._lib = lib_path, lib
+
+
+@pytest.fixture()
+def host(linked):
+    linked[0].fake_reset()
+    return Host(*linked)
+
+
+def test_image_occurrences_without_page_views_are_refused(host):
+    """A batch of no views with image IDs: the occurrences' rows exist nowhere.  Refused before anything is enqueued."""
+    gb = host.gb
+    for mode in (gb.GEAR_ACC_SORT, gb.GEAR_ACC_ATOMIC):
+        ctx = host.ctx(mode=mode)
+        host.log()
+        rc = host.lib.gear_step(ctx, host.batch(B=0, nnz=5), 0.1, host.out(), host.lists(), 1, 1, 1, None, STREAM)
+        assert rc == gb.GEAR_ERR_STATE and host.log() == []
+        assert host.lib.gear_step(ctx, host.batch(B=0, nnz=0), 0.1, host.out(), host.lists(), 1, 1, 1, None, STREAM) == 0
+        assert host.lib.gear_destroy(ctx) == 0
+    plan, batches, ctxs = host.shard()
+    assert host.shard_step(plan, batches) == 0
+    host.log()
+    batches[1].B = 0
+    assert host.shard_step(plan, batches) == gb.GEAR_ERR_ARG and host.log() == []
+    batches[1].nnz = 0
+    assert host.shard_step(plan, batches) == 0
+    for c in ctxs:
+        assert host.lib.gear_destroy(c) == 0
