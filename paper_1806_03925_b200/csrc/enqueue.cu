@@ -160,6 +160,9 @@ cudaError_t Player::play(OpList& l, Profiler* prof) {
     if (l.ops.empty()) return cudaSuccess;
     if (prof && prof->on) return direct(l, prof);
     if (l.n_kernels < MIN_KERNELS) return direct(l, prof);
+    // a stream that its owner is capturing is left to the owner's graph (the legacy default stream cannot be captured)
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (l.streams[0] && (cudaStreamIsCapturing(l.streams[0], &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) return direct(l, prof);
     Entry* e = nullptr;
     for (Entry& x : entry_)
         if (x.seen && same_shape(x.last, l)) { e = &x; break; }
@@ -170,10 +173,7 @@ cudaError_t Player::play(OpList& l, Profiler* prof) {
     }
     e->used = ++clock_;
     if (!e->exec) {
-        // a stream that its owner is capturing is left to the owner's graph
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        if (++e->seen <= GRAPH_AFTER || (l.streams[0] && (cudaStreamIsCapturing(l.streams[0], &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)) ||
-            !build(*e, l)) {
+        if (++e->seen <= GRAPH_AFTER || !build(*e, l)) {
             const cudaError_t r = direct(l, prof);
             if (!e->seen) e->seen = 1;
             std::swap(e->last, l);

@@ -3,7 +3,7 @@
 // A call first writes down what it wants enqueued -- kernels with their arguments, memsets, copies, events between
 // streams -- in an OpList, and the list is then played.  Played directly, every entry is one runtime call (about 2 us each:
 // a step of 20 kernels on three streams cost the host 80 us, more than the GPU needs for a few thousand views).  A list whose
-// shape (which kernels, on which streams, in which order) has come up GRAPH_AFTER times in a row is captured into a
+// shape (which kernels, on which streams, in which order) has come up GRAPH_AFTER times, in a row or not, is captured into a
 // CUDA graph once; from then on a call compares its entries with those of the call before, sets the parameters of the
 // nodes that differ (pointers, sizes, grids of a new batch) and launches the graph with one call.
 #pragma once

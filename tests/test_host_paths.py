@@ -136,3 +136,30 @@ def test_image_occurrences_without_page_views_are_refused(host):
     assert host.shard_step(plan, batches) == 0
     for c in ctxs:
         assert host.lib.gear_destroy(c) == 0
+
+
+def _store_call(host, ctx, n=40_001, ids=None, grads=None):
+    lists = host.lists(cap=n)
+    return host.lib.gear_accumulate_collect(ctx, ids or host.address(), grads or host.address(), 64, None, None, n, lists.ids, lists.seq,
+                                            lists.avg, n, lists.d_n, None, STREAM)
+
+
+def test_a_capturing_stream_gets_kernels_also_of_a_shape_with_a_graph(host):
+    """Its owner's graph holds the call's own kernels, and the call's graph is left as it was."""
+    ctx = host.ctx(nnz=50_000, max_nnz=50_000)
+    kernels = []
+    for call in range(6):
+        host.log()
+        assert _store_call(host, ctx) == 0
+        seen = [line[0] for line in host.log()]
+        assert ("graph" in seen) == (call >= 3), (call, seen)
+    host.lib.fake_user_capture(STREAM, 1)
+    assert _store_call(host, ctx) == 0
+    host.lib.fake_user_capture(None, 0)
+    log = host.log()
+    assert all(line[0] == "node" and line[1] == "%x" % STREAM for line in log), log
+    kernels = [line[2] for line in log]
+    assert len(kernels) == 4 and "coop_sort_kernel" in kernels[0] and "acc_reduce_kernel" in kernels[3]
+    assert _store_call(host, ctx) == 0
+    assert [line[0] for line in host.log()].count("graph") == 1
+    assert host.lib.gear_destroy(ctx) == 0
