@@ -583,7 +583,7 @@ static cudaError_t launch_accumulate_to(const gear_ctx_impl& c, const int32_t* i
         batch.name = "sort_img";
         planned = sort_small_fits(batch);
         if (planned) { se = launch_sort_small(c, batch, plan_args(c, n, src_row, scale), st); cur = 0; }
-        else cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
+        else cur = sort_jobs(batch, st, &c.prof, &se);
         if (se != cudaSuccess) return se;
         c.img_sort_valid = resort_batch;
         if (resort_batch) c.img_sorted_buf = cur;
@@ -992,7 +992,7 @@ cudaError_t launch_collect_ready(const gear_ctx_impl& c, int32_t* ids, int32_t* 
             batch.job[0].n_max = n_max;
             batch.job[0].n_dev = &state->sort_n;
             batch.name = "sort_ready";
-            cur = sort_jobs(batch, &c.gbs, st, &c.prof, &e);
+            cur = sort_jobs(batch, st, &c.prof, &e);
             if (e != cudaSuccess) return e;
         }
     }

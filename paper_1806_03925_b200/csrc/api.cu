@@ -248,7 +248,7 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
         }
         batch.name = "sort_ids";
         small_sort = batch.n_jobs > 0 && sort_small_fits(batch);
-        if (batch.n_jobs > 0 && !small_sort) sorted_buf = sort_jobs(batch, &c.gbs, side, &c.prof, &e);
+        if (batch.n_jobs > 0 && !small_sort) sorted_buf = sort_jobs(batch, side, &c.prof, &e);
         if (e != cudaSuccess) return e;
         if (b.nnz > 0) {
             c.img_sorted = true; c.img_sorted_n = b.nnz; c.img_sorted_buf = sorted_buf; c.last_img_id = b.img_id;
@@ -370,7 +370,7 @@ static cudaError_t enqueue_owner_plan(gear_ctx_impl& c, const Arrivals& user, co
     if (small_sort) GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, img.n, nullptr, nullptr) : PlanArgs{}, st));
     else if (batch.n_jobs > 0) {
         cudaError_t se;
-        *sorted_buf = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
+        *sorted_buf = sort_jobs(batch, st, &c.prof, &se);
         if (se != cudaSuccess) return se;
     }
     if (plan) {
@@ -419,11 +419,9 @@ static void forget_batch(gear_ctx_impl& c) {
 // Writes a call down and plays it.
 template <typename Fn> static int run_call(gear_ctx_impl& c, const char* where, cudaStream_t st, Fn&& enqueue) {
     c.last_stream = st;
-    const unsigned long long base = c.gbs.host_base;
     Recording rec(c.player, st);
     cudaError_t e = enqueue();
-    if (e != cudaSuccess) c.gbs.host_base = base;            // nothing has been enqueued
-    else e = rec.play(&c.prof);
+    if (e == cudaSuccess) e = rec.play(&c.prof);             // (else nothing has been enqueued)
     if (e == cudaSuccess) return GEAR_OK;
     forget_batch(c);
     return cuda_fail(e, where);
@@ -475,8 +473,6 @@ int gear_init_tables(gear_ctx** out_ctx, const gear_config* cfg, const gear_buff
     c.alive = true;
     c.tma = new_tma_cache();
     if (!c.tma) { delete ctx; return arg_fail("out of host memory"); }
-    c.gbs.device_counter = &c.state()->grid_barrier;
-    c.gbs.host_base = 0;
     c.img_sorted = false;
     c.img_sort_valid = false;
     c.img_sorted_n = 0;
@@ -757,16 +753,10 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
         r.table[t].src_stride = t < 2 ? p.max_batch : p.max_nnz;
     }
     gear_ctx_impl &w0 = p.workers[0]->impl, &o0 = p.owners[0]->impl;
-    unsigned long long base[2 * GEAR_MAX_LOCAL_RANKS];
-    for (int s = 0; s < W; ++s) {
-        base[2 * s] = p.workers[s]->impl.gbs.host_base; base[2 * s + 1] = p.owners[s]->impl.gbs.host_base;
-        p.workers[s]->impl.last_stream = p.owners[s]->impl.last_stream = st;
-    }
-    auto fail = [&](cudaError_t err, bool enqueued) {
-        for (int s = 0; s < W; ++s) {
-            if (!enqueued) { p.workers[s]->impl.gbs.host_base = base[2 * s]; p.owners[s]->impl.gbs.host_base = base[2 * s + 1]; }
+    for (int s = 0; s < W; ++s) p.workers[s]->impl.last_stream = p.owners[s]->impl.last_stream = st;
+    auto fail = [&](cudaError_t err) {
+        for (int s = 0; s < W; ++s)
             for (gear_ctx_impl* c : {&p.workers[s]->impl, &p.owners[s]->impl}) forget_batch(*c);
-        }
         return cuda_fail(err, "shard_step");
     };
     enum { EV_RANKS = 8, EV_ROUTED = 9 };
@@ -787,7 +777,7 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
     else if (e == cudaSuccess) e = cudaMemsetAsync(r.counts, 0, sizeof(int32_t) * 3 * W, early);
     if (e == cudaSuccess) e = cudaMemcpyAsync(p.host_stage + at.counts, r.counts, sizeof(int32_t) * 3 * W, cudaMemcpyDeviceToHost, early);
     if (e == cudaSuccess) e = cudaEventRecord(w0.ev[EV_ROUTED], early);
-    if (e != cudaSuccess) return fail(e, true);
+    if (e != cudaSuccess) return fail(e);
     auto stream_of = [&](int s) { return s == 0 ? st : p.owners[s]->impl.rank_stream; };
 #define GEAR_TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return e_; } while (0)
     // ---- events 1 to 4 on the workers, side by side
@@ -810,11 +800,11 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
             }
             return cudaSuccess;
         }();
-        if (e != cudaSuccess) return fail(e, false);
+        if (e != cudaSuccess) return fail(e);
         e = rec.play(&w0.prof);
     }
     if (e == cudaSuccess) e = cudaEventSynchronize(w0.ev[EV_ROUTED]);
-    if (e != cudaSuccess) return fail(e, true);
+    if (e != cudaSuccess) return fail(e);
     // ---- events 4 (push), 5 and 6 at the owners, side by side
     Arrivals arrived[GEAR_MAX_LOCAL_RANKS][3];
     int sorted_buf[GEAR_MAX_LOCAL_RANKS] = {};
@@ -847,10 +837,10 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
             return enqueue_owner_apply(c, arrived[s][0], arrived[s][1], arrived[s][2], sorted_buf[s], p.out[0].dX, w0.d_in, p.out[0].dfv_grad,
                                        g0->dfv_dim, lr, p.lists[s], where);
         });
-    if (e != cudaSuccess) return fail(e, true);
+    if (e != cudaSuccess) return fail(e);
 #undef GEAR_TRY
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return fail(e, true);
+    if (e != cudaSuccess) return fail(e);
     int rc = GEAR_OK;
     for (int s = 0; s < W; ++s) {
         const gear_ctx_impl& c = p.owners[s]->impl;
@@ -908,11 +898,6 @@ int gear_status(gear_ctx* ctx, int32_t* device_status, int64_t* pending_ready) {
     if (e != cudaSuccess) return cuda_fail(e, "gear_status");      // h holds nothing to look at
     if (h.tc_error != 0) h.status |= GEAR_DEV_TIMEOUT;
     if (e == cudaSuccess && h.status != 0) e = cudaMemset(c.state(), 0, 2 * sizeof(int32_t));   // status, tc_error
-    if (e == cudaSuccess && h.tc_error != 0) {
-        // an abandoned grid barrier leaves its arrival counter short: start the count again
-        e = cudaMemset(&c.state()->grid_barrier, 0, sizeof(unsigned long long));
-        c.gbs.host_base = 0;
-    }
     if (e != cudaSuccess) return cuda_fail(e, "gear_status");
     if (device_status) *device_status = h.status;
     if (pending_ready) *pending_ready = h.q_count;

@@ -26,7 +26,8 @@ struct DevState {
     int64_t plan_base;     // accumulate: length of the ready queue that the plan goes by
     int64_t pad0;
     int64_t collect_n;     // collect_ready: entries moved by the running call
-    unsigned long long grid_barrier;   // arrival counter of the cooperative sort's grid barrier
+    unsigned int barrier_arrived;      // the cooperative sort's grid barrier: arrivals; blocks that have left the launch
+    unsigned int barrier_left;         // (both zero between launches)
     unsigned int n_copies; // order-free store: records of repeated averages still to be written
     unsigned int pad32;                // blocks of a solo collect_move_kernel that have finished (wraps to 0)
     int64_t q_calls;       // accumulate calls that added to the ready queue since the last collect
@@ -277,21 +278,14 @@ struct SortBatch {
     SortJob job[3];
     int n_jobs;
     const char* name;                 // host only: the name the launch is timed under
-    int passes, n_barriers;           // filled in by sort_jobs
-    unsigned long long* barrier_ctr;  // filled in by sort_jobs
-    unsigned long long barrier_base;
+    int passes;                       // filled in by sort_jobs
+    unsigned int* barrier;            // two device words, zero before and after every launch: arrivals, blocks that have left
     int32_t* err;                     // device word that receives a non-zero code when a grid barrier gives up
-};
-
-// Arrival counter of the grid barrier (device) and what all launches so far will have added to it (host).
-struct GridBarrierState {
-    unsigned long long* device_counter;
-    unsigned long long host_base;
 };
 
 // Sorts every job of the batch in one cooperative launch.  Returns the index (0 or 1) of the keys/vals
 // buffer pair that holds the sorted result of every job.
-int sort_jobs(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st, Profiler* prof, cudaError_t* err_out);
+int sort_jobs(SortBatch& batch, cudaStream_t st, Profiler* prof, cudaError_t* err_out);
 
 inline int bits_for(int64_t max_key_inclusive) {
     int b = 1;

@@ -165,7 +165,7 @@ cudaError_t launch_apply_emb_grad(const gear_ctx_impl& c, int which, const int32
     cudaError_t se;
     int cur = 0;
     if (sort_small_fits(batch)) se = launch_sort_small(c, batch, PlanArgs{}, st);
-    else cur = sort_jobs(batch, &c.gbs, st, &c.prof, &se);
+    else cur = sort_jobs(batch, st, &c.prof, &se);
     if (se != cudaSuccess) return se;
     const EmbTable t{batch.job[0].keys[cur], batch.job[0].vals[cur], (uint32_t)vocab, (int)n, rows, ld, user ? c.buf.user_emb : c.buf.url_emb};
     EmbTable none = t;

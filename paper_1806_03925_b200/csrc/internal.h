@@ -79,7 +79,6 @@ struct gear_ctx_impl {
     int64_t* h_counts;                 // two counts on their way to the caller (pinned)
     Player player;                     // plays what a call has written down
     mutable Profiler prof;
-    mutable GridBarrierState gbs;
     mutable int plan_sections_dirty = 0;    // section counts a plan has added to and no reduce pass has cleared yet
     mutable int expiry_set = 0;             // which set of section counts the last expiry scan used
     // image IDs of the last gear_forward_backward batch, already sorted (reused by gear_accumulate_dfv_grad)
@@ -112,6 +111,7 @@ struct gear_ctx_impl {
     }
     SortBatch sort_batch() const {
         SortBatch b{};
+        b.barrier = &state()->barrier_arrived;
         b.err = &state()->tc_error;
         return b;
     }

@@ -13,10 +13,10 @@
 // separate key-building launch is needed.  Arrays whose live size (known only on the device) fits a few
 // tiles are sorted by block 0 alone, with block-level barriers only.
 //
-// The grid barrier is a monotonically increasing 64-bit arrival counter: barrier k of a launch completes
-// when the counter reaches base + grid * (k + 1), where the host knows `base` (it adds up what every
-// earlier launch contributes).  The kernel is launched cooperatively, so all blocks are resident; the spin is bounded all
-// the same, and a block that gives up records an error and makes every later wait of the launch fall through.
+// The grid barrier is an arrival counter: barrier k of a launch completes when it reaches grid * (k + 1); the last block to
+// leave the launch puts it back to zero, so that a launch needs nothing from the host and may be replayed.  The kernel is
+// launched cooperatively, so all blocks are resident; the spin is bounded all the same, and a block that gives up records an
+// error and makes every later wait of the launch fall through.
 #include <type_traits>
 
 #include "common.cuh"
@@ -32,15 +32,15 @@ __device__ __forceinline__ int64_t effective_n(int64_t n_max, const int64_t* n_d
 }
 
 // All threads of every participating block call this.  Returns false once the launch has been abandoned.
-__device__ __forceinline__ bool grid_barrier(unsigned long long* ctr, unsigned long long target, int32_t* err) {
+__device__ __forceinline__ bool grid_barrier(unsigned int* ctr, unsigned int target, int32_t* err) {
     __shared__ int ok_flag;
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
         __threadfence();
-        atomicAdd(ctr, 1ull);
+        atomicAdd(ctr, 1u);
         uint32_t spin = 0;
-        while (*reinterpret_cast<volatile unsigned long long*>(ctr) < target) {
+        while (*reinterpret_cast<volatile unsigned int*>(ctr) < target) {
             if (++spin > GRID_SPIN_LIMIT) { atomicCAS(err, 0, 100); ok = 0; break; }
             if ((spin & 1023u) == 1023u && *reinterpret_cast<volatile int32_t*>(err) != 0) { ok = 0; break; }
         }
@@ -261,27 +261,25 @@ coop_sort_kernel(const SortBatch batch) {
     int64_t live_tiles = 0;
     for (int q = 0; q < batch.n_jobs; ++q) live_tiles += ceil_div(live_n[q], TILE);
     if (live_tiles <= RS_SOLO_TILES) {
-        // a few tiles in all: block 0 sorts everything without a grid barrier (and advances the arrival counter on behalf of all)
+        // a few tiles in all: block 0 sorts everything without a grid barrier
         if (blockIdx.x != 0) return;
         for (int q = 0; q < batch.n_jobs; ++q)
             if (live_n[q] > 0) {
                 __syncthreads();
                 sort_job<ITEMS, KEYS>(batch.job[q], live_n[q], batch.passes, 0, 1, dyn, scratch, [] { __syncthreads(); return true; });
             }
-        if (threadIdx.x == 0) {
-            // the host has already booked this launch's arrivals: deliver them
-            __threadfence();
-            atomicAdd(batch.barrier_ctr, (unsigned long long)gridDim.x * (unsigned long long)batch.n_barriers);
-        }
         return;
     }
-    unsigned long long target = batch.barrier_base;
+    unsigned int target = 0;             // at most 512 blocks * 12 barriers
     int q = 0;
     while (q + 1 < batch.n_jobs && (int)blockIdx.x >= batch.job[q + 1].block0) ++q;
     sort_job<ITEMS, KEYS>(batch.job[q], live_n[q], batch.passes, (int)blockIdx.x - batch.job[q].block0, batch.job[q].n_blocks, dyn, scratch, [&]() -> bool {
         target += gridDim.x;
-        return grid_barrier(batch.barrier_ctr, target, batch.err);
+        return grid_barrier(batch.barrier, target, batch.err);
     });
+    // nobody arrives or looks any more once all have come here (a block that gave up too): the counts start again from zero
+    __syncthreads();
+    if (threadIdx.x == 0 && atomicInc(batch.barrier + 1, gridDim.x - 1) == gridDim.x - 1) batch.barrier[0] = 0u;
 }
 
 template <int ITEMS, int KEYS> static int coop_grid_limit() {
@@ -296,7 +294,7 @@ template <int ITEMS, int KEYS> static int coop_grid_limit() {
     return limit;
 }
 
-template <int ITEMS, int KEYS> static cudaError_t launch_sort(SortBatch& batch, int width, GridBarrierState* gbs, cudaStream_t st) {
+template <int ITEMS, int KEYS> static cudaError_t launch_sort(SortBatch& batch, int width, cudaStream_t st) {
     // every job gets blocks in proportion to its tiles, at least one and at most one per tile
     const int limit = coop_grid_limit<ITEMS, KEYS>();
     int64_t tiles[3], total = 0;
@@ -314,14 +312,10 @@ template <int ITEMS, int KEYS> static cudaError_t launch_sort(SortBatch& batch, 
     }
     if (grid > limit) { batch.job[big].n_blocks -= grid - limit; grid = limit; }      // (very small jobs beside a very large one)
     for (int j = 0, at = 0; j < batch.n_jobs; ++j) { batch.job[j].block0 = at; at += batch.job[j].n_blocks; }
-    batch.n_barriers = 3 * batch.passes - 1;            // per pass: counts, running totals, the next order
-    batch.barrier_ctr = gbs->device_counter;
-    batch.barrier_base = gbs->host_base;
-    gbs->host_base += (unsigned long long)grid * (unsigned long long)batch.n_barriers;
     return launch_as(Op::COOPERATIVE, coop_sort_kernel<ITEMS, KEYS>, dim3(grid), dim3(RS_THREADS), rs_smem_bytes<ITEMS>(width, KEYS), st, batch);
 }
 
-int sort_jobs(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st, Profiler* prof, cudaError_t* err_out) {
+int sort_jobs(SortBatch& batch, cudaStream_t st, Profiler* prof, cudaError_t* err_out) {
     int passes = 1;
     int64_t n = 0;
     for (int j = 0; j < batch.n_jobs; ++j) {
@@ -339,7 +333,7 @@ int sort_jobs(SortBatch& batch, GridBarrierState* gbs, cudaStream_t st, Profiler
     // smaller tiles while the larger ones would leave blocks idle
     auto launch = [&](auto keys) {
         constexpr int K = decltype(keys)::value;
-        return n <= (int64_t)RS_THREADS * 4 * coop_grid_limit<4, K>() ? launch_sort<4, K>(batch, width, gbs, st) : launch_sort<8, K>(batch, width, gbs, st);
+        return n <= (int64_t)RS_THREADS * 4 * coop_grid_limit<4, K>() ? launch_sort<4, K>(batch, width, st) : launch_sort<8, K>(batch, width, st);
     };
     *err_out = rs_keys(width) == 2 ? launch(std::integral_constant<int, 2>{}) : launch(std::integral_constant<int, 1>{});
     return passes & 1;

@@ -186,3 +186,48 @@ def test_dense_forward_at_tile_edges(n, R, D):
         np.testing.assert_allclose(rows.cpu().numpy(), want, rtol=0, atol=R * R * 2.0 ** -24)
     finally:
         s.close()
+
+
+def _replays(call, *sessions):
+    """The call captured on its owner's graph, as a function that replays it."""
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        call()
+    return g.replay
+
+
+# one cluster's sort, the multi-block sort with its grid barrier
+@pytest.mark.parametrize("n,vocab", [(1000, 500), (40_001, 60_000)])
+def test_a_captured_store_call_can_be_replayed(n, vocab):
+    """Replays with new rows, other calls between them, against the same calls one by one: the order of a sum is fixed, so the
+    results are the same numbers."""
+    M, D = 3, 8
+    a, c = (_store_session(vocab, D, M, n) for _ in range(2))
+    try:
+        ids, rows = torch.zeros(n, dtype=torch.int32, device="cuda"), torch.zeros((n, D), device="cuda")
+
+        def fresh(seed):
+            ids.copy_(torch.from_numpy(_ids(vocab, n, seed)))
+            rows.copy_(torch.from_numpy(np.random.default_rng(seed).uniform(-1, 1, (n, D)).astype(np.float32)))
+        fresh(0)
+        for k in range(5):                                   # past the point where the call has a graph of its own
+            for s in (a, c):
+                s.accumulate_collect_rows(ids, rows)
+        replay = _replays(lambda: a.accumulate_collect_rows(ids, rows, sync=False))
+        for k in range(1, 7):
+            fresh(k)
+            if k % 3 == 0:
+                a.accumulate_collect_rows(ids, rows)
+            else:
+                replay()
+            want = c.accumulate_collect_rows(ids, rows)
+            torch.cuda.synchronize()
+            assert int(a.d_counts[0]) == want, k
+            for name in ("ready_ids", "ready_seq", "ready_avg"):
+                assert torch.equal(getattr(a, name)[:want], getattr(c, name)[:want]), (k, name)
+            assert torch.equal(a.dfv_gcnt, c.dfv_gcnt) and torch.equal(a.dfv_gsum, c.dfv_gsum), k
+        assert a.status()[1] & ~1 == 0                       # (the IDs out of range were noted)
+    finally:
+        a.close()
+        c.close()
