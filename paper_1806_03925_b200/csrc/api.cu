@@ -410,8 +410,10 @@ static cudaError_t enqueue_owner_apply(gear_ctx_impl& c, const Arrivals& user, c
 #undef GEAR_TRY
 }
 
-// The ctx forgets the batch whose order it may have been in the middle of.
+// After a call that failed: the ctx forgets the batch whose order it may have been in the middle of, and whatever else the call
+// may have left half done starts anew.
 static void forget_batch(gear_ctx_impl& c) {
+    c.scan_cut_off = true;
     c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
     c.plan_sections_dirty = (int)((c.ws.grp_rec - c.ws.plan_sections) / 8);
 }
@@ -621,7 +623,7 @@ int gear_collect_expired(gear_ctx* ctx, int64_t now, int restamp, int32_t* ids, 
     c.note_stream(st);             // may differ from the stream of the training calls: the scan shares nothing with them
     int64_t* d_cnt = d_n ? d_n : &c.state()->pad[1];
     cudaError_t e = launch_collect_expired(c, now, restamp, ids, cap, d_cnt, st);
-    if (e != cudaSuccess) return cuda_fail(e, "collect_expired");
+    if (e != cudaSuccess) { c.scan_cut_off = true; return cuda_fail(e, "collect_expired"); }
     return finish_count(c, d_cnt, cap, h_n, st);
 }
 

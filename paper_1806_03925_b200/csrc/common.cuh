@@ -24,7 +24,8 @@ struct DevState {
     int64_t direct_done;   // accumulate + collect as one call: 1 while the hand-over pass that follows has nothing to do
                            // (the reduce pass wrote the averages straight into the caller's lists)
     int64_t plan_base;     // accumulate: length of the ready queue that the plan goes by
-    int64_t pad0;
+    uint32_t scan_next;    // expiry scan: which set of section counts the next mark pass adds to (written by the write pass)
+    uint32_t scan_set;     // ... and which one the last mark pass added to (written by that pass)
     int64_t collect_n;     // collect_ready: entries moved by the running call
     unsigned int barrier_arrived;      // the cooperative sort's grid barrier: arrivals; blocks that have left the launch
     unsigned int barrier_left;         // (both zero between launches)

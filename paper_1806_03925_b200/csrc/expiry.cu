@@ -20,10 +20,12 @@ constexpr int EXP_MARK_ITEMS = EXP_MARK_TILE / EXP_THREADS;
 static_assert(EXP_TILE == EXP_THREADS * 32, "one bitmap word per thread in the write pass");
 static_assert(EXP_MARK_TILE % (EXP_THREADS * 1) == 0 && EXP_TILE % EXP_MARK_TILE == 0, "mark tiles nest in write tiles");
 
-// Per-tile counts, then the sections' counts twice over: a scan adds to one set and clears the other for the next scan.
+// Per-tile counts, then the sections' counts twice over: a scan adds to one set and clears the other for the next scan.  Which
+// set it is stands in the device state, so that a scan that is replayed, or was written down and never ran, leaves nothing
+// behind: the mark pass reads scan_next and notes it in scan_set, the write pass reads that and turns scan_next over.
 struct ExpiryCounts {
-    uint32_t* tile; uint32_t* section; uint32_t* section_next;
-    int64_t n_tiles;
+    uint32_t* tile; uint32_t* section;
+    int64_t n_tiles, n_sections;
 };
 constexpr int EXP_SECTION = 64;           // mark tiles per section
 
@@ -31,8 +33,9 @@ constexpr int EXP_SECTION = 64;           // mark tiles per section
 // block keeps its whole 16 KB tile in flight; the small tiles leave the balancing to the block scheduler.
 __global__ void __launch_bounds__(EXP_THREADS)
 expiry_mark_kernel(const int64_t* __restrict__ ts, int64_t vocab, int64_t now, int64_t expire,
-                   uint32_t* __restrict__ bits, const ExpiryCounts cnt) {
+                   uint32_t* __restrict__ bits, const ExpiryCounts cnt, DevState* __restrict__ state) {
     wait_for_predecessor();
+    const uint32_t set = state->scan_next & 1u;
     __shared__ uint32_t warp_cnt[EXP_THREADS / 32];
     const int64_t tile0 = (int64_t)blockIdx.x * EXP_MARK_TILE;
     const unsigned lane = lane_id(), warp = threadIdx.x >> 5;
@@ -61,8 +64,9 @@ expiry_mark_kernel(const int64_t* __restrict__ ts, int64_t vocab, int64_t now, i
 #pragma unroll
         for (int w = 0; w < EXP_THREADS / 32; ++w) total += warp_cnt[w];
         cnt.tile[blockIdx.x] = total;
-        if (total) atomicAdd(cnt.section + blockIdx.x / EXP_SECTION, total);
-        if (blockIdx.x % EXP_SECTION == 0) cnt.section_next[blockIdx.x / EXP_SECTION] = 0u;
+        if (total) atomicAdd(cnt.section + set * cnt.n_sections + blockIdx.x / EXP_SECTION, total);
+        if (blockIdx.x % EXP_SECTION == 0) cnt.section[(set ^ 1u) * cnt.n_sections + blockIdx.x / EXP_SECTION] = 0u;
+        if (blockIdx.x == 0) state->scan_set = set;
     }
 }
 
@@ -77,10 +81,10 @@ expiry_write_kernel(const uint32_t* __restrict__ bits, int64_t vocab, const Expi
     const int64_t w = (int64_t)blockIdx.x * EXP_THREADS + threadIdx.x;
     uint32_t word = (w * 32 < vocab) ? bits[w] : 0u;
     const int64_t my_tile = (int64_t)blockIdx.x * (EXP_TILE / EXP_MARK_TILE), my_section = my_tile / EXP_SECTION;
-    const int64_t sections = ceil_div(cnt.n_tiles, EXP_SECTION);
+    const uint32_t set = state->scan_set & 1u;
     uint32_t before = 0, after = 0;                         // this thread's share
-    for (int64_t s = threadIdx.x; s < sections; s += EXP_THREADS) {
-        const uint32_t v = cnt.section[s];
+    for (int64_t s = threadIdx.x; s < cnt.n_sections; s += EXP_THREADS) {
+        const uint32_t v0 = cnt.section[s], v1 = cnt.section[cnt.n_sections + s], v = set ? v1 : v0;     // (no load waits for `set`)
         if (s < my_section) before += v; else after += v;
     }
     const int64_t t = my_section * EXP_SECTION + threadIdx.x;
@@ -90,6 +94,7 @@ expiry_write_kernel(const uint32_t* __restrict__ bits, int64_t vocab, const Expi
     block_exclusive_scan(after, scratch, &n_after);
     const int64_t total = (int64_t)(n_before + n_after);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
+        state->scan_next = set ^ 1u;                        // the mark pass behind this one finds that set cleared
         if (d_n) *d_n = total;
         if (total > cap) atomicOr(&state->status, GEAR_DEV_OUT_CAPACITY);
     }
@@ -111,24 +116,29 @@ static cudaError_t enqueue_expiry_scan(int64_t* ts, int64_t vocab, int64_t expir
     const int64_t n_write = ceil_div(vocab, EXP_TILE);
     cudaError_t e;
     { KernelScope k(prof, "expiry_mark", st);
-    e = launch_dependent(expiry_mark_kernel, dim3((unsigned)cnt.n_tiles), dim3(EXP_THREADS), 0, st, ts, vocab, now, expire, bits, cnt); }
+    e = launch_dependent(expiry_mark_kernel, dim3((unsigned)cnt.n_tiles), dim3(EXP_THREADS), 0, st, ts, vocab, now, expire, bits, cnt, state); }
     if (e != cudaSuccess) return e;
     KernelScope k(prof, "expiry_write", st);
     return launch_dependent(expiry_write_kernel, dim3((unsigned)n_write), dim3(EXP_THREADS), 0, st, bits, vocab, cnt, cap, d_n, state, now,
                             restamp, ts, ids);
 }
 
-// counts: [n_tiles] tile counts, then two sets of section counts; the sections of `set` are zero before the scan
-static ExpiryCounts expiry_counts(uint32_t* counts, int64_t vocab, int set) {
-    const int64_t n = ceil_div(vocab, EXP_MARK_TILE), sections = ceil_div(n, EXP_SECTION);
-    return ExpiryCounts{counts, counts + n + set * sections, counts + n + (set ^ 1) * sections, n};
+// counts: [n_tiles] tile counts, then two sets of section counts; the set that scan_next names is zero before the scan
+static ExpiryCounts expiry_counts(uint32_t* counts, int64_t vocab) {
+    const int64_t n = ceil_div(vocab, EXP_MARK_TILE);
+    return ExpiryCounts{counts, counts + n, n, ceil_div(n, EXP_SECTION)};
 }
 
 cudaError_t launch_collect_expired(const gear_ctx_impl& c, int64_t now, int restamp, int32_t* ids, int64_t cap,
                                    int64_t* d_n, cudaStream_t st) {
-    c.expiry_set ^= 1;
+    const ExpiryCounts cnt = expiry_counts(c.at<uint32_t>(c.ws.exp_cnt), c.cfg.img_vocab);
+    if (c.scan_cut_off) {                                   // a mark pass may have run whose write pass did not
+        const cudaError_t e = enqueue_memset(cnt.section, 2 * sizeof(uint32_t) * (size_t)cnt.n_sections, st);
+        if (e != cudaSuccess) return e;
+        c.scan_cut_off = false;
+    }
     return enqueue_expiry_scan(c.buf.dfv_ts, c.cfg.img_vocab, c.cfg.expire, now, restamp, ids, cap, d_n, c.at<uint32_t>(c.ws.exp_bits),
-                               expiry_counts(c.at<uint32_t>(c.ws.exp_cnt), c.cfg.img_vocab, c.expiry_set), c.state(), &c.prof, st);
+                               cnt, c.state(), &c.prof, st);
 }
 
 }  // namespace gear
@@ -196,9 +206,9 @@ extern "C" int gear_collect_expired_static(int64_t* dfv_ts, int64_t img_vocab, i
 
     // the array keeps what the previous call left: the state block and the section counts have to start from zero, the
     // bitmap words and tile counts of this table size are all rewritten by the mark pass
-    const ExpiryCounts cnt = expiry_counts(counts, img_vocab, 0);
+    const ExpiryCounts cnt = expiry_counts(counts, img_vocab);
     if (enqueue_memset(state, STATIC_STATE_BYTES, st) != cudaSuccess) return GEAR_ERR_CUDA;
-    if (enqueue_memset(cnt.section, sizeof(uint32_t) * (size_t)ceil_div(cnt.n_tiles, EXP_SECTION), st) != cudaSuccess) return GEAR_ERR_CUDA;
+    if (enqueue_memset(cnt.section, sizeof(uint32_t) * (size_t)cnt.n_sections, st) != cudaSuccess) return GEAR_ERR_CUDA;
     int64_t* d_cnt = d_n ? d_n : &state->pad[1];
     if (enqueue_expiry_scan(dfv_ts, img_vocab, expire, now, restamp, ids, cap, d_cnt, bits, cnt, state, nullptr, st) !=
         cudaSuccess)

@@ -79,8 +79,8 @@ struct gear_ctx_impl {
     int64_t* h_counts;                 // two counts on their way to the caller (pinned)
     Player player;                     // plays what a call has written down
     mutable Profiler prof;
+    mutable bool scan_cut_off = false;      // a call failed: its expiry scan may have been enqueued in part
     mutable int plan_sections_dirty = 0;    // section counts a plan has added to and no reduce pass has cleared yet
-    mutable int expiry_set = 0;             // which set of section counts the last expiry scan used
     // image IDs of the last gear_forward_backward batch, already sorted (reused by gear_accumulate_dfv_grad)
     const int32_t* last_img_id;         // img_id array of that batch (the atomic mode reads it unsorted)
     bool img_sorted;

@@ -231,3 +231,32 @@ def test_a_captured_store_call_can_be_replayed(n, vocab):
     finally:
         a.close()
         c.close()
+
+
+def test_a_captured_expiry_scan_can_be_replayed():
+    """A scan adds to one of two sets of section counts (64 tiles of 2048 timestamps) and clears the other: replays, the same scan
+    over and over, with scans of a step's kind between them, against the timestamps on the host."""
+    from paper_1806_03925_b200.session import GearSession
+    V, T = 300_007, 5
+    p = PRESETS["tiny"].scaled(user_vocab=64, url_vocab=64, img_vocab=V, expire=T)
+    s = GearSession(p, workloads.head_params(p, 0), max_batch=8, max_nnz=32)
+    try:
+        replay = None
+        for k in range(8):
+            ts = np.random.default_rng(k).integers(-9, 10, V)
+            if k == 2:
+                replay = _replays(lambda: s.collect_expired(10, restamp=True, sync=False))
+            s.dfv_ts.copy_(torch.from_numpy(ts))
+            if k in (0, 1, 5):
+                s.collect_expired(10, restamp=True)
+            else:
+                replay()
+            torch.cuda.synchronize()
+            want = np.flatnonzero(10 - ts >= T)
+            assert int(s.d_counts[1]) == want.size, k
+            assert np.array_equal(s.expired_ids[:want.size].cpu().numpy(), want), k
+            ts[want] = 10
+            assert np.array_equal(s.dfv_ts.cpu().numpy(), ts), k
+        assert s.status()[1] == 0
+    finally:
+        s.close()

@@ -163,3 +163,20 @@ def test_a_capturing_stream_gets_kernels_also_of_a_shape_with_a_graph(host):
     assert _store_call(host, ctx) == 0
     assert [line[0] for line in host.log()].count("graph") == 1
     assert host.lib.gear_destroy(ctx) == 0
+
+
+def test_an_expiry_scan_that_was_cut_off_leaves_no_counts(host):
+    """A mark pass without its write pass: the next scan clears the counts first; one that ran whole costs nothing more."""
+    lib, ctx = host.lib, host.ctx()
+    scan = lambda: lib.gear_collect_expired(ctx, 1, 1, host.address(), 1000, host.address(), None, STREAM)
+    names = lambda: [("expiry_" + line[2].split("expiry_")[1].split("_")[0]) if line[0] == "launch" else line[0] for line in host.log()]
+    host.log()
+    assert scan() == 0 and scan() == 0
+    assert names() == ["expiry_mark", "expiry_write"] * 2
+    lib.fake_fail_at(2)
+    assert scan() == host.gb.GEAR_ERR_CUDA
+    lib.fake_fail_at(-1)
+    assert names() == ["expiry_mark", "FAIL"]
+    assert scan() == 0 and scan() == 0
+    assert names() == ["memset", "expiry_mark", "expiry_write", "expiry_mark", "expiry_write"]
+    assert lib.gear_destroy(ctx) == 0
