@@ -410,9 +410,23 @@ static cudaError_t enqueue_owner_apply(gear_ctx_impl& c, const Arrivals& user, c
 #undef GEAR_TRY
 }
 
-// After a call that failed: the ctx forgets the batch whose order it may have been in the middle of, and whatever else the call
-// may have left half done starts anew.
+// Waits for everything the ctx has enqueued: the stream of the training calls and, if the expiry scan went to a
+// stream of its own, that one too (a call's own streams are joined to it).
+static cudaError_t sync_streams(const gear_ctx_impl& c) {
+    cudaError_t e = cudaStreamSynchronize(c.last_stream);
+    for (int i = 0; i < c.n_seen && e == cudaSuccess; ++i)
+        if (c.seen_stream[i] != c.last_stream) e = cudaStreamSynchronize(c.seen_stream[i]);
+    return e;
+}
+// The ctx's own streams, which a call that failed may have left unjoined.
+static void sync_own_streams(const gear_ctx_impl& c) {
+    for (cudaStream_t s : {c.side_stream, c.aux_stream, c.rank_stream}) if (s) cudaStreamSynchronize(s);
+}
+
+// After a call that failed: nothing of it runs on a stream that the caller cannot wait for; the ctx forgets the batch whose order
+// it may have been in the middle of, and whatever else the call may have left half done starts anew.
 static void forget_batch(gear_ctx_impl& c) {
+    sync_own_streams(c);
     c.scan_cut_off = true;
     c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
     c.plan_sections_dirty = (int)((c.ws.grp_rec - c.ws.plan_sections) / 8);
@@ -584,15 +598,6 @@ int gear_step(gear_ctx* ctx, const gear_batch* batch, float lr, const gear_step_
     return check_capacity(l.expired_cap, h_n[1]);
 }
 
-// Waits for everything the ctx has enqueued: the stream of the training calls and, if the expiry scan went to a
-// stream of its own, that one too.
-static cudaError_t sync_streams(const gear_ctx_impl& c) {
-    cudaError_t e = cudaStreamSynchronize(c.last_stream);
-    for (int i = 0; i < c.n_seen && e == cudaSuccess; ++i)
-        if (c.seen_stream[i] != c.last_stream) e = cudaStreamSynchronize(c.seen_stream[i]);
-    return e;
-}
-
 static int finish_count(gear_ctx_impl& c, const int64_t* d_src, int64_t cap, int64_t* h_n, cudaStream_t st) {
     if (!h_n) return GEAR_OK;
     cudaError_t e = cudaMemcpyAsync(c.h_counts, d_src, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
@@ -756,7 +761,9 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
     }
     gear_ctx_impl &w0 = p.workers[0]->impl, &o0 = p.owners[0]->impl;
     for (int s = 0; s < W; ++s) p.workers[s]->impl.last_stream = p.owners[s]->impl.last_stream = st;
+    // Whatever has been enqueued is waited for, so that a caller that gives up may free the tables or use the staging buffer again
     auto fail = [&](cudaError_t err) {
+        cudaStreamSynchronize(st);
         for (int s = 0; s < W; ++s)
             for (gear_ctx_impl* c : {&p.workers[s]->impl, &p.owners[s]->impl}) forget_batch(*c);
         return cuda_fail(err, "shard_step");
@@ -988,8 +995,7 @@ int gear_destroy(gear_ctx* ctx) {
     if (!ctx->impl.alive) return GEAR_ERR_STATE;     // a ctx that failed half-way through its set-up; a destroyed
                                                      // ctx is freed memory and must not be passed in again
     sync_streams(ctx->impl);
-    cudaStreamSynchronize(ctx->impl.side_stream);
-    cudaStreamSynchronize(ctx->impl.aux_stream);
+    sync_own_streams(ctx->impl);
     release_host_objects(ctx->impl);
     ctx->impl.alive = false;
     delete ctx;

@@ -63,7 +63,7 @@ class Host:
         """A plan, its batches (host arrays), the contexts; `arrivals` is what every owner finds in the staging buffer's counts."""
         gb, lib = self.gb, self.lib
         owners = [self.ctx(batch * world, nnz * world, head=head, img_vocab=100_000) for _ in range(world)]
-        workers = [self.ctx(batch, nnz, head=head, mode=gb.GEAR_ACC_ATOMIC) for _ in range(world)]
+        workers = [self.ctx(batch, nnz, head=head, mode=gb.GEAR_ACC_ATOMIC, img_vocab=100_000) for _ in range(world)]
         words = C.c_int64()
         assert lib.gear_shard_stage_words(world, batch, nnz, C.byref(words)) == 0
         stage = (C.c_int32 * words.value)(*([arrivals] * words.value))
@@ -180,3 +180,34 @@ def test_an_expiry_scan_that_was_cut_off_leaves_no_counts(host):
     assert scan() == 0 and scan() == 0
     assert names() == ["memset", "expiry_mark", "expiry_write", "expiry_mark", "expiry_write"]
     assert lib.gear_destroy(ctx) == 0
+
+
+def _failing_call(host, call, k):
+    host.lib.fake_fail_at(k)
+    rc = call()
+    hit = host.lib.fake_calls() >= k
+    host.lib.fake_fail_at(-1)
+    return rc, hit
+
+
+@pytest.mark.parametrize("warm", [0, 5])                       # one launch after the other; as graphs
+@pytest.mark.parametrize("arrivals,nnz", [(100, 512), (40_000, 25_000)])
+def test_a_partitioned_step_that_fails_leaves_nothing_running(host, arrivals, nnz, warm):
+    """Whichever of its calls to the runtime fails: when gear_shard_step has returned, no stream holds work that the host has not
+    waited for (the caller may free the tables or use the staging buffer again), and the next step goes through."""
+    gb, lib = host.gb, host.lib
+    live, failed, k, hit = lib.fake_live(), 0, 0, True
+    while hit:
+        k += 1
+        plan, batches, ctxs = host.shard(nnz=nnz, arrivals=arrivals)
+        for _ in range(warm):
+            assert host.shard_step(plan, batches) == 0, lib.gear_last_error()
+            assert lib.fake_unfinished() == 0
+        rc, hit = _failing_call(host, lambda: host.shard_step(plan, batches), k)
+        failed += rc != 0                                        # (a graph that cannot be updated is played launch by launch)
+        assert rc in (0, gb.GEAR_ERR_CUDA) and lib.fake_unfinished() == 0, k
+        assert host.shard_step(plan, batches) == 0 and lib.fake_unfinished() == 0, k
+        for c in ctxs:
+            assert lib.gear_destroy(c) == 0
+        host.log()
+    assert failed > (5 if warm else 50) and lib.fake_live() == live
