@@ -428,6 +428,7 @@ static void sync_own_streams(const gear_ctx_impl& c) {
 static void forget_batch(gear_ctx_impl& c) {
     sync_own_streams(c);
     c.scan_cut_off = true;
+    c.acc_calls_pending = 2;                    // nothing is known of the ready queue
     c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
     c.plan_sections_dirty = (int)((c.ws.grp_rec - c.ws.plan_sections) / 8);
 }

@@ -199,6 +199,7 @@ collect_sort_kernel(const SortJob j, int64_t cap, int64_t* __restrict__ d_n, Dev
         if (d_n) *d_n = n;
         if (n > cap) atomicOr(&state->status, GEAR_DEV_OUT_CAPACITY);
         state->collect_n = n > cap ? -1 : n;
+        state->direct_done = 0;                 // (left by a reduce pass whose hand-over was never enqueued)
         state->sort_n = here ? -1 : sort ? n : 0;
     }
     if (here) s.sort(j, (int)n);

@@ -211,3 +211,30 @@ def test_a_partitioned_step_that_fails_leaves_nothing_running(host, arrivals, nn
             assert lib.gear_destroy(c) == 0
         host.log()
     assert failed > (5 if warm else 50) and lib.fake_live() == live
+
+
+@pytest.mark.parametrize("warm", [0, 5])
+@pytest.mark.parametrize("head,B,nnz", [(0, 64, 200), (1, 5000, 40_000)])
+def test_a_step_that_fails_is_joined_to_its_stream(host, head, B, nnz, warm):
+    """Whichever of its calls to the runtime fails: the caller's stream covers what was enqueued, and the next step does not take
+    the ready queue to be empty."""
+    lib = host.lib
+    failed, k, hit = 0, 0, True
+    while hit:
+        k += 1
+        ctx = host.ctx(B, nnz, hidden=(128, 64), head=head)
+        out, lists = host.out(), host.lists(nnz)
+        step = lambda: lib.gear_step(ctx, host.batch(B, nnz), 0.1, out, lists, 1, 1, 1, None, STREAM)
+        for _ in range(warm):
+            assert step() == 0
+        rc, hit = _failing_call(host, step, k)
+        lib.cudaStreamSynchronize(C.c_void_p(STREAM))
+        assert lib.fake_unfinished() == 0, k
+        host.log()
+        assert step() == 0
+        log = " ".join(" ".join(line) for line in host.log())
+        if rc != 0:
+            failed += 1
+            assert "collect_sort" in log and "collect_move" in log, k         # whatever the queue holds is handed over, in order
+        assert lib.gear_destroy(ctx) == 0
+    assert failed > (0 if warm else 30)
