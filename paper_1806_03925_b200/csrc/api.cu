@@ -433,12 +433,19 @@ static void forget_batch(gear_ctx_impl& c) {
     c.plan_sections_dirty = (int)((c.ws.grp_rec - c.ws.plan_sections) / 8);
 }
 
+// Writing a call down takes host memory; that it can run out is for the caller to hear, not an exception.
+template <typename Fn> static cudaError_t no_throw(Fn&& fn) {
+    try { return fn(); } catch (const std::bad_alloc&) { return cudaErrorMemoryAllocation; }
+}
+
 // Writes a call down and plays it.
 template <typename Fn> static int run_call(gear_ctx_impl& c, const char* where, cudaStream_t st, Fn&& enqueue) {
     c.last_stream = st;
-    Recording rec(c.player, st);
-    cudaError_t e = enqueue();
-    if (e == cudaSuccess) e = rec.play(&c.prof);             // (else nothing has been enqueued)
+    const cudaError_t e = no_throw([&] {
+        Recording rec(c.player, st);
+        const cudaError_t we = enqueue();
+        return we == cudaSuccess ? rec.play(&c.prof) : we;   // (else nothing has been enqueued)
+    });
     if (e == cudaSuccess) return GEAR_OK;
     forget_batch(c);
     return cuda_fail(e, where);
@@ -628,7 +635,7 @@ int gear_collect_expired(gear_ctx* ctx, int64_t now, int restamp, int32_t* ids, 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c.note_stream(st);             // may differ from the stream of the training calls: the scan shares nothing with them
     int64_t* d_cnt = d_n ? d_n : &c.state()->pad[1];
-    cudaError_t e = launch_collect_expired(c, now, restamp, ids, cap, d_cnt, st);
+    cudaError_t e = no_throw([&] { return launch_collect_expired(c, now, restamp, ids, cap, d_cnt, st); });
     if (e != cudaSuccess) { c.scan_cut_off = true; return cuda_fail(e, "collect_expired"); }
     return finish_count(c, d_cnt, cap, h_n, st);
 }
@@ -643,7 +650,7 @@ int gear_refresh_dfv(gear_ctx* ctx, const int32_t* ids, const float* rows, int64
     if (ld < c.cfg.dfv_dim || (ld & 3) || !aligned16(rows)) return arg_fail("rows must be 16-byte aligned, ld >= dfv_dim and a multiple of 4");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c.note_stream(st);
-    cudaError_t e = launch_refresh_dfv(c, ids, rows, ld, n, d_n, now, st);
+    cudaError_t e = no_throw([&] { return launch_refresh_dfv(c, ids, rows, ld, n, d_n, now, st); });
     if (e != cudaSuccess) return cuda_fail(e, "refresh_dfv");
     return GEAR_OK;
 }
@@ -657,7 +664,7 @@ int gear_fetch_rows(gear_ctx* ctx, int32_t which, const int32_t* ids, int64_t n,
     if (!ids || !out || !aligned16(out)) return arg_fail("NULL or misaligned pointer");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c.note_stream(st);
-    cudaError_t e = launch_fetch_rows(c, which, ids, n, out, st);
+    cudaError_t e = no_throw([&] { return launch_fetch_rows(c, which, ids, n, out, st); });
     return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "fetch_rows");
 }
 
@@ -783,7 +790,7 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
     };
     e = cudaMemcpyAsync(p.stage, p.host_stage, (size_t)pos[4] * 4, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess) e = order(st, early);
-    if (e == cudaSuccess && total[0] + total[1] + total[2] > 0) e = launch_shard_route(&w0.prof, r, early);
+    if (e == cudaSuccess && total[0] + total[1] + total[2] > 0) e = no_throw([&] { return launch_shard_route(&w0.prof, r, early); });
     else if (e == cudaSuccess) e = cudaMemsetAsync(r.counts, 0, sizeof(int32_t) * 3 * W, early);
     if (e == cudaSuccess) e = cudaMemcpyAsync(p.host_stage + at.counts, r.counts, sizeof(int32_t) * 3 * W, cudaMemcpyDeviceToHost, early);
     if (e == cudaSuccess) e = cudaEventRecord(w0.ev[EV_ROUTED], early);
@@ -791,9 +798,9 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
     auto stream_of = [&](int s) { return s == 0 ? st : p.owners[s]->impl.rank_stream; };
 #define GEAR_TRY(x) do { cudaError_t e_ = (x); if (e_ != cudaSuccess) return e_; } while (0)
     // ---- events 1 to 4 on the workers, side by side
-    {
+    e = no_throw([&] {
         Recording rec(w0.player, st);
-        e = [&]() -> cudaError_t {
+        const cudaError_t we = [&]() -> cudaError_t {
             if (total[0] + total[1] + total[2] > 0) GEAR_TRY(launch_shard_fetch(&w0.prof, f, st));
             if (W > 1) GEAR_TRY(enqueue_record(w0.ev[EV_RANKS], st));
             for (int s = 1; s < W; ++s) GEAR_TRY(enqueue_wait(stream_of(s), w0.ev[EV_RANKS]));
@@ -810,9 +817,8 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
             }
             return cudaSuccess;
         }();
-        if (e != cudaSuccess) return fail(e);
-        e = rec.play(&w0.prof);
-    }
+        return we == cudaSuccess ? rec.play(&w0.prof) : we;
+    });
     if (e == cudaSuccess) e = cudaEventSynchronize(w0.ev[EV_ROUTED]);
     if (e != cudaSuccess) return fail(e);
     // ---- events 4 (push), 5 and 6 at the owners, side by side
@@ -821,7 +827,7 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
     for (int s = 0; s < W; ++s)
         for (int t = 0; t < 3; ++t)
             arrived[s][t] = Arrivals{r.table[t].local + s * total[t], r.table[t].src + s * total[t], (int64_t)p.host_stage[at.counts + t * W + s]};
-    auto at_owners = [&](auto of, auto work) -> cudaError_t {
+    auto at_owners = [&](auto of, auto work) -> cudaError_t { return no_throw([&] {
         Recording rec(o0.player, of(0));
         const cudaError_t we = [&]() -> cudaError_t {
             if (W > 1) GEAR_TRY(enqueue_record(o0.ev[EV_RANKS], of(0)));
@@ -837,7 +843,7 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
             return cudaSuccess;
         }();
         return we == cudaSuccess ? rec.play(&o0.prof) : we;
-    };
+    }); };
     e = at_owners(early_of, [&](int s, gear_ctx_impl& c, cudaStream_t where) {
         return enqueue_owner_plan(c, arrived[s][0], arrived[s][1], arrived[s][2], p.lists[s], now, &sorted_buf[s], where);
     });
@@ -870,7 +876,7 @@ int gear_dense_forward(gear_ctx* ctx, const float* raw, int32_t raw_dim, const f
     if (!raw || !Wd || !ids || !rows || ld < c.cfg.dfv_dim) return arg_fail("NULL pointer or ld < dfv_dim");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c.note_stream(st);
-    cudaError_t e = launch_dense_forward(c, raw, raw_dim, Wd, ids, n, d_n, rows, ld, st);
+    cudaError_t e = no_throw([&] { return launch_dense_forward(c, raw, raw_dim, Wd, ids, n, d_n, rows, ld, st); });
     return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "dense_forward");
 }
 
@@ -883,7 +889,7 @@ int gear_dense_backward(gear_ctx* ctx, const float* raw, int32_t raw_dim, const 
     if (!raw || !ids || !avg || !Wd_grad) return arg_fail("NULL pointer");
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     c.note_stream(st);
-    cudaError_t e = launch_dense_backward(c, raw, raw_dim, ids, avg, c.cfg.dfv_dim, n, d_n, Wd_grad, st);
+    cudaError_t e = no_throw([&] { return launch_dense_backward(c, raw, raw_dim, ids, avg, c.cfg.dfv_dim, n, d_n, Wd_grad, st); });
     return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "dense_backward");
 }
 
@@ -894,7 +900,7 @@ int gear_adam_dense(float* param, const float* grad, float* m, float* v, int64_t
     if (!param || !grad || !m || !v) return arg_fail("NULL pointer");
     if (!(cfg->beta1 >= 0.f && cfg->beta1 < 1.f && cfg->beta2 >= 0.f && cfg->beta2 < 1.f && cfg->eps >= 0.f))
         return arg_fail("adam: beta1, beta2 in [0, 1), eps >= 0");
-    cudaError_t e = launch_adam_dense(nullptr, param, grad, m, v, n, t, *cfg, static_cast<cudaStream_t>(stream));
+    cudaError_t e = no_throw([&] { return launch_adam_dense(nullptr, param, grad, m, v, n, t, *cfg, static_cast<cudaStream_t>(stream)); });
     return e == cudaSuccess ? GEAR_OK : cuda_fail(e, "adam_dense");
 }
 

@@ -103,10 +103,10 @@ static bool same_shape(const OpList& a, const OpList& b) {
 // The list captured into a graph (nothing is enqueued).  The caller's stream is stood in for by a stream of the player's
 // own, since the default stream cannot be captured.
 bool Player::build(Entry& e, OpList& l) {
+    e.node.assign(l.ops.size(), nullptr);                // (nothing below allocates: a capture that has begun is ended)
     if (!capture_ && cudaStreamCreateWithFlags(&capture_, cudaStreamNonBlocking) != cudaSuccess) return false;
     if (cudaStreamBeginCapture(capture_, cudaStreamCaptureModeRelaxed) != cudaSuccess) return false;
     bool ok = true;
-    e.node.assign(l.ops.size(), nullptr);
     for (size_t i = 0; i < l.ops.size() && ok; ++i) {
         const Op& o = l.ops[i];
         const cudaStream_t st = o.role == 0 ? capture_ : l.streams[o.role];

@@ -155,6 +155,7 @@ cudaError_t launch_collect_expired(const gear_ctx_impl& c, int64_t now, int rest
 // process exits.  The price is a bound on the table size and one shared scratch per device.
 // ---------------------------------------------------------------------------------------------------
 #include <mutex>
+#include <new>
 
 namespace gear {
 
@@ -210,9 +211,10 @@ extern "C" int gear_collect_expired_static(int64_t* dfv_ts, int64_t img_vocab, i
     if (enqueue_memset(state, STATIC_STATE_BYTES, st) != cudaSuccess) return GEAR_ERR_CUDA;
     if (enqueue_memset(cnt.section, sizeof(uint32_t) * (size_t)cnt.n_sections, st) != cudaSuccess) return GEAR_ERR_CUDA;
     int64_t* d_cnt = d_n ? d_n : &state->pad[1];
-    if (enqueue_expiry_scan(dfv_ts, img_vocab, expire, now, restamp, ids, cap, d_cnt, bits, cnt, state, nullptr, st) !=
-        cudaSuccess)
-        return GEAR_ERR_CUDA;
+    try {                                            // (a launch is written down in host memory, which may run out)
+        if (enqueue_expiry_scan(dfv_ts, img_vocab, expire, now, restamp, ids, cap, d_cnt, bits, cnt, state, nullptr, st) != cudaSuccess)
+            return GEAR_ERR_CUDA;
+    } catch (const std::bad_alloc&) { return GEAR_ERR_CUDA; }
     if (h_n) {
         if (cudaMemcpyAsync(h_n, d_cnt, sizeof(int64_t), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)

@@ -16,8 +16,8 @@ class Host:
     def __init__(self, lib, gb):
         self.lib, self.gb = lib, gb
         lib.fake_unfinished.restype = C.c_int
-        lib.fake_calls.restype = lib.fake_live.restype = lib.fake_log.restype = C.c_long
-        lib.fake_fail_at.argtypes = [C.c_long]
+        lib.fake_calls.restype = lib.fake_live.restype = lib.fake_log.restype = lib.fake_news.restype = C.c_long
+        lib.fake_fail_at.argtypes = lib.fake_no_memory_at.argtypes = [C.c_long]
         lib.fake_user_capture.argtypes = [C.c_void_p, C.c_int]
         self.next = 1 << 40
         self.keep = []
@@ -238,3 +238,54 @@ def test_a_step_that_fails_is_joined_to_its_stream(host, head, B, nnz, warm):
             assert "collect_sort" in log and "collect_move" in log, k         # whatever the queue holds is handed over, in order
         assert lib.gear_destroy(ctx) == 0
     assert failed > (0 if warm else 30)
+
+
+@pytest.mark.parametrize("warm", [0, 3, 5])                    # ... where the graph is made; with it
+def test_no_call_throws_when_the_host_is_out_of_memory(host, warm):
+    """Whichever allocation of a call fails, the call returns GEAR_ERR_CUDA (an exception would end the process here), the caller's
+    stream covers what was enqueued, and the calls that follow go through."""
+    gb, lib = host.gb, host.lib
+    calls = {
+        "step": lambda c: lib.gear_step(c, host.batch(5000, 40_000), 0.1, host.out(), host.lists(40_000), 1, 1, 1, None, STREAM),
+        "forward_backward": lambda c: lib.gear_forward_backward(c, host.batch(), 0.1, host.out(), STREAM),
+        "collect_expired": lambda c: lib.gear_collect_expired(c, 1, 1, host.address(), 1000, None, None, STREAM),
+        "refresh": lambda c: lib.gear_refresh_dfv(c, host.address(), host.address(), 64, 10, None, 1, STREAM),
+        "fetch": lambda c: lib.gear_fetch_rows(c, 0, host.address(), 10, host.address(), STREAM),
+        "dense_forward": lambda c: lib.gear_dense_forward(c, host.address(), 32, host.address(), host.address(), 10, None, host.address(), 64, STREAM),
+        "dense_backward": lambda c: lib.gear_dense_backward(c, host.address(), 32, host.address(), host.address(), 10, None, host.address(), STREAM),
+        "adam": lambda c: lib.gear_adam_dense(host.address(), host.address(), host.address(), host.address(), 10, 1, C.byref(gb.make_adam()), STREAM),
+        "expired_static": lambda c: lib.gear_collect_expired_static(host.address(), 1000, 1, 1, 1, host.address(), 1000, None, None, STREAM),
+    }
+    for name, call in calls.items():
+        failed, k, hit = 0, 0, True
+        while hit:
+            k += 1
+            ctx = host.ctx(5000, 40_000, hidden=(128, 64))
+            for _ in range(warm):
+                assert call(ctx) == 0, (name, lib.gear_last_error())
+            lib.fake_no_memory_at(k)
+            rc = call(ctx)
+            hit = lib.fake_news() >= k
+            lib.fake_no_memory_at(-1)
+            assert rc == (gb.GEAR_ERR_CUDA if hit else 0), (name, k)
+            failed += hit
+            lib.cudaStreamSynchronize(C.c_void_p(STREAM))
+            assert lib.fake_unfinished() == 0, (name, k)
+            for _ in range(2):
+                assert call(ctx) == 0, (name, k)
+            assert lib.gear_destroy(ctx) == 0
+            host.log()
+        assert failed > 0 or (warm and name in ("step", "forward_backward")), name
+    plan, batches, ctxs = host.shard(nnz=25_000, arrivals=40_000)
+    for _ in range(warm):
+        assert host.shard_step(plan, batches) == 0
+    k, hit = 0, True
+    while hit:
+        k += 1
+        lib.fake_no_memory_at(k)
+        rc = host.shard_step(plan, batches)
+        hit = lib.fake_news() >= k
+        lib.fake_no_memory_at(-1)
+        assert rc == (gb.GEAR_ERR_CUDA if hit else 0) and lib.fake_unfinished() == 0, k
+    for c in ctxs:
+        assert lib.gear_destroy(c) == 0
