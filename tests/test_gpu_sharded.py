@@ -1,0 +1,62 @@
+"""The step with the tables partitioned by ID and all ranks in this process: the native call (gear_shard_step) against the same step
+exchange by exchange, which goes by the same rules through other calls."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1806_03925_b200 import workloads
+from paper_1806_03925_b200.workloads import BF16, PRESETS, Batch, BatchSource
+
+pytestmark = pytest.mark.gpu
+
+TABLES = ("user_emb", "url_emb", "dfv_gsum", "dfv_gcnt", "dfv_ts")
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _device():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+
+
+def _exchange(world):
+    """An in-process exchange with a method of its own: the step goes through its calls."""
+    from paper_1806_03925_b200.sharded import LoopbackExchange
+
+    class Counting(LoopbackExchange):
+        routed = 0
+
+        def route(self, ids):
+            self.routed += 1
+            return super().route(ids)
+    return Counting(world)
+
+
+def _jobs(p, world, max_batch, max_nnz, **more):
+    from paper_1806_03925_b200.sharded import LoopbackExchange, ShardedGear
+    return [ShardedGear(p, workloads.head_params(p, 2), ex, max_batch_local=max_batch, max_nnz_local=max_nnz, seed=5, **more)
+            for ex in (LoopbackExchange(world), _exchange(world))]
+
+
+def _small(world, **more):
+    p = PRESETS["tiny"].scaled(user_vocab=501, url_vocab=400, img_vocab=603, batch=60, expire=3, **more)
+    return p, [BatchSource(p, 3 + r).batch(0) for r in range(world)]
+
+
+def _same(a, c, tol):
+    from gpu_harness import _np, assert_close
+    for oa, oc in zip(a.owners, c.owners):
+        for name in TABLES:
+            x, y = _np(getattr(oa, name)), _np(getattr(oc, name))
+            assert np.array_equal(x, y) if x.dtype.kind == "i" else assert_close(x, y, tol, name) is None, name
+
+
+def test_an_exchange_with_methods_of_its_own_is_used():
+    p, batches = _small(2)
+    native, by_hand = _jobs(p, 2, p.batch, p.batch * p.img_hi)
+    try:
+        assert native.step(batches, 1) == by_hand.step(batches, 1)
+        assert by_hand.ex.routed == 3 and by_hand._in_process is None
+        _same(native, by_hand, 1e-5)
+    finally:
+        native.close()
+        by_hand.close()
