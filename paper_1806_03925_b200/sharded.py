@@ -289,16 +289,20 @@ class _InProcessStep:
         self.batches, self.counts = (gb.gear_host_batch * W)(), (C.c_int64 * (2 * W))()
 
     def step(self, batches: Sequence[Batch], now: int, lr: float, mean_head_grad: bool):
+        if len(batches) < len(self.batches):
+            raise IndexError("%d batches for %d ranks" % (len(batches), len(self.batches)))
         keep = []                                    # converted arrays live until the call has copied them
 
-        def at(a, dtype):
+        def at(a, dtype, n):
             a = np.ascontiguousarray(a, dtype)
+            if a.size < n:                           # the call copies n entries
+                raise ValueError("a batch array holds %d entries, its batch needs %d" % (a.size, n))
             keep.append(a)
             return a.__array_interface__["data"][0]
         for c, b in zip(self.batches, batches):
-            c.B, c.nnz = b.B, b.nnz
-            c.user_id, c.url_id, c.img_off = at(b.user_id, np.int32), at(b.url_id, np.int32), at(b.img_off, np.int32)
-            c.img_id, c.label = at(b.img_id, np.int32), at(b.label, np.float32)
+            B, nnz = c.B, c.nnz = b.B, b.nnz
+            c.user_id, c.url_id, c.img_id = at(b.user_id, np.int32, B), at(b.url_id, np.int32, B), at(b.img_id, np.int32, nnz)
+            c.img_off, c.label = at(b.img_off, np.int32, B + 1 if B else 0), at(b.label, np.float32, B)
         gb.gear_shard_step(self.plan, self.batches, lr, now, mean_head_grad, self.counts)
         v = list(self.counts)
         return list(zip(v[0::2], v[1::2]))

@@ -60,3 +60,23 @@ def test_an_exchange_with_methods_of_its_own_is_used():
     finally:
         native.close()
         by_hand.close()
+
+
+def test_a_step_needs_a_batch_for_every_rank_and_whole_arrays():
+    p, batches = _small(3)
+    (native, by_hand) = _jobs(p, 3, p.batch, p.batch * p.img_hi)
+    try:
+        for job in (native, by_hand):
+            job.step(batches, 1)
+            with pytest.raises(IndexError):
+                job.step(batches[:2], 2)
+        whole = batches[1]
+        for name in ("url_id", "img_off", "label"):
+            cut = Batch(whole.user_id, whole.url_id, whole.img_off, whole.img_id, whole.label)
+            setattr(cut, name, getattr(whole, name)[:-1])
+            with pytest.raises(ValueError):
+                native.step([batches[0], cut, batches[2]], 2)
+        assert native.step(batches, 2) == by_hand.step(batches, 2)
+    finally:
+        native.close()
+        by_hand.close()
