@@ -224,8 +224,9 @@ class ShardedGear:
         rank (averages handed over by its owner, IDs its owner's scan listed)."""
         p, ex = self.p, self.ex
         lr = p.lr if lr is None else lr
-        # the short way takes all ranks in this process; an exchange with methods of its own goes its own way
-        if type(ex) is LoopbackExchange and self.world <= gb.GEAR_MAX_LOCAL_RANKS:
+        # The short way takes all ranks in this process and int32 IDs; an exchange with methods of its own goes its own way, and so
+        # do IDs of a table with more rows than int32 can name (every shard is smaller than that).
+        if type(ex) is LoopbackExchange and self.world <= gb.GEAR_MAX_LOCAL_RANKS and _ids_fit_int32(batches):
             if self._in_process is None:
                 self._in_process = _InProcessStep(self)
             return self._in_process.step(batches, now, lr, mean_head_grad)
@@ -270,6 +271,14 @@ class ShardedGear:
     def close(self):
         for s in self.owners + self.workers:
             s.close()
+
+
+def _ids_fit_int32(batches: Sequence[Batch]) -> bool:
+    for b in batches:
+        for a in map(np.asarray, (b.user_id, b.url_id, b.img_id)):
+            if not np.can_cast(a.dtype, np.int32) and a.size and (a.max() > 2 ** 31 - 1 or a.min() < -2 ** 31):
+                return False
+    return True
 
 
 class _InProcessStep:

@@ -80,3 +80,26 @@ def test_a_step_needs_a_batch_for_every_rank_and_whole_arrays():
     finally:
         native.close()
         by_hand.close()
+
+
+def test_ids_beyond_int32_are_not_wrapped_around():
+    """An int64 list with an ID of 2^32 + 6: no shard holds it, its row counts as zeros.  (As int32 it would be ID 6.)"""
+    p, batches = _small(2)
+    native, by_hand = _jobs(p, 2, p.batch, p.batch * p.img_hi)
+    try:
+        wide = batches[0].user_id.astype(np.int64)
+        wide[:] = 2 ** 32 + 6
+        odd = Batch(wide, batches[0].url_id, batches[0].img_off, batches[0].img_id, batches[0].label)
+        before = native.owners[0].user_emb.clone()
+        quiet = Batch(np.full_like(batches[1].user_id, 7), *(getattr(batches[1], n) for n in ("url_id", "img_off", "img_id", "label")))
+        assert native.step([odd, quiet], 1) == by_hand.step([odd, quiet], 1)
+        assert torch.equal(native.owners[0].user_emb, before)              # (the other rank names ID 7, of owner 1)
+        _same(native, by_hand, 1e-5)
+        # 64-bit lists that int32 can hold take the short way
+        narrow = Batch(batches[0].user_id.astype(np.int64), *(getattr(batches[0], n) for n in ("url_id", "img_off", "img_id", "label")))
+        assert native.step([narrow, batches[1]], 2) == by_hand.step([narrow, batches[1]], 2)
+        assert native._in_process is not None
+        _same(native, by_hand, 1e-5)
+    finally:
+        native.close()
+        by_hand.close()
