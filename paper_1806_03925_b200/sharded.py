@@ -205,12 +205,12 @@ class ShardedGear:
             self.owners.append(GearSession(sp, head_params, max_batch=max_batch_local * W, max_nnz=max_nnz_local * W,
                                            seed=seed + r, fill=True, now=now, tables=mine, device=device,
                                            scalars=self._scalars[3 * len(self.owners):3 * len(self.owners) + 3]))
-            wp = replace(p, user_vocab=max_batch_local, url_vocab=max_batch_local, img_vocab=max_nnz_local)
+            wp = replace(p, user_vocab=max_batch_local, url_vocab=max_batch_local, img_vocab=max_nnz_local, M=1)
             i = len(self.workers)
             rows = slice(i * max_batch_local, (i + 1) * max_batch_local), slice(i * max_nnz_local, (i + 1) * max_nnz_local)
             blank = dict(user_emb=self._user_rows[rows[0]], url_emb=self._url_rows[rows[0]], dfv=self._dfv_rows[rows[1]],
                          ts=torch.zeros(max_nnz_local, dtype=torch.int64, device=dev))
-            # a worker keeps no gradient store (GEAR_ACC_ATOMIC: its image IDs are not sorted)
+            # a worker keeps no gradient store (GEAR_ACC_ATOMIC: its image IDs are not sorted), so that M means nothing to it
             wk = GearSession(wp, head_params, max_batch=max_batch_local, max_nnz=max_nnz_local, tables=blank,
                              expired_cap=1, ready_cap=1, device=device, accum_mode=gb.GEAR_ACC_ATOMIC)
             wk.dX, wk.dfv_grad, wk.head_grad = self._dX[rows[0]], self._dfv_grad[rows[1]], self._head_grads[i]

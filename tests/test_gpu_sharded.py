@@ -103,3 +103,17 @@ def test_ids_beyond_int32_are_not_wrapped_around():
     finally:
         native.close()
         by_hand.close()
+
+
+def test_stores_of_any_m_are_taken():
+    """Workers keep no store: what a store of their kind could not take (M from 2^29 on) does not matter to them."""
+    p, batches = _small(2, M=1 << 30)
+    native, by_hand = _jobs(p, 2, p.batch, p.batch * p.img_hi)
+    try:
+        got = native.step(batches, 1)
+        assert got == by_hand.step(batches, 1) and all(n_ready == 0 for n_ready, _ in got)
+        _same(native, by_hand, 1e-5)
+        assert sum(int(o.dfv_gcnt.sum()) for o in native.owners) == sum(b.nnz for b in batches)
+    finally:
+        native.close()
+        by_hand.close()
