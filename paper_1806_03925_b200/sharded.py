@@ -224,6 +224,8 @@ class ShardedGear:
         rank (averages handed over by its owner, IDs its owner's scan listed)."""
         p, ex = self.p, self.ex
         lr = p.lr if lr is None else lr
+        if any(s.ctx is None for s in self.owners + self.workers):
+            raise gb.GearError(gb.GEAR_ERR_STATE, "ShardedGear.step", "a session has been closed")
         # The short way takes all ranks in this process and int32 IDs; an exchange with methods of its own goes its own way, and so
         # do IDs of a table with more rows than int32 can name (every shard is smaller than that).
         if type(ex) is LoopbackExchange and self.world <= gb.GEAR_MAX_LOCAL_RANKS and _ids_fit_int32(batches):
@@ -269,6 +271,7 @@ class ShardedGear:
         return out
 
     def close(self):
+        self._in_process = None                      # it holds the contexts' addresses
         for s in self.owners + self.workers:
             s.close()
 

@@ -117,3 +117,18 @@ def test_stores_of_any_m_are_taken():
     finally:
         native.close()
         by_hand.close()
+
+
+def test_a_closed_job_is_refused():
+    from paper_1806_03925_b200 import binding as gb
+    p, batches = _small(2)
+    for job in _jobs(p, 2, p.batch, p.batch * p.img_hi):
+        job.step(batches, 1)
+        job.owners[1].close()
+        with pytest.raises(gb.GearError) as e:
+            job.step(batches, 2)
+        assert e.value.code == gb.GEAR_ERR_STATE
+        job.close()
+        with pytest.raises(gb.GearError) as e:
+            job.step(batches, 2)
+        assert e.value.code == gb.GEAR_ERR_STATE
