@@ -260,3 +260,33 @@ def test_a_captured_expiry_scan_can_be_replayed():
         assert s.status()[1] == 0
     finally:
         s.close()
+
+
+def test_a_host_batch_may_be_used_on_any_stream():
+    """Made on a stream that is busy for some milliseconds; its tensors read, or the batch handed to a session, on another one."""
+    from paper_1806_03925_b200.session import DeviceBatch, GearSession
+    p = PRESETS["tiny"]
+    b = BatchSource(p, 3).batch(0)
+    names = ("user_id", "url_id", "img_off", "img_id", "label")
+    busy, other = torch.cuda.Stream(), torch.cuda.Stream()
+    a, c = (GearSession(p, workloads.head_params(p, 3), max_nnz=b.nnz, seed=3) for _ in range(2))
+    try:
+        DeviceBatch.from_host(b)                                         # (the pools have their blocks)
+        torch.cuda.synchronize()
+        with torch.cuda.stream(busy):
+            torch.cuda._sleep(20_000_000)
+            read, used, mixed = (DeviceBatch.from_host(b) for _ in range(3))
+            mixed.label = 1 - torch.from_numpy(b.label).cuda()
+        with torch.cuda.stream(other):
+            got = {name: getattr(read, name).clone() for name in names}
+            n_ready, n_exp = a.step(used, 1, sync=True)
+            assert GearSession._c_batch(mixed).label == mixed.label.data_ptr()
+        torch.cuda.synchronize()
+        for name, t in got.items():
+            assert np.array_equal(t.cpu().numpy(), getattr(b, name)), name
+        assert np.array_equal(mixed.label.cpu().numpy(), 1 - b.label) and np.array_equal(mixed.img_id.cpu().numpy(), b.img_id)
+        assert (n_ready, n_exp) == c.step(DeviceBatch(*(torch.from_numpy(getattr(b, n)).cuda() for n in names), b.B, b.nnz), 1, sync=True)
+        assert torch.equal(a.prob, c.prob)
+    finally:
+        a.close()
+        c.close()
