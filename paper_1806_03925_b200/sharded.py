@@ -37,6 +37,8 @@ from . import binding as gb
 from .session import DeviceBatch, GearSession
 from .workloads import BF16, Batch, GearPreset
 
+_WORD = np.dtype(np.int32)
+
 
 @dataclass
 class Route:
@@ -224,7 +226,7 @@ class ShardedGear:
         rank (averages handed over by its owner, IDs its owner's scan listed)."""
         p, ex = self.p, self.ex
         lr = p.lr if lr is None else lr
-        if any(s.ctx is None for s in self.owners + self.workers):
+        if None in [s.ctx for s in self.owners] or None in [s.ctx for s in self.workers]:
             raise gb.GearError(gb.GEAR_ERR_STATE, "ShardedGear.step", "a session has been closed")
         # The short way takes all ranks in this process and int32 IDs; an exchange with methods of its own goes its own way, and so
         # do IDs of a table with more rows than int32 can name (every shard is smaller than that).
@@ -278,8 +280,10 @@ class ShardedGear:
 
 def _ids_fit_int32(batches: Sequence[Batch]) -> bool:
     for b in batches:
-        for a in map(np.asarray, (b.user_id, b.url_id, b.img_id)):
-            if not np.can_cast(a.dtype, np.int32) and a.size and (a.max() > 2 ** 31 - 1 or a.min() < -2 ** 31):
+        for a in (b.user_id, b.url_id, b.img_id):
+            if a.dtype == _WORD or np.can_cast(a.dtype, _WORD) or not a.size:
+                continue
+            if a.max() > 2 ** 31 - 1 or a.min() < -2 ** 31:
                 return False
     return True
 
