@@ -167,7 +167,7 @@ class GearSession:
         self._expired_ids_g = torch.full((self.expired_cap + 1,), self.GUARD_I, dtype=torch.int32, device=dev)
         self.expired_ids = self._expired_ids_g[:self.expired_cap]
         self.d_counts = self.scalars[1:3]
-        self._step_out = self._step_lists = None
+        self._step_out = self._step_lists = self._lists_at = None
 
     # ---- the four calls of a step ---------------------------------------------------------------
     def forward_backward(self, b: DeviceBatch, lr: Optional[float] = None):
@@ -177,7 +177,7 @@ class GearSession:
             o.adam_step = self.adam_step
         return gb.gear_forward_backward_structs(self.ctx, self._c_batch(b), self.p.lr if lr is None else lr, o)
 
-    # the structs of the outputs never change and a batch's struct only in its counts: all are made once
+    # structs are made once: a step's outputs never change, a batch only in its counts
     def _make_step_out(self):
         self._step_out = gb.make_step_out(self.loss, self.head_grad, self.dX, prob=self.prob, row_view=self.row_view,
                                               inv_n=self.inv_n, x_debug=self.x_debug, user_grad=self.user_grad,
@@ -185,9 +185,14 @@ class GearSession:
                                               user_v=self.user_v, url_m=self.url_m, url_v=self.url_v)
         return self._step_out
 
-    def _make_step_lists(self):
-        self._step_lists = gb.make_step_lists(self.ready_ids, self.ready_seq, self.ready_avg, self.ready_cap, self.expired_ids,
-                                              self.expired_cap, d_n=self.d_counts[0:1], d_expired=self.d_counts[1:2])
+    def _lists(self):
+        """The struct of the output lists, made anew when a program has put other tensors in their place."""
+        at = (self.ready_ids.data_ptr(), self.ready_seq.data_ptr(), self.ready_avg.data_ptr(), self.ready_cap,
+              self.expired_ids.data_ptr(), self.expired_cap, self.d_counts.data_ptr())
+        if at != self._lists_at:
+            self._step_lists = gb.make_step_lists(self.ready_ids, self.ready_seq, self.ready_avg, self.ready_cap, self.expired_ids,
+                                                  self.expired_cap, d_n=self.d_counts[0:1], d_expired=self.d_counts[1:2])
+            self._lists_at = at
         return self._step_lists
 
     @staticmethod
@@ -258,7 +263,7 @@ class GearSession:
         """One pass of the whole hot path over one batch (gear_step).  The expiry scan depends on nothing the training
         calls produce and runs beside them (expiry_beside=False: behind them)."""
         beside = True if expiry_beside is None else expiry_beside
-        o, lists = self._step_out or self._make_step_out(), self._step_lists or self._make_step_lists()
+        o, lists = self._step_out or self._make_step_out(), self._lists()
         if self.adam is not None:
             self.adam_step += 1
             o.adam_step = self.adam_step

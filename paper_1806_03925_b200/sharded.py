@@ -37,7 +37,7 @@ from . import binding as gb
 from .session import DeviceBatch, GearSession
 from .workloads import BF16, Batch, GearPreset
 
-_WORD = np.dtype(np.int32)
+_WORD, _FLOAT = np.dtype(np.int32), np.dtype(np.float32)
 
 
 @dataclass
@@ -299,7 +299,8 @@ class _InProcessStep:
         self.host, self.dev = torch.zeros(words, dtype=torch.int32).pin_memory(), torch.zeros(words, dtype=torch.int32, device=sg.workers[0].dev)
         self.ctxs = [(C.c_void_p * W)(*(s.ctx.value for s in side)) for side in (sg.owners, sg.workers)]
         self.out = (gb.gear_step_out * W)(*(w._make_step_out() for w in sg.workers))
-        self.lists = (gb.gear_step_lists * W)(*(o._make_step_lists() for o in sg.owners))
+        self.lists_made = [o._lists() for o in sg.owners]
+        self.lists = (gb.gear_step_lists * W)(*self.lists_made)
         self.plan = gb.gear_shard_plan(W, sg.max_batch_local, sg.max_nnz_local, self.ctxs[0], self.ctxs[1], self.host.data_ptr(),
                                        self.dev.data_ptr(), sg._iota.data_ptr(), self.out, self.lists)
         self.batches, self.counts = (gb.gear_host_batch * W)(), (C.c_int64 * (2 * W))()
@@ -310,15 +311,19 @@ class _InProcessStep:
         keep = []                                    # converted arrays live until the call has copied them
 
         def at(a, dtype, n):
-            a = np.ascontiguousarray(a, dtype)
+            if getattr(a, "dtype", None) != dtype or not a.flags.c_contiguous:
+                a = np.ascontiguousarray(a, dtype)
             if a.size < n:                           # the call copies n entries
                 raise ValueError("a batch array holds %d entries, its batch needs %d" % (a.size, n))
             keep.append(a)
             return a.__array_interface__["data"][0]
         for c, b in zip(self.batches, batches):
             B, nnz = c.B, c.nnz = b.B, b.nnz
-            c.user_id, c.url_id, c.img_id = at(b.user_id, np.int32, B), at(b.url_id, np.int32, B), at(b.img_id, np.int32, nnz)
-            c.img_off, c.label = at(b.img_off, np.int32, B + 1 if B else 0), at(b.label, np.float32, B)
+            c.user_id, c.url_id, c.img_id = at(b.user_id, _WORD, B), at(b.url_id, _WORD, B), at(b.img_id, _WORD, nnz)
+            c.img_off, c.label = at(b.img_off, _WORD, B + 1 if B else 0), at(b.label, _FLOAT, B)
+        made = [o._lists() for o in self.sg.owners]
+        if made != self.lists_made:                  # other tensors have been put in place of an owner's lists
+            self.lists_made, self.lists[:] = made, made
         gb.gear_shard_step(self.plan, self.batches, lr, now, mean_head_grad, self.counts)
         v = list(self.counts)
         return list(zip(v[0::2], v[1::2]))

@@ -290,3 +290,28 @@ def test_a_host_batch_may_be_used_on_any_stream():
     finally:
         a.close()
         c.close()
+
+
+def test_a_step_writes_to_the_lists_a_session_has_now():
+    """A program that keeps a step's lists and puts fresh ones in their place."""
+    from paper_1806_03925_b200.session import DeviceBatch, GearSession
+    p = PRESETS["tiny"].scaled(expire=1, M=1)
+    batches = [DeviceBatch.from_host(BatchSource(p, 3).batch(k)) for k in range(2)]
+    a, c = (GearSession(p, workloads.head_params(p, 3), max_nnz=max(b.nnz for b in batches), seed=3) for _ in range(2))
+    try:
+        names = ("ready_ids", "ready_seq", "ready_avg", "expired_ids", "d_counts")
+        assert a.step(batches[0], 1, sync=True) == c.step(batches[0], 1, sync=True)
+        kept = {n: getattr(a, n) for n in names}
+        held = {n: t.clone() for n, t in kept.items()}
+        for n in names:
+            setattr(a, n, torch.full_like(kept[n], -3))
+        got = a.step(batches[1], 2, sync=True)
+        assert got == c.step(batches[1], 2, sync=True) and got[0] == batches[1].nnz and got[1] == p.img_vocab
+        assert a.d_counts.tolist() == list(got)
+        for n, m in (("ready_ids", got[0]), ("ready_seq", got[0]), ("ready_avg", got[0]), ("expired_ids", got[1])):
+            assert torch.equal(getattr(a, n)[:m], getattr(c, n)[:m]), n
+        for n in names:
+            assert torch.equal(kept[n], held[n]), n
+    finally:
+        a.close()
+        c.close()
