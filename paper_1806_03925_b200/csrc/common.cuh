@@ -3,6 +3,7 @@
 
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
+#include <cfloat>
 #include <stdint.h>
 
 #include <utility>
@@ -107,11 +108,20 @@ __device__ __forceinline__ float4 ld_stream_f4(const float* p) {
 // An fp32 matrix held as three bf16 matrices `stride` elements apart, whose sum it is (head_tc3.cu)
 struct Planes { __nv_bfloat16* p; int64_t stride; };
 
-// two fp32 values as three packed pairs of bf16 (each part rounded to nearest; the three parts of a value sum to it)
+// two fp32 values as three packed pairs of bf16 (each part rounded to nearest; the three parts of a value sum to it).  A value that
+// rounds to infinity has its leading part cut off instead; an infinity or NaN is its leading part alone (inf - inf would make
+// NaN of an infinity).
 __device__ __forceinline__ void split3_pair(float x, float y, uint32_t& p0, uint32_t& p1, uint32_t& p2) {
     const __nv_bfloat162 h0 = __floats2bfloat162_rn(x, y);
     p0 = *reinterpret_cast<const uint32_t*>(&h0);
-    const float rx = x - __uint_as_float(p0 << 16), ry = y - __uint_as_float(p0 & 0xffff0000u);
+    float rx = x - __uint_as_float(p0 << 16), ry = y - __uint_as_float(p0 & 0xffff0000u);
+    if (!(fabsf(rx) + fabsf(ry) <= FLT_MAX)) {               // the rests of values in range are below 2^120
+        const float hx = fabsf(x) <= FLT_MAX ? __uint_as_float(__float_as_uint(x) & 0xffff0000u) : x;
+        const float hy = fabsf(y) <= FLT_MAX ? __uint_as_float(__float_as_uint(y) & 0xffff0000u) : y;
+        const __nv_bfloat162 cut = __floats2bfloat162_rn(hx, hy);
+        p0 = *reinterpret_cast<const uint32_t*>(&cut);
+        rx = fabsf(x) <= FLT_MAX ? x - hx : 0.f; ry = fabsf(y) <= FLT_MAX ? y - hy : 0.f;
+    }
     const __nv_bfloat162 h1 = __floats2bfloat162_rn(rx, ry);
     p1 = *reinterpret_cast<const uint32_t*>(&h1);
     const __nv_bfloat162 h2 = __floats2bfloat162_rn(rx - __uint_as_float(p1 << 16), ry - __uint_as_float(p1 & 0xffff0000u));

@@ -1,5 +1,6 @@
 """Products of the head at the edges of their tiles, against the oracle: fp32 heads (three bf16 planes per matrix) at the fp32
 tolerance (1e-5 of the largest value of a tensor), bf16 heads at theirs."""
+import numpy as np
 import pytest
 import torch
 
@@ -53,3 +54,55 @@ def test_bf16_products_at_tile_edges(B, E, D, hidden):
         pair.step_and_compare(batch, now=1)
     finally:
         pair.close()
+
+
+@pytest.mark.parametrize("bias", [float("inf"), 3.4e38, -float("inf")])
+@pytest.mark.parametrize("head", [F32, BF16])
+def test_units_beyond_the_largest_value(head, bias):
+    """One unit of the top layer saturated by its bias: infinite, or finite but above the largest bf16 value (3.39e38; a bf16 head
+    rounds it to infinity).  The views' probabilities and all gradients but the unit's own output weight are finite: 1e-5 of
+    the largest value against fp64, bf16 1e-2."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1806_03925_b200 import workloads
+    from paper_1806_03925_b200.session import DeviceBatch, GearSession
+    p = PRESETS["tiny"].scaled(dfv_dtype=head, head_dtype=head, hidden=(128, 64))
+    b = BatchSource(p, 3).batch(0)
+    params = workloads.head_params(p, 3)
+    n0, n1 = p.d_in * 128 + 128, 128 * 64
+    params[n0 + n1 + 5] = bias
+    w_out = params[n0 + n1 + 64:-1]
+    w_out[5] = 1e-38
+    s = GearSession(p, params, max_nnz=b.nnz, seed=3, want_debug=True, want_emb_grad=True)
+    try:
+        s.forward_backward(DeviceBatch.from_host(b))
+        t = [torch.from_numpy(a.astype(np.float64)).requires_grad_() for a in
+             (params[:n0 - 128].reshape(p.d_in, 128), params[n0 - 128:n0], params[n0:n0 + n1].reshape(128, 64),
+              params[n0 + n1:n0 + n1 + 64], w_out, params[-1:])]
+        rnd = (lambda v: v) if head == F32 else (lambda v: v + (v.to(torch.bfloat16).to(torch.float64) - v).detach().nan_to_num(0.0))
+        x = s.x_debug.double().cpu().requires_grad_()
+        h = rnd(torch.relu(x @ rnd(t[0]) + t[1]))
+        h = rnd(torch.relu(h @ rnd(t[2]) + t[3]))
+        if head == BF16 and bias == 3.4e38:
+            h = torch.where(h > 3.39e38, torch.full_like(h, float("inf")), h)          # as bf16 rounds it
+        z = h @ t[4] + t[5]
+        y = torch.from_numpy(b.label).double()
+        prob = torch.sigmoid(z)
+        dz = ((prob - y) / b.B).detach()
+        z.backward(dz)                                               # dLoss/dz is p - y, also where the loss is not finite
+        tol = 1e-5 if head == F32 else 1e-2
+        close = lambda got, want: np.testing.assert_allclose(got, want, rtol=0, atol=tol * max(np.abs(want).max(), 1e-30))
+        close(s.prob[:b.B].cpu().numpy(), prob.detach().numpy())
+        grads = [a.grad.numpy().ravel() for a in t]
+        got = s.head_grad.cpu().numpy()
+        own = n0 + n1 + 64 + 5
+        assert np.isfinite(got[own]) == np.isfinite(grads[4][5])
+        if np.isfinite(got[own]):
+            np.testing.assert_allclose(got[own], grads[4][5], rtol=1e-4 if head == F32 else 1e-2)
+        want = np.concatenate(grads)
+        got[own] = want[own] = 0.0
+        for lo, hi in ((0, n0 - 128), (n0 - 128, n0), (n0, n0 + n1), (n0 + n1, n0 + n1 + 64), (n0 + n1 + 64, want.size)):
+            close(got[lo:hi], want[lo:hi])
+        close(s.dX[:b.B].cpu().numpy(), x.grad.numpy())
+    finally:
+        s.close()
