@@ -47,7 +47,7 @@ template <bool HB, int N> __device__ __forceinline__ void store_x(__nv_bfloat16*
         if constexpr (HB) {
             __nv_bfloat162 h = __floats2bfloat162_rn(v[2 * k], v[2 * k + 1]);
             w[0][k] = *reinterpret_cast<uint32_t*>(&h);
-        } else split3_pair(v[2 * k], v[2 * k + 1], w[0][k], w[1][k], w[2][k]);
+        } else split3_pair_any(v[2 * k], v[2 * k + 1], w[0][k], w[1][k], w[2][k]);
     }
     auto put = [&](__nv_bfloat16* dst, const uint32_t* q) {
         if constexpr (N == 8) *reinterpret_cast<uint4*>(dst) = make_uint4(q[0], q[1], q[2], q[3]);

@@ -39,8 +39,8 @@ fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __rest
             const float4 h = make_float4(fmaxf(T::value(acc, i, 4 * j) + b0, 0.f), fmaxf(T::value(acc, i, 4 * j + 1) + b1, 0.f),
                                          fmaxf(T::value(acc, i, 4 * j + 2) + b2, 0.f), fmaxf(T::value(acc, i, 4 * j + 3) + b3, 0.f));
             uint2 p[3];
-            split3_pair(h.x, h.y, p[0].x, p[1].x, p[2].x);
-            split3_pair(h.z, h.w, p[0].y, p[1].y, p[2].y);
+            split3_pair_relu(h.x, h.y, p[0].x, p[1].x, p[2].x);
+            split3_pair_relu(h.z, h.w, p[0].y, p[1].y, p[2].y);
             const int64_t at = (int64_t)m * N + n;
 #pragma unroll
             for (int q = 0; q < 3; ++q) *reinterpret_cast<uint2*>(H + q * h_stride + at) = p[q];

@@ -59,8 +59,8 @@ def test_bf16_products_at_tile_edges(B, E, D, hidden):
 @pytest.mark.parametrize("bias", [float("inf"), 3.4e38, -float("inf")])
 @pytest.mark.parametrize("head", [F32, BF16])
 def test_units_beyond_the_largest_value(head, bias):
-    """One unit of the top layer saturated by its bias: infinite, or finite but above the largest bf16 value (3.39e38; a bf16 head
-    rounds it to infinity).  The views' probabilities and all gradients but the unit's own output weight are finite: 1e-5 of
+    """One unit of the top layer saturated by its bias: infinite, or finite but above the largest bf16 value (3.39e38), which counts
+    as infinite.  The views' probabilities and all gradients but the unit's own output weight are finite: 1e-5 of
     the largest value against fp64, bf16 1e-2."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -83,8 +83,7 @@ def test_units_beyond_the_largest_value(head, bias):
         x = s.x_debug.double().cpu().requires_grad_()
         h = rnd(torch.relu(x @ rnd(t[0]) + t[1]))
         h = rnd(torch.relu(h @ rnd(t[2]) + t[3]))
-        if head == BF16 and bias == 3.4e38:
-            h = torch.where(h > 3.39e38, torch.full_like(h, float("inf")), h)          # as bf16 rounds it
+        h = torch.where(h > 3.39e38, torch.full_like(h, float("inf")), h)
         z = h @ t[4] + t[5]
         y = torch.from_numpy(b.label).double()
         prob = torch.sigmoid(z)
