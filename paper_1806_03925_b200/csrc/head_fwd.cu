@@ -21,7 +21,8 @@ fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __rest
     wait_for_predecessor();
     using T = ChainTile<BM, BN, TM, TN, BK, DEPTH, AHEAD>;
     __shared__ __align__(16) typename T::Smem smem;
-    const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
+    const int m0 = (int)(blockIdx.y + gridDim.y * blockIdx.z) * BM, n0 = blockIdx.x * BN;
+    if (m0 >= M) return;                                            // (the last layer of more row tiles than a grid dimension takes)
     typename T::Acc acc;
 #pragma unroll
     for (int i = 0; i < TM * TN / 2; ++i) acc[i] = 0ull;
@@ -61,10 +62,14 @@ cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const fl
     KernelScope ks(&c.prof, "f32_gemm_fwd", st);
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     auto tiles = [&](int bm, int bn) { return ceil_div(M, bm) * ceil_div(N, bn); };
+    auto grid = [&](int bm, int bn) {
+        const int64_t rows = ceil_div(M, bm), y = rows < 65535 ? rows : 65535;
+        return dim3((unsigned)ceil_div(N, bn), (unsigned)y, (unsigned)ceil_div(rows, y));
+    };
 #define GEAR_FWD(BM, BN, TM, TN, BK, DEPTH, AH, MB) \
-    (wvec ? launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, true>, dim3((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM)), \
+    (wvec ? launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, true>, grid(BM, BN), \
                              dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, A, W, bias, H.p, H.stride, Hf) \
-          : launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, false>, dim3((unsigned)ceil_div(N, BN), (unsigned)ceil_div(M, BM)), \
+          : launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, false>, grid(BM, BN), \
                              dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, A, W, bias, H.p, H.stride, Hf))
     if (2 * tiles(64, 64) >= 3 * sm_count()) return GEAR_FWD(64, 128, 16, 4, 16, 1, 1, 4);
     if (5 * tiles(32, 64) >= 4 * sm_count()) return GEAR_FWD(32, 64, 4, 4, 32, 4, 2, 1);

@@ -289,3 +289,12 @@ def test_no_call_throws_when_the_host_is_out_of_memory(host, warm):
         assert rc == (gb.GEAR_ERR_CUDA if hit else 0) and lib.fake_unfinished() == 0, k
     for c in ctxs:
         assert lib.gear_destroy(c) == 0
+
+
+@pytest.mark.parametrize("head", [0, 1])
+def test_batches_of_millions_of_views_fit_every_grid(host, head):
+    """65536 row tiles of 64 views and one more: no launch has a second or third dimension above 65535."""
+    B = 65_536 * 64 + 1
+    ctx = host.ctx(B, 2 * B, hidden=(128,), head=head)
+    assert host.lib.gear_step(ctx, host.batch(B, 2 * B), 0.1, host.out(), host.lists(2 * B), 1, 1, 1, None, STREAM) == 0
+    assert host.lib.gear_destroy(ctx) == 0
