@@ -48,8 +48,10 @@ def measured_peaks():
     return dict(hbm_gbs=6650.0, bf16_tflops=1590.0, bf16_sustained=1400.0, source="fallback")
 
 
-# an fp32 product of an fp32 head is six bf16 tensor-core products
+# fp32 heads: a backward product is six bf16 tensor-core products; the forward ones are fp32 multiply-adds on the ordinary
+# lanes (SMs x lanes x 2 flop x largest SM clock)
 F32_PRODUCTS = 6
+ALU_F32_TFLOPS = 148 * 128 * 2 * 1.965e9 / 1e12
 
 
 class ClockSampler:
@@ -209,12 +211,15 @@ def roofline_for(name, ms_per_launch, p, stats, peaks):
                 "peak_source": peaks["source"], "work_per_launch": work}
     if name.startswith(("tc_gemm", "tc3_gemm", "f32_gemm")):
         # The head's products are dense contractions: rated by their flops against the tensor peak (bf16 heads; the
-        # sustained figure, since they run inside a long step; a sixth of it for fp32 heads).  memory_frac is
-        # the secondary figure: every operand and the output once, over the measured copy rate.
+        # sustained figure, since they run inside a long step; a sixth of it for the backward products of fp32 heads) or
+        # the fp32 multiply-add peak (their forward ones).  memory_frac is the secondary figure: every operand and the
+        # output once, over the measured copy rate.
         flops, nbytes = models["gemm"][name.rsplit("_", 1)[1]]
         peak, bound, src = peaks["bf16_sustained"] or peaks["bf16_tflops"], "tensor", peaks["source"] + " (sustained bf16)"
         if name.startswith("tc3_gemm"):
             peak, src = peak / F32_PRODUCTS, src + " / %d" % F32_PRODUCTS
+        elif name.startswith("f32_gemm"):
+            peak, bound, src = ALU_F32_TFLOPS, "alu", "148 SMs x 128 FMA lanes x 2 x 1.965 GHz"
         ach = flops / sec / 1e12
         traffic, source = ncu_traffic(name, p, None)
         return {"kernel": name, "bound": bound, "achieved": round(ach, 2), "peak": round(peak, 1), "unit": "TFLOP/s",
@@ -233,12 +238,15 @@ def step_roofline(p, stats, ms_per_step, peaks):
     fan = [p.d_in] + list(p.hidden)
     flops = 6.0 * stats["B"] * (sum(fan[l] * fan[l + 1] for l in range(len(p.hidden))) + fan[-1])
     sec = ms_per_step * 1e-3
-    tensor_peak = (peaks["bf16_sustained"] or peaks["bf16_tflops"]) / (1 if p.head_dtype == "bf16" else F32_PRODUCTS)
+    # an fp32 head's forward third of the flops is rated at the multiply-add peak, the other two thirds at a sixth of the tensor one
+    tensor_peak = peaks["bf16_sustained"] or peaks["bf16_tflops"]
+    bf16 = p.head_dtype == "bf16"
+    math_peak = tensor_peak if bf16 else 3.0 / (1.0 / ALU_F32_TFLOPS + 2.0 * F32_PRODUCTS / tensor_peak)
     return {"bytes_per_step": round(nbytes), "flops_per_step": round(flops),
             "hbm_GB/s": round(nbytes / sec / 1e9, 1), "hbm_frac": round(nbytes / sec / 1e9 / peaks["hbm_gbs"], 4),
-            "math_TFLOP/s": round(flops / sec / 1e12, 2), "math_frac": round(flops / sec / 1e12 / tensor_peak, 4),
-            "math_peak": round(tensor_peak, 1), "math_bound": "tensor",
-            "lower_bound_ms": round(max(nbytes / (peaks["hbm_gbs"] * 1e9), flops / (tensor_peak * 1e12)) * 1e3, 4),
+            "math_TFLOP/s": round(flops / sec / 1e12, 2), "math_frac": round(flops / sec / 1e12 / math_peak, 4),
+            "math_peak": round(math_peak, 1), "math_bound": "tensor" if bf16 else "alu + tensor",
+            "lower_bound_ms": round(max(nbytes / (peaks["hbm_gbs"] * 1e9), flops / (math_peak * 1e12)) * 1e3, 4),
             "peak_source": peaks["source"]}
 
 
@@ -490,7 +498,7 @@ def run_ours(args):
     roof = None
     for kd in kernels:
         r = roofline_for(kd["name"], kd["ms_per_launch"], p, stats, peaks)
-        if r["bound"] in ("hbm", "tensor"):
+        if r["bound"] in ("hbm", "tensor", "alu"):
             roof = r
             roof["share_of_step"] = round(kd["share"], 4)
             break
