@@ -330,7 +330,8 @@ typedef struct {
     int32_t max_batch; int64_t max_nnz;      /* per worker (the workers' own max_batch and max_nnz are at least these) */
     gear_ctx* const* owners;                 /* [world] */
     gear_ctx* const* workers;                /* [world] tables of max_batch / max_batch / max_nnz rows */
-    int32_t* host_stage; int32_t* stage;     /* pinned host memory and device memory of gear_shard_stage_words words each */
+    int32_t* host_stage; int32_t* stage;     /* pinned host memory of gear_shard_host_words words, device memory of
+                                                gear_shard_stage_words words */
     const int32_t* iota;                     /* device: 0, 1, 2, ... max(max_batch, max_nnz) - 1 */
     const gear_step_out* out;                /* [world] workers' outputs (host array).  dX of worker s starts s * max_batch rows behind
                                                 that of worker 0, dfv_grad s * max_nnz rows; prob optional as always */
@@ -341,6 +342,7 @@ typedef struct {                             /* host arrays of one worker's batc
     const int32_t* user_id; const int32_t* url_id; const int32_t* img_off; const int32_t* img_id; const float* label;
 } gear_host_batch;
 int gear_shard_stage_words(int32_t world, int32_t max_batch, int64_t max_nnz, int64_t* words);
+int gear_shard_host_words(int32_t world, int32_t max_batch, int64_t max_nnz, int64_t* words);
 int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches, float lr, int64_t now, int mean_head_grad,
                     int64_t* counts, void* stream);
 

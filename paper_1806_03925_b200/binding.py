@@ -28,7 +28,7 @@ EXPORTS = ("gear_workspace_bytes", "gear_init_tables", "gear_forward_backward", 
            "gear_last_error", "gear_profile_enable", "gear_profile_read", "gear_launch_count",
            "gear_collect_expired_static", "gear_refresh_dfv", "gear_accumulate_collect", "gear_dense_forward",
            "gear_dense_backward", "gear_adam_dense", "gear_fetch_rows", "gear_apply_emb_grad", "gear_profile_timeline", "gear_step",
-           "gear_shard_stage_words", "gear_shard_step")
+           "gear_shard_stage_words", "gear_shard_host_words", "gear_shard_step")
 GEAR_STATIC_EXPIRY_MAX_VOCAB = 16777216
 GEAR_MAX_LOCAL_RANKS = 8
 
@@ -117,6 +117,8 @@ def load() -> C.CDLL:
                             C.c_int, C.POINTER(i64), vp]
     L.gear_shard_stage_words.restype = C.c_int
     L.gear_shard_stage_words.argtypes = [i32, i32, i64, C.POINTER(i64)]
+    L.gear_shard_host_words.restype = C.c_int
+    L.gear_shard_host_words.argtypes = [i32, i32, i64, C.POINTER(i64)]
     L.gear_shard_step.restype = C.c_int
     L.gear_shard_step.argtypes = [C.POINTER(gear_shard_plan), C.POINTER(gear_host_batch), C.c_float, i64, C.c_int, C.POINTER(i64), vp]
     L.gear_fetch_rows.restype = C.c_int
@@ -319,6 +321,12 @@ def gear_step_structs(ctx, bt: gear_batch, lr: float, o: gear_step_out, lists: g
 def gear_shard_stage_words(world: int, max_batch: int, max_nnz: int) -> int:
     n = C.c_int64(0)
     _check(load().gear_shard_stage_words(world, max_batch, max_nnz, C.byref(n)), "gear_shard_stage_words")
+    return n.value
+
+
+def gear_shard_host_words(world: int, max_batch: int, max_nnz: int) -> int:
+    n = C.c_int64(0)
+    _check(load().gear_shard_host_words(world, max_batch, max_nnz, C.byref(n)), "gear_shard_host_words")
     return n.value
 
 

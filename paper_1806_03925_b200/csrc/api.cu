@@ -53,6 +53,8 @@ static int64_t param_count(const gear_config& c) {
     return n + fan + 1;
 }
 
+static int64_t plan_section_count(int64_t max_nnz) { return ceil_div(ceil_div(max_nnz, 1024), 64) + 1; }
+
 int plan_workspace(const gear_config& c, WsPlan* p) {
     memset(p, 0, sizeof(*p));
     size_t off = 0;
@@ -64,7 +66,11 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
     p->loss_blocks = (int)ceil_div(c.max_batch, 8);
     if (p->loss_blocks > 2 * sm_count()) p->loss_blocks = 2 * sm_count();   // two resident blocks of the output-unit kernel per SM
 
+    // what a ctx starts with at zero, one behind the other
     p->state = take(sizeof(DevState));
+    p->plan_sections = take((size_t)plan_section_count(c.max_nnz) * 8);
+    p->exp_cnt = take((size_t)(ceil_div(c.img_vocab, EXP_MARK_TILE) + 1) * sizeof(uint2));
+    p->cleared = off;
     p->x = take(B * d_in * hsz);
     int fan = d_in;
     for (int l = 0; l < c.n_hidden; ++l) {
@@ -89,7 +95,6 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
         p->sort_tot[s] = take((size_t)RS_BUCKETS * 4);
     }
     p->tile_cnt = take((size_t)(ceil_div(c.max_nnz, 1024) + 1) * sizeof(uint2));
-    p->plan_sections = take((size_t)(ceil_div(ceil_div(c.max_nnz, 1024), 64) + 1) * 8);
     p->grp_rec = take((size_t)c.max_nnz * 16);
     p->pmeta = take((size_t)c.max_nnz * 8);
     p->blk_first = take((size_t)acc_max_spans(c.max_nnz) * 4);
@@ -99,7 +104,6 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
     p->emb_gsum[0] = take(B * c.emb_dim * 4);
     p->emb_gsum[1] = take(B * c.emb_dim * 4);
     p->exp_bits = take((size_t)ceil_div(c.img_vocab, 32) * 4);
-    p->exp_cnt = take((size_t)(ceil_div(c.img_vocab, EXP_MARK_TILE) + 1) * sizeof(uint2));
     p->total = off;
     return GEAR_OK;
 }
@@ -319,24 +323,31 @@ static int check_capacity(int64_t cap, int64_t n) {
     return GEAR_ERR_CAPACITY;
 }
 
-// Where things lie in the staging buffer of a partitioned job (words): the five lists of the batches, the numbers of arrivals, and
-// on the device each owner's arrivals per table.
+// Where things lie in the staging buffer of a partitioned job (words): the five lists of the batches, the numbers of arrivals, the
+// owners' results (two 64-bit counts each), and on the device only each owner's arrivals per table.
 struct ShardStage {
-    int64_t list[5], counts, local[3], src[3], words = 0;
+    int64_t list[5], counts, results, local[3], src[3], host_words, words = 0;
     ShardStage(int W, int64_t max_batch, int64_t max_nnz) {
         auto take = [&](int64_t n) { const int64_t at = words; words += (n + 3) / 4 * 4; return at; };
         const int64_t cap[5] = {W * max_batch, W * max_batch, W * max_nnz, W * (max_batch + 1), W * max_batch};
         for (int t = 0; t < 5; ++t) list[t] = take(cap[t]);
         counts = take(3 * W);
+        results = take(4 * W);
+        host_words = words;
         for (int t = 0; t < 3; ++t) { local[t] = take(W * cap[t]); src[t] = take(W * cap[t]); }
     }
 };
 
-// both counts of a step to the ctx's pinned words (one copy where they lie side by side)
-static cudaError_t enqueue_counts(gear_ctx_impl& c, const int64_t* d_n, const int64_t* d_expired, cudaStream_t st) {
-    if (d_expired == d_n + 1) return enqueue_copy(c.h_counts, d_n, 2 * sizeof(int64_t), st);
-    cudaError_t e = enqueue_copy(c.h_counts, d_n, sizeof(int64_t), st);
-    return e == cudaSuccess ? enqueue_copy(c.h_counts + 1, d_expired, sizeof(int64_t), st) : e;
+// both counts of a step to two pinned words (one copy where they lie side by side)
+static cudaError_t enqueue_counts(void* to, const int64_t* d_n, const int64_t* d_expired, cudaStream_t st) {
+    if (d_expired == d_n + 1) return enqueue_copy(to, d_n, 2 * sizeof(int64_t), st);
+    cudaError_t e = enqueue_copy(to, d_n, sizeof(int64_t), st);
+    return e == cudaSuccess ? enqueue_copy(static_cast<char*>(to) + sizeof(int64_t), d_expired, sizeof(int64_t), st) : e;
+}
+// The ctx's two pinned words.  Made when a call first waits for a count: page-locking 16 bytes takes as long as all else that
+// gear_init_tables does besides filling the tables, and the contexts of a partitioned job never need them.
+static cudaError_t pinned_counts(gear_ctx_impl& c) {
+    return c.h_counts ? cudaSuccess : cudaHostAlloc(reinterpret_cast<void**>(&c.h_counts), 2 * sizeof(int64_t), cudaHostAllocDefault);
 }
 
 // What one owner of a partitioned job does with its arrivals.  First what their IDs alone decide: the sort (the sorted values are
@@ -388,7 +399,7 @@ static cudaError_t enqueue_owner_plan(gear_ctx_impl& c, const Arrivals& user, co
 // Then what their gradients do: embedding rows, gradient store and hand-over.
 static cudaError_t enqueue_owner_apply(gear_ctx_impl& c, const Arrivals& user, const Arrivals& url, const Arrivals& img, int sorted_buf,
                                        const float* emb_rows, int64_t emb_ld, const float* img_rows, int64_t img_ld, float lr,
-                                       const gear_step_lists& lists, cudaStream_t st) {
+                                       const gear_step_lists& lists, void* h_counts, cudaStream_t st) {
     int64_t* d_n = lists.d_n ? lists.d_n : &c.state()->pad[0];
     int64_t* d_expired = lists.d_expired ? lists.d_expired : &c.state()->pad[1];
     const bool apart = !c.prof.on || c.prof.keep_streams, plan = c.cfg.accum_mode == GEAR_ACC_SORT && img.n > 0;
@@ -406,7 +417,7 @@ static cudaError_t enqueue_owner_apply(gear_ctx_impl& c, const Arrivals& user, c
         GEAR_TRY(enqueue_record(c.ev[2], side));
         GEAR_TRY(enqueue_wait(st, c.ev[2]));
     }
-    return enqueue_counts(c, d_n, d_expired, st);
+    return enqueue_counts(h_counts, d_n, d_expired, st);
 #undef GEAR_TRY
 }
 
@@ -430,7 +441,7 @@ static void forget_batch(gear_ctx_impl& c) {
     c.scan_cut_off = true;
     c.acc_calls_pending = 2;                    // nothing is known of the ready queue
     c.img_sorted = false; c.img_sort_valid = false; c.plan_ready = false;
-    c.plan_sections_dirty = (int)((c.ws.grp_rec - c.ws.plan_sections) / 8);
+    c.plan_sections_dirty = (int)plan_section_count(c.cfg.max_nnz);
 }
 
 // Writing a call down takes host memory; that it can run out is for the caller to hear, not an exception.
@@ -509,16 +520,12 @@ int gear_init_tables(gear_ctx** out_ctx, const gear_config* cfg, const gear_buff
     for (cudaEvent_t& ev : c.ev) ev = nullptr;
     c.plan_ready = false; c.plan_n = 0; c.plan_src_row = nullptr; c.plan_scale = nullptr;
 
-    c.h_counts = nullptr;
-    cudaError_t e = cudaHostAlloc(reinterpret_cast<void**>(&c.h_counts), 2 * sizeof(int64_t), cudaHostAllocDefault);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c.side_stream, cudaStreamNonBlocking);
+    c.h_counts = nullptr;                                    // made when a count is first asked for
+    cudaError_t e = cudaStreamCreateWithFlags(&c.side_stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c.aux_stream, cudaStreamNonBlocking);
     for (cudaEvent_t& ev : c.ev)
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = enqueue_memset(c.state(), sizeof(DevState), st);
-    // section counts start from zero
-    if (e == cudaSuccess) e = enqueue_memset(c.at<char>(c.ws.plan_sections), c.ws.grp_rec - c.ws.plan_sections, st);
-    if (e == cudaSuccess) e = enqueue_memset(c.at<char>(c.ws.exp_cnt), c.ws.total - c.ws.exp_cnt, st);
+    if (e == cudaSuccess) e = enqueue_memset(c.state(), c.ws.cleared, st);
     if (e == cudaSuccess && fill) {
         const double amp = 0.17320508075688773;   // uniform half-width for standard deviation 0.1
         e = launch_fill_uniform(buf->user_emb, GEAR_F32, cfg->user_vocab * cfg->emb_dim, seed, GEAR_TAG_USER, amp, st);
@@ -594,8 +601,9 @@ int gear_step(gear_ctx* ctx, const gear_batch* batch, float lr, const gear_step_
                       lists->expired, lists->expired_cap, lists->d_expired ? lists->d_expired : &c.state()->pad[1],
                       now, restamp, scan_beside != 0};
     if (int rc = run_call(c, "step", st, [&]() -> cudaError_t {
-            cudaError_t e = enqueue_step(c, *batch, lr, *out, &l, st);
-            return e == cudaSuccess && h_n ? enqueue_counts(c, l.d_n, l.d_expired, st) : e;
+            cudaError_t e = h_n ? pinned_counts(c) : cudaSuccess;
+            if (e == cudaSuccess) e = enqueue_step(c, *batch, lr, *out, &l, st);
+            return e == cudaSuccess && h_n ? enqueue_counts(c.h_counts, l.d_n, l.d_expired, st) : e;
         }))
         return rc;
     if (!h_n) return GEAR_OK;
@@ -608,7 +616,8 @@ int gear_step(gear_ctx* ctx, const gear_batch* batch, float lr, const gear_step_
 
 static int finish_count(gear_ctx_impl& c, const int64_t* d_src, int64_t cap, int64_t* h_n, cudaStream_t st) {
     if (!h_n) return GEAR_OK;
-    cudaError_t e = cudaMemcpyAsync(c.h_counts, d_src, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
+    cudaError_t e = pinned_counts(c);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c.h_counts, d_src, sizeof(int64_t), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_fail(e, "read count");
     *h_n = c.h_counts[0];
@@ -686,6 +695,12 @@ int gear_shard_stage_words(int32_t world, int32_t max_batch, int64_t max_nnz, in
     return GEAR_OK;
 }
 
+int gear_shard_host_words(int32_t world, int32_t max_batch, int64_t max_nnz, int64_t* words) {
+    if (!words || world < 1 || world > GEAR_MAX_LOCAL_RANKS || max_batch < 1 || max_nnz < 1) return arg_fail("gear_shard_host_words");
+    *words = ShardStage(world, max_batch, max_nnz).host_words;
+    return GEAR_OK;
+}
+
 int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches, float lr, int64_t now, int mean_head_grad, int64_t* counts,
                     void* stream) {
     if (!plan || !batches || !counts) return arg_fail("NULL pointer");
@@ -727,7 +742,8 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
     cudaError_t e = cudaSuccess;
     for (int s = 0; s < W; ++s)
         for (gear_ctx_impl* c : {&p.owners[s]->impl, &p.workers[s]->impl})
-            if (e == cudaSuccess && !c->rank_stream) e = cudaStreamCreateWithFlags(&c->rank_stream, cudaStreamNonBlocking);
+            if (e == cudaSuccess && !c->rank_stream && c != &p.owners[0]->impl)           // (owner 0 works on the caller's)
+                e = cudaStreamCreateWithFlags(&c->rank_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cuda_fail(e, "shard_step");
     // ---- the batches: lists sender by sender in the staging buffer, one copy
     const ShardStage at(W, p.max_batch, p.max_nnz);
@@ -851,7 +867,7 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
     if (e == cudaSuccess)
         e = at_owners(stream_of, [&](int s, gear_ctx_impl& c, cudaStream_t where) {
             return enqueue_owner_apply(c, arrived[s][0], arrived[s][1], arrived[s][2], sorted_buf[s], p.out[0].dX, w0.d_in, p.out[0].dfv_grad,
-                                       g0->dfv_dim, lr, p.lists[s], where);
+                                       g0->dfv_dim, lr, p.lists[s], p.host_stage + at.results + 4 * s, where);
         });
     if (e != cudaSuccess) return fail(e);
 #undef GEAR_TRY
@@ -859,8 +875,7 @@ int gear_shard_step(const gear_shard_plan* plan, const gear_host_batch* batches,
     if (e != cudaSuccess) return fail(e);
     int rc = GEAR_OK;
     for (int s = 0; s < W; ++s) {
-        const gear_ctx_impl& c = p.owners[s]->impl;
-        counts[2 * s] = c.h_counts[0]; counts[2 * s + 1] = c.h_counts[1];
+        memcpy(counts + 2 * s, p.host_stage + at.results + 4 * s, 2 * sizeof(int64_t));
         for (int q = 0; q < 2; ++q)
             if (int bad = check_capacity(q ? p.lists[s].expired_cap : p.lists[s].cap, counts[2 * s + q])) rc = bad;
     }

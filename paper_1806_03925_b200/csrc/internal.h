@@ -42,6 +42,7 @@ struct WsPlan {
                                         // batch, in the row of the sorted position where the ID's run starts (Adam only)
     size_t exp_bits;                    // [ceil(img_vocab / 32)] uint32 expired bitmap
     size_t exp_cnt;                     // [expiry mark tiles + 1][2] words: tile counts, two sets of section counts
+    size_t cleared;                     // bytes from the start that a new ctx clears
     size_t total;
     int64_t ready_cap;
     int loss_blocks;
@@ -74,9 +75,9 @@ struct gear_ctx_impl {
     TmaCache* tma;      // tensor maps of the head's products (tc_ptx.cuh)
     cudaStream_t side_stream;          // runs the ID sort of a step beside the gather and the head
     cudaStream_t aux_stream;           // runs the expiry scan and, for small batches, the weight gradients
-    cudaStream_t rank_stream = nullptr;  // a partitioned job's rank other than the first (made on demand)
+    cudaStream_t rank_stream = nullptr;  // a partitioned job's ranks (made on demand)
     cudaEvent_t ev[10];                // between the streams of a step (enqueue_step, gear_shard_step in api.cu)
-    int64_t* h_counts;                 // two counts on their way to the caller (pinned)
+    int64_t* h_counts;                 // two counts on their way to the caller (pinned; made on demand)
     Player player;                     // plays what a call has written down
     mutable Profiler prof;
     mutable bool scan_cut_off = false;      // a call failed: its expiry scan may have been enqueued in part

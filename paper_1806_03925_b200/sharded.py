@@ -295,8 +295,9 @@ class _InProcessStep:
     def __init__(self, sg: ShardedGear):
         self.sg = sg
         W, C = sg.world, gb.C
-        words = gb.gear_shard_stage_words(W, sg.max_batch_local, sg.max_nnz_local)
-        self.host, self.dev = torch.zeros(words, dtype=torch.int32).pin_memory(), torch.zeros(words, dtype=torch.int32, device=sg.workers[0].dev)
+        words = [f(W, sg.max_batch_local, sg.max_nnz_local) for f in (gb.gear_shard_host_words, gb.gear_shard_stage_words)]
+        self.host = torch.empty(words[0], dtype=torch.int32, pin_memory=True)
+        self.dev = torch.empty(words[1], dtype=torch.int32, device=sg.workers[0].dev)
         self.ctxs = [(C.c_void_p * W)(*(s.ctx.value for s in side)) for side in (sg.owners, sg.workers)]
         self.out = (gb.gear_step_out * W)(*(w._make_step_out() for w in sg.workers))
         self.lists_made = [o._lists() for o in sg.owners]

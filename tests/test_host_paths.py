@@ -65,8 +65,8 @@ class Host:
         owners = [self.ctx(batch * world, nnz * world, head=head, img_vocab=100_000) for _ in range(world)]
         workers = [self.ctx(batch, nnz, head=head, mode=gb.GEAR_ACC_ATOMIC, img_vocab=100_000) for _ in range(world)]
         words = C.c_int64()
-        assert lib.gear_shard_stage_words(world, batch, nnz, C.byref(words)) == 0
-        stage = (C.c_int32 * words.value)(*([arrivals] * words.value))
+        assert lib.gear_shard_host_words(world, batch, nnz, C.byref(words)) == 0
+        stage = (C.c_int32 * words.value)(*([arrivals] * (words.value - 4 * world)))          # (the owners' results: zeros)
         dX, rows = self.address(), self.address(1 << 30)
         outs = (gb.gear_step_out * world)(*(self.out(dX=dX + 4 * s * batch * 96, dfv_grad=rows + 4 * s * nnz * 64) for s in range(world)))
         lists = (gb.gear_step_lists * world)(*(self.lists(nnz * world) for _ in range(world)))
@@ -298,3 +298,21 @@ def test_batches_of_millions_of_views_fit_every_grid(host, head):
     ctx = host.ctx(B, 2 * B, hidden=(128,), head=head)
     assert host.lib.gear_step(ctx, host.batch(B, 2 * B), 0.1, host.out(), host.lists(2 * B), 1, 1, 1, None, STREAM) == 0
     assert host.lib.gear_destroy(ctx) == 0
+
+
+def test_a_context_costs_no_pinned_memory_before_a_count_is_waited_for(host):
+    """One clear besides the tables', no page-locked block; the block comes with the first h_n, and a partitioned step needs none
+    (its counts lie in the plan's staging buffer)."""
+    lib = host.lib
+    plan, batches, ctxs = host.shard()
+    log = [line[0] for line in host.log()]
+    assert "pinned" not in log and log.count("memset") == len(ctxs)
+    for _ in range(5):
+        assert host.shard_step(plan, batches) == 0
+    assert "pinned" not in [line[0] for line in host.log()]
+    n = C.c_int64()
+    for k in range(3):
+        assert lib.gear_collect_expired(ctxs[0], 1, 1, host.address(), 1000, None, C.byref(n), STREAM) == 0
+    assert [line[0] for line in host.log()].count("pinned") == 1
+    for c in ctxs:
+        assert lib.gear_destroy(c) == 0
