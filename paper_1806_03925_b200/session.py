@@ -15,6 +15,8 @@ from .workloads import BF16, Batch, GearPreset
 
 
 _WORD = np.dtype(np.int32)
+_NAMES = ("user_id", "url_id", "img_off", "img_id", "label", "fast")
+_FAST_FIRST = ("fast",) + _NAMES[:5]                  # the order of a host batch's copy
 _TORCH = {np.dtype(np.int32): torch.int32, np.dtype(np.float32): torch.float32}
 
 
@@ -29,11 +31,11 @@ class DeviceBatch:
     nnz: int
     fast: Optional[torch.Tensor] = field(default_factory=lambda: None)       # [B][fast_dim] fp32: the views' own dense input
 
-    # A batch whose copy to the device is still on its way (from_host) has its tensors in _arriving: whoever asks for one waits
-    # for the copy and may use it on any stream; GearSession asks for none and is ordered behind the copy by its stream.
+    # A batch whose copy to the device is still on its way (from_host) has no tensors yet, only what they are made from, in _arriving:
+    # whoever asks for one waits for the copy and may use it on any stream; GearSession asks for none and is ordered behind the
+    # copy by its stream.
     def __getattr__(self, name):                      # (called for what is not there yet)
-        arriving = self.__dict__.get("_arriving")
-        if arriving is not None and name in arriving[1]:
+        if name in _NAMES and "_arriving" in self.__dict__:
             self._arrive()
         try:
             return self.__dict__[name]
@@ -42,12 +44,17 @@ class DeviceBatch:
 
     def _arrive(self):
         arriving = self.__dict__.get("_arriving")
-        if arriving is not None:                      # (a second thread may come here meanwhile: taken down last)
-            (device, raw_stream), tensors = arriving
-            torch.cuda.ExternalStream(raw_stream, device).synchronize()
-            for name, t in tensors.items():
-                self.__dict__.setdefault(name, t)
-            self.__dict__.pop("_arriving", None)
+        if arriving is None:
+            return
+        raw_stream, there, sizes, dtypes, fast_shape = arriving
+        torch.cuda.ExternalStream(raw_stream, there.device).synchronize()
+        parts = [t if d == _WORD else t.view(_TORCH.get(d) or getattr(torch, d.name))
+                 for d, t in zip(dtypes, there.split_with_sizes(sizes))]
+        parts.append(parts.pop(0).view(fast_shape) if fast_shape is not None else None)
+        self.__dict__["_c_struct"] = self.__dict__["_c_struct"][0], tuple(parts)
+        for name, t in zip(_NAMES, parts):
+            self.__dict__.setdefault(name, t)
+        self.__dict__.pop("_arriving", None)          # last: a second thread may come here meanwhile
 
     @staticmethod
     def from_host(b: Batch, device="cuda") -> "DeviceBatch":
@@ -66,19 +73,15 @@ class DeviceBatch:
         np.concatenate([(a if a.flags.c_contiguous else np.ascontiguousarray(a)).reshape(-1).view(_WORD) for a in arrays],
                        out=host.numpy())
         there = host.to(device, non_blocking=True)
-        parts = [t if a.dtype == _WORD else t.view(_TORCH.get(a.dtype) or getattr(torch, a.dtype.name))
-                 for a, t in zip(arrays, there.split_with_sizes(sizes))]
-        fast = parts.pop(0).view(b.fast.shape) if b.fast is not None else None
-        names = ("user_id", "url_id", "img_off", "img_id", "label")
-        out = DeviceBatch.__new__(DeviceBatch)
-        out.__dict__.update(B=b.B, nnz=b.nnz, _arriving=((there.device, torch._C._cuda_getCurrentRawStream(there.device.index)),
-                                                         dict(zip(names, parts), fast=fast)))
         # the C struct of the batch: the pointers follow from where the copy went
         c, at = gb.gear_batch(), there.data_ptr()
-        for name, n in zip(("fast",) * (fast is not None) + names, sizes):
+        for name, n in zip(_NAMES if b.fast is None else _FAST_FIRST, sizes):
             setattr(c, name, at)
             at += 4 * n
-        out.__dict__["_c_struct"] = c, (*parts, fast)
+        out = DeviceBatch.__new__(DeviceBatch)
+        out.__dict__.update(B=b.B, nnz=b.nnz, _c_struct=(c, None),
+                            _arriving=(torch._C._cuda_getCurrentRawStream(there.get_device()), there, sizes, [a.dtype for a in arrays],
+                                       None if b.fast is None else b.fast.shape))
         return out
 
 
@@ -197,12 +200,13 @@ class GearSession:
 
     @staticmethod
     def _c_batch(b: DeviceBatch):
-        bt, of = b.__dict__.get("_c_struct", (None, None))
         if "_arriving" in b.__dict__:
-            if len(b.__dict__) == 4 and b.__dict__["_arriving"][0][1] == gb._raw_stream(None):      # no tensor has been put in its place
+            if len(b.__dict__) == 4 and b.__dict__["_arriving"][0] == gb._raw_stream(None):      # no tensor has been put in its place
+                bt = b.__dict__["_c_struct"][0]
                 bt.B, bt.nnz = b.B, b.nnz
                 return bt
             b._arrive()
+        bt, of = b.__dict__.get("_c_struct", (None, None))
         if bt is None or not (of[0] is b.user_id and of[1] is b.url_id and of[2] is b.img_off and of[3] is b.img_id and
                               of[4] is b.label and of[5] is b.fast):
             of = (b.user_id, b.url_id, b.img_off, b.img_id, b.label, b.fast)
