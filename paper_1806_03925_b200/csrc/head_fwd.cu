@@ -50,12 +50,17 @@ fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __rest
     }
 }
 
-// The chain over the reduction cannot be split, so a small batch is spread over as many SMs as it has tiles, in smaller ones the
-// fewer it has, and the fewer warps an SM gets the further ahead it fetches (kernel time; before: one step ahead, at most 32 x 32
-// tiles with 4 x 4 outputs per thread): 32768 views, 192-256-128: 143 -> 139 us; 1024 views, 1632-256-64: 65 -> 52; 1237 views,
-// 120-136 and 256 views, 96-64: steps 39.1 -> 38.8 and 26.5 -> 24.8.  The large tiles issue multiply-adds in half of the
-// cycles; 8 x 4, 8 x 8 and 16 x 4 outputs per thread, pairs along rows or columns, doubled operands in shared memory (178 us)
-// made no other difference.
+// The chain over the reduction cannot be split, so a product takes as long as its fullest SM: the smallest tiles while they are one
+// wave, then the next larger ones, whose blocks have an SM to themselves and fetch further ahead; large tiles, which issue
+// multiply-adds in half of the cycles, from three waves of 64 x 64 on, where their last wave no longer counts.  Measured on
+// either side of each line (us, the form below the line / above it):
+//   16 x 32 | 32 x 32   one wave of 16 x 32:    256 x 256 outputs, depth 192 (0.86 waves) 9.1 / 10.8; 512 x 256 (1.73) 10.7 / 10.9
+//   32 x 32 | 32 x 64   one wave of 32 x 32:    512 x 256 (0.86) 10.9 / 11.2, depth 1632 39.4 / 41.4; 1024 x 256 (1.73) 12.8 / 10.7,
+//                                               depth 1632 53.7 / 42.2; 1536 x 128 (1.30) 12.7 / 10.8
+//   32 x 64 | 64 x 128  three waves of 64 x 64: 5632 x 256 (2.4) 27.1 / 29.9, depth 1632 171 / 196; 7168 x 256 (3.0) 31.3 / 31.3, depth
+//                                               1632 207 / 199; 9472 x 256 (4.0) 35.6 / 31.8; 16384 x 128 (3.5) 35.2 / 31.1
+// (8 x 4, 8 x 8 and 16 x 4 outputs per thread, pairs along rows or columns, doubled operands in shared memory made no other
+// difference to the large ones: 32768 views, 192-256-128: 139 us.)
 cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
                            const Planes& H, float* Hf, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
@@ -71,10 +76,10 @@ cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const fl
                              dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, A, W, bias, H.p, H.stride, Hf) \
           : launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, false>, grid(BM, BN), \
                              dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, A, W, bias, H.p, H.stride, Hf))
-    if (2 * tiles(64, 64) >= 3 * sm_count()) return GEAR_FWD(64, 128, 16, 4, 16, 1, 1, 4);
-    if (5 * tiles(32, 64) >= 4 * sm_count()) return GEAR_FWD(32, 64, 4, 4, 32, 4, 2, 1);
-    if (tiles(16, 32) > sm_count()) return GEAR_FWD(32, 32, 2, 4, 32, 2, 3, 2);
-    return GEAR_FWD(16, 32, 2, 4, 32, 2, 3, 2);
+    if (tiles(16, 32) <= sm_count()) return GEAR_FWD(16, 32, 2, 4, 32, 2, 3, 2);
+    if (tiles(32, 32) <= sm_count()) return GEAR_FWD(32, 32, 2, 4, 32, 2, 3, 2);
+    if (tiles(64, 64) < 3 * sm_count()) return GEAR_FWD(32, 64, 4, 4, 32, 4, 2, 1);
+    return GEAR_FWD(64, 128, 16, 4, 16, 1, 1, 4);
 #undef GEAR_FWD
 }
 

@@ -17,8 +17,9 @@ pytestmark = pytest.mark.gpu
     (256, 16, 480, (136, 120)),             # head input 512 wide: two segments' worth in one, columns one step past 128
     (640, 16, 512, (128, 64)),              # head input 544 wide: the first width that is cut into segments
     (20_000, 4, 24, (1024,)),               # widest layer, a long reduction over the batch
-    # forward tiles of 16 x 32 up to 148 of them, 32 x 32, 32 x 64 from 119 of those, 64 x 128 from 222 tiles of 64 x 64
+    # forward tiles of 16 x 32 up to 148 of them, 32 x 32 up to 148, 32 x 64, 64 x 128 from 444 tiles of 64 x 64
     (1184, 4, 16, (64,)), (1185, 4, 16, (64, 40)), (1889, 8, 88, (128,)), (7105, 4, 24, (120, 136)),
+    (2368, 4, 24, (64,)), (2369, 4, 24, (64, 40)), (14_144, 4, 24, (128,)), (14_145, 4, 24, (120, 136)),
 ])
 def test_fp32_products_at_tile_edges(B, E, D, hidden):
     if not torch.cuda.is_available():
