@@ -106,3 +106,29 @@ def test_struct_layouts_of_the_binding_match_the_header(gb, tmp_path):
             names[0] = names[0].split()[-1]                      # drop the type of the first declarator
             fields += [re.sub(r"\[.*\]", "", n).strip().lstrip("*").strip() for n in names]
         assert fields == [f for f, _ in st._fields_], (name, fields)
+
+
+def test_struct_layouts_of_the_step_calls_match_the_header(gb, tmp_path):
+    """The same for the structures of gear_step and gear_shard_step (every field, in order)."""
+    import shutil
+    import subprocess
+    cc = shutil.which("gcc") or shutil.which("cc")
+    if cc is None:
+        pytest.skip("no C compiler")
+    structs = {"gear_step_lists": gb.gear_step_lists, "gear_shard_plan": gb.gear_shard_plan, "gear_host_batch": gb.gear_host_batch}
+    body = "".join('  printf("%s %%zu\\n", sizeof(%s));\n' % (n, n) +
+                   "".join('  printf("%s.%s %%zu\\n", offsetof(%s, %s));\n' % (n, f[0], n, f[0]) for f in st._fields_)
+                   for n, st in structs.items())
+    src = tmp_path / "layout.c"
+    src.write_text('#include <stdio.h>\n#include <stddef.h>\n#include "gear.h"\nint main(void) {\n%s  return 0;\n}\n' % body)
+    exe = tmp_path / "layout"
+    subprocess.check_call([cc, "-std=c99", "-I", os.path.join(ROOT, "include"), str(src), "-o", str(exe)])
+    seen = dict(line.split() for line in subprocess.check_output([str(exe)], text=True).splitlines())
+    text = re.sub(r"/\*.*?\*/", "", open(os.path.join(ROOT, "include", "gear.h")).read(), flags=re.S)
+    for name, st in structs.items():
+        assert int(seen[name]) == C.sizeof(st), name
+        for field, _ in st._fields_:
+            assert int(seen["%s.%s" % (name, field)]) == getattr(st, field).offset, "%s.%s" % (name, field)
+        decls = re.search(r"typedef struct \{([^}]*)\}\s*%s;" % name, text).group(1)
+        fields = [re.search(r"(\w+)\s*$", part).group(1) for decl in decls.split(";") if decl.strip() for part in decl.split(",")]
+        assert fields == [f for f, _ in st._fields_], name
