@@ -19,6 +19,8 @@
  *                             every completed group.
  *   gear_accumulate_collect   events 5 and 6 as one call.
  *   gear_step                 events 1 to 6 and the expiry scan as one call.
+ *   gear_shard_step           the same for tables partitioned by ID, all ranks on
+ *                             this device.
  *   gear_refresh_dfv          Section 1 / Section 3: recomputed DFVs replace
  *                             expired ones and restart their clocks.
  *   gear_dense_forward /      events 2-3 and the second half of event 6 for a
@@ -45,8 +47,14 @@
  *     GEAR_DEV_BAD_ID bit of the device status word.
  *   - Calls on one ctx must be issued from one host thread at a time and on
  *     one stream (or on streams the caller orders with events).
- *   - A call whose kernels and streams are the same as before (a training loop's) is replayed as a CUDA graph with the new
- *     batch's pointers and sizes; a stream that its owner is capturing gets the kernels one by one.
+ *   - A call whose kernels and streams have come up three times (a training loop's) is replayed as a CUDA graph with the new
+ *     batch's pointers and sizes.
+ *   - Capture: a stream that its owner is capturing gets the kernels one by one.  The owner's graph holds what the call was
+ *     given by value (pointers, sizes, now, lr, adam_step) and the path that the ctx took: capture after a few calls of the
+ *     same kind, with every accumulate call's averages handed over, and replay it in the place of such calls.  A call that
+ *     waits (h_n, gear_status, gear_shard_step) cannot be captured.
+ *   - After GEAR_ERR_CUDA nothing of the call runs on a stream of the library's own any more; the tables may hold a part of
+ *     the call's updates.
  */
 #ifndef GEAR_H
 #define GEAR_H
@@ -107,7 +115,9 @@ typedef struct {
     int32_t emb_dim;       /* columns of the user and URL-hash tables (fp32); multiple of 4, <= 1024 */
     int32_t dfv_dim;       /* columns of the DFV table; multiple of 8, <= 1024 */
     int32_t dfv_dtype;     /* GEAR_F32 | GEAR_BF16: storage type of the DFV table */
-    int32_t head_dtype;    /* GEAR_F32: fp32 FMA head.  GEAR_BF16: operands of the head's matrix products
+    int32_t head_dtype;    /* GEAR_F32: fp32 head (forward products in fp32 multiply-adds, backward ones on the
+                              tensor cores as sums of bf16 parts; an activation above 3.39e38 counts as
+                              infinite).  GEAR_BF16: operands of the head's matrix products
                               (head input, weights, hidden activations, activation gradients) are rounded
                               to bfloat16 (nearest-even); products accumulate in fp32 */
     int32_t n_hidden;      /* 1 or 2 hidden ReLU layers; the output layer is one logistic unit */

@@ -644,7 +644,7 @@ cudaError_t launch_accumulate(const gear_ctx_impl& c, const int32_t* img_id, con
 
 // Events 5 and 6 in one call.  When the host knows the ready queue to be empty (no accumulate call since a collect that
 // could not be refused) and the caller's lists can take every group the n rows could complete, the reduce pass writes
-// ids, emission numbers and averages straight into the caller's lists and its last block reports the count: no
+// ids, emission numbers and averages straight into the caller's lists and its first thread reports the count: no
 // hand-over pass, and the averages cross memory once.  Otherwise: accumulate into the queue, then hand the queue over.
 cudaError_t launch_accumulate_collect(const gear_ctx_impl& c, const int32_t* img_id, const float* grads, int64_t ld,
                                       const int32_t* src_row, const float* scale, int64_t n, int32_t* ids, int32_t* seq,

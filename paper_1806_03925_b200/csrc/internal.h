@@ -73,8 +73,8 @@ struct gear_ctx_impl {
     }
     bool alive;
     TmaCache* tma;      // tensor maps of the head's products (tc_ptx.cuh)
-    cudaStream_t side_stream;          // runs the ID sort of a step beside the gather and the head
-    cudaStream_t aux_stream;           // runs the expiry scan and, for small batches, the weight gradients
+    cudaStream_t side_stream;          // ID sorts, accumulate plan and embedding scatter, beside the gather and the head
+    cudaStream_t aux_stream;           // expiry scan and weight gradients; for small batches the weights' copies as well
     cudaStream_t rank_stream = nullptr;  // a partitioned job's ranks (made on demand)
     cudaEvent_t ev[10];                // between the streams of a step (enqueue_step, gear_shard_step in api.cu)
     int64_t* h_counts;                 // two counts on their way to the caller (pinned; made on demand)
@@ -118,8 +118,8 @@ struct gear_ctx_impl {
     }
 };
 
-// sort_small.cu: one block per array (raw IDs, at most 16384 of them), sorted into the first buffer pair of each job; the block
-// of the last job also plans the accumulate call where plan.totals is set.
+// sort_small.cu: a cluster of eight blocks (one block up to 2048 IDs) per array of at most 32768 raw IDs, sorted into the first
+// buffer pair of each job; the cluster of the last job also plans the accumulate call where plan.totals is set.
 // What a plan is made from and where it goes (plan.cuh).
 struct PlanArgs {
     uint2* totals; uint32_t vocab; const int32_t* cnt; uint4* grp_rec; const int32_t* src_row; const float* scale;
@@ -141,11 +141,10 @@ cudaError_t launch_fill_ts(int64_t* ts, int64_t n, uint64_t seed, int64_t expire
 cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* row_view, float* inv_n,
                           void* x_debug, cudaStream_t st);
 
-// head.cu: forward + backward of the head.  The weights' copies must have been made and head_grad cleared earlier on the same
-// stream (launch_round_weights).  after_dx(arg) is called once dX has been enqueued.  dw_stream: where the weight gradients go;
-// if it is not the head's own stream, it is made to wait for what they read (one event of dw_ev per layer).
-// after_dx: called once dX is on its way.  The weight gradients go to dw_stream (dw_ev: an event per layer, if that is not the
-// head's own stream), each as soon as its operands exist or, dw_last, all of them after dX.
+// head.cu: forward + backward of the head.  The weights' copies must have been made and head_grad cleared before it on its stream
+// (launch_round_weights).  after_dx(arg) is called once dX is on its way.  The weight gradients go to dw_stream; if that is not the
+// head's own stream it is made to wait for what they read (dw_ev: an event per layer), each as soon as its operands exist or,
+// dw_last, all of them after dX.
 struct HeadHooks { cudaError_t (*after_dx)(void*); void* arg; cudaStream_t dw_stream; cudaEvent_t* dw_ev; bool dw_last; };
 cudaError_t launch_head(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o, cudaStream_t st, const HeadHooks& hooks);
 // the weights as the products read them; clears head_grad (all of it, also for an empty batch)
