@@ -160,17 +160,17 @@ def kernel_models(p, stats):
     return m
 
 
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the ncu --set full captures summarised under
-# profiles/, taken on the large_2m workload (same batch and head, 4.6 GB of tables; a full-set capture of the 48.9 GB
-# workload would save and restore tens of GB per pass).  Second entry: what the figure scales with when the bench
+# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the ncu capture of a whole step under profiles/
+# (step_launches_large_2m.md), taken on the large_2m workload (same batch and head, 4.6 GB of tables; a capture of the 48.9 GB
+# workload could save and restore tens of GB per pass).  Second entry: what the figure scales with when the bench
 # runs another workload -- "work" = the kernel's algorithmic bytes (table-bound kernels: traffic grows with the rows
 # touched), "vocab" = image vocabulary, None = same shapes, taken as is.  ncu flushes the L2 before every pass, so
 # re-reads that hit the L2 in a real step count as DRAM traffic here.  A kernel that has changed since its capture
 # must be taken out of this table (traffic is then reported as null).
 NCU_TRAFFIC_LARGE_2M = {
-    "gather_pool": (64.1e6, "l2"), "acc_reduce": (238.0e6, "work"), "expiry_mark": (16.0e6, "vocab"),
-    "head_out": (34.5e6, None), "emb_reduce": (46.9e6, "work"),
-    "tc_gemm_fwd": (69.0e6, None), "tc_gemm_dw": (113.6e6, None), "tc_gemm_dh": (130.4e6, None), "tc_gemm_dx": (110.3e6, None),
+    "gather_pool": (60.4e6, "l2"), "acc_reduce": (235.0e6, "work"), "expiry_mark": (16.0e6, "vocab"),
+    "emb_reduce": (46.8e6, "work"), "tc_gemm_fwd": (61.0e6, None), "tc_gemm_top": (68.1e6, None), "tc_gemm_dw": (110.3e6, None),
+    "tc_gemm_dh": (126.3e6, None), "tc_gemm_dx": (105.5e6, None),
 }
 # algorithmic bytes per launch of the table-bound kernels on large_2m (kernel_models on that workload's batches)
 NCU_WORK_LARGE_2M = {"gather_pool": 222.0e6, "acc_reduce": 224.5e6, "emb_reduce": 58.9e6}
@@ -185,7 +185,7 @@ def ncu_traffic(name, p, work):
         return None, "ncu captures exist for the large-table shapes only"
     bytes_2m, scales_with = NCU_TRAFFIC_LARGE_2M[name]
     if p.name == "large_2m":
-        return round(bytes_2m), "ncu --set full on this workload (large_2m)"
+        return round(bytes_2m), "ncu on this workload (large_2m)"
     if scales_with == "vocab":
         return round(bytes_2m * p.img_vocab / 2_000_000), "ncu on large_2m, scaled by the image vocabulary"
     if scales_with == "work":
