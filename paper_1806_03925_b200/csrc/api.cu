@@ -66,6 +66,10 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
     p->loss_blocks = (int)ceil_div(c.max_batch, 8);
     if (p->loss_blocks > 2 * sm_count()) p->loss_blocks = 2 * sm_count();   // two resident blocks of the output-unit kernel per SM
 
+    // an fp32 head's top layer leaves one per block, up to four resident blocks per SM
+    p->loss_slots = c.head_dtype == GEAR_F32 && ceil_div(c.max_batch, 8) > p->loss_blocks ? (int)ceil_div(c.max_batch, 8) : p->loss_blocks;
+    if (p->loss_slots > 4 * sm_count()) p->loss_slots = 4 * sm_count();
+
     // what a ctx starts with at zero, one behind the other
     p->state = take(sizeof(DevState));
     p->plan_sections = take((size_t)plan_section_count(c.max_nnz) * 8);
@@ -81,7 +85,7 @@ int plan_workspace(const gear_config& c, WsPlan* p) {
         p->wbt[l] = take((size_t)fan * c.hidden[l] * hsz);
         fan = c.hidden[l];
     }
-    p->loss_part = take((size_t)p->loss_blocks * 4);
+    p->loss_part = take((size_t)p->loss_slots * 4);
     if (c.head_dtype == GEAR_F32) p->head_grad = take((size_t)param_count(c) * 4);
     p->sort_n[0] = p->sort_n[1] = c.max_batch;
     p->sort_n[2] = c.max_nnz;

@@ -21,16 +21,17 @@ constexpr int DK = 16;     // tile depth
 // rows[k][c] = sum_r raw[ids[k]][r] * Wd[r][c],  k < min(n, *d_n),  c < D.  An ID outside [0, vocab) gives a zero row.
 // A chain of R multiply-adds per output cannot be cut, so small tiles spread the live rows over the SMs (2500 rows of 1536
 // values, 64 columns: 40 blocks of 64 x 64 took 242 us), and blocks walk the tiles so that a capacity far above the live
-// count costs nothing.  Fetching two steps ahead and reading shared memory four rounds early: 70 -> 57 us for those rows.  AVEC / BVEC: raw rows / Wd rows may be read 16 bytes at a time.
+// count costs nothing.  32 x 32 tiles, 4 x 4 outputs per lane: bound by shared-memory reads (2 x 4 outputs in 16 x 64: 57 us for
+// those rows, this 29).  AVEC / BVEC: raw rows / Wd rows may be read 16 bytes at a time.
+typedef ChainTile<4, 4, 8, 4, 1, 2, 32, 4> DenseTile;
 template <bool AVEC, bool BVEC>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(DenseTile::THREADS)
 dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const float* __restrict__ Wd, int D,
                      const int32_t* __restrict__ ids, int64_t n, const int64_t* __restrict__ d_n,
                      float* __restrict__ rows, int64_t ld, DevState* __restrict__ state) {
     wait_for_predecessor();
-    constexpr int BM = 16, BN = 64, TM = 2, TN = 4;
-    using T = ChainTile<BM, BN, TM, TN, 32, 2, 4>;
-    __shared__ __align__(16) typename T::Smem smem;
+    constexpr int BM = DenseTile::BM, BN = DenseTile::BN;
+    extern __shared__ float4 dyn_smem[];
     __shared__ int64_t row_of[BM];
     if (d_n) { const int64_t live = *d_n; n = live < n ? (live < 0 ? 0 : live) : n; }
     const int n0 = blockIdx.y * BN;
@@ -47,23 +48,25 @@ dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const 
         __syncthreads();
         // the tile's rows are random lines of a large table: all of them on their way at once, so that the steps of the chain wait
         // for the L2 only
-        for (int q = threadIdx.x; q < BM * (int)ceil_div(R, 32); q += 128) {
+        for (int q = threadIdx.x; q < BM * (int)ceil_div(R, 32); q += DenseTile::THREADS) {
             const int64_t id = row_of[q % BM];
             if (id >= 0) asm volatile("prefetch.global.L2 [%0];" :: "l"(raw + id * R + 32 * (q / BM)));
         }
-        typename T::Acc acc;
+        DenseTile::Acc acc;
+        DenseTile::product<AVEC, BVEC>(acc, R, reinterpret_cast<float*>(dyn_smem),
+                                       [&](int r) -> const float* { const int64_t id = row_of[r]; return id >= 0 ? raw + id * R : nullptr; },
+                                       Wd + n0, D, D - n0);
 #pragma unroll
-        for (int i = 0; i < TM * TN / 2; ++i) acc[i] = 0ull;
-        T::product(acc, R, smem, [&](int r, int k) { const int64_t id = row_of[r]; return load4<AVEC>(raw + id * R + k, id >= 0 ? R - k : 0); },
-                   [&](int k, int c) { return load4<BVEC>(Wd + (int64_t)k * D + n0 + c, k < R ? D - (n0 + c) : 0); });
+        for (int i = 0; i < DenseTile::TM; ++i) {
+            const int64_t m = m0 + DenseTile::row(i);
 #pragma unroll
-        for (int i = 0; i < TM; ++i) {
-            const int64_t m = m0 + T::row(i);
-            const int c = n0 + T::col(0);
-            if (m >= n || c >= D) continue;                       // D is a multiple of 8: whole strips
-            float* dst = rows + m * ld + c;
+            for (int j = 0; j < DenseTile::TN / 4; ++j) {
+                const int c = n0 + DenseTile::col(j);
+                if (m >= n || c >= D) continue;                   // D is a multiple of 8: whole strips
+                float* dst = rows + m * ld + c;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) dst[j] = T::value(acc, i, j);
+                for (int e = 0; e < 4; ++e) dst[e] = DenseTile::value(acc, i, 4 * j + e);
+            }
         }
     }
 }
@@ -132,10 +135,15 @@ cudaError_t launch_dense_forward(const gear_ctx_impl& c, const float* raw, int R
                                  int64_t n, const int64_t* d_n, float* rows, int64_t ld, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     KernelScope k(&c.prof, "dense_forward", st);
-    const int64_t want = ceil_div(n, 16), cap = (int64_t)sm_count() * 8;
-    const dim3 grid((unsigned)(want < cap ? want : cap), (unsigned)ceil_div(c.cfg.dfv_dim, 64));
+    const int64_t want = ceil_div(n, DenseTile::BM), cap = (int64_t)sm_count() * 4;
+    const dim3 grid((unsigned)(want < cap ? want : cap), (unsigned)ceil_div(c.cfg.dfv_dim, DenseTile::BN));
     const bool avec = (R & 3) == 0 && (reinterpret_cast<uintptr_t>(raw) & 15u) == 0, bvec = (reinterpret_cast<uintptr_t>(Wd) & 15u) == 0;
-#define GEAR_DF(A, B) launch_dependent(dense_forward_kernel<A, B>, grid, dim3(128), 0, st, raw, c.cfg.img_vocab, R, Wd, c.cfg.dfv_dim, ids, n, d_n, rows, ld, c.state())
+    cudaError_t e = allow_smem<dense_forward_kernel<true, true>>(DenseTile::SMEM);
+    if (e == cudaSuccess) e = allow_smem<dense_forward_kernel<true, false>>(DenseTile::SMEM);
+    if (e == cudaSuccess) e = allow_smem<dense_forward_kernel<false, true>>(DenseTile::SMEM);
+    if (e == cudaSuccess) e = allow_smem<dense_forward_kernel<false, false>>(DenseTile::SMEM);
+    if (e != cudaSuccess) return e;
+#define GEAR_DF(A, B) launch_dependent(dense_forward_kernel<A, B>, grid, dim3(DenseTile::THREADS), (size_t)DenseTile::SMEM, st, raw, c.cfg.img_vocab, R, Wd, c.cfg.dfv_dim, ids, n, d_n, rows, ld, c.state())
     return avec ? (bvec ? GEAR_DF(true, true) : GEAR_DF(true, false)) : (bvec ? GEAR_DF(false, true) : GEAR_DF(false, false));
 #undef GEAR_DF
 }

@@ -321,15 +321,16 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
 
     // forward
     const int HT = p.fan[L];
-    // a bf16 top layer whose columns are one tile of its product takes the output unit along
-    const bool top_fused = BF && HT <= TC_TOP_N;
+    // a top layer whose columns are one tile of its product takes the output unit along
+    const bool top_fused = HT <= (BF ? TC_TOP_N : F32_TOP_N);
     int n_part = 0;                                       // partial losses it leaves
     for (int l = 0; l < L; ++l) {
         const int K = p.fan[l], N = p.fan[l + 1];
-        if (top_fused && l + 1 == L)
-            err = tc_gemm_top(c, "tc_gemm_top", B, N, K, H[l].p, K, Wt[l].p, K, p.b[l], dA[L].p,
-                              TopArgs{p.w_out, p.b_out, bt.label, o.prob, loss_part, p.gw_out, p.gb[l], p.gb_out}, &n_part, st);
-        else if constexpr (BF)
+        if (top_fused && l + 1 == L) {
+            const TopArgs top{p.w_out, p.b_out, bt.label, o.prob, loss_part, p.gw_out, p.gb[l], p.gb_out};
+            if constexpr (BF) err = tc_gemm_top(c, "tc_gemm_top", B, N, K, H[l].p, K, Wt[l].p, K, p.b[l], dA[L].p, top, &n_part, st);
+            else err = launch_fwd_top_f32(c, B, N, K, c.at<float>(c.ws.xf[l]), p.W[l], p.b[l], dA[L], top, &n_part, st);
+        } else if constexpr (BF)
             err = tc_gemm_kmajor(c, "tc_gemm_fwd", B, N, K, H[l].p, K, Wt[l].p, K, 0, H[l + 1].p, N, p.b[l], nullptr, 0, nullptr, LossSum{}, st);
         else
             err = launch_fwd_f32(c, B, N, K, c.at<float>(c.ws.xf[l]), p.W[l], p.b[l], H[l + 1], l + 1 < L ? c.at<float>(c.ws.xf[l + 1]) : nullptr, st);

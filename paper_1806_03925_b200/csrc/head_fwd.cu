@@ -1,5 +1,5 @@
 // Forward products of fp32 heads: H = ReLU(X W + b) with fp32 multiply-adds, every output one chain over the reduction
-// in ascending order.
+// in ascending order; the top layer takes the output unit along.
 //
 // The backward products run on the tensor cores (head_tc3.cu); the forward ones stay on the ordinary lanes because the sign of
 // a pre-activation decides a ReLU branch: a view's gradient depends on it as a whole, so a value that is rounded in another
@@ -14,27 +14,24 @@
 namespace gear {
 
 // WVEC: the weights may be read 16 bytes at a time (the head input and the activations always can).
-template <int BM, int BN, int TM, int TN, int BK, int DEPTH, int AHEAD, int MIN_BLOCKS, bool WVEC>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN), MIN_BLOCKS)
+template <class T, int MIN_BLOCKS, bool WVEC>
+__global__ void __launch_bounds__(T::THREADS, MIN_BLOCKS)
 fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ bias,
            __nv_bfloat16* __restrict__ H, int64_t h_stride, float* __restrict__ Hf) {
     wait_for_predecessor();
-    using T = ChainTile<BM, BN, TM, TN, BK, DEPTH, AHEAD>;
-    __shared__ __align__(16) typename T::Smem smem;
-    const int m0 = (int)(blockIdx.y + gridDim.y * blockIdx.z) * BM, n0 = blockIdx.x * BN;
+    extern __shared__ float4 dyn_smem[];
+    const int m0 = (int)(blockIdx.y + gridDim.y * blockIdx.z) * T::BM, n0 = blockIdx.x * T::BN;
     if (m0 >= M) return;                                            // (the last layer of more row tiles than a grid dimension takes)
     typename T::Acc acc;
+    T::template product<true, WVEC>(acc, K, reinterpret_cast<float*>(dyn_smem),
+                                    [&](int r) -> const float* { return m0 + r < M ? A + (int64_t)(m0 + r) * K : nullptr; }, W + n0, N, N - n0);
 #pragma unroll
-    for (int i = 0; i < TM * TN / 2; ++i) acc[i] = 0ull;
-    T::product(acc, K, smem, [&](int r, int k) { return load4<true>(A + (int64_t)(m0 + r) * K + k, m0 + r < M ? K - k : 0); },
-               [&](int k, int c) { return load4<WVEC>(W + (int64_t)k * N + n0 + c, k < K ? N - (n0 + c) : 0); });
-#pragma unroll
-    for (int j = 0; j < TN / 4; ++j) {
+    for (int j = 0; j < T::TN / 4; ++j) {
         const int n = n0 + T::col(j);
         if (n >= N) continue;                                       // N is a multiple of 8: whole strips
         const float b0 = __ldg(bias + n), b1 = __ldg(bias + n + 1), b2 = __ldg(bias + n + 2), b3 = __ldg(bias + n + 3);
 #pragma unroll
-        for (int i = 0; i < TM; ++i) {
+        for (int i = 0; i < T::TM; ++i) {
             const int m = m0 + T::row(i);
             if (m >= M) continue;
             const float4 h = make_float4(fmaxf(T::value(acc, i, 4 * j) + b0, 0.f), fmaxf(T::value(acc, i, 4 * j + 1) + b1, 0.f),
@@ -50,37 +47,189 @@ fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __rest
     }
 }
 
-// The chain over the reduction cannot be split, so a product takes as long as its fullest SM: the smallest tiles while they are one
-// wave, then the next larger ones, whose blocks have an SM to themselves and fetch further ahead; large tiles, which issue
-// multiply-adds in half of the cycles, from three waves of 64 x 64 on, where their last wave no longer counts.  Measured on
-// either side of each line (us, the form below the line / above it):
-//   16 x 32 | 32 x 32   one wave of 16 x 32:    256 x 256 outputs, depth 192 (0.86 waves) 9.1 / 10.8; 512 x 256 (1.73) 10.7 / 10.9
-//   32 x 32 | 32 x 64   one wave of 32 x 32:    512 x 256 (0.86) 10.9 / 11.2, depth 1632 39.4 / 41.4; 1024 x 256 (1.73) 12.8 / 10.7,
-//                                               depth 1632 53.7 / 42.2; 1536 x 128 (1.30) 12.7 / 10.8
-//   32 x 64 | 64 x 128  three waves of 64 x 64: 5632 x 256 (2.4) 27.1 / 29.9, depth 1632 171 / 196; 7168 x 256 (3.0) 31.3 / 31.3, depth
-//                                               1632 207 / 199; 9472 x 256 (4.0) 35.6 / 31.8; 16384 x 128 (3.5) 35.2 / 31.1
-// (8 x 4, 8 x 8 and 16 x 4 outputs per thread, pairs along rows or columns, doubled operands in shared memory made no other
-// difference to the large ones: 32768 views, 192-256-128: 139 us.)
+// The top hidden layer (its columns are one tile) with all that hangs off it:
+//   h = ReLU(A W + bias);  z = h . w_out + b_out;  p = sigmoid(z);  BCE in its overflow-safe form;  dz = (p - y) / M;
+//   dA[b][j] = dz * w_out[j] where h[b][j] > 0, else 0 (in planes);  gw_out[j] += sum_b h dz;  gb_top[j] += sum_b dA
+// h goes nowhere: nothing after this reads it.  Blocks walk the row tiles, so that the sums of a block leave it once.
+template <class T, int MIN_BLOCKS, bool WVEC>
+__global__ void __launch_bounds__(T::THREADS, MIN_BLOCKS)
+fwd_top_kernel(int M, int N, int K, const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ bias,
+               __nv_bfloat16* __restrict__ dA, int64_t stride, const TopArgs top) {
+    wait_for_predecessor();
+    extern __shared__ float4 dyn_smem[];
+    static_assert(T::TM <= T::LANES_C, "a lane per row of a thread's outputs");
+    constexpr int WARPS = T::WR * T::WC;
+    __shared__ float s_gw[T::WR][T::BN], s_gb[T::WR][T::BN];        // column sums, a row per row of warps
+    __shared__ float s_z[T::WC][T::BM], s_part[2][WARPS];
+    const int lane = (int)lane_id(), lc = lane % T::LANES_C, wr = T::warp_row(), wc = T::warp_col();
+    for (int i = threadIdx.x; i < T::WR * T::BN; i += T::THREADS) { (&s_gw[0][0])[i] = 0.f; (&s_gb[0][0])[i] = 0.f; }
+    float loss = 0.f, dz_sum = 0.f;
+    const float b_out = __ldg(top.b_out);
+    const int m_tiles = (M + T::BM - 1) / T::BM;
+    for (int mt = blockIdx.x; mt < m_tiles; mt += gridDim.x) {
+        const int m0 = mt * T::BM;
+        typename T::Acc acc;
+        T::template product<true, WVEC>(acc, K, reinterpret_cast<float*>(dyn_smem),
+                                        [&](int r) -> const float* { return m0 + r < M ? A + (int64_t)(m0 + r) * K : nullptr; }, W, N, N);
+        // activations; a lane's part of its rows' dot products
+        float z[T::TM];
+#pragma unroll
+        for (int i = 0; i < T::TM; ++i) z[i] = 0.f;
+        float h[T::TM][T::TN];
+#pragma unroll
+        for (int c = 0; c < T::TN; ++c) {
+            const int n = T::col(c / 4) + c % 4;
+            const bool on = n < N;
+            const float b = on ? __ldg(bias + n) : 0.f, w = on ? __ldg(top.w_out + n) : 0.f;
+#pragma unroll
+            for (int i = 0; i < T::TM; ++i) {
+                const float v = fmaxf(T::value(acc, i, c) + b, 0.f);
+                h[i][c] = v >= 0x1.ffp127f ? __int_as_float(0x7f800000) : v;       // beyond the largest bf16 value: as infinite as in planes
+                if (on) z[i] = fmaf(h[i][c], w, z[i]);
+            }
+        }
+#pragma unroll
+        for (int s = 1; s < T::LANES_C; s <<= 1)
+#pragma unroll
+            for (int i = 0; i < T::TM; ++i) z[i] += __shfl_xor_sync(0xffffffffu, z[i], s);
+        if (T::WC > 1) {
+            if (lc == 0)
+#pragma unroll
+                for (int i = 0; i < T::TM; ++i) s_z[wc][T::row(i)] = z[i];
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < T::TM; ++i) {
+                z[i] = s_z[0][T::row(i)];
+#pragma unroll
+                for (int q = 1; q < T::WC; ++q) z[i] += s_z[q][T::row(i)];
+            }
+        }
+        // lane lc of a row group works out row lc: sigmoid, loss, dz
+        float zz = z[0];
+        int m = m0 + T::row(0);
+#pragma unroll
+        for (int i = 1; i < T::TM; ++i) if (lc == i) { zz = z[i]; m = m0 + T::row(i); }
+        zz += b_out;
+        const float y = m < M ? __ldg(top.label + m) : 0.f;
+        const float p = 1.0f / (1.0f + expf(-zz));
+        const float dz = m < M ? (p - y) / (float)M : 0.f;
+        if (lc < T::TM && wc == 0 && m < M) {
+            loss += fmaxf(zz, 0.f) - zz * y + log1pf(expf(-fabsf(zz)));
+            dz_sum += dz;
+            if (top.prob) top.prob[m] = p;
+        }
+        float g[T::TM];
+#pragma unroll
+        for (int i = 0; i < T::TM; ++i) g[i] = __shfl_sync(0xffffffffu, dz, (lane - lc) + i);
+#pragma unroll
+        for (int j = 0; j < T::TN / 4; ++j) {
+            const int n = T::col(j);
+            float gw[4], gb[4], w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) { gw[e] = gb[e] = 0.f; w[e] = n < N ? __ldg(top.w_out + n + e) : 0.f; }
+#pragma unroll
+            for (int i = 0; i < T::TM; ++i) {
+                const int row = m0 + T::row(i);
+                if (row >= M || n >= N) continue;                    // N is a multiple of 8: whole strips
+                float d[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const float v = h[i][4 * j + e];
+                    gw[e] = fmaf(v, g[i], gw[e]);
+                    d[e] = v > 0.f ? g[i] * w[e] : 0.f;
+                    gb[e] += d[e];
+                }
+                uint2 q[3];
+                split3_pair(d[0], d[1], q[0].x, q[1].x, q[2].x);
+                split3_pair(d[2], d[3], q[0].y, q[1].y, q[2].y);
+#pragma unroll
+                for (int t = 0; t < 3; ++t) *reinterpret_cast<uint2*>(dA + t * stride + (int64_t)row * N + n) = q[t];
+            }
+#pragma unroll
+            for (int s = T::LANES_C; s < 32; s <<= 1)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { gw[e] += __shfl_xor_sync(0xffffffffu, gw[e], s); gb[e] += __shfl_xor_sync(0xffffffffu, gb[e], s); }
+            if (lane < T::LANES_C)                                  // the warp's own words: nobody else adds to them
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { s_gw[wr][n + e] += gw[e]; s_gb[wr][n + e] += gb[e]; }
+        }
+    }
+    loss = warp_sum(loss);
+    dz_sum = warp_sum(dz_sum);
+    if (lane == 0) { s_part[0][threadIdx.x / 32] = loss; s_part[1][threadIdx.x / 32] = dz_sum; }
+    __syncthreads();
+    for (int n = threadIdx.x; n < N; n += T::THREADS) {
+        float gw = s_gw[0][n], gb = s_gb[0][n];
+#pragma unroll
+        for (int q = 1; q < T::WR; ++q) { gw += s_gw[q][n]; gb += s_gb[q][n]; }
+        atomicAdd(top.gw_out + n, gw);
+        atomicAdd(top.gb_top + n, gb);
+    }
+    if (threadIdx.x == 0) {
+        float l = 0.f, t = 0.f;
+        for (int q = 0; q < WARPS; ++q) { l += s_part[0][q]; t += s_part[1][q]; }
+        top.loss_part[blockIdx.x] = l;
+        atomicAdd(top.gb_out, t);
+    }
+}
+
+template <class T, int MIN_BLOCKS, bool WVEC>
+static cudaError_t launch_form(int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& H, float* Hf, cudaStream_t st) {
+    constexpr auto kernel = fwd_kernel<T, MIN_BLOCKS, WVEC>;
+    if (const cudaError_t e = allow_smem<kernel>(T::SMEM)) return e;
+    const int64_t rows = ceil_div(M, T::BM), y = rows < 65535 ? rows : 65535;
+    return launch_dependent(kernel, dim3((unsigned)ceil_div(N, T::BN), (unsigned)y, (unsigned)ceil_div(rows, y)), dim3(T::THREADS),
+                            (size_t)T::SMEM, st, M, N, K, A, W, bias, H.p, H.stride, Hf);
+}
+
+template <class T, int MIN_BLOCKS, bool WVEC>
+static cudaError_t launch_top_form(int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& dA, const TopArgs& top,
+                                   int slots, int* n_part, cudaStream_t st) {
+    constexpr auto kernel = fwd_top_kernel<T, MIN_BLOCKS, WVEC>;
+    if (const cudaError_t e = allow_smem<kernel>(T::SMEM)) return e;
+    const int64_t tiles = ceil_div(M, T::BM), resident = (int64_t)sm_count() * MIN_BLOCKS;
+    const int64_t most = resident < slots ? resident : slots;
+    *n_part = (int)(tiles < most ? tiles : most);
+    return launch_dependent(kernel, dim3((unsigned)*n_part), dim3(T::THREADS), (size_t)T::SMEM, st, M, N, K, A, W, bias, dA.p, dA.stride, top);
+}
+
+// Forms of a tile: outputs per lane, lanes, warps, steps per buffer, buffers.
+typedef ChainTile<2, 4, 4, 8, 2, 1, 32, 4> F16x32;
+typedef ChainTile<4, 4, 8, 4, 1, 2, 32, 4> F32x32;
+typedef ChainTile<8, 8, 4, 8, 2, 2, 32, 2> F64x128;
+typedef ChainTile<2, 4, 4, 8, 1, 2, 32, 4> F8x64;
+typedef ChainTile<4, 4, 4, 8, 1, 2, 32, 4> F16x64;
+typedef ChainTile<8, 8, 4, 8, 2, 1, 32, 2> F64x64;
+typedef ChainTile<2, 4, 4, 8, 1, 4, 32, 3> F8x128;
+typedef ChainTile<4, 4, 4, 8, 1, 4, 32, 3> F16x128;
+typedef ChainTile<4, 4, 4, 8, 1, 8, 32, 3> F16x256;
+typedef ChainTile<8, 8, 4, 8, 1, 4, 32, 2> F32x256;
+
 cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
                            const Planes& H, float* Hf, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     KernelScope ks(&c.prof, "f32_gemm_fwd", st);
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     auto tiles = [&](int bm, int bn) { return ceil_div(M, bm) * ceil_div(N, bn); };
-    auto grid = [&](int bm, int bn) {
-        const int64_t rows = ceil_div(M, bm), y = rows < 65535 ? rows : 65535;
-        return dim3((unsigned)ceil_div(N, bn), (unsigned)y, (unsigned)ceil_div(rows, y));
-    };
-#define GEAR_FWD(BM, BN, TM, TN, BK, DEPTH, AH, MB) \
-    (wvec ? launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, true>, grid(BM, BN), \
-                             dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, A, W, bias, H.p, H.stride, Hf) \
-          : launch_dependent(fwd_kernel<BM, BN, TM, TN, BK, DEPTH, AH, MB, false>, grid(BM, BN), \
-                             dim3((BM / TM) * (BN / TN)), 0, st, M, N, K, A, W, bias, H.p, H.stride, Hf))
-    if (tiles(16, 32) <= sm_count()) return GEAR_FWD(16, 32, 2, 4, 32, 2, 3, 2);
-    if (tiles(32, 32) <= sm_count()) return GEAR_FWD(32, 32, 2, 4, 32, 2, 3, 2);
-    if (tiles(64, 64) < 3 * sm_count()) return GEAR_FWD(32, 64, 4, 4, 32, 4, 2, 1);
-    return GEAR_FWD(64, 128, 16, 4, 16, 1, 1, 4);
+#define GEAR_FWD(T, MB) (wvec ? launch_form<T, MB, true>(M, N, K, A, W, bias, H, Hf, st) : launch_form<T, MB, false>(M, N, K, A, W, bias, H, Hf, st))
+    if (tiles(16, 32) <= sm_count()) return GEAR_FWD(F16x32, 4);
+    if (tiles(64, 128) <= sm_count()) return GEAR_FWD(F32x32, 4);
+    return GEAR_FWD(F64x128, 3);
 #undef GEAR_FWD
+}
+
+cudaError_t launch_fwd_top_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
+                               const Planes& dA, const TopArgs& top, int* n_part, cudaStream_t st) {
+    KernelScope ks(&c.prof, "f32_gemm_top", st);
+    const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
+    const int slots = c.ws.loss_slots;
+#define GEAR_TOP(T, MB) (wvec ? launch_top_form<T, MB, true>(M, N, K, A, W, bias, dA, top, slots, n_part, st) \
+                              : launch_top_form<T, MB, false>(M, N, K, A, W, bias, dA, top, slots, n_part, st))
+    if (N <= 32) return ceil_div(M, 16) <= sm_count() ? GEAR_TOP(F16x32, 4) : GEAR_TOP(F32x32, 4);
+    if (N <= 64) return ceil_div(M, 8) <= sm_count() ? GEAR_TOP(F8x64, 4) : ceil_div(M, 64) <= sm_count() ? GEAR_TOP(F16x64, 4) : GEAR_TOP(F64x64, 4);
+    if (N <= 128) return ceil_div(M, 8) <= sm_count() ? GEAR_TOP(F8x128, 3) : ceil_div(M, 64) <= sm_count() ? GEAR_TOP(F16x128, 3) : GEAR_TOP(F64x128, 3);
+    return ceil_div(M, 32) <= sm_count() ? GEAR_TOP(F16x256, 2) : GEAR_TOP(F32x256, 2);
+#undef GEAR_TOP
 }
 
 }  // namespace gear

@@ -22,7 +22,7 @@ struct WsPlan {
     size_t h[MAX_LAYERS];               // [max_batch][hidden[l]] post-ReLU activations
     size_t da[MAX_LAYERS];              // [max_batch][hidden[l]] gradient at the pre-activation
     size_t xf[MAX_LAYERS];              // fp32 head: the inputs of its layers (head input, lower hidden activations) in fp32
-    size_t loss_part;                   // [loss_blocks] fp32 per-block partial losses
+    size_t loss_part;                   // [loss_slots] fp32 per-block partial losses
     size_t head_grad;                   // fp32 head: the parameters' gradient, when the caller's array is not 16-byte aligned
     size_t wb[MAX_LAYERS];              // W_l as [in][out]
     size_t wbt[MAX_LAYERS];             // W_l as [out][in]
@@ -46,6 +46,7 @@ struct WsPlan {
     size_t total;
     int64_t ready_cap;
     int loss_blocks;
+    int loss_slots;                // words of loss_part: most partial losses a batch can have
 };
 
 int plan_workspace(const gear_config& c, WsPlan* p);
@@ -176,6 +177,11 @@ cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int
 // head_fwd.cu: H = ReLU(A W + bias), A [M][K], W [K][N] fp32; H in planes and, if Hf is given, in fp32
 cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
                            const Planes& H, float* Hf, cudaStream_t st);
+// The same for the top hidden layer, N at most F32_TOP_N, with the output unit behind it (as tc_gemm_top): dA gets, in planes, the
+// gradient with respect to its pre-activations.
+constexpr int F32_TOP_N = 256;
+cudaError_t launch_fwd_top_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
+                               const Planes& dA, const TopArgs& top, int* n_part, cudaStream_t st);
 
 // head_tc3.cu: the backward products of fp32 matrices held as three bf16 planes.  With a mask (the leading plane of the
 // activations) the output goes to planes, masked, and colsum[n] += its column sums; without, to out_f32.
