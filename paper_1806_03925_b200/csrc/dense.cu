@@ -34,8 +34,13 @@ dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const 
     extern __shared__ float4 dyn_smem[];
     __shared__ int64_t row_of[BM];
     if (d_n) { const int64_t live = *d_n; n = live < n ? (live < 0 ? 0 : live) : n; }
-    const int n0 = blockIdx.y * BN;
-    for (int64_t m0 = (int64_t)blockIdx.x * BM; m0 < n; m0 += (int64_t)gridDim.x * BM) {
+    // Column tiles of a row tile are neighbours in the order, and the live tiles the first blocks', which sit on different SMs (with
+    // a grid dimension for the columns the live blocks of its second half piled up four to an SM: 29 us became 57)
+    const int n_tiles = (D + BN - 1) / BN;
+    const int64_t tiles = (n + BM - 1) / BM * n_tiles;
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int64_t m0 = t / n_tiles * BM;
+        const int n0 = (int)(t % n_tiles) * BN;
         __syncthreads();                                          // the tile before this one has been read
         if (threadIdx.x < BM) {
             int64_t id = -1;
@@ -135,8 +140,8 @@ cudaError_t launch_dense_forward(const gear_ctx_impl& c, const float* raw, int R
                                  int64_t n, const int64_t* d_n, float* rows, int64_t ld, cudaStream_t st) {
     if (n <= 0) return cudaSuccess;
     KernelScope k(&c.prof, "dense_forward", st);
-    const int64_t want = ceil_div(n, DenseTile::BM), cap = (int64_t)sm_count() * 4;
-    const dim3 grid((unsigned)(want < cap ? want : cap), (unsigned)ceil_div(c.cfg.dfv_dim, DenseTile::BN));
+    const int64_t want = ceil_div(n, DenseTile::BM) * ceil_div(c.cfg.dfv_dim, DenseTile::BN), cap = (int64_t)sm_count() * 4;
+    const dim3 grid((unsigned)(want < cap ? want : cap));
     const bool avec = (R & 3) == 0 && (reinterpret_cast<uintptr_t>(raw) & 15u) == 0, bvec = (reinterpret_cast<uintptr_t>(Wd) & 15u) == 0;
     cudaError_t e = allow_smem<dense_forward_kernel<true, true>>(DenseTile::SMEM);
     if (e == cudaSuccess) e = allow_smem<dense_forward_kernel<true, false>>(DenseTile::SMEM);

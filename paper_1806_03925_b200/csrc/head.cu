@@ -202,7 +202,7 @@ struct RoundArgs {
 // 32 x 32 tiles through shared memory, so that both copies are written with coalesced rows
 template <int PLANES>
 __global__ void __launch_bounds__(256)
-round_weights_kernel(const RoundArgs a) {
+round_weights_kernel(const __grid_constant__ RoundArgs a) {
     wait_for_predecessor();
     {
         const int64_t blk = blockIdx.x + (int64_t)gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
