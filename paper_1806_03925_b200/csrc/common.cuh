@@ -185,6 +185,12 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
 // block of such a kernel must make the call, first thing, or the chain of completions would break.
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// The next kernel in the stream may be set up beside this one from here on.  It still waits for this one to complete, and, since this
+// is called behind wait_for_predecessor(), for all before it.  For launches that leave SMs to it: on SMs that are full, blocks
+// which only wait keep the kernels of other streams out.
+constexpr unsigned FEW_BLOCKS = 128;
+__device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_as(Op::Attr attr, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
     OpList local;

@@ -153,6 +153,7 @@ template <typename TD, bool HB, int NQ, bool FULL>
 __global__ void __launch_bounds__(GP_WARPS * 32, NQ <= 2 ? 3 : 2)
 gather_pool_kernel(const GatherArgs a) {
     wait_for_predecessor();
+    if (gridDim.x <= FEW_BLOCKS) let_successor_start();
     constexpr int PER = Chunk<TD>::PER;
     constexpr int KMAX = NQ >= 8 ? 1 : 8 / NQ;               // rows in flight per warp
     const int lane = (int)lane_id();

@@ -19,6 +19,7 @@ __global__ void __launch_bounds__(T::THREADS, MIN_BLOCKS)
 fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ bias,
            __nv_bfloat16* __restrict__ H, int64_t h_stride, float* __restrict__ Hf) {
     wait_for_predecessor();
+    if (gridDim.x * gridDim.y <= FEW_BLOCKS) let_successor_start();
     extern __shared__ float4 dyn_smem[];
     const int m0 = (int)(blockIdx.y + gridDim.y * blockIdx.z) * T::BM, n0 = blockIdx.x * T::BN;
     if (m0 >= M) return;                                            // (the last layer of more row tiles than a grid dimension takes)
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(T::THREADS, MIN_BLOCKS)
 fwd_top_kernel(int M, int N, int K, const float* __restrict__ A, const float* __restrict__ W, const float* __restrict__ bias,
                __nv_bfloat16* __restrict__ dA, int64_t stride, const TopArgs top) {
     wait_for_predecessor();
+    if (gridDim.x * gridDim.y <= FEW_BLOCKS) let_successor_start();
     extern __shared__ float4 dyn_smem[];
     static_assert(T::TM <= T::LANES_C, "a lane per row of a thread's outputs");
     constexpr int WARPS = T::WR * T::WC;

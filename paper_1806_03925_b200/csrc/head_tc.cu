@@ -53,17 +53,23 @@ template <int BN, int EW, int EPI> struct TcCfg {
     static constexpr int B_BYTES = BN * TC_BK * 2;               // 32 KB or 16 KB
     static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
     // one output block per epilogue warp; the top layer's epilogue holds a warp's whole part of the tile
-    static constexpr int OUT_BYTES = EW * TC_OUT_BLOCK * (EPI == TC_EPI_TOP ? BN / (EW / 4) / 64 : 1);
-    static constexpr int MASK_BYTES = EPI == TC_EPI_MASK ? EW * 2 * TC_MASK_BLOCK : 0;
+    // (64-column tiles in bf16: blocks of 64 bytes a row, one mask block)
+    static constexpr bool NARROW = BN == 64;
+    static constexpr int OUT_BYTES = EW * TC_OUT_BLOCK * (EPI == TC_EPI_TOP ? BN / (EW / 4) / 64 : 1) / (NARROW && (EPI == TC_EPI_BIAS_RELU || EPI == TC_EPI_MASK) ? 2 : 1);
+    static constexpr int MASK_BYTES = EPI == TC_EPI_MASK ? EW * (NARROW ? 1 : 2) * TC_MASK_BLOCK : 0;
     // per-CTA column sums of the masked product; the top layer's vectors and sums
     static constexpr int COLSUM_BYTES = EPI == TC_EPI_MASK ? TC_MAX_N * 4 : EPI == TC_EPI_TOP ? (int)sizeof(TopSmem) : 0;
     static constexpr int FIXED = 1024 /*alignment slack*/ + 512 /*barriers*/ + COLSUM_BYTES + OUT_BYTES + MASK_BYTES;
     static constexpr int ROOM = (227 * 1024 - FIXED) / STAGE_BYTES;
-    static constexpr int STAGES = ROOM > (BN == 256 ? 4 : 6) ? (BN == 256 ? 4 : 6) : ROOM;
+    // Tiles of 64 columns take half an SM's shared memory: the next product's CTA is set up beside this one's (4096 views: the step
+    // 54.3 -> 52.1 us, 3001 views: 51.2 -> 48.4).
+    static constexpr int MOST = BN == 256 ? 4 : NARROW ? 3 : 6;
+    static constexpr int STAGES = ROOM > MOST ? MOST : ROOM;
     static constexpr int SMEM = STAGES * STAGE_BYTES + FIXED;
     static constexpr int TMEM_COLS = BN == 192 ? 512 : 2 * BN;   // two accumulator buffers (a power of two is allocated)
     static_assert(STAGES >= 3, "operand ring too short");
-    static_assert(SMEM > 116 * 1024, "one CTA per SM: two CTAs would both ask for tensor memory");
+    static_assert(NARROW || SMEM > 116 * 1024, "one CTA per SM: two CTAs would both ask for tensor memory");
+    static_assert(!NARROW || SMEM <= 112 * 1024, "two CTAs per SM");
     static_assert(SMEM <= 227 * 1024, "shared memory budget");
 };
 
@@ -77,6 +83,7 @@ struct TcArgs {
     int32_t* err;             // device word that receives a non-zero code on a timeout
     TopArgs top;              // top layer only
     LossSum loss;             // the loss to finish
+    int let_next;             // the next kernel in the stream may be set up beside this one
 };
 
 // Epilogue of one finished accumulator buffer `a`, as run by one of the epilogue warps: warp w reads
@@ -413,6 +420,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
     tc_fence_after();
     const uint32_t tmem_base = *tmem_word_ptr;
     wait_for_predecessor();      // barriers, tensor memory and descriptors are set up while the previous kernel drains
+    if (g.let_next) let_successor_start();
 
     if (warp == 0) {
         // ---------------- TMA producer
@@ -497,7 +505,7 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
         // where this warp's part of tile t starts
         auto part_m0 = [&](int t) { return ((t / g.n_tiles) % g.m_tiles) * TC_BM + (warp & 3) * 32; };
         auto part_col0 = [&](int t) { return (t % g.n_tiles) * BN + ((warp - 2) >> 2) * COLS; };
-        MaskPipe mp{&map_mask, mask_blocks + (uint32_t)((warp - 2) * 2 * TC_MASK_BLOCK), mask_bar(warp - 2, 0), 0u, 0u, -1, -1};
+        MaskPipe mp{&map_mask, mask_blocks + (uint32_t)((warp - 2) * (Cfg::MASK_BYTES / EW)), mask_bar(warp - 2, 0), 0u, 0u, -1, -1};
         if (EPI == TC_EPI_MASK && (int)blockIdx.x < total_tiles) {
             // the masks of the first tile's first two blocks (after the wait for the previous kernel, which wrote them)
             mask_request(mp, 0, part_col0(blockIdx.x), part_m0(blockIdx.x), lane);
@@ -570,8 +578,9 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
 
 // Eight epilogue warps, at most 128 registers per thread: a CTA (320 threads) then fits on an SM beside a block of
 // the ID sort.  One CTA per SM follows from the shared-memory footprint.
+// (64-column tiles: few enough for two CTAs, the top layer's of 128 columns for one of each.)
 template <int BN, bool MN_MAJOR, int EPI>
-__global__ void __maxnreg__(128)
+__global__ void __maxnreg__(BN == 64 ? 88 : EPI == TC_EPI_TOP && BN == 128 ? 112 : 128)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_mask, const TcArgs g) {
     tc_gemm_body<BN, MN_MAJOR, EPI, 8>(map_a, map_b, map_out, map_mask, g);
@@ -631,7 +640,7 @@ static bool make_map_mask(const gear_ctx_impl& c, CUtensorMap* m, const void* pt
 
 template <int BN, bool MN, int EPI, int EW>
 static cudaError_t launch_variant(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mo, const CUtensorMap& mm,
-                                  const TcArgs& g, cudaStream_t st) {
+                                  TcArgs g, cudaStream_t st) {
     using Cfg = TcCfg<BN, EW, EPI>;
     static_assert(EW == 8, "one kernel entry point: eight epilogue warps");
     auto kernel = tc_gemm_kernel<BN, MN, EPI>;
@@ -643,6 +652,9 @@ static cudaError_t launch_variant(const CUtensorMap& ma, const CUtensorMap& mb, 
     }
     const int tiles = g.m_tiles * g.n_tiles * g.k_splits;
     const int grid = tiles < sm_count() ? tiles : sm_count();
+    // (Larger products gain nothing, and CTAs that wait on an SM keep the kernels of other streams from it: 65 k views, all products:
+    // step 369 -> 373 us.  dX: its successor is the store, which would keep the weight gradients out.)
+    if (BN == 64 && EPI != TC_EPI_F32 && !MN) g.let_next = 1;
     return launch_dependent(kernel, dim3(grid), dim3(tc_threads(EW)), (size_t)Cfg::SMEM, st, ma, mb, mo, mm, g);
 }
 

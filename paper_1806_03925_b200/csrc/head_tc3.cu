@@ -185,6 +185,7 @@ t3_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     tc_fence_after();
     const uint32_t tmem_base = *tmem_word_ptr;
     wait_for_predecessor();
+    if (EPI != T3_F32 && gridDim.x <= FEW_BLOCKS) let_successor_start();
 
     if (warp == 0) {
         // ---------------- TMA producer
