@@ -195,7 +195,20 @@ static cudaError_t launch_top_form(int M, int N, int K, const float* A, const fl
     return launch_dependent(kernel, dim3((unsigned)*n_part), dim3(T::THREADS), (size_t)T::SMEM, st, M, N, K, A, W, bias, dA.p, dA.stride, top);
 }
 
-// Forms of a tile: outputs per lane, lanes, warps, steps per buffer, buffers.
+// Forms of a tile: outputs per lane, lanes, warps, steps per buffer, buffers.  The chain over the reduction cannot be split, so a
+// product takes as long as its fullest SM: small tiles while they are about one wave, then 4 x 4 outputs per lane, then 8 x 8, which
+// need several warps per scheduler to hide their longer rounds.  Measured on either side of each line, depth 192 (us, the form below
+// the line / above it):
+//   16 x 32 | 32 x 32   one wave of 16 x 32:      1024 x 64 (0.9 waves) 3.5 / 4.8; 1024 x 256 (3.5) 6.3 / 5.4
+//   32 x 32 | 64 x 128  six waves of 32 x 32:     2048 x 256 (3.5) 8.3 / 13.2; 4096 x 256 (6.9) 15.0 / 13.5; 8192 x 256 24.4 / 21.4
+// and with the output unit (all columns in one tile):
+//   16 x 32 | 32 x 32   two waves of 16 rows:     4096 views (1.7) 6.2 / 6.9; 8192 (3.5) 9.5 / 7.7
+//   8 x 64 | 16 x 64    one wave of 8 rows:       1024 (0.9) 6.0 / 6.9; 2048 (1.7) 7.5 / 7.1
+//   16 x 64 | 64 x 64   four waves of 16 rows:    9472 (4.0) 14.8 / 16.0; 16384 (6.9) 22.8 / 17.3
+//   8 x 128 | 16 x 128  one wave of 8 rows:       1024 (0.9) 6.9 / 7.7; 1237 (1.05) 8.6 / 7.7
+//   16 x 128 | 64 x 128 three waves of 16 rows:   4096 (1.7) 10.6 / 15.9; 8192 (3.5) 17.9 / 16.5
+//   16 x 256 | 32 x 256 1.5 waves of 16 rows:     2048 (0.9) 11.6 / 16.6; 4096 (1.7) 17.6 / 17.1
+// (32 x 128 tiles of 64 threads, which would share out 32768 views more evenly, were slower: 72 against 64 us.)
 typedef ChainTile<2, 4, 4, 8, 2, 1, 32, 4> F16x32;
 typedef ChainTile<4, 4, 8, 4, 1, 2, 32, 4> F32x32;
 typedef ChainTile<8, 8, 4, 8, 2, 2, 32, 2> F64x128;
@@ -215,8 +228,8 @@ cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const fl
     auto tiles = [&](int bm, int bn) { return ceil_div(M, bm) * ceil_div(N, bn); };
 #define GEAR_FWD(T, MB) (wvec ? launch_form<T, MB, true>(M, N, K, A, W, bias, H, Hf, st) : launch_form<T, MB, false>(M, N, K, A, W, bias, H, Hf, st))
     if (tiles(16, 32) <= sm_count()) return GEAR_FWD(F16x32, 4);
-    if (tiles(64, 128) <= sm_count()) return GEAR_FWD(F32x32, 4);
-    return GEAR_FWD(F64x128, 3);
+    if (tiles(32, 32) <= 6 * sm_count()) return GEAR_FWD(F32x32, 4);
+    return N % 128 == 0 || N % 128 > 64 ? GEAR_FWD(F64x128, 3) : GEAR_FWD(F64x64, 4);
 #undef GEAR_FWD
 }
 
@@ -227,10 +240,11 @@ cudaError_t launch_fwd_top_f32(const gear_ctx_impl& c, int M, int N, int K, cons
     const int slots = c.ws.loss_slots;
 #define GEAR_TOP(T, MB) (wvec ? launch_top_form<T, MB, true>(M, N, K, A, W, bias, dA, top, slots, n_part, st) \
                               : launch_top_form<T, MB, false>(M, N, K, A, W, bias, dA, top, slots, n_part, st))
-    if (N <= 32) return ceil_div(M, 16) <= sm_count() ? GEAR_TOP(F16x32, 4) : GEAR_TOP(F32x32, 4);
-    if (N <= 64) return ceil_div(M, 8) <= sm_count() ? GEAR_TOP(F8x64, 4) : ceil_div(M, 64) <= sm_count() ? GEAR_TOP(F16x64, 4) : GEAR_TOP(F64x64, 4);
-    if (N <= 128) return ceil_div(M, 8) <= sm_count() ? GEAR_TOP(F8x128, 3) : ceil_div(M, 64) <= sm_count() ? GEAR_TOP(F16x128, 3) : GEAR_TOP(F64x128, 3);
-    return ceil_div(M, 32) <= sm_count() ? GEAR_TOP(F16x256, 2) : GEAR_TOP(F32x256, 2);
+    const int64_t t8 = ceil_div(M, 8), t16 = ceil_div(M, 16), sms = sm_count();
+    if (N <= 32) return t16 <= 2 * sms ? GEAR_TOP(F16x32, 4) : GEAR_TOP(F32x32, 4);
+    if (N <= 64) return t8 <= sms ? GEAR_TOP(F8x64, 4) : t16 <= 4 * sms ? GEAR_TOP(F16x64, 4) : GEAR_TOP(F64x64, 4);
+    if (N <= 128) return t8 <= sms ? GEAR_TOP(F8x128, 3) : t16 <= 3 * sms ? GEAR_TOP(F16x128, 3) : GEAR_TOP(F64x128, 3);
+    return 2 * t16 <= 3 * sms ? GEAR_TOP(F16x256, 2) : GEAR_TOP(F32x256, 2);
 #undef GEAR_TOP
 }
 

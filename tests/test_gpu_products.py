@@ -35,6 +35,16 @@ def test_fp32_products_at_tile_edges(B, E, D, hidden):
         pair.close()
 
 
+# the same at the lines between the forms of a top layer's tile (8, 16, 32 or 64 rows of at most 32, 64, 128, 256 columns; wider ones in
+# a launch of their own) and of a lower layer's (32 x 32 up to six waves, then 64 x 128, or 64 x 64 where columns fill half a tile)
+@pytest.mark.parametrize("B,hidden", [
+    (4736, (24,)), (4737, (32,)), (9472, (64,)), (9473, (40,)), (1184, (128,)), (1185, (72,)), (7104, (128, 120)), (7105, (128, 72)),
+    (3552, (256,)), (3553, (136,)), (300, (264,)), (14_208, (64, 8)), (14_209, (64, 16)),
+])
+def test_fp32_forward_forms(B, hidden):
+    test_fp32_products_at_tile_edges(B, 4, 24, hidden)
+
+
 # column tiles are 64 wide while 64-column tiles are no more than the SMs (148), then 128, then 256 (dX: 192 where that fits);
 # weight gradients take 64 to 256 columns and cut the batch into slices
 @pytest.mark.parametrize("B,E,D,hidden", [
