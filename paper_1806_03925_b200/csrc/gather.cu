@@ -265,14 +265,32 @@ gather_pool_kernel(const GatherArgs a) {
             }
         }
         if (a.inv_n && lane == 0) a.inv_n[b] = rinv;
-        // ---- the view's own dense input (the part of the image the Fastgear side keeps), eight columns per lane and pass
-        for (int c = lane * 8; c < a.F; c += 256) {
-            const float4 f0 = ld_stream_f4(a.fast + (int64_t)b * a.F + c), f1 = ld_stream_f4(a.fast + (int64_t)b * a.F + c + 4);
-            const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-            store_x<HB, 8>(a.X, a.x_stride, a.Xf, a.x_debug, x0 + 2 * a.E + a.D + c, f);
-        }
-
         cur = nxt; nxt = nxt2; ids_cur = ids_nxt;
+    }
+    // ---- the views' own dense input (the part of the image the Fastgear side keeps): eight columns at a time over all threads, three
+    // of them asked for before the first is stored (inside the views' loop, a view of 1536 columns waited for memory six times, and
+    // 128 blocks held 1024 views: their loop pass was 3 to 4 us longer)
+    if (a.F > 0) {
+        constexpr int FK = 3;
+        const int per = a.F / 8;
+        const int64_t units = (int64_t)a.B * per, threads = (int64_t)gridDim.x * blockDim.x;
+        for (int64_t u0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < units; u0 += FK * threads) {
+            float4 f[FK][2];
+#pragma unroll
+            for (int t = 0; t < FK; ++t)
+                if (u0 + t * threads < units) {
+                    const float* src = a.fast + (u0 + t * threads) * 8;
+                    f[t][0] = ld_stream_f4(src); f[t][1] = ld_stream_f4(src + 4);
+                }
+#pragma unroll
+            for (int t = 0; t < FK; ++t) {
+                const int64_t u = u0 + t * threads;
+                if (u >= units) continue;
+                const int64_t v = u / per;
+                const float x[8] = {f[t][0].x, f[t][0].y, f[t][0].z, f[t][0].w, f[t][1].x, f[t][1].y, f[t][1].z, f[t][1].w};
+                store_x<HB, 8>(a.X, a.x_stride, a.Xf, a.x_debug, v * Din + 2 * a.E + a.D + (u - v * per) * 8, x);
+            }
+        }
     }
     if (flags) atomicOr(&a.state->status, flags);
 }
@@ -284,7 +302,8 @@ static cudaError_t dispatch_nq(const GatherArgs& a, cudaStream_t st, Profiler* p
     const int nq = (n_chunks + 31) / 32;
     // every block stays resident: three (two for wide rows) per SM
     const int64_t resident = (int64_t)sm_count() * (nq <= 2 ? 3 : 2);
-    const int grid = (int)std::min<int64_t>(ceil_div(a.B, GP_WARPS), resident);
+    const int64_t want = std::max(ceil_div(a.B, GP_WARPS), ceil_div((int64_t)a.B * a.F, 8 * 3 * 32 * GP_WARPS));
+    const int grid = (int)std::min<int64_t>(want, resident);
     KernelScope ks(prof, "gather_pool", st);
     // FULL only when a row fills the instantiated width exactly (n_chunks == NQ * 32): every lane then owns a chunk of
     // every DFV row; widths that round up to the next instantiation (3, 5, 6, 7 chunks per lane) keep the guard
