@@ -257,14 +257,15 @@ struct KernelScope {
     ~KernelScope() { if (stop) cudaEventRecord(stop, st); }
 };
 
-// Sorted positions per unit of work (span) of the accumulate's reduce pass: 16, or as few as 2 while longer spans would leave
-// warps idle (12 k rows in spans of 16 kept 768 of 3552 warps busy, each with a serial chain of 16 rows).  The workspace
-// holds one word per span.
+// Sorted positions per unit of work (span) of the accumulate's reduce pass: 16, or as few as 2 while longer spans would leave more
+// than half of the warps idle (12 k rows in spans of 16 kept 768 of 3552 warps busy, each with a serial chain of 16 rows; in spans of
+// 2 a warp went through the latencies of a span's start twice: step of 4096 views 52.1 us, spans of 4: 50.6, of 8: 51.1).
+// The workspace holds one word per span.
 constexpr int ACC_SPAN = 16;
 constexpr int64_t ACC_WARPS = 3552;        // warps of a full reduce grid: 148 SMs x 3 blocks x 8
 inline int acc_span_log2(int64_t n) {
     int s = 4;
-    while (s > 1 && (n >> s) < ACC_WARPS) --s;
+    while (s > 1 && (n >> s) < ACC_WARPS / 2) --s;
     return s;
 }
 // words of the span table for any n up to n_max
