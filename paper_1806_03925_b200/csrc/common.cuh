@@ -205,10 +205,10 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
     return launch_as(Op::DEPENDENT, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
-// Lets a kernel take `bytes` of dynamic shared memory (asked for once per process, again where that failed).
+// Lets a kernel take `bytes` of dynamic shared memory beside its static one (asked for once per process, again where that failed).
 template <auto Kernel> inline cudaError_t allow_smem(int bytes) {
     static bool done = false;
-    if (done || bytes <= 48 * 1024) return cudaSuccess;
+    if (done) return cudaSuccess;
     const cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     done = e == cudaSuccess;
     return e;
