@@ -145,11 +145,14 @@ def kernel_models(p, stats):
     def avg(xs):
         return sum(xs) / max(len(xs), 1)
     layers = range(L)
-    # bf16 top layers of at most 256 columns take the output unit along (a product of its own name)
+    # top layers of at most 256 columns take the output unit along (a product of its own name; fp32 heads: the others are "low" then)
     plain = range(L - 1) if p.head_dtype == "bf16" and fan[L] <= 256 else layers
     m["gemm"] = {
         "fwd": (avg([2 * B * fan[l] * fan[l + 1] for l in plain]),
                 avg([(B * fan[l] + fan[l] * fan[l + 1] + B * fan[l + 1]) * xsz for l in plain])),
+        # fp32 heads whose top layer takes the output unit along: the layers below it
+        "low": (avg([2 * B * fan[l] * fan[l + 1] for l in range(L - 1)]),
+                avg([(B * fan[l] + fan[l] * fan[l + 1] + B * fan[l + 1]) * xsz for l in range(L - 1)])),
         "top": (2 * B * (fan[L - 1] + 1) * fan[L], (B * fan[L - 1] + fan[L - 1] * fan[L] + B * fan[L]) * xsz + B * 8),
         "dw": (avg([2 * B * fan[l] * fan[l + 1] for l in layers]),
                avg([(B * fan[l] + B * fan[l + 1]) * xsz + fan[l] * fan[l + 1] * 4 for l in layers])),

@@ -333,7 +333,7 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
         } else if constexpr (BF)
             err = tc_gemm_kmajor(c, "tc_gemm_fwd", B, N, K, H[l].p, K, Wt[l].p, K, 0, H[l + 1].p, N, p.b[l], nullptr, 0, nullptr, LossSum{}, st);
         else
-            err = launch_fwd_f32(c, B, N, K, c.at<float>(c.ws.xf[l]), p.W[l], p.b[l], H[l + 1], l + 1 < L ? c.at<float>(c.ws.xf[l + 1]) : nullptr, st);
+            err = launch_fwd_f32(c, top_fused ? "f32_gemm_low" : "f32_gemm_fwd", B, N, K, c.at<float>(c.ws.xf[l]), p.W[l], p.b[l], H[l + 1], l + 1 < L ? c.at<float>(c.ws.xf[l + 1]) : nullptr, st);
         if (err != cudaSuccess) return err;
     }
     if (!top_fused) {
@@ -369,7 +369,7 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
     // backward.  The weight gradients run on a stream of their own, where the caller has one: as soon as dA_{l+1} exists, or after
     // dX, beside what the caller does with dX.  On one stream the gradient that the layers below wait for (dA_l, at the bottom
     // dX) comes first: once dX exists the caller's hook may start the embedding scatter on another stream.  The bias gradient of a lower layer is summed in the epilogue of the product
-    // that makes its dA (the top layer's came out of head_out_kernel).
+    // that makes its dA (the top layer's came with the output unit).
     for (int l = L - 1; l >= 0; --l) {
         const int K = p.fan[l], N = p.fan[l + 1];
         if (beside && !hooks.dw_last && (err = weight_grad(l)) != cudaSuccess) return err;

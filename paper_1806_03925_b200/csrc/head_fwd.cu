@@ -220,10 +220,10 @@ typedef ChainTile<4, 4, 4, 8, 1, 4, 32, 3> F16x128;
 typedef ChainTile<4, 4, 4, 8, 1, 8, 32, 3> F16x256;
 typedef ChainTile<8, 8, 4, 8, 1, 4, 32, 2> F32x256;
 
-cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
+cudaError_t launch_fwd_f32(const gear_ctx_impl& c, const char* name, int M, int N, int K, const float* A, const float* W, const float* bias,
                            const Planes& H, float* Hf, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
-    KernelScope ks(&c.prof, "f32_gemm_fwd", st);
+    KernelScope ks(&c.prof, name, st);
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     auto tiles = [&](int bm, int bn) { return ceil_div(M, bm) * ceil_div(N, bn); };
 #define GEAR_FWD(T, MB) (wvec ? launch_form<T, MB, true>(M, N, K, A, W, bias, H, Hf, st) : launch_form<T, MB, false>(M, N, K, A, W, bias, H, Hf, st))

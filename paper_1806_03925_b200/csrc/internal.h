@@ -175,7 +175,7 @@ cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int
                             const __nv_bfloat16* Bm, int64_t ldb, float* out, int64_t ldo, cudaStream_t st);
 
 // head_fwd.cu: H = ReLU(A W + bias), A [M][K], W [K][N] fp32; H in planes and, if Hf is given, in fp32
-cudaError_t launch_fwd_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
+cudaError_t launch_fwd_f32(const gear_ctx_impl& c, const char* name, int M, int N, int K, const float* A, const float* W, const float* bias,
                            const Planes& H, float* Hf, cudaStream_t st);
 // The same for the top hidden layer, N at most F32_TOP_N, with the output unit behind it (as tc_gemm_top): dA gets, in planes, the
 // gradient with respect to its pre-activations.
