@@ -188,6 +188,9 @@ static int check_lists(const int32_t* ids, const int32_t* seq, const float* avg,
 //                 idle, the weight gradients, which nothing but the caller waits for
 // The caller's stream waits for the other two before the call ends.  With per-kernel timing on, everything stays on the
 // caller's stream so that each kernel is timed alone.
+// Where one cluster sorts and plans, it does so beside the gather from more image occurrences than one block sorts by itself on, for
+// bf16 heads, whose products then no longer wait for it (see enqueue_step).
+constexpr int64_t EARLY_SORT_FROM = 2048;
 struct StepLists {
     int32_t* ids; int32_t* seq; float* avg; int64_t cap; int64_t* d_n;
     int32_t* expired; int64_t expired_cap; int64_t* d_expired;
@@ -219,13 +222,14 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     auto scan = [&](cudaStream_t where) {
         return launch_collect_expired(c, lists->now, lists->restamp, lists->expired, lists->expired_cap, lists->d_expired, where);
     };
-    // The weights in the form the head's products read: first on the caller's stream, ahead of the gather.  The gather keeps
-    // every SM busy for its whole duration, so a small kernel on another stream would get its blocks placed only when the
-    // gather ends, and the first product of the head would wait for it.
-    // (Small batches leave SMs free: there the copies run beside the gather.)
-    if (dw_beside && !scan_beside) GEAR_TRY(enqueue_wait(aux, c.ev[EV_FORK]));
-    GEAR_TRY(launch_round_weights(c, o, dw_beside ? aux : st));
-    if (dw_beside) GEAR_TRY(enqueue_record(c.ev[EV_AUX], aux));
+    // The weights in the form the head's products read.  bf16: in the gather's launch.  (On a stream of its own a small kernel gets its
+    // blocks placed only when the gather's leave room, in front of the gather it delays that by its own length, and a product
+    // behind two streams starts some microseconds after the later of them.)  fp32, three planes: ahead of the gather, or, small batches,
+    // which leave SMs free, beside it.
+    const bool with_gather = b.B > 0 && c.cfg.head_dtype == GEAR_BF16, weights_aside = dw_beside && !with_gather;
+    if (weights_aside && !scan_beside) GEAR_TRY(enqueue_wait(aux, c.ev[EV_FORK]));
+    if (!with_gather) GEAR_TRY(launch_round_weights(c, o, weights_aside ? aux : st));
+    if (weights_aside) GEAR_TRY(enqueue_record(c.ev[EV_AUX], aux));
     // The expiry scan reads the whole table of time stamps.  Beside the gather it slows that down; a large fp32 head's forward
     // products wait for the ALUs and leave the memory to it (32 k views: step 327 -> 316 us).  bf16 products do not (65 k views:
     // 376 us there, 386 behind the gather).
@@ -267,21 +271,27 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     // rows and queue slot are).  Only where a row's gradient lies and its scale come from the gather (row_view, inv_n): behind a
     // multi-block sort they are put in by a launch of its own, so that the plan runs beside the gather instead of beside the
     // head's first products (65 k views: step 387 -> 381 us).  Small arrays are sorted and planned by one kernel behind the
-    // gather: there the extra launch costs more than the earlier start gives (4 k views: 56.6 us against 58.0).
-    if (plan && forked && !small_sort) GEAR_TRY(launch_accumulate_plan_ahead(c, b.nnz, side));
-    GEAR_TRY(launch_gather(c, b, o.row_view, o.inv_n, o.x_debug, st));
+    // gather: there the extra launch costs more than the earlier start gives (256 views +3.4 us, 1237 views fp32 34.0 / 34.3), unless
+    // the head is done sooner than such a sort would be, as bf16 ones are since their weights come with the gather (4096 views: 51.4
+    // behind it, 49.1 beside it; 3001 views: 47.7, 47.3).
+    const bool early = forked && small_sort && with_gather && b.nnz > EARLY_SORT_FROM;
+    if (early) {
+        GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, nullptr, nullptr) : PlanArgs{}, side));
+        if (plan) note_plan(c, b.nnz, nullptr, nullptr);
+    } else if (plan && forked && !small_sort) GEAR_TRY(launch_accumulate_plan_ahead(c, b.nnz, side));
+    GEAR_TRY(launch_gather(c, b, o, with_gather, st));
     if (forked) GEAR_TRY(enqueue_record(c.ev[EV_GATHER], st));
     if (scan_late) {
         GEAR_TRY(enqueue_wait(aux, c.ev[EV_GATHER]));
         GEAR_TRY(scan(aux));
     }
-    if (dw_beside) GEAR_TRY(enqueue_wait(st, c.ev[EV_AUX]));
+    if (weights_aside) GEAR_TRY(enqueue_wait(st, c.ev[EV_AUX]));
     if (small_sort || (forked && plan)) {
         if (forked) GEAR_TRY(enqueue_wait(side, c.ev[EV_GATHER]));
-        if (small_sort) {
+        if (small_sort && !early) {
             GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, o.row_view, o.inv_n) : PlanArgs{}, side));
             if (plan) note_plan(c, b.nnz, o.row_view, o.inv_n);
-        } else GEAR_TRY(launch_accumulate_resolve_ahead(c, b.nnz, o.row_view, o.inv_n, side));
+        } else if (plan) GEAR_TRY(launch_accumulate_resolve_ahead(c, b.nnz, o.row_view, o.inv_n, side));
     }
     if (forked && lists) GEAR_TRY(enqueue_record(c.ev[EV_PLAN], side));
     // the embedding scatter: enqueued by the head as soon as dX is on its way

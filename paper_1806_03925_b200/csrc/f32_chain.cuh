@@ -1,10 +1,11 @@
 // Products of fp32 matrices with one ascending chain of multiply-adds per output (head_fwd.cu, dense.cu).
 //
 // Multiply-adds are issued in pairs (fma.rn.f32x2: two independent fp32 multiply-adds, each rounded like fmaf), which
-// leaves issue slots for the shared-memory reads.  Bound: those reads.  A 16-byte read costs a warp four clocks of the SM's 128
-// bytes per clock however many of its lanes ask for the same words, so a step of the reduction costs a warp TM + TN clocks there and
-// TM * TN / 4 in the multiply-add lanes: outputs of 8 x 8 per lane balance the two (37888 x 128 x 2048: 54 TFLOP/s, of 65 to 69
-// that multiply-adds on registers alone reach; 16 x 4, as before: 40), smaller ones are bound by shared memory.
+// leaves issue slots for the shared-memory reads.  A 16-byte read costs a warp about four clocks of the SM's 128 bytes per clock
+// however many of its lanes ask for the same words (1 x 8 outputs per lane: 4.6 measured), so a step of the reduction costs a warp
+// TM + TN clocks there and TM * TN / 4 in the multiply-add lanes.  Bound: 8 x 8 outputs per lane wait for the multiply-add pipe first
+// (shared memory 58 % of its rate; 37888 x 128 x 2048: 54 TFLOP/s, of 65 to 69 that multiply-adds on registers alone reach; 16 x 4,
+// as before: 40); 4 x 4 with a warp per scheduler, of products too small for more, for shared memory and their own latencies.
 #pragma once
 
 #include "common.cuh"

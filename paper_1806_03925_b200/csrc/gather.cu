@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "weights.cuh"
 
 namespace gear {
 
@@ -88,6 +89,7 @@ struct GatherArgs {
     __nv_bfloat16* X; int64_t x_stride; float* Xf; void* x_debug;      // X: bf16, or three planes x_stride apart and fp32 at Xf
     int32_t* row_view; float* inv_n;
     DevState* state;
+    RoundArgs weights; int w_blocks;      // the launch's first w_blocks blocks make the weights' copies
 };
 
 // Adds rows j .. j + K - 1 of the view to acc, in order; their IDs, all valid, sit in lanes (j + t) % 32 of my_id.
@@ -151,13 +153,16 @@ __device__ __forceinline__ ViewRec load_view(const GatherArgs& a, int b) {
 // round trip (the rows themselves) is exposed.
 template <typename TD, bool HB, int NQ, bool FULL>
 __global__ void __launch_bounds__(GP_WARPS * 32, NQ <= 2 ? 3 : 2)
-gather_pool_kernel(const GatherArgs a) {
+gather_pool_kernel(const __grid_constant__ GatherArgs a) {
     wait_for_predecessor();
     if (gridDim.x <= FEW_BLOCKS) let_successor_start();
+    if constexpr (HB)
+        if ((int)blockIdx.x < a.w_blocks) { round_weights_block<1>(a.weights, (int)blockIdx.x, a.w_blocks); return; }
+    const int block = (int)blockIdx.x - a.w_blocks, blocks = (int)gridDim.x - a.w_blocks;
     constexpr int PER = Chunk<TD>::PER;
     constexpr int KMAX = NQ >= 8 ? 1 : 8 / NQ;               // rows in flight per warp
     const int lane = (int)lane_id();
-    const int W = gridDim.x * GP_WARPS;
+    const int W = blocks * GP_WARPS;
     const int Din = 2 * a.E + a.D + a.F;
     const int n_chunks = a.D / PER;
     const int ce = a.E / 4;                                    // 16-byte chunks per embedding row
@@ -169,7 +174,7 @@ gather_pool_kernel(const GatherArgs a) {
         return (ok && j0 + lane < r.n) ? __ldg(a.img_id + r.s + j0 + lane) : -1;
     };
 
-    int b = blockIdx.x * GP_WARPS + (int)(threadIdx.x >> 5);
+    int b = block * GP_WARPS + (int)(threadIdx.x >> 5);
     ViewRec cur = load_view(a, b), nxt = load_view(a, b + W);
     int ids_cur = load_ids(cur, 0);
 
@@ -273,8 +278,8 @@ gather_pool_kernel(const GatherArgs a) {
     if (a.F > 0) {
         constexpr int FK = 3;
         const int per = a.F / 8;
-        const int64_t units = (int64_t)a.B * per, threads = (int64_t)gridDim.x * blockDim.x;
-        for (int64_t u0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u0 < units; u0 += FK * threads) {
+        const int64_t units = (int64_t)a.B * per, threads = (int64_t)blocks * blockDim.x;
+        for (int64_t u0 = (int64_t)block * blockDim.x + threadIdx.x; u0 < units; u0 += FK * threads) {
             float4 f[FK][2];
 #pragma unroll
             for (int t = 0; t < FK; ++t)
@@ -303,7 +308,7 @@ static cudaError_t dispatch_nq(const GatherArgs& a, cudaStream_t st, Profiler* p
     // every block stays resident: three (two for wide rows) per SM
     const int64_t resident = (int64_t)sm_count() * (nq <= 2 ? 3 : 2);
     const int64_t want = std::max(ceil_div(a.B, GP_WARPS), ceil_div((int64_t)a.B * a.F, 8 * 3 * 32 * GP_WARPS));
-    const int grid = (int)std::min<int64_t>(want, resident);
+    const int grid = a.w_blocks + (int)std::min<int64_t>(want, resident);
     KernelScope ks(prof, "gather_pool", st);
     // FULL only when a row fills the instantiated width exactly (n_chunks == NQ * 32): every lane then owns a chunk of
     // every DFV row; widths that round up to the next instantiation (3, 5, 6, 7 chunks per lane) keep the guard
@@ -318,16 +323,16 @@ static cudaError_t dispatch_nq(const GatherArgs& a, cudaStream_t st, Profiler* p
     return cudaGetLastError();
 }
 
-cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* row_view, float* inv_n,
-                          void* x_debug, cudaStream_t st) {
+cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o, bool with_weights, cudaStream_t st) {
     if (b.B <= 0) return cudaSuccess;
     GatherArgs a;
     a.user_emb = c.buf.user_emb; a.url_emb = c.buf.url_emb; a.dfv = c.buf.dfv;
     a.user_vocab = c.cfg.user_vocab; a.url_vocab = c.cfg.url_vocab; a.img_vocab = c.cfg.img_vocab;
     a.E = c.cfg.emb_dim; a.D = c.cfg.dfv_dim; a.B = b.B; a.nnz = b.nnz; a.F = c.cfg.fast_dim; a.fast = b.fast;
     a.user_id = b.user_id; a.url_id = b.url_id; a.img_off = b.img_off; a.img_id = b.img_id;
-    a.X = c.at<__nv_bfloat16>(c.ws.x); a.x_stride = (int64_t)c.cfg.max_batch * c.d_in; a.Xf = c.cfg.head_dtype == GEAR_F32 ? c.at<float>(c.ws.xf[0]) : nullptr; a.x_debug = x_debug; a.row_view = row_view; a.inv_n = inv_n;
+    a.X = c.at<__nv_bfloat16>(c.ws.x); a.x_stride = (int64_t)c.cfg.max_batch * c.d_in; a.Xf = c.cfg.head_dtype == GEAR_F32 ? c.at<float>(c.ws.xf[0]) : nullptr; a.x_debug = o.x_debug; a.row_view = o.row_view; a.inv_n = o.inv_n;
     a.state = c.state();
+    a.weights = round_args(c, o); a.w_blocks = with_weights ? a.weights.blocks() : 0;
     const bool dbf = c.cfg.dfv_dtype == GEAR_BF16, xbf = c.cfg.head_dtype == GEAR_BF16;
     if (dbf && xbf) return dispatch_nq<__nv_bfloat16, true>(a, st, &c.prof);
     if (dbf && !xbf) return dispatch_nq<__nv_bfloat16, false>(a, st, &c.prof);

@@ -9,6 +9,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "weights.cuh"
 
 namespace gear {
 
@@ -189,56 +190,12 @@ head_out_kernel(int B, int H, const __nv_bfloat16* __restrict__ h, int64_t strid
     }
 }
 
-// fp32 master weights -> bf16 in both orientations, all hidden layers in one launch (blockIdx.z = layer).
-// PLANES 1: rounded to bf16 (bf16 heads); 3: split into three planes, fan_in * fan_out elements apart (fp32 heads).
-struct RoundArgs {
-    int fan_in[MAX_LAYERS], fan_out[MAX_LAYERS];
-    const float* W[MAX_LAYERS];
-    __nv_bfloat16* wb[MAX_LAYERS];
-    __nv_bfloat16* wbt[MAX_LAYERS];
-    float* grad; int64_t n_grad;                // the parameters' gradient, cleared by the same launch
-    float* loss;                                // empty batch only: its loss (0)
-};
-// 32 x 32 tiles through shared memory, so that both copies are written with coalesced rows
+// The weights' copies by themselves: of fp32 heads, and of an empty batch, which has no gather.
 template <int PLANES>
 __global__ void __launch_bounds__(256)
 round_weights_kernel(const __grid_constant__ RoundArgs a) {
     wait_for_predecessor();
-    {
-        const int64_t blk = blockIdx.x + (int64_t)gridDim.x * (blockIdx.y + (int64_t)gridDim.y * blockIdx.z);
-        const int64_t threads = (int64_t)gridDim.x * gridDim.y * gridDim.z * blockDim.x;
-        for (int64_t i = blk * blockDim.x + threadIdx.x; i < a.n_grad; i += threads) a.grad[i] = 0.f;
-        if (a.loss && blk == 0 && threadIdx.x == 0) *a.loss = 0.f;
-    }
-    __shared__ __nv_bfloat16 tile[PLANES][32][33];
-    const int l = blockIdx.z;
-    const int fan_in = a.fan_in[l], fan_out = a.fan_out[l];
-    const int64_t stride = (int64_t)fan_in * fan_out;
-    const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
-    if (r0 >= fan_in || c0 >= fan_out) return;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int r = r0 + ty + 8 * k, c = c0 + tx;
-        if (r < fan_in && c < fan_out) {
-            float w = a.W[l][(int64_t)r * fan_out + c];
-#pragma unroll
-            for (int p = 0; p < PLANES; ++p) {
-                const __nv_bfloat16 v = __float2bfloat16_rn(w);
-                a.wb[l][p * stride + (int64_t)r * fan_out + c] = v;
-                tile[p][ty + 8 * k][tx] = v;
-                w -= __bfloat162float(v);
-            }
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int c = c0 + ty + 8 * k, r = r0 + tx;
-        if (r < fan_in && c < fan_out)
-#pragma unroll
-            for (int p = 0; p < PLANES; ++p) a.wbt[l][p * stride + (int64_t)c * fan_in + r] = tile[p][tx][ty + 8 * k];
-    }
+    round_weights_block<PLANES>(a, (int)blockIdx.x, (int)gridDim.x);
 }
 
 struct HeadParams {
@@ -270,26 +227,28 @@ static float* grad_array(const gear_ctx_impl& c, const gear_step_out& o) {
     return (reinterpret_cast<uintptr_t>(o.head_grad) & 15u) == 0 ? o.head_grad : c.at<float>(c.ws.head_grad);
 }
 
-// bf16 copies or planes of the hidden layers' weights in both orientations (what the tensor-core products read).  Depends
-// on head_params only, so a step runs it ahead of the gather.  Clears head_grad on the way.
-cudaError_t launch_round_weights(const gear_ctx_impl& c, const gear_step_out& o, cudaStream_t st) {
-    const int L = c.cfg.n_hidden;
-    RoundArgs ra;
+// bf16 copies or planes of the hidden layers' weights in both orientations (what the tensor-core products read).  Clears
+// head_grad on the way.
+RoundArgs round_args(const gear_ctx_impl& c, const gear_step_out& o) {
+    RoundArgs ra = {};
     ra.grad = grad_array(c, o); ra.n_grad = c.n_params; ra.loss = o.loss;     // the loss of a batch is written after this
-    int max_in = 0, max_out = 0, fan = c.d_in;
+    int fan = c.d_in;
     int64_t pos = 0;
-    for (int l = 0; l < L; ++l) {
+    for (int l = 0; l < c.cfg.n_hidden; ++l) {
         const int h = c.cfg.hidden[l];
         ra.fan_in[l] = fan; ra.fan_out[l] = h; ra.W[l] = c.buf.head_params + pos;
         ra.wb[l] = c.at<__nv_bfloat16>(c.ws.wb[l]); ra.wbt[l] = c.at<__nv_bfloat16>(c.ws.wbt[l]);
-        if (fan > max_in) max_in = fan;
-        if (h > max_out) max_out = h;
+        ra.tiles[l] = (int)(ceil_div(fan, 32) * ceil_div(h, 32));
         pos += (int64_t)fan * h + h;
         fan = h;
     }
+    return ra;
+}
+cudaError_t launch_round_weights(const gear_ctx_impl& c, const gear_step_out& o, cudaStream_t st) {
+    const RoundArgs ra = round_args(c, o);
     KernelScope ks(&c.prof, "round_weights", st);
     return launch_dependent(c.cfg.head_dtype == GEAR_BF16 ? round_weights_kernel<1> : round_weights_kernel<3>,
-                            dim3((unsigned)ceil_div(max_out, 32), (unsigned)ceil_div(max_in, 32), (unsigned)L), dim3(256), 0, st, ra);
+                            dim3((unsigned)ra.blocks()), dim3(256), 0, st, ra);
 }
 
 // The head's matrices in the form the products take: bf16, or planes of an fp32 matrix

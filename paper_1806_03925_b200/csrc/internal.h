@@ -138,9 +138,21 @@ cudaError_t launch_fill_uniform(void* dst, int dtype, int64_t n_elems, uint64_t 
                                 cudaStream_t st);
 cudaError_t launch_fill_ts(int64_t* ts, int64_t n, uint64_t seed, int64_t expire, int64_t now, cudaStream_t st);
 
-// gather.cu
-cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* row_view, float* inv_n,
-                          void* x_debug, cudaStream_t st);
+// What the weights' copies are made from (weights.cuh)
+struct RoundArgs {
+    int fan_in[MAX_LAYERS], fan_out[MAX_LAYERS];
+    const float* W[MAX_LAYERS];
+    __nv_bfloat16* wb[MAX_LAYERS];
+    __nv_bfloat16* wbt[MAX_LAYERS];
+    int tiles[MAX_LAYERS];                      // of 32 x 32 weights
+    float* grad; int64_t n_grad;                // the parameters' gradient, cleared by the same launch
+    float* loss;                                // empty batch only: its loss (0)
+    int blocks() const { int n = 0; for (int t : tiles) n += t; return n; }
+};
+RoundArgs round_args(const gear_ctx_impl& c, const gear_step_out& o);
+
+// gather.cu.  with_weights: the first blocks of the launch make the weights' copies and clear head_grad (bf16 heads).
+cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o, bool with_weights, cudaStream_t st);
 
 // head.cu: forward + backward of the head.  The weights' copies must have been made and head_grad cleared before it on its stream
 // (launch_round_weights).  after_dx(arg) is called once dX is on its way.  The weight gradients go to dw_stream; if that is not the
@@ -148,7 +160,7 @@ cudaError_t launch_gather(const gear_ctx_impl& c, const gear_batch& b, int32_t* 
 // dw_last, all of them after dX.
 struct HeadHooks { cudaError_t (*after_dx)(void*); void* arg; cudaStream_t dw_stream; cudaEvent_t* dw_ev; bool dw_last; };
 cudaError_t launch_head(const gear_ctx_impl& c, const gear_batch& b, const gear_step_out& o, cudaStream_t st, const HeadHooks& hooks);
-// the weights as the products read them; clears head_grad (all of it, also for an empty batch)
+// the weights as the products read them, in a launch of their own; clears head_grad (all of it, also for an empty batch)
 cudaError_t launch_round_weights(const gear_ctx_impl& c, const gear_step_out& o, cudaStream_t st);
 
 // The blocks' partial losses of the batch, added up in a fixed order by a block of the product that follows the output unit (a
