@@ -274,7 +274,7 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     // gather: there the extra launch costs more than the earlier start gives (256 views +3.4 us, 1237 views fp32 34.0 / 34.3), unless
     // the head is done sooner than such a sort would be, as bf16 ones are since their weights come with the gather (4096 views: 51.4
     // behind it, 49.1 beside it; 3001 views: 47.7, 47.3).
-    const bool early = forked && small_sort && with_gather && b.nnz > EARLY_SORT_FROM;
+    const bool early = small_sort && with_gather && b.nnz > EARLY_SORT_FROM;
     if (early) {
         GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, nullptr, nullptr) : PlanArgs{}, side));
         if (plan) note_plan(c, b.nnz, nullptr, nullptr);
