@@ -60,7 +60,7 @@ dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const 
         DenseTile::Acc acc;
         DenseTile::product<AVEC, BVEC>(acc, R, reinterpret_cast<float*>(dyn_smem),
                                        [&](int r) -> const float* { const int64_t id = row_of[r]; return id >= 0 ? raw + id * R : nullptr; },
-                                       Wd + n0, D, D - n0);
+                                       raw, Wd + n0, D, D - n0);
 #pragma unroll
         for (int i = 0; i < DenseTile::TM; ++i) {
             const int64_t m = m0 + DenseTile::row(i);

@@ -42,11 +42,14 @@ template <int TM_, int TN_, int LR, int LC, int WR_, int WC_, int BK_, int STAGE
     static __device__ __forceinline__ int row(int i) { return warp_row() * (TM * LR) + i * LR + (int)(threadIdx.x % 32) / LC; }
     static __device__ __forceinline__ int col(int j) { return warp_col() * (TN * LC) + j * (4 * LC) + (int)(threadIdx.x % LC) * 4; }
 
-    // acc = A . B over k < K.  a_row(r): row r of the tile in memory, or null (zeros); b: element (0, first column of the tile),
-    // rows ldb apart, n_cols columns exist.  AVEC / BVEC: A's rows / B's rows may be read 16 bytes at a time (lengths and strides
-    // are multiples of four then).  smem: SMEM bytes, free when the block enters and when it leaves.
+    // acc = A . B over k < K.  a_row(r): row r of the tile in memory, or null (zeros); a: any row of A; b: element (0, first column
+    // of the tile), rows ldb apart, n_cols columns exist.  AVEC / BVEC: A's rows / B's rows may be read 16 bytes at a time (lengths
+    // and strides are multiples of four then).  smem: SMEM bytes, free when the block enters and when it leaves.
+    // A copy that fills with zeros names an address of its own operand: a copy's source has to be aligned to the copy's size also
+    // where nothing is read, and either operand may be the one that is not.
     template <bool AVEC, bool BVEC, typename ARow>
-    static __device__ __forceinline__ void product(Acc& acc, int K, float* smem, ARow a_row, const float* __restrict__ b, int64_t ldb, int n_cols) {
+    static __device__ __forceinline__ void product(Acc& acc, int K, float* smem, ARow a_row, const float* __restrict__ a, const float* __restrict__ b,
+                                                   int64_t ldb, int n_cols) {
         const int tid = threadIdx.x;
         const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
         const float* pa[A_PIECES];
@@ -64,10 +67,10 @@ template <int TM_, int TN_, int LR, int LC, int WR_, int WC_, int BK_, int STAGE
                 if (A_QUADS % THREADS != 0 && p >= A_QUADS) break;
                 const int k = k0 + 4 * (p % (BK / 4));
                 const uint32_t dst = sa + (uint32_t)((p / (BK / 4)) * PITCH + 4 * (p % (BK / 4))) * 4u;
-                if (AVEC) { const bool on = pa[q] && k < K; cp_async_16(dst, on ? pa[q] + k0 : b, on ? 16 : 0); }
+                if (AVEC) { const bool on = pa[q] && k < K; cp_async_16(dst, on ? pa[q] + k0 : a, on ? 16 : 0); }
                 else
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) { const bool on = pa[q] && k + e < K; cp_async_4(dst + 4u * e, on ? pa[q] + k0 + e : b, on ? 4 : 0); }
+                    for (int e = 0; e < 4; ++e) { const bool on = pa[q] && k + e < K; cp_async_4(dst + 4u * e, on ? pa[q] + k0 + e : a, on ? 4 : 0); }
             }
 #pragma unroll
             for (int q = 0; q < B_PIECES; ++q) {
@@ -98,11 +101,11 @@ template <int TM_, int TN_, int LR, int LC, int WR_, int WC_, int BK_, int STAGE
             const float* sa = smem + stage * STAGE_WORDS + a_at;
             const float* sb = smem + stage * STAGE_WORDS + A_WORDS + b_at;
             stage = stage + 1 == STAGES ? 0 : stage + 1;
-            float4 a[2][TM];
+            float4 av[2][TM];
             f32x2 bv[2][TN / 2];
             auto read_a = [&](int f, int kq) {
 #pragma unroll
-                for (int i = 0; i < TM; ++i) a[f][i] = *reinterpret_cast<const float4*>(sa + i * (LR * PITCH) + 4 * kq);
+                for (int i = 0; i < TM; ++i) av[f][i] = *reinterpret_cast<const float4*>(sa + i * (LR * PITCH) + 4 * kq);
             };
             auto read_b = [&](int f, int k) {
 #pragma unroll
@@ -118,7 +121,7 @@ template <int TM_, int TN_, int LR, int LC, int WR_, int WC_, int BK_, int STAGE
                 if (k + 1 < BK) read_b((k + 1) & 1, k + 1);
 #pragma unroll
                 for (int i = 0; i < TM; ++i) {
-                    const float4 v = a[(k / 4) & 1][i];
+                    const float4 v = av[(k / 4) & 1][i];
                     const f32x2 vv = dup2(k % 4 == 0 ? v.x : k % 4 == 1 ? v.y : k % 4 == 2 ? v.z : v.w);
 #pragma unroll
                     for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], vv, bv[k & 1][j]);

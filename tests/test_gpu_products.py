@@ -45,6 +45,72 @@ def test_fp32_forward_forms(B, hidden):
     test_fp32_products_at_tile_edges(B, 4, 24, hidden)
 
 
+def _off_by_one_float(t):
+    out = torch.empty(t.numel() + 1, device=t.device)[1:].view(t.shape)
+    assert out.data_ptr() % 16 == 4
+    return out.copy_(t)
+
+
+def _with_params_off(s):
+    """The session's ctx made anew with head parameters that start 4 bytes past a 16-byte boundary (fp32 heads take any address)."""
+    from paper_1806_03925_b200 import binding as gb
+    gb.gear_destroy(s.ctx)
+    s.head_params = _off_by_one_float(s.head_params)
+    s.ctx = gb.gear_init_tables(s.cfg, s.user_emb, s.url_emb, s.dfv, s.dfv_gsum, s.dfv_gcnt, s.dfv_ts, s.head_params, s.workspace, fill=False)
+
+
+# Every form of a forward tile, 304 terms deep (nine and a half steps of the operand ring), on batches that end inside a tile:
+# weights read 16 bytes at a time and one by one.
+@pytest.mark.parametrize("off", [False, True])
+@pytest.mark.parametrize("B,hidden", [
+    (33, (24,)), (9473, (32,)), (1000, (64,)), (1187, (40,)), (9473, (64,)), (1001, (128,)), (1187, (72,)), (7105, (128,)), (301, (256,)), (3553, (136,)),
+    (300, (64, 8)), (1889, (128, 8)), (14_211, (64, 8)), (14_211, (128, 8)),
+])
+def test_fp32_forward_forms_in_deep_layers(B, hidden, off):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from gpu_harness import Pair
+    p = PRESETS["skew"].scaled(emb_dim=4, dfv_dim=296, dfv_dtype=F32, head_dtype=F32, hidden=hidden, M=3, user_vocab=3000,
+                               url_vocab=2000, img_vocab=4000, expire=2)
+    batch = BatchSource(p, B).batch(0, B)
+    pair = Pair(p, [batch], seed=1, want_emb_grad=True)
+    try:
+        if off:
+            _with_params_off(pair.gpu)
+        pair.step_and_compare(batch, now=1)
+    finally:
+        pair.close()
+
+
+# the Dense Part's products over more steps than the ring of four has buffers, with rows and weights off a 16-byte boundary or not
+@pytest.mark.parametrize("raw_off,w_off", [(False, False), (False, True), (True, False), (True, True)])
+@pytest.mark.parametrize("n,R,D", [(33, 300, 72), (2401, 288, 64), (31, 301, 8)])
+def test_dense_forward_of_unaligned_operands(n, R, D, raw_off, w_off):
+    """Against fp64; R products of values in (-1, 1) added one by one in fp32 are off by at most R * 2^-24 * R.  An ID out of range
+    gives a row of zeros."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1806_03925_b200 import workloads
+    from paper_1806_03925_b200.session import GearSession
+    p = PRESETS["tiny"].scaled(user_vocab=64, url_vocab=64, img_vocab=500, dfv_dim=D)
+    s = GearSession(p, workloads.head_params(p, 0), max_batch=8, max_nnz=32)
+    try:
+        rng = np.random.default_rng(R)
+        raw, Wd = rng.uniform(-1, 1, (500, R)).astype(np.float32), rng.uniform(-1, 1, (R, D)).astype(np.float32)
+        ids = rng.integers(0, 500, n).astype(np.int32)
+        ids[::7] = -1
+        ids[5] = 500
+        at = lambda a, off: _off_by_one_float(torch.from_numpy(a).cuda()) if off else torch.from_numpy(a).cuda()
+        rows = torch.full((n, D), 7.0, device="cuda")
+        s.dense_forward(at(raw, raw_off), at(Wd, w_off), torch.from_numpy(ids).cuda(), rows, n=n)
+        ok = (ids >= 0) & (ids < 500)
+        want = raw[np.where(ok, ids, 0)].astype(np.float64) @ Wd.astype(np.float64) * ok[:, None]
+        np.testing.assert_allclose(rows.cpu().numpy(), want, rtol=0, atol=R * R * 2.0 ** -24)
+        assert s.status()[1] == 1
+    finally:
+        s.close()
+
+
 # column tiles are 64 wide while 64-column tiles are no more than the SMs (148), then 128, then 256 (dX: 192 where that fits);
 # weight gradients take 64 to 256 columns and cut the batch into slices
 @pytest.mark.parametrize("B,E,D,hidden", [
