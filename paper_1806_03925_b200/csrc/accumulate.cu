@@ -535,7 +535,8 @@ plan_resolve_kernel(int n, const DevState* __restrict__ state, const uint32_t* _
     if (i >= min(n, (int)state->n_valid)) return;          // rows without a valid image have no record
     int src = (int)__ldg(perm + i);
     if (src_row) src = __ldg(src_row + src);
-    pmeta[i] = make_int2(src, __float_as_int(scale ? __ldg(scale + src) : 1.f));
+    // (below zero: as in plan_tile)
+    pmeta[i] = make_int2(max(src, 0), __float_as_int(src < 0 ? 0.f : scale ? __ldg(scale + src) : 1.f));
 }
 static cudaError_t launch_plan_resolve(const gear_ctx_impl& c, const uint32_t* perm, int64_t n, const int32_t* src_row, const float* scale, cudaStream_t st) {
     KernelScope k(&c.prof, "plan_resolve", st);

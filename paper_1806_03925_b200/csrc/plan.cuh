@@ -71,23 +71,27 @@ __device__ __forceinline__ void plan_tile(const PlanArgs& p, int n, int tile0, K
     uint32_t g0, f0;
     base(__reduce_add_sync(0xffffffffu, (uint32_t)g_warp), __reduce_add_sync(0xffffffffu, (uint32_t)f_warp), g0, f0);
     // where the gradient row of every sorted position lives and what it is scaled by (one 8-byte record), where the call names
-    // either; every level of the chain is requested for all positions at once
+    // either; every level of the chain is requested for all positions at once.  A source row below zero (an occurrence that no page
+    // view of a malformed batch covers): row 0 times zero.
     if (p.src_row || p.scale) {
         int src[ITEMS];
         float scale[ITEMS];
+        uint32_t live = 0;
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it) {
             const int i = seg0 + it * 32 + lane;
-            src[it] = i < n && key_at(i) < p.vocab ? (int)perm_at(i) : -1;          // a row without a valid image has no record
+            const bool on = i < n && key_at(i) < p.vocab;                            // a row without a valid image has no record
+            live |= (uint32_t)on << it;
+            src[it] = on ? (int)perm_at(i) : -1;
         }
         if (p.src_row)
 #pragma unroll
             for (int it = 0; it < ITEMS; ++it) if (src[it] >= 0) src[it] = __ldg(p.src_row + src[it]);
 #pragma unroll
-        for (int it = 0; it < ITEMS; ++it) scale[it] = p.scale && src[it] >= 0 ? __ldg(p.scale + src[it]) : 1.f;
+        for (int it = 0; it < ITEMS; ++it) scale[it] = src[it] < 0 ? 0.f : p.scale ? __ldg(p.scale + src[it]) : 1.f;
 #pragma unroll
         for (int it = 0; it < ITEMS; ++it)
-            if (src[it] >= 0) p.pmeta[seg0 + it * 32 + lane] = make_int2(src[it], __float_as_int(scale[it]));
+            if ((live >> it) & 1u) p.pmeta[seg0 + it * 32 + lane] = make_int2(max(src[it], 0), __float_as_int(scale[it]));
     }
     uint32_t gi = g0 + __reduce_add_sync(0xffffffffu, (uint32_t)(lane < warp ? g_warp : 0));
     uint32_t ci = f0 + __reduce_add_sync(0xffffffffu, (uint32_t)(lane < warp ? f_warp : 0));

@@ -84,6 +84,41 @@ def test_sorted_store_at_sort_and_plan_edges(n, vocab, M):
         s.close()
 
 
+# sorted and planned by one block, by one cluster (bf16: beside the gather, the rows put in behind both), by the multi-block sort
+@pytest.mark.parametrize("head,B", [(F32, 300), (BF16, 300), (F32, 1500), (BF16, 1500), (BF16, 12_000)])
+def test_occurrences_that_no_page_view_covers(head, B):
+    """Two views with offsets beyond the batch: their occurrences' entries of row_view stay what they were (-1).  The rows count as
+    zeros, the others as always: k values of an image, each rounded once, added one by one in fp32, are off by at most (k + 1) * 2^-24
+    of the sum of their sizes."""
+    from paper_1806_03925_b200 import binding as gb
+    from paper_1806_03925_b200.session import DeviceBatch, GearSession
+    p = PRESETS["medium"].scaled(batch=B, user_vocab=500, url_vocab=500, img_vocab=2000, M=50_000, dfv_dim=72, dfv_dtype=head, head_dtype=head,
+                                 hidden=(64,))
+    b = BatchSource(p, 3).batch(0, B)
+    lo, hi = int(b.img_off[B // 2]), int(b.img_off[B // 2 + 2])
+    b.img_off[B // 2 + 1] = b.nnz + 100                                  # view B / 2 ends past the batch, the next one starts there
+    s = GearSession(p, workloads.head_params(p, 0), max_batch=B, max_nnz=b.nnz, seed=3)
+    try:
+        for now in (1, 2):
+            s.row_view.fill_(-1)
+            s.dfv_gsum.zero_()
+            s.dfv_gcnt.zero_()
+            s.step(DeviceBatch.from_host(b), now)
+            torch.cuda.synchronize()
+            assert s.status()[1] == gb.GEAR_DEV_BAD_CSR
+            view = s.row_view[:b.nnz].cpu().numpy()
+            assert (view[lo:hi] == -1).all() and (np.delete(view, np.arange(lo, hi)) >= 0).all()
+            g = s.dX[:, 2 * p.emb_dim:].double().cpu().numpy()[view] * s.inv_n.double().cpu().numpy()[view][:, None] * (view >= 0)[:, None]
+            want, size = np.zeros((2, p.img_vocab, p.dfv_dim))
+            np.add.at(want, b.img_id, g)
+            np.add.at(size, b.img_id, np.abs(g))
+            k = np.bincount(b.img_id, minlength=p.img_vocab)
+            assert np.array_equal(s.dfv_gcnt.cpu().numpy(), k)
+            assert np.all(np.abs(s.dfv_gsum.cpu().numpy() - want) <= (k + 1)[:, None] * 2.0 ** -24 * size + 1e-37)
+    finally:
+        s.close()
+
+
 # blocks take 256 rows, warps 32 of them; rows of 72 columns leave lanes idle, of 136 take a second round
 @pytest.mark.parametrize("n,vocab,M,D", [(1, 1000, 1, 8), (255, 1000, 4, 72), (256, 5, 3, 128), (257, 1000, 2, 136), (20_011, 3, 64, 72),
                                          (33_000, 40_000, 1, 64)])
