@@ -6,6 +6,7 @@
 #include <cfloat>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 #include <vector>
 
@@ -205,12 +206,16 @@ inline cudaError_t launch_dependent(void (*kernel)(KArgs...), dim3 grid, dim3 bl
     return launch_as(Op::DEPENDENT, kernel, grid, block, smem, st, std::forward<Args>(args)...);
 }
 
-// Lets a kernel take `bytes` of dynamic shared memory beside its static one (asked for once per process, again where that failed).
+// Lets a kernel take `bytes` of dynamic shared memory beside its static one.  The attribute belongs to the kernel on one device: it is
+// asked for once on each, again where that failed.
 template <auto Kernel> inline cudaError_t allow_smem(int bytes) {
-    static bool done = false;
-    if (done) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    done = e == cudaSuccess;
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0ull;
+    if (e != cudaSuccess || (done.load(std::memory_order_relaxed) & bit)) return e;
+    e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
     return e;
 }
 

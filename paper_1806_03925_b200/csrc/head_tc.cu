@@ -643,13 +643,8 @@ static cudaError_t launch_variant(const CUtensorMap& ma, const CUtensorMap& mb, 
                                   TcArgs g, cudaStream_t st) {
     using Cfg = TcCfg<BN, EW, EPI>;
     static_assert(EW == 8, "one kernel entry point: eight epilogue warps");
-    auto kernel = tc_gemm_kernel<BN, MN, EPI>;
-    static bool configured = false;
-    if (!configured) {
-        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    constexpr auto kernel = tc_gemm_kernel<BN, MN, EPI>;
+    if (const cudaError_t e = allow_smem<kernel>(Cfg::SMEM)) return e;
     const int tiles = g.m_tiles * g.n_tiles * g.k_splits;
     const int grid = tiles < sm_count() ? tiles : sm_count();
     // (Larger products gain nothing, and CTAs that wait on an SM keep the kernels of other streams from it: 65 k views, all products:

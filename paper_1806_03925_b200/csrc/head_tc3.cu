@@ -354,9 +354,8 @@ t3_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 template <int BN, bool MN, int EPI, bool SEG>
 static cudaError_t t3_launch_as(const CUtensorMap& ma, const CUtensorMap& mb, const CUtensorMap& mo, const T3Args& g, cudaStream_t st) {
     using Cfg = T3Cfg<BN, EPI>;
-    auto kernel = t3_gemm_kernel<BN, MN, EPI, SEG>;
-    static const cudaError_t configured = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
-    if (configured != cudaSuccess) return configured;
+    constexpr auto kernel = t3_gemm_kernel<BN, MN, EPI, SEG>;
+    if (const cudaError_t e = allow_smem<kernel>(Cfg::SMEM)) return e;
     const int tiles = g.m_tiles * g.n_tiles * g.k_splits;
     return launch_dependent(kernel, dim3(tiles < sm_count() ? tiles : sm_count()), dim3(T3_THREADS), (size_t)Cfg::SMEM, st, ma, mb, mo, g);
 }

@@ -282,11 +282,12 @@ coop_sort_kernel(const SortBatch batch) {
     if (threadIdx.x == 0 && atomicInc(batch.barrier + 1, gridDim.x - 1) == gridDim.x - 1) batch.barrier[0] = 0u;
 }
 
+template <int ITEMS, int KEYS> constexpr int coop_smem() { return rs_smem_bytes<ITEMS>(KEYS == 2 ? 8 : RS_RADIX_BITS, KEYS); }      // of the widest digit
 template <int ITEMS, int KEYS> static int coop_grid_limit() {
     static const int limit = [] {
         int per_sm = 0;
-        const int smem = rs_smem_bytes<ITEMS>(KEYS == 2 ? 8 : RS_RADIX_BITS, KEYS);
-        cudaFuncSetAttribute(coop_sort_kernel<ITEMS, KEYS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        constexpr int smem = coop_smem<ITEMS, KEYS>();
+        allow_smem<coop_sort_kernel<ITEMS, KEYS>>(smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, coop_sort_kernel<ITEMS, KEYS>, RS_THREADS, smem);
         const int n = sm_count() * (per_sm < 1 ? 1 : per_sm > 2 ? 2 : per_sm);
         return n < RS_MAX_BLOCKS ? n : RS_MAX_BLOCKS;
@@ -297,6 +298,7 @@ template <int ITEMS, int KEYS> static int coop_grid_limit() {
 template <int ITEMS, int KEYS> static cudaError_t launch_sort(SortBatch& batch, int width, cudaStream_t st) {
     // every job gets blocks in proportion to its tiles, at least one and at most one per tile
     const int limit = coop_grid_limit<ITEMS, KEYS>();
+    if (const cudaError_t e = allow_smem<coop_sort_kernel<ITEMS, KEYS>>(coop_smem<ITEMS, KEYS>())) return e;
     int64_t tiles[3], total = 0;
     for (int j = 0; j < batch.n_jobs; ++j) {
         tiles[j] = ceil_div(batch.job[j].n_max, RS_THREADS * ITEMS);

@@ -29,6 +29,8 @@ void* g_capture_origin = nullptr;
 std::vector<std::string> g_log;
 std::map<const void*, std::string> g_kernel;
 long g_calls = 0, g_fail_at = -1, g_handles = 0, g_live = 0;
+int g_device = 0;
+std::map<std::pair<int, const void*>, int> g_smem;   // dynamic shared memory that a kernel has been allowed on a device
 int g_nodes[4096];
 int g_n_nodes = 0;
 
@@ -83,6 +85,7 @@ int fake_unfinished() {
     }
     return n;
 }
+void fake_device(int d) { g_device = d; }
 long fake_log(char* out, long cap) {
     std::string all;
     for (const auto& l : g_log) all += l + "\n";
@@ -101,9 +104,12 @@ void __cudaRegisterVar(void**, char*, char*, const char*, int, size_t, int, int)
 unsigned __cudaPushCallConfiguration(dim3, dim3, size_t, cudaStream_t) { return 0; }
 cudaError_t __cudaPopCallConfiguration(dim3*, dim3*, size_t*, void*) { return cudaSuccess; }
 
-cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaGetDevice(int* d) { *d = g_device; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 148; return cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void*, cudaFuncAttribute, int) { return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int bytes) { Own own;
+    if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) g_smem[{g_device, f}] = bytes;
+    return cudaSuccess;
+}
 cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) { *n = 2; return cudaSuccess; }
 cudaError_t cudaGetDriverEntryPoint(const char*, void** p, unsigned long long, cudaDriverEntryPointQueryResult* q) {
     *p = reinterpret_cast<void*>(&encode_tiled);
@@ -116,6 +122,7 @@ cudaError_t cudaGetLastError() { return cudaSuccess; }
 
 cudaError_t cudaLaunchKernel(const void* f, dim3, dim3, void**, size_t, cudaStream_t s) { Own own; return work("launch", s, g_kernel[f].c_str()); }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { Own own;
+    if (c->dynamicSmemBytes > 48 * 1024 && (int)c->dynamicSmemBytes > g_smem[{g_device, f}]) return cudaErrorInvalidValue;
     if (c->gridDim.x == 0 || c->gridDim.y > 65535 || c->gridDim.z > 65535) return cudaErrorInvalidConfiguration;
     return work("launch", c->stream, g_kernel[f].c_str());
 }

@@ -18,6 +18,7 @@ class Host:
         lib.fake_unfinished.restype = C.c_int
         lib.fake_calls.restype = lib.fake_live.restype = lib.fake_log.restype = lib.fake_news.restype = C.c_long
         lib.fake_fail_at.argtypes = lib.fake_no_memory_at.argtypes = [C.c_long]
+        lib.fake_device.argtypes = [C.c_int]
         lib.fake_user_capture.argtypes = [C.c_void_p, C.c_int]
         self.next = 1 << 40
         self.keep = []
@@ -289,6 +290,23 @@ def test_no_call_throws_when_the_host_is_out_of_memory(host, warm):
         assert rc == (gb.GEAR_ERR_CUDA if hit else 0) and lib.fake_unfinished() == 0, k
     for c in ctxs:
         assert lib.gear_destroy(c) == 0
+
+
+def test_kernels_get_their_shared_memory_on_every_device(host):
+    """Contexts on a second device of the process: what a kernel may take beyond 48 KB is asked for there too."""
+    lib = host.lib
+    for device in (0, 1):
+        lib.fake_device(device)
+        for head in (0, 1):
+            for hidden in ((64,), (128, 64), (256, 192), (512, 256), (512, 320)) + (((24,), (256, 136)) if head == 0 else ()):
+                for B, nnz in ((64, 200), (1200, 3600), (2400, 7000), (8000, 40_000), (60_000, 600_000)):
+                    ctx = host.ctx(B, nnz, hidden=hidden, head=head)
+                    rc = lib.gear_step(ctx, host.batch(B, nnz), 0.1, host.out(), host.lists(nnz), 1, 1, 1, None, STREAM)
+                    assert rc == 0, (device, head, hidden, B, lib.gear_last_error())
+                    assert lib.gear_dense_forward(ctx, host.address(), 32, host.address(), host.address(), 10, None, host.address(), 64, STREAM) == 0
+                    assert lib.gear_dense_forward(ctx, host.address(), 33, host.address() + 4, host.address(), 10, None, host.address(), 64, STREAM) == 0
+                    assert lib.gear_destroy(ctx) == 0
+    lib.fake_device(0)
 
 
 @pytest.mark.parametrize("head", [0, 1])
