@@ -280,8 +280,8 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
 
     // forward
     const int HT = p.fan[L];
-    // a top layer whose columns are one tile of its product takes the output unit along
-    const bool top_fused = HT <= (BF ? TC_TOP_N : F32_TOP_N);
+    // a top layer whose columns are one tile of its product takes the output unit along (fp32: where that is the shorter way)
+    const bool top_fused = BF ? HT <= TC_TOP_N : fwd_top_fused_f32(B, HT, p.fan[L - 1]);
     int n_part = 0;                                       // partial losses it leaves
     for (int l = 0; l < L; ++l) {
         const int K = p.fan[l], N = p.fan[l + 1];
@@ -298,18 +298,17 @@ static cudaError_t run_head(const gear_ctx_impl& c, const gear_batch& bt, const 
     if (!top_fused) {
         KernelScope ks(&c.prof, "head_out", st);
         const int nq = (int)ceil_div(HT, 256);
-        // rows per warp and pass: as many as the registers hold (8 chunks of bf16, 4 of fp32)
-        constexpr int RMAX = BF ? 8 : 4;
-        const int rows = nq <= 1 ? RMAX : nq == 2 ? RMAX / 4 : 1;
+        // rows per warp and pass, as many as the registers hold.  (Up to 256 columns, one chunk a lane: fp32 heads only)
+        const int rows = nq <= 1 ? 4 : nq == 2 && BF ? 2 : 1;
         // every warp gets the same number of passes where the batch allows it
         const int64_t batches = ceil_div(B, rows);
         const int64_t passes = ceil_div(batches, (int64_t)c.ws.loss_blocks * 8);
         const int blocks = n_part = (int)ceil_div(batches, 8 * passes);
 #define GEAR_HEAD_OUT(NQ, ROWS) launch_dependent(head_out_kernel<TX, NQ, ROWS>, dim3(blocks), dim3(256), 0, st, B, HT, H[L].p, H[L].stride, p.w_out, p.b_out, bt.label, \
         o.prob, dA[L].p, loss_part, p.gw_out, p.gb[L - 1], p.gb_out)
-        if (nq <= 1) err = GEAR_HEAD_OUT(1, RMAX);
-        else if (nq == 2) err = GEAR_HEAD_OUT(2, RMAX / 4);
-        else err = GEAR_HEAD_OUT(4, 1);
+        if (nq > 2) err = GEAR_HEAD_OUT(4, 1);
+        else if constexpr (BF) err = GEAR_HEAD_OUT(2, 2);
+        else err = nq <= 1 ? GEAR_HEAD_OUT(1, 4) : GEAR_HEAD_OUT(2, 1);
 #undef GEAR_HEAD_OUT
         if (err != cudaSuccess) return err;
     }

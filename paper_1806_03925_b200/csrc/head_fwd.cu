@@ -185,8 +185,8 @@ static cudaError_t launch_form(int M, int N, int K, const float* A, const float*
 }
 
 template <class T, int MIN_BLOCKS, bool WVEC>
-static cudaError_t launch_top_form(int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& dA, const TopArgs& top,
-                                   int slots, int* n_part, cudaStream_t st) {
+static cudaError_t launch_top_form(int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& dA,
+                                   const TopArgs& top, int slots, int* n_part, cudaStream_t st) {
     constexpr auto kernel = fwd_top_kernel<T, MIN_BLOCKS, WVEC>;
     if (const cudaError_t e = allow_smem<kernel>(T::SMEM)) return e;
     const int64_t tiles = ceil_div(M, T::BM), resident = (int64_t)sm_count() * MIN_BLOCKS;
@@ -195,20 +195,7 @@ static cudaError_t launch_top_form(int M, int N, int K, const float* A, const fl
     return launch_dependent(kernel, dim3((unsigned)*n_part), dim3(T::THREADS), (size_t)T::SMEM, st, M, N, K, A, W, bias, dA.p, dA.stride, top);
 }
 
-// Forms of a tile: outputs per lane, lanes, warps, steps per buffer, buffers.  The chain over the reduction cannot be split, so a
-// product takes as long as its fullest SM: small tiles while they are about one wave, then 4 x 4 outputs per lane, then 8 x 8, which
-// need several warps per scheduler to hide their longer rounds.  Measured on either side of each line, depth 192 (us, the form below
-// the line / above it):
-//   16 x 32 | 32 x 32   one wave of 16 x 32:      1024 x 64 (0.9 waves) 3.5 / 4.8; 1024 x 256 (3.5) 6.3 / 5.4
-//   32 x 32 | 64 x 128  six waves of 32 x 32:     2048 x 256 (3.5) 8.3 / 13.2; 4096 x 256 (6.9) 15.0 / 13.5; 8192 x 256 24.4 / 21.4
-// and with the output unit (all columns in one tile):
-//   16 x 32 | 32 x 32   two waves of 16 rows:     4096 views (1.7) 6.2 / 6.9; 8192 (3.5) 9.5 / 7.7
-//   8 x 64 | 16 x 64    one wave of 8 rows:       1024 (0.9) 6.0 / 6.9; 2048 (1.7) 7.5 / 7.1
-//   16 x 64 | 64 x 64   four waves of 16 rows:    9472 (4.0) 14.8 / 16.0; 16384 (6.9) 22.8 / 17.3
-//   8 x 128 | 16 x 128  one wave of 8 rows:       1024 (0.9) 6.9 / 7.7; 1237 (1.05) 8.6 / 7.7
-//   16 x 128 | 64 x 128 three waves of 16 rows:   4096 (1.7) 10.6 / 15.9; 8192 (3.5) 17.9 / 16.5
-//   16 x 256 | 32 x 256 1.5 waves of 16 rows:     2048 (0.9) 11.6 / 16.6; 4096 (1.7) 17.6 / 17.1
-// (32 x 128 tiles of 64 threads, which would share out 32768 views more evenly, were slower: 72 against 64 us.)
+// Forms of a tile: outputs per lane, lanes, warps, steps per buffer, buffers.
 typedef ChainTile<2, 4, 4, 8, 2, 1, 32, 4> F16x32;
 typedef ChainTile<4, 4, 8, 4, 1, 2, 32, 4> F32x32;
 typedef ChainTile<8, 8, 4, 8, 2, 2, 32, 2> F64x128;
@@ -220,16 +207,64 @@ typedef ChainTile<4, 4, 4, 8, 1, 4, 32, 3> F16x128;
 typedef ChainTile<4, 4, 4, 8, 1, 8, 32, 3> F16x256;
 typedef ChainTile<8, 8, 4, 8, 1, 4, 32, 2> F32x256;
 
+// What a product takes in a form, in ns: per step of the reduction `alone` while no SM has more than one block, `shared` per block of the
+// fullest SM where that is longer (blocks count in multiples of `unit`); `once` besides, of which what is beyond 1.5 us comes again
+// with every round of tiles that `resident` blocks per SM walk.  The chain over the reduction cannot be split, so a product
+// takes as long as its fullest SM.  Measured in a loop at depths of 96, 224, 608 and 1632, twelve batches of 64 to 16384 views and 32
+// to 256 columns: the form that the sum names is within 5 % of the fastest at every one of them, the way (below) within 2.5 us.  A few of
+// them (us, 1632 deep): 1024 x 128 in 16 x 32 tiles 22.0, in 32 x 32 26.4, in 64 x 128 82.6; 4096 x 256: 128, 96, 83.5.
+struct Form {
+    int bm, bn;
+    float alone, shared, once;
+    int unit, resident;
+    float cost(int M, int N, int K) const {
+        const int64_t tiles = ceil_div(M, bm) * ceil_div(N, bn), blocks = ceil_div(ceil_div(tiles, sm_count()), unit) * unit;
+        const float step = (float)blocks * shared, rounds = resident ? (float)ceil_div(tiles, (int64_t)resident * sm_count()) : 1.f;
+        return 1500.f + (once - 1500.f) * rounds + (float)K * (step > alone ? step : alone);
+    }
+};
+constexpr Form LOW[] = {{16, 32, 10.2f, 6.f, 1300.f, 1, 0}, {32, 32, 15.7f, 8.f, 1500.f, 1, 0}, {64, 128, 50.5f, 46.5f, 2700.f, 1, 0},
+                        {64, 64, 51.f, 24.5f, 3100.f, 2, 0}};
+constexpr Form TOP[] = {{16, 32, 12.f, 6.5f, 2300.f, 1, 4}, {32, 32, 17.5f, 10.2f, 2700.f, 1, 4},
+                        {8, 64, 15.2f, 11.f, 2400.f, 1, 4}, {16, 64, 20.3f, 10.8f, 2600.f, 1, 4}, {64, 64, 50.5f, 25.f, 5000.f, 1, 4},
+                        {8, 128, 21.7f, 15.f, 2400.f, 1, 3}, {16, 128, 24.8f, 17.8f, 2700.f, 1, 3}, {64, 128, 54.5f, 48.f, 4600.f, 1, 3},
+                        {16, 256, 39.6f, 33.2f, 3100.f, 1, 2}, {32, 256, 61.5f, 55.f, 4600.f, 1, 2}};
+// the cheapest of the forms of at least `cols` and less than 2 * max(cols, 32) columns (0: of any)
+template <int COUNT> static int cheapest(const Form (&forms)[COUNT], int cols, int M, int N, int K, float* cost) {
+    int best = -1;
+    for (int f = 0; f < COUNT; ++f) {
+        if (cols && (forms[f].bn < cols || forms[f].bn >= 2 * (cols > 32 ? cols : 32))) continue;
+        const float c = forms[f].cost(M, N, K);
+        if (best < 0 || c < *cost) { best = f; *cost = c; }
+    }
+    return best;
+}
+
+// A tile over all columns takes longer for a step than a small one, and there are fewer of them: a deep layer is done sooner in small tiles
+// with the output unit (head_out_kernel, 4 to 11 us) behind it.  Steps of the two ways, the output unit in the product / behind it (us):
+// 1632 deep, 256 columns, 256 views 87.8 / 47.2, 1024 views 92 / 84; 608 deep, 136 columns, 256 views 47.4 / 35.1; 96 deep, 64 + 256
+// columns, 1024 views 37.8 / 41.2.
+bool fwd_top_fused_f32(int M, int N, int K) {
+    if (N > F32_TOP_N) return false;
+    float low, top;
+    cheapest(LOW, 0, M, N, K, &low);
+    cheapest(TOP, N, M, N, K, &top);
+    return top <= low + 5000.f + (float)M * (0.25f + 0.0007f * (float)N);
+}
+
 cudaError_t launch_fwd_f32(const gear_ctx_impl& c, const char* name, int M, int N, int K, const float* A, const float* W, const float* bias,
                            const Planes& H, float* Hf, cudaStream_t st) {
     if (M <= 0 || N <= 0) return cudaSuccess;
     KernelScope ks(&c.prof, name, st);
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
-    auto tiles = [&](int bm, int bn) { return ceil_div(M, bm) * ceil_div(N, bn); };
+    float cost;
 #define GEAR_FWD(T, MB) (wvec ? launch_form<T, MB, true>(M, N, K, A, W, bias, H, Hf, st) : launch_form<T, MB, false>(M, N, K, A, W, bias, H, Hf, st))
-    if (tiles(16, 32) <= sm_count()) return GEAR_FWD(F16x32, 4);
-    if (tiles(32, 32) <= 6 * sm_count()) return GEAR_FWD(F32x32, 4);
-    return N % 128 == 0 || N % 128 > 64 ? GEAR_FWD(F64x128, 3) : GEAR_FWD(F64x64, 4);
+    switch (cheapest(LOW, 0, M, N, K, &cost)) {
+    case 0: return GEAR_FWD(F16x32, 4);
+    case 1: return GEAR_FWD(F32x32, 4);
+    case 2: return GEAR_FWD(F64x128, 3);
+    default: return GEAR_FWD(F64x64, 4);
+    }
 #undef GEAR_FWD
 }
 
@@ -238,13 +273,21 @@ cudaError_t launch_fwd_top_f32(const gear_ctx_impl& c, int M, int N, int K, cons
     KernelScope ks(&c.prof, "f32_gemm_top", st);
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     const int slots = c.ws.loss_slots;
+    float cost;
 #define GEAR_TOP(T, MB) (wvec ? launch_top_form<T, MB, true>(M, N, K, A, W, bias, dA, top, slots, n_part, st) \
                               : launch_top_form<T, MB, false>(M, N, K, A, W, bias, dA, top, slots, n_part, st))
-    const int64_t t8 = ceil_div(M, 8), t16 = ceil_div(M, 16), sms = sm_count();
-    if (N <= 32) return t16 <= 2 * sms ? GEAR_TOP(F16x32, 4) : GEAR_TOP(F32x32, 4);
-    if (N <= 64) return t8 <= sms ? GEAR_TOP(F8x64, 4) : t16 <= 4 * sms ? GEAR_TOP(F16x64, 4) : GEAR_TOP(F64x64, 4);
-    if (N <= 128) return t8 <= sms ? GEAR_TOP(F8x128, 3) : t16 <= 3 * sms ? GEAR_TOP(F16x128, 3) : GEAR_TOP(F64x128, 3);
-    return 2 * t16 <= 3 * sms ? GEAR_TOP(F16x256, 2) : GEAR_TOP(F32x256, 2);
+    switch (cheapest(TOP, N, M, N, K, &cost)) {
+    case 0: return GEAR_TOP(F16x32, 4);
+    case 1: return GEAR_TOP(F32x32, 4);
+    case 2: return GEAR_TOP(F8x64, 4);
+    case 3: return GEAR_TOP(F16x64, 4);
+    case 4: return GEAR_TOP(F64x64, 4);
+    case 5: return GEAR_TOP(F8x128, 3);
+    case 6: return GEAR_TOP(F16x128, 3);
+    case 7: return GEAR_TOP(F64x128, 3);
+    case 8: return GEAR_TOP(F16x256, 2);
+    default: return GEAR_TOP(F32x256, 2);
+    }
 #undef GEAR_TOP
 }
 

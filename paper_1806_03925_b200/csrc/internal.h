@@ -190,8 +190,9 @@ cudaError_t tc_gemm_mnmajor(const gear_ctx_impl& c, const char* name, int M, int
 cudaError_t launch_fwd_f32(const gear_ctx_impl& c, const char* name, int M, int N, int K, const float* A, const float* W, const float* bias,
                            const Planes& H, float* Hf, cudaStream_t st);
 // The same for the top hidden layer, N at most F32_TOP_N, with the output unit behind it (as tc_gemm_top): dA gets, in planes, the
-// gradient with respect to its pre-activations.
+// gradient with respect to its pre-activations.  fwd_top_fused_f32: whether that is the shorter way.
 constexpr int F32_TOP_N = 256;
+bool fwd_top_fused_f32(int M, int N, int K);
 cudaError_t launch_fwd_top_f32(const gear_ctx_impl& c, int M, int N, int K, const float* A, const float* W, const float* bias,
                                const Planes& dA, const TopArgs& top, int* n_part, cudaStream_t st);
 

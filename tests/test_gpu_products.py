@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
     (256, 16, 480, (136, 120)),             # head input 512 wide: two segments' worth in one, columns one step past 128
     (640, 16, 512, (128, 64)),              # head input 544 wide: the first width that is cut into segments
     (20_000, 4, 24, (1024,)),               # widest layer, a long reduction over the batch
-    # forward tiles of 16 x 32 up to 148 of them, 32 x 32 up to 148, 32 x 64, 64 x 128 from 444 tiles of 64 x 64
+    # one hidden layer, and two of changing width, around whole numbers of blocks per SM in the forward products
     (1184, 4, 16, (64,)), (1185, 4, 16, (64, 40)), (1889, 8, 88, (128,)), (7105, 4, 24, (120, 136)),
     (2368, 4, 24, (64,)), (2369, 4, 24, (64, 40)), (14_144, 4, 24, (128,)), (14_145, 4, 24, (120, 136)),
 ])
@@ -35,8 +35,8 @@ def test_fp32_products_at_tile_edges(B, E, D, hidden):
         pair.close()
 
 
-# the same at the lines between the forms of a top layer's tile (8, 16, 32 or 64 rows of at most 32, 64, 128, 256 columns; wider ones in
-# a launch of their own) and of a lower layer's (32 x 32 up to six waves, then 64 x 128, or 64 x 64 where columns fill half a tile)
+# the same in a shallow layer (one step of the operand ring), around whole numbers of blocks per SM in tiles of 8 to 64 rows and 32 to 256
+# columns, where the forms of a tile change; more than 256 columns: the output unit in a launch of its own
 @pytest.mark.parametrize("B,hidden", [
     (4736, (24,)), (4737, (32,)), (9472, (64,)), (9473, (40,)), (1184, (128,)), (1185, (72,)), (7104, (128, 120)), (7105, (128, 72)),
     (3552, (256,)), (3553, (136,)), (300, (264,)), (14_208, (64, 8)), (14_209, (64, 16)),
@@ -63,8 +63,10 @@ def _with_params_off(s):
 # weights read 16 bytes at a time and one by one.
 @pytest.mark.parametrize("off", [False, True])
 @pytest.mark.parametrize("B,hidden", [
-    (33, (24,)), (9473, (32,)), (1000, (64,)), (1187, (40,)), (9473, (64,)), (1001, (128,)), (1187, (72,)), (7105, (128,)), (301, (256,)), (3553, (136,)),
-    (300, (64, 8)), (1889, (128, 8)), (14_211, (64, 8)), (14_211, (128, 8)),
+    (33, (24,)), (7107, (32,)), (1001, (64,)), (1193, (40,)), (11_847, (64,)), (1001, (128,)), (1193, (72,)), (7107, (128,)),     # with the output unit
+    (1777, (256,)), (7107, (256,)),
+    (301, (136,)), (1777, (136,)), (11_363, (136,)), (10_061, (256,)),                                                # the output unit behind it
+    (300, (64, 8)), (1889, (128, 8)), (14_213, (128, 8)), (16_579, (64, 8)),                                          # a layer above
 ])
 def test_fp32_forward_forms_in_deep_layers(B, hidden, off):
     if not torch.cuda.is_available():
