@@ -175,24 +175,38 @@ fwd_top_kernel(int M, int N, int K, const float* __restrict__ A, const float* __
     }
 }
 
-template <class T, int MIN_BLOCKS, bool WVEC>
-static cudaError_t launch_form(int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& H, float* Hf, cudaStream_t st) {
-    constexpr auto kernel = fwd_kernel<T, MIN_BLOCKS, WVEC>;
-    if (const cudaError_t e = allow_smem<kernel>(T::SMEM)) return e;
-    const int64_t rows = ceil_div(M, T::BM), y = rows < 65535 ? rows : 65535;
-    return launch_dependent(kernel, dim3((unsigned)ceil_div(N, T::BN), (unsigned)y, (unsigned)ceil_div(rows, y)), dim3(T::THREADS),
-                            (size_t)T::SMEM, st, M, N, K, A, W, bias, H.p, H.stride, Hf);
+// Shared memory a block asks for.  All blocks of a wave are placed within a microsecond, on the SMs that are free at that moment: 256 of
+// them went to 75 SMs, four each, while the ID sort and the expiry scan had begun on the other 73 (4096 x 1632 x 256: 164 us instead
+// of 97, step 265 us instead of 199; 1024 x 1632 x 256: 46 and 32 us).  A block of a long product asks for so much that no SM
+// takes more blocks than an even spread gives it.  Short products have ended by the time it matters, and keep the sort waiting
+// (1024 x 608 x 64, 12 us: step 37.0 us as it comes, 39.3 spread; 2048 views, 15 us: 45.2, 47.3).
+constexpr int SM_SMEM = 228 * 1024, EVEN_SMEM_MAX = SM_SMEM / 2 - 512;
+static int even_smem(int own, int64_t blocks, float cost) {
+    const int share = SM_SMEM / (int)(ceil_div(blocks, sm_count()) + 1) - 512;          // (a block takes 1 KB more than it asks for)
+    return cost < 16000.f || share < own ? own : share;
 }
 
 template <class T, int MIN_BLOCKS, bool WVEC>
-static cudaError_t launch_top_form(int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& dA,
+static cudaError_t launch_form(float cost, int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& H, float* Hf,
+                               cudaStream_t st) {
+    constexpr auto kernel = fwd_kernel<T, MIN_BLOCKS, WVEC>;
+    static_assert(T::SMEM <= EVEN_SMEM_MAX, "two blocks per SM");
+    if (const cudaError_t e = allow_smem<kernel>(EVEN_SMEM_MAX)) return e;
+    const int64_t rows = ceil_div(M, T::BM), y = rows < 65535 ? rows : 65535;
+    return launch_dependent(kernel, dim3((unsigned)ceil_div(N, T::BN), (unsigned)y, (unsigned)ceil_div(rows, y)), dim3(T::THREADS),
+                            (size_t)even_smem(T::SMEM, rows * ceil_div(N, T::BN), cost), st, M, N, K, A, W, bias, H.p, H.stride, Hf);
+}
+
+template <class T, int MIN_BLOCKS, bool WVEC>
+static cudaError_t launch_top_form(float cost, int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& dA,
                                    const TopArgs& top, int slots, int* n_part, cudaStream_t st) {
     constexpr auto kernel = fwd_top_kernel<T, MIN_BLOCKS, WVEC>;
-    if (const cudaError_t e = allow_smem<kernel>(T::SMEM)) return e;
+    static_assert(T::SMEM <= EVEN_SMEM_MAX, "two blocks per SM");
+    if (const cudaError_t e = allow_smem<kernel>(EVEN_SMEM_MAX)) return e;
     const int64_t tiles = ceil_div(M, T::BM), resident = (int64_t)sm_count() * MIN_BLOCKS;
     const int64_t most = resident < slots ? resident : slots;
     *n_part = (int)(tiles < most ? tiles : most);
-    return launch_dependent(kernel, dim3((unsigned)*n_part), dim3(T::THREADS), (size_t)T::SMEM, st, M, N, K, A, W, bias, dA.p, dA.stride, top);
+    return launch_dependent(kernel, dim3((unsigned)*n_part), dim3(T::THREADS), (size_t)even_smem(T::SMEM, *n_part, cost), st, M, N, K, A, W, bias, dA.p, dA.stride, top);
 }
 
 // Forms of a tile: outputs per lane, lanes, warps, steps per buffer, buffers.
@@ -258,7 +272,7 @@ cudaError_t launch_fwd_f32(const gear_ctx_impl& c, const char* name, int M, int 
     KernelScope ks(&c.prof, name, st);
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     float cost;
-#define GEAR_FWD(T, MB) (wvec ? launch_form<T, MB, true>(M, N, K, A, W, bias, H, Hf, st) : launch_form<T, MB, false>(M, N, K, A, W, bias, H, Hf, st))
+#define GEAR_FWD(T, MB) (wvec ? launch_form<T, MB, true>(cost, M, N, K, A, W, bias, H, Hf, st) : launch_form<T, MB, false>(cost, M, N, K, A, W, bias, H, Hf, st))
     switch (cheapest(LOW, 0, M, N, K, &cost)) {
     case 0: return GEAR_FWD(F16x32, 4);
     case 1: return GEAR_FWD(F32x32, 4);
@@ -274,8 +288,8 @@ cudaError_t launch_fwd_top_f32(const gear_ctx_impl& c, int M, int N, int K, cons
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     const int slots = c.ws.loss_slots;
     float cost;
-#define GEAR_TOP(T, MB) (wvec ? launch_top_form<T, MB, true>(M, N, K, A, W, bias, dA, top, slots, n_part, st) \
-                              : launch_top_form<T, MB, false>(M, N, K, A, W, bias, dA, top, slots, n_part, st))
+#define GEAR_TOP(T, MB) (wvec ? launch_top_form<T, MB, true>(cost, M, N, K, A, W, bias, dA, top, slots, n_part, st) \
+                              : launch_top_form<T, MB, false>(cost, M, N, K, A, W, bias, dA, top, slots, n_part, st))
     switch (cheapest(TOP, N, M, N, K, &cost)) {
     case 0: return GEAR_TOP(F16x32, 4);
     case 1: return GEAR_TOP(F32x32, 4);
