@@ -155,7 +155,7 @@ template <typename TD, bool HB, int NQ, bool FULL>
 __global__ void __launch_bounds__(GP_WARPS * 32, NQ <= 2 ? 3 : 2)
 gather_pool_kernel(const __grid_constant__ GatherArgs a) {
     wait_for_predecessor();
-    if (gridDim.x <= FEW_BLOCKS) let_successor_start();
+    if (gridDim.x - (unsigned)a.w_blocks <= FEW_BLOCKS) let_successor_start();       // (the weights' blocks are soon gone)
     if constexpr (HB)
         if ((int)blockIdx.x < a.w_blocks) { round_weights_block<1>(a.weights, (int)blockIdx.x, a.w_blocks); return; }
     const int block = (int)blockIdx.x - a.w_blocks, blocks = (int)gridDim.x - a.w_blocks;
