@@ -1,7 +1,7 @@
 // bf16 matrix products of the head on the 5th-generation tensor cores (sm_100a):
 // tcgen05.mma with fp32 accumulators in tensor memory, operands staged in shared memory by TMA.
 //
-// One persistent kernel, one CTA per SM, three roles:
+// One persistent kernel, one CTA per SM (two where tiles are 64 columns wide), three roles:
 //   warp 0     TMA producer: streams 128 x 64 (A) and BN x 64 (B) bf16 tiles through a ring of
 //              shared-memory stages (128-byte swizzle), one mbarrier pair per stage;
 //   warp 1     MMA issuer: one elected lane issues tcgen05.mma (M 128, N BN, K 16) into one of two
@@ -577,10 +577,9 @@ __device__ __forceinline__ void tc_gemm_body(const CUtensorMap& map_a, const CUt
 }
 
 // Eight epilogue warps, at most 128 registers per thread: a CTA (320 threads) then fits on an SM beside a block of
-// the ID sort.  One CTA per SM follows from the shared-memory footprint.
-// (64-column tiles: few enough for two CTAs, the top layer's of 128 columns for one of each.)
+// the ID sort.  One CTA per SM follows from the shared-memory footprint; of 64-column tiles two fit, in registers too.
 template <int BN, bool MN_MAJOR, int EPI>
-__global__ void __maxnreg__(BN == 64 ? 88 : EPI == TC_EPI_TOP && BN == 128 ? 112 : 128)
+__global__ void __maxnreg__(BN == 64 ? 88 : 128)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
                const __grid_constant__ CUtensorMap map_out, const __grid_constant__ CUtensorMap map_mask, const TcArgs g) {
     tc_gemm_body<BN, MN_MAJOR, EPI, 8>(map_a, map_b, map_out, map_mask, g);
