@@ -60,7 +60,7 @@ dense_forward_kernel(const float* __restrict__ raw, int64_t vocab, int R, const 
         DenseTile::Acc acc;
         DenseTile::product<AVEC, BVEC>(acc, R, reinterpret_cast<float*>(dyn_smem),
                                        [&](int r) -> const float* { const int64_t id = row_of[r]; return id >= 0 ? raw + id * R : nullptr; },
-                                       raw, Wd + n0, D, D - n0);
+                                       Wd + n0, D, D - n0);
 #pragma unroll
         for (int i = 0; i < DenseTile::TM; ++i) {
             const int64_t m = m0 + DenseTile::row(i);
@@ -155,11 +155,7 @@ cudaError_t launch_dense_forward(const gear_ctx_impl& c, const float* raw, int R
     const int64_t want = ceil_div(n, DenseTile::BM) * ceil_div(c.cfg.dfv_dim, DenseTile::BN), cap = (int64_t)sm_count() * 4;
     const dim3 grid((unsigned)(want < cap ? want : cap));
     const bool avec = (R & 3) == 0 && (reinterpret_cast<uintptr_t>(raw) & 15u) == 0, bvec = (reinterpret_cast<uintptr_t>(Wd) & 15u) == 0;
-    cudaError_t e = allow_smem<dense_forward_kernel<true, true>>(DenseTile::SMEM);
-    if (e == cudaSuccess) e = allow_smem<dense_forward_kernel<true, false>>(DenseTile::SMEM);
-    if (e == cudaSuccess) e = allow_smem<dense_forward_kernel<false, true>>(DenseTile::SMEM);
-    if (e == cudaSuccess) e = allow_smem<dense_forward_kernel<false, false>>(DenseTile::SMEM);
-    if (e != cudaSuccess) return e;
+    static_assert(DenseTile::SMEM + DenseTile::BM * 8 <= 48 * 1024, "a launch may have this much without asking");
 #define GEAR_DF(A, B) launch_dependent(dense_forward_kernel<A, B>, grid, dim3(DenseTile::THREADS), (size_t)DenseTile::SMEM, st, raw, c.cfg.img_vocab, R, Wd, c.cfg.dfv_dim, ids, n, d_n, rows, ld, c.state())
     return avec ? (bvec ? GEAR_DF(true, true) : GEAR_DF(true, false)) : (bvec ? GEAR_DF(false, true) : GEAR_DF(false, false));
 #undef GEAR_DF

@@ -42,16 +42,16 @@ template <int TM_, int TN_, int LR, int LC, int WR_, int WC_, int BK_, int STAGE
     static __device__ __forceinline__ int row(int i) { return warp_row() * (TM * LR) + i * LR + (int)(threadIdx.x % 32) / LC; }
     static __device__ __forceinline__ int col(int j) { return warp_col() * (TN * LC) + j * (4 * LC) + (int)(threadIdx.x % LC) * 4; }
 
-    // acc = A . B over k < K.  a_row(r): row r of the tile in memory, or null (zeros); a: any row of A; b: element (0, first column
-    // of the tile), rows ldb apart, n_cols columns exist.  AVEC / BVEC: A's rows / B's rows may be read 16 bytes at a time (lengths
-    // and strides are multiples of four then).  smem: SMEM bytes, free when the block enters and when it leaves.
-    // A copy that fills with zeros names an address of its own operand: a copy's source has to be aligned to the copy's size also
-    // where nothing is read, and either operand may be the one that is not.
+    // acc = A . B over k < K.  a_row(r): row r of the tile in memory, or null (zeros); b: element (0, first column of the tile),
+    // rows ldb apart, n_cols columns exist.  AVEC / BVEC: A's rows / B's rows may be read 16 bytes at a time (lengths and strides
+    // are multiples of four then).  smem: SMEM bytes, free when the block enters and when it leaves.
     template <bool AVEC, bool BVEC, typename ARow>
-    static __device__ __forceinline__ void product(Acc& acc, int K, float* smem, ARow a_row, const float* __restrict__ a, const float* __restrict__ b,
-                                                   int64_t ldb, int n_cols) {
+    static __device__ __forceinline__ void product(Acc& acc, int K, float* smem, ARow a_row, const float* __restrict__ b, int64_t ldb, int n_cols) {
         const int tid = threadIdx.x;
         const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(smem);
+        // What a copy that fills with zeros names as its source: that has to be aligned to the copy's size also where nothing is read.  (A
+        // pointer to A in its place, one more register pair in the loop: 32 x 256 tiles 8 % slower.)
+        const float* none = AVEC && !BVEC ? reinterpret_cast<const float*>(reinterpret_cast<uintptr_t>(b) & ~(uintptr_t)15) : b;
         const float* pa[A_PIECES];
 #pragma unroll
         for (int q = 0; q < A_PIECES; ++q) {
@@ -67,10 +67,10 @@ template <int TM_, int TN_, int LR, int LC, int WR_, int WC_, int BK_, int STAGE
                 if (A_QUADS % THREADS != 0 && p >= A_QUADS) break;
                 const int k = k0 + 4 * (p % (BK / 4));
                 const uint32_t dst = sa + (uint32_t)((p / (BK / 4)) * PITCH + 4 * (p % (BK / 4))) * 4u;
-                if (AVEC) { const bool on = pa[q] && k < K; cp_async_16(dst, on ? pa[q] + k0 : a, on ? 16 : 0); }
+                if (AVEC) { const bool on = pa[q] && k < K; cp_async_16(dst, on ? pa[q] + k0 : none, on ? 16 : 0); }
                 else
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) { const bool on = pa[q] && k + e < K; cp_async_4(dst + 4u * e, on ? pa[q] + k0 + e : a, on ? 4 : 0); }
+                    for (int e = 0; e < 4; ++e) { const bool on = pa[q] && k + e < K; cp_async_4(dst + 4u * e, on ? pa[q] + k0 + e : none, on ? 4 : 0); }
             }
 #pragma unroll
             for (int q = 0; q < B_PIECES; ++q) {

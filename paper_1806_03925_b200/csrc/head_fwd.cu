@@ -25,7 +25,7 @@ fwd_kernel(int M, int N, int K, const float* __restrict__ A, const float* __rest
     if (m0 >= M) return;                                            // (the last layer of more row tiles than a grid dimension takes)
     typename T::Acc acc;
     T::template product<true, WVEC>(acc, K, reinterpret_cast<float*>(dyn_smem),
-                                    [&](int r) -> const float* { return m0 + r < M ? A + (int64_t)(m0 + r) * K : nullptr; }, A, W + n0, N, N - n0);
+                                    [&](int r) -> const float* { return m0 + r < M ? A + (int64_t)(m0 + r) * K : nullptr; }, W + n0, N, N - n0);
 #pragma unroll
     for (int j = 0; j < T::TN / 4; ++j) {
         const int n = n0 + T::col(j);
@@ -72,7 +72,7 @@ fwd_top_kernel(int M, int N, int K, const float* __restrict__ A, const float* __
         const int m0 = mt * T::BM;
         typename T::Acc acc;
         T::template product<true, WVEC>(acc, K, reinterpret_cast<float*>(dyn_smem),
-                                        [&](int r) -> const float* { return m0 + r < M ? A + (int64_t)(m0 + r) * K : nullptr; }, A, W, N, N);
+                                        [&](int r) -> const float* { return m0 + r < M ? A + (int64_t)(m0 + r) * K : nullptr; }, W, N, N);
         // activations; a lane's part of its rows' dot products
         float z[T::TM];
 #pragma unroll
