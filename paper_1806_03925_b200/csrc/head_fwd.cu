@@ -175,30 +175,27 @@ fwd_top_kernel(int M, int N, int K, const float* __restrict__ A, const float* __
     }
 }
 
-// Shared memory a block asks for.  All blocks of a wave are placed within a microsecond, on the SMs that are free at that moment: 256 of
-// them went to 75 SMs, four each, while the ID sort and the expiry scan had begun on the other 73 (4096 x 1632 x 256: 164 us instead
-// of 97, step 265 us instead of 199; 1024 x 1632 x 256: 46 and 32 us).  A block of a long product asks for so much that no SM
-// takes more blocks than an even spread gives it.  Short products have ended by the time it matters, and keep the sort waiting
-// (1024 x 608 x 64, 12 us: step 37.0 us as it comes, 39.3 spread; 2048 views, 15 us: 45.2, 47.3).
+// Shared memory a block asks for: so much, where `even`, that no SM takes more of them than an even spread gives it.
 constexpr int SM_SMEM = 228 * 1024, EVEN_SMEM_MAX = SM_SMEM / 2 - 512;
-static int even_smem(int own, int64_t blocks, float cost) {
-    const int share = SM_SMEM / (int)(ceil_div(blocks, sm_count()) + 1) - 512;          // (a block takes 1 KB more than it asks for)
-    return cost < 16000.f || share < own ? own : share;
+template <auto Kernel> static int even_smem(int own, int threads, int64_t blocks, bool even) {
+    static const int fit = [&] { int n = 0; return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, Kernel, threads, own) == cudaSuccess ? n : 0; }();
+    const int64_t per = ceil_div(blocks, sm_count());
+    return even && per < fit ? (int)(SM_SMEM / (per + 1)) - 512 : own;                   // (a block takes 1 KB more than it asks for)
 }
 
 template <class T, int MIN_BLOCKS, bool WVEC>
-static cudaError_t launch_form(float cost, int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& H, float* Hf,
+static cudaError_t launch_form(bool even, int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& H, float* Hf,
                                cudaStream_t st) {
     constexpr auto kernel = fwd_kernel<T, MIN_BLOCKS, WVEC>;
     static_assert(T::SMEM <= EVEN_SMEM_MAX, "two blocks per SM");
     if (const cudaError_t e = allow_smem<kernel>(EVEN_SMEM_MAX)) return e;
     const int64_t rows = ceil_div(M, T::BM), y = rows < 65535 ? rows : 65535;
     return launch_dependent(kernel, dim3((unsigned)ceil_div(N, T::BN), (unsigned)y, (unsigned)ceil_div(rows, y)), dim3(T::THREADS),
-                            (size_t)even_smem(T::SMEM, rows * ceil_div(N, T::BN), cost), st, M, N, K, A, W, bias, H.p, H.stride, Hf);
+                            (size_t)even_smem<kernel>(T::SMEM, T::THREADS, rows * ceil_div(N, T::BN), even), st, M, N, K, A, W, bias, H.p, H.stride, Hf);
 }
 
 template <class T, int MIN_BLOCKS, bool WVEC>
-static cudaError_t launch_top_form(float cost, int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& dA,
+static cudaError_t launch_top_form(bool even, int M, int N, int K, const float* A, const float* W, const float* bias, const Planes& dA,
                                    const TopArgs& top, int slots, int* n_part, cudaStream_t st) {
     constexpr auto kernel = fwd_top_kernel<T, MIN_BLOCKS, WVEC>;
     static_assert(T::SMEM <= EVEN_SMEM_MAX, "two blocks per SM");
@@ -206,7 +203,7 @@ static cudaError_t launch_top_form(float cost, int M, int N, int K, const float*
     const int64_t tiles = ceil_div(M, T::BM), resident = (int64_t)sm_count() * MIN_BLOCKS;
     const int64_t most = resident < slots ? resident : slots;
     *n_part = (int)(tiles < most ? tiles : most);
-    return launch_dependent(kernel, dim3((unsigned)*n_part), dim3(T::THREADS), (size_t)even_smem(T::SMEM, *n_part, cost), st, M, N, K, A, W, bias, dA.p, dA.stride, top);
+    return launch_dependent(kernel, dim3((unsigned)*n_part), dim3(T::THREADS), (size_t)even_smem<kernel>(T::SMEM, T::THREADS, *n_part, even), st, M, N, K, A, W, bias, dA.p, dA.stride, top);
 }
 
 // Forms of a tile: outputs per lane, lanes, warps, steps per buffer, buffers.
@@ -231,11 +228,18 @@ struct Form {
     int bm, bn;
     float alone, shared, once;
     int unit, resident;
-    float cost(int M, int N, int K) const {
-        const int64_t tiles = ceil_div(M, bm) * ceil_div(N, bn), blocks = ceil_div(ceil_div(tiles, sm_count()), unit) * unit;
+    // (sms: on so many SMs)
+    float cost(int M, int N, int K, int sms) const {
+        const int64_t tiles = ceil_div(M, bm) * ceil_div(N, bn), blocks = ceil_div(ceil_div(tiles, sms), unit) * unit;
         const float step = (float)blocks * shared, rounds = resident ? (float)ceil_div(tiles, (int64_t)resident * sm_count()) : 1.f;
         return 1500.f + (once - 1500.f) * rounds + (float)K * (step > alone ? step : alone);
     }
+    // All blocks of a wave are placed within a microsecond, on the SMs that are free at that moment: 256 of them went to 75 SMs, four each,
+    // while the ID sort and the expiry scan had begun on the other 73 (4096 x 1632 x 256: 164 us instead of 97, step 265 us instead of
+    // 197; 1024 x 1632 x 256: 46 us and 32).  They are spread evenly where half of the SMs would take 8 us longer.  Elsewhere that
+    // costs more than it gives, since the sort then waits for room (128 blocks of 16 x 32 outputs, 1632 deep: step 59.5 us as it comes,
+    // 65.3 spread; of 8 x 64, 608 deep: 37.0, 39.3).
+    bool even(int M, int N, int K) const { return cost(M, N, K, (sm_count() + 1) / 2) - cost(M, N, K, sm_count()) >= 8000.f; }
 };
 constexpr Form LOW[] = {{16, 32, 10.2f, 6.f, 1300.f, 1, 0}, {32, 32, 15.7f, 8.f, 1500.f, 1, 0}, {64, 128, 50.5f, 46.5f, 2700.f, 1, 0},
                         {64, 64, 51.f, 24.5f, 3100.f, 2, 0}};
@@ -248,7 +252,7 @@ template <int COUNT> static int cheapest(const Form (&forms)[COUNT], int cols, i
     int best = -1;
     for (int f = 0; f < COUNT; ++f) {
         if (cols && (forms[f].bn < cols || forms[f].bn >= 2 * (cols > 32 ? cols : 32))) continue;
-        const float c = forms[f].cost(M, N, K);
+        const float c = forms[f].cost(M, N, K, sm_count());
         if (best < 0 || c < *cost) { best = f; *cost = c; }
     }
     return best;
@@ -272,8 +276,10 @@ cudaError_t launch_fwd_f32(const gear_ctx_impl& c, const char* name, int M, int 
     KernelScope ks(&c.prof, name, st);
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     float cost;
-#define GEAR_FWD(T, MB) (wvec ? launch_form<T, MB, true>(cost, M, N, K, A, W, bias, H, Hf, st) : launch_form<T, MB, false>(cost, M, N, K, A, W, bias, H, Hf, st))
-    switch (cheapest(LOW, 0, M, N, K, &cost)) {
+#define GEAR_FWD(T, MB) (wvec ? launch_form<T, MB, true>(even, M, N, K, A, W, bias, H, Hf, st) : launch_form<T, MB, false>(even, M, N, K, A, W, bias, H, Hf, st))
+    const int f = cheapest(LOW, 0, M, N, K, &cost);
+    const bool even = LOW[f].even(M, N, K);
+    switch (f) {
     case 0: return GEAR_FWD(F16x32, 4);
     case 1: return GEAR_FWD(F32x32, 4);
     case 2: return GEAR_FWD(F64x128, 3);
@@ -288,9 +294,11 @@ cudaError_t launch_fwd_top_f32(const gear_ctx_impl& c, int M, int N, int K, cons
     const bool wvec = (reinterpret_cast<uintptr_t>(W) & 15u) == 0;
     const int slots = c.ws.loss_slots;
     float cost;
-#define GEAR_TOP(T, MB) (wvec ? launch_top_form<T, MB, true>(cost, M, N, K, A, W, bias, dA, top, slots, n_part, st) \
-                              : launch_top_form<T, MB, false>(cost, M, N, K, A, W, bias, dA, top, slots, n_part, st))
-    switch (cheapest(TOP, N, M, N, K, &cost)) {
+#define GEAR_TOP(T, MB) (wvec ? launch_top_form<T, MB, true>(even, M, N, K, A, W, bias, dA, top, slots, n_part, st) \
+                              : launch_top_form<T, MB, false>(even, M, N, K, A, W, bias, dA, top, slots, n_part, st))
+    const int f = cheapest(TOP, N, M, N, K, &cost);
+    const bool even = TOP[f].even(M, N, K);
+    switch (f) {
     case 0: return GEAR_TOP(F16x32, 4);
     case 1: return GEAR_TOP(F32x32, 4);
     case 2: return GEAR_TOP(F8x64, 4);
