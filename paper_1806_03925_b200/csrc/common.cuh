@@ -187,11 +187,11 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // The next kernel in the stream may be set up beside this one from here on.  It still waits for this one to complete, and, since this
-// is called behind wait_for_predecessor(), for all before it.  For launches that leave half of the SMs to it: elsewhere, blocks
-// which only wait keep the kernels of other streams out.  Steps in fp32 with this line at 128 blocks / at 74 (us): 4096 views, 256 + 64
-// units 61.8 / 59.6, 256 + 200 units 80.4 / 76.2; 1024 views, 64 to 256 units 33.3 / 33.0; 256 views the same.  40 in its place: the same
-// but 512 units in bf16 at 300 views (30.6 / 29.2) and 1632 inputs at 256 views (43.8 / 45.8).
-constexpr unsigned FEW_BLOCKS = 74;
+// is called behind wait_for_predecessor(), for all before it.  For launches that leave a third of the SMs to it: elsewhere, blocks
+// which only wait keep the kernels of other streams out.  Steps in fp32 with this line at 128 blocks / at 98 / at 74 (us): 4096 views,
+// 256 + 64 units 61.8 / 59.6 / 59.6, 256 + 200 units 80.4 / 76.2 / 76.2; 1024 views, 64 to 256 units 33.3 / 33.0 / 33.0; 780 views,
+// 256 + 64 units 39.2 / 39.1 / 40.7, 128 + 128 units 37.1 / 35.4 / 36.1; 256 views no difference.
+constexpr unsigned FEW_BLOCKS = 98;
 __device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
