@@ -129,14 +129,16 @@ def kernel_models(p, stats):
     dsz = 2 if p.dfv_dtype == "bf16" else 4
     xsz = 2 if p.head_dtype == "bf16" else 4
     m = {}
+    fan = [Din] + list(p.hidden)
     m["gather_pool"] = ("hbm", B * 2 * E * 4 + nnz * D * dsz + B * Din * xsz + (3 * B + 1 + 2 * nnz) * 4 + B * 4)
+    if p.head_dtype == "bf16":      # the launch also makes the weights' copies (both orientations) and clears the head's gradient
+        m["gather_pool"] = ("hbm", m["gather_pool"][1] + sum(a * b for a, b in zip(fan, fan[1:])) * (4 + 2 * 2) + p.n_params * 4)
     # gradient rows: the B pooled-gradient rows are read (each once from HBM; repeats hit L2), one accumulator row
     # is read (if open) and written per distinct image, complete groups write one averaged row
     m["acc_reduce"] = ("hbm", B * D * 4 + nnz * 8 + stats["uniq_img"] * (D * 4 + 4) * 2 + stats["n_ready"] * (D * 4 + 4))
     m["expiry_mark"] = ("hbm", p.img_vocab * 8 + p.img_vocab // 8)
     m["emb_reduce"] = ("hbm", 2 * (B * E * 4 + B * 8 + stats["uniq_emb"] * E * 4 * 2))      # both tables, one launch
     m["collect_move"] = ("hbm", stats["n_ready"] * (D * 4 * 2 + 16))
-    fan = [Din] + list(p.hidden)
     L = len(p.hidden)
     m["head_out"] = ("hbm", B * fan[L] * xsz * 2 + B * 12)          # top activations in, their gradients out
     # the head's products: (flops, bytes) per launch.  Launches of one name share the step's products of that kind

@@ -272,8 +272,10 @@ static cudaError_t enqueue_step(gear_ctx_impl& c, const gear_batch& b, float lr,
     // multi-block sort they are put in by a launch of its own, so that the plan runs beside the gather instead of beside the
     // head's first products (65 k views: step 387 -> 381 us).  Small arrays are sorted and planned by one kernel behind the
     // gather: there the extra launch costs more than the earlier start gives (256 views +3.4 us, 1237 views fp32 34.0 / 34.3), unless
-    // the head is done sooner than such a sort would be, as bf16 ones are since their weights come with the gather (4096 views: 51.4
-    // behind it, 49.1 beside it; 3001 views: 47.7, 47.3).
+    // the head is done sooner than such a sort would be, as bf16 ones are since their weights come with the gather.  Steps of about 3
+    // images a view with the sort behind the gather / beside it (us).  Below the line: 500 views, 64 units 23.4 / 25.0, 256 + 128 33.0 / 34.9,
+    // 512 + 256 39.3 / 41.4.  Above it: 700 views 31.5 / 29.4, 33.9 / 34.8, 40.9 / 41.6; 1500 views 35.4 / 33.1, 37.1 / 36.4, 44.4 / 45.9;
+    // 4096 views, 256 + 128 51.4 / 49.1; 7000 views 58.9 / 52.7, 59.6 / 54.0, 69.9 / 73.8; 10000 views 63.8 / 56.6, 65.8 / 59.2, 94.8 / 94.4.
     const bool early = small_sort && with_gather && b.nnz > EARLY_SORT_FROM;
     if (early) {
         GEAR_TRY(launch_sort_small(c, batch, plan ? plan_args(c, b.nnz, nullptr, nullptr) : PlanArgs{}, side));

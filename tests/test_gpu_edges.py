@@ -206,7 +206,8 @@ def test_host_batch_arrives_as_it_is(fast):
         assert GearSession._c_batch(d).label == d.label.data_ptr()
 
 
-# tiles of 16 rows x 64 columns, 32 values deep, two steps ahead; rows that are no multiple of 16 bytes
+# tiles of 32 rows x 32 columns, up to three of the ring's four buffers of 32 values (deeper: test_dense_forward_of_unaligned_operands) or,
+# 129 values, five; rows that are no multiple of 16 bytes
 @pytest.mark.parametrize("n,R,D", [(1, 1, 8), (16, 32, 64), (17, 33, 72), (15, 64, 8), (40, 31, 136), (33, 96, 64), (2400, 129, 64)])
 def test_dense_forward_at_tile_edges(n, R, D):
     """Against fp64; R products of values in (-1, 1) added one by one in fp32 are off by at most R * 2^-24 * R."""
