@@ -22,7 +22,7 @@ constexpr int DK = 16;     // tile depth
 // A chain of R multiply-adds per output cannot be cut, so small tiles spread the live rows over the SMs (2500 rows of 1536
 // values, 64 columns: 40 blocks of 64 x 64 took 242 us), and blocks walk the tiles so that a capacity far above the live
 // count costs nothing.  32 x 32 tiles, 4 x 4 outputs per lane: bound by shared-memory reads (2 x 4 outputs in 16 x 64: 57 us for
-// those rows, this 29).  AVEC / BVEC: raw rows / Wd rows may be read 16 bytes at a time.
+// those rows, this 29, the same rows over and over; 38 in a loop pass, whose rows are other ones of a large table each time).  AVEC / BVEC: raw rows / Wd rows may be read 16 bytes at a time.
 typedef ChainTile<4, 4, 8, 4, 1, 2, 32, 4> DenseTile;
 template <bool AVEC, bool BVEC>
 __global__ void __launch_bounds__(DenseTile::THREADS)
